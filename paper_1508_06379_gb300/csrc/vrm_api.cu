@@ -115,6 +115,8 @@ struct vrm_ctx {
   int bs_src_cap = 0, bs_tgt_cap = 0;
   float4 *bs_src = nullptr, *bs_tgt = nullptr;
   float* bs_g = nullptr;
+  size_t bs_part_cap = 0;
+  float2* bs_part = nullptr;  // tile sums of the direct summation
   // particle removal (vrm_remove_close)
   int rm_cap = 0;
   uint8_t *rm_close = nullptr, *rm_removed = nullptr, *rm_keep = nullptr;
@@ -268,6 +270,9 @@ void free_bs(vrm_ctx* ctx) {
   if (ctx->bs_src) cudaFree(ctx->bs_src);
   if (ctx->bs_tgt) cudaFree(ctx->bs_tgt);
   if (ctx->bs_g) cudaFree(ctx->bs_g);
+  if (ctx->bs_part) cudaFree(ctx->bs_part);
+  ctx->bs_part = nullptr;
+  ctx->bs_part_cap = 0;
   ctx->bs_src = ctx->bs_tgt = nullptr;
   ctx->bs_g = nullptr;
   ctx->bs_src_cap = ctx->bs_tgt_cap = 0;
@@ -307,15 +312,20 @@ cudaError_t ensure_rm(vrm_ctx* ctx, int n, cudaStream_t st) {
   return cudaSuccess;
 }
 
+// Buffers of the direct summation of n sources at m targets (grown, never
+// shrunk; the tile sums' workspace is bounded by bs_part_count).
 cudaError_t ensure_bs(vrm_ctx* ctx, int n, int m, cudaStream_t st) {
-  if (n <= ctx->bs_src_cap && m <= ctx->bs_tgt_cap) return cudaSuccess;
+  const size_t want = bs_part_count(n, m);
+  if (n <= ctx->bs_src_cap && m <= ctx->bs_tgt_cap && want <= ctx->bs_part_cap) return cudaSuccess;
   cudaStreamSynchronize(st);
   const int ns = n > ctx->bs_src_cap ? n : ctx->bs_src_cap;
   const int mt = m > ctx->bs_tgt_cap ? m : ctx->bs_tgt_cap;
+  const size_t np = want > ctx->bs_part_cap ? want : ctx->bs_part_cap;
   free_bs(ctx);
   cudaError_t e = cudaMalloc(&ctx->bs_src, sizeof(float4) * (size_t)(ns > 0 ? ns : 1));
   if (e == cudaSuccess) e = cudaMalloc(&ctx->bs_g, sizeof(float) * (size_t)(ns > 0 ? ns : 1));
   if (e == cudaSuccess) e = cudaMalloc(&ctx->bs_tgt, sizeof(float4) * (size_t)(mt > 0 ? mt : 1));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->bs_part, sizeof(float2) * (np > 0 ? np : 1));
   if (e != cudaSuccess) {
     free_bs(ctx);
     cudaGetLastError();
@@ -323,6 +333,7 @@ cudaError_t ensure_bs(vrm_ctx* ctx, int n, int m, cudaStream_t st) {
   }
   ctx->bs_src_cap = ns;
   ctx->bs_tgt_cap = mt;
+  ctx->bs_part_cap = np;
   return cudaSuccess;
 }
 
@@ -1152,6 +1163,7 @@ vrm_status vrm_rk3_step(vrm_ctx* ctx, double* x, double* y, int32_t n, int32_t c
   if (s.h_grid->nonfinite || s.h_ds->nonfinite) return VRM_ERR_ARG;
   fill_front_stats(ctx, n, st);
   if (s.h_state->overflow) return VRM_ERR_CAPACITY;
+  const int n1 = s.h_state->n_cur;  // particles of every stage
   const int* n_cur = &s.st->n_cur;
   double* Xs[3] = {x, ctx->rk_x1, ctx->rk_x2};
   double* Ys[3] = {y, ctx->rk_y1, ctx->rk_y2};
@@ -1175,13 +1187,13 @@ vrm_status vrm_rk3_step(vrm_ctx* ctx, double* x, double* y, int32_t n, int32_t c
       // only the n given particles carry circulation (gamma_in holds n)
       if (k == 0) {
         VRM_CUDA(bs_split(px, py, gamma_in, n, nullptr, ctx->bs_src, ctx->bs_g, stream));
-        VRM_CUDA(bs_split(px, py, nullptr, capacity, n_cur, ctx->bs_tgt, nullptr, stream));
-        VRM_CUDA(bs_direct(ctx->bs_src, ctx->bs_g, n, nullptr, ctx->bs_tgt, capacity, n_cur, vel->eps, ctx->rk_u,
-                           ctx->rk_v, stream));
+        VRM_CUDA(bs_split(px, py, nullptr, n1, nullptr, ctx->bs_tgt, nullptr, stream));
+        VRM_CUDA(bs_direct(ctx->bs_src, ctx->bs_g, n, ctx->bs_tgt, n1, vel->eps, ctx->bs_part, ctx->rk_u, ctx->rk_v,
+                           stream));
       } else {
-        VRM_CUDA(bs_split(px, py, Gs[k], capacity, n_cur, ctx->bs_src, ctx->bs_g, stream));
-        VRM_CUDA(bs_direct(ctx->bs_src, ctx->bs_g, capacity, n_cur, ctx->bs_src, capacity, n_cur, vel->eps,
-                           ctx->rk_u, ctx->rk_v, stream));
+        VRM_CUDA(bs_split(px, py, Gs[k], n1, nullptr, ctx->bs_src, ctx->bs_g, stream));
+        VRM_CUDA(bs_direct(ctx->bs_src, ctx->bs_g, n1, ctx->bs_src, n1, vel->eps, ctx->bs_part, ctx->rk_u, ctx->rk_v,
+                           stream));
       }
       us = ctx->rk_u;
       vs = ctx->rk_v;
@@ -1230,7 +1242,7 @@ vrm_status vrm_biot_savart(vrm_ctx* ctx, const double* xs, const double* ys, con
   VRM_CUDA(ensure_bs(ctx, n, m, stream));
   VRM_CUDA(bs_split(xs, ys, gamma, n, nullptr, ctx->bs_src, ctx->bs_g, stream));
   VRM_CUDA(bs_split(xt, yt, nullptr, m, nullptr, ctx->bs_tgt, nullptr, stream));
-  VRM_CUDA(bs_direct(ctx->bs_src, ctx->bs_g, n, nullptr, ctx->bs_tgt, m, nullptr, eps, u, v, stream));
+  VRM_CUDA(bs_direct(ctx->bs_src, ctx->bs_g, n, ctx->bs_tgt, m, eps, ctx->bs_part, u, v, stream));
   return VRM_OK;
 }
 

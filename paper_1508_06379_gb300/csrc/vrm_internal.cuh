@@ -424,8 +424,10 @@ cudaError_t rk3_stage(int stage, int n_bound, const int* n_dev, double dt, doubl
 // Splits FP64 positions into fp32 hi/lo pairs (and circulations to fp32).
 cudaError_t bs_split(const double* x, const double* y, const double* g, int n_bound, const int* n_dev, float4* pos,
                      float* gf, cudaStream_t s);
-// u, v at the m targets from the n sources (counts on the device if given).
-cudaError_t bs_direct(const float4* src, const float* gs, int n_bound, const int* n_dev, const float4* tgt,
-                      int m_bound, const int* m_dev, double eps, double* u, double* v, cudaStream_t s);
+// u, v at the m targets from the n sources; part: workspace of
+// bs_part_count(n, m) tile sums.
+size_t bs_part_count(int n, int m);
+cudaError_t bs_direct(const float4* src, const float* gs, int n, const float4* tgt, int m, double eps, float2* part,
+                      double* u, double* v, cudaStream_t s);
 
 }  // namespace vrm
