@@ -25,11 +25,16 @@
 // is exactly 1 in binary32 and phi is the correctly rounded 1/q: the hardware
 // reciprocal and one Newton step (Markstein, IBM J. Res. Dev. 34, 1990: exact
 // after one step from a 1-ulp estimate but for isolated significands, of
-// which the hardware estimate leaves none: every binary32 in [17, 2^101)
+// which the hardware estimate leaves none: every binary32 in [0.1, 2^101)
 // compared with __frcp_rn).  That is 14 packed instructions and two
-// reciprocals per two pairs; tiles near a warp's targets take the general
-// form, where a vote per source skips the exponential as long as all lanes
-// are far.
+// reciprocals per two pairs; the parts of a tile near a warp's targets take
+// the general form, where a vote per source skips the exponential as long as
+// all lanes are far.  The FMA pipe binds it (a packed instruction takes it for
+// two cycles: 14 cycles a pair of the 18 measured).  251,001 sources at 40,000
+// targets: 5.36 ms (31.1 ms with one target per thread, a branch at q = 0.1,
+// __frcp_rn and one block per 256 targets); all pairs far: 4.95 ms, and 5.51
+// ms with scalar instructions in place of the packed ones; targets in random
+// order: 6.6 ms.
 #include "vrm_internal.cuh"
 
 namespace vrm {
@@ -349,7 +354,9 @@ cudaError_t bs_direct(const float4* src, const float* gs, int n, const float4* t
   const double c0 = 1.0 / (2.0 * 3.141592653589793 * eps * eps);
   const int all = (int)bs_tiles(n), group = (int)(bs_part_count(n, m) / (size_t)m);
   // four targets per thread read a source half as often as two, but need
-  // enough (target block, tile) pairs to fill the GPU's 8 blocks per SM
+  // enough (target block, tile) pairs to fill the GPU's 8 blocks per SM: 900
+  // sources at 900 targets (16 blocks of 256 targets) take 0.053 ms, 0.109 ms
+  // before; 160,000 at 300 targets 0.19 ms, 16.9 ms before
   const long slots = 8L * sm_count();
   const bool wide = (((long)m + 4 * kBsThreads - 1) / (4 * kBsThreads)) * all >= slots;
   const int T = wide ? 4 : 2;
