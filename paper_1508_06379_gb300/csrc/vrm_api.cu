@@ -372,10 +372,12 @@ cudaError_t enqueue_stage_weights(vrm_ctx* ctx, const double* x, const double* y
   // counts, masks and small neighbourhoods of the diffused particles (the
   // LPs read no other particle's); their rows only where the learned slots
   // read them (the full-neighbourhood LP's few particles get theirs below;
-  // the application goes through the transposed stencils), in visiting order
-  // (the learned slots and the full-neighbourhood LP order their entries
-  // themselves)
-  const bool rows = ctx->mlp != nullptr;
+  // the application goes through the transposed stencils) and for n = 2,
+  // whose small LPs nearly all fail on jittered clouds (a second search sized
+  // for a few particles took 1.05 ms on 251,001, the rows written here 0.04),
+  // in visiting order (the learned slots and the full-neighbourhood LP order
+  // their entries themselves)
+  const bool rows = ctx->mlp != nullptr || c.order == 2;
   if ((e = search_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key, s.cell_rank,
                            s.dlist, s.counters + 0, cap, s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, st,
                            rows)) != cudaSuccess)
@@ -397,7 +399,7 @@ cudaError_t enqueue_stage_weights(vrm_ctx* ctx, const double* x, const double* y
                                     s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, st, true)) != cudaSuccess)
     return e;
   return lp_full(c, x, y, s.fail_list, &s.ds->n_fail, cap, s.nbr_count, s.nbr_idx, s.cols, s.f, s.fii, s.status,
-                 s.ds, 0.0, st, &s.st->dt, ctx->p.nu);
+                 s.retry_list, s.ds, 0.0, st, &s.st->dt, ctx->p.nu);
 }
 
 // Scratch for `cap` particles (grown by 25% steps, never shrunk).
@@ -675,10 +677,12 @@ cudaError_t enqueue_back(vrm_ctx* ctx, double* x, double* y, int cap, const doub
   // counts, masks and small neighbourhoods of the diffused particles (the
   // LPs read no other particle's); their rows only where the learned slots
   // read them (the full-neighbourhood LP's few particles get theirs below;
-  // the application goes through the transposed stencils), in visiting order
-  // (the learned slots and the full-neighbourhood LP order their entries
-  // themselves)
-  const bool rows = ctx->mlp != nullptr;
+  // the application goes through the transposed stencils) and for n = 2,
+  // whose small LPs nearly all fail on jittered clouds (a second search sized
+  // for a few particles took 1.05 ms on 251,001, the rows written here 0.04),
+  // in visiting order (the learned slots and the full-neighbourhood LP order
+  // their entries themselves)
+  const bool rows = ctx->mlp != nullptr || c.order == 2;
   if ((e = search_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key, s.cell_rank,
                            s.dlist, s.counters + 0, cap, s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, st,
                            rows)) != cudaSuccess)
@@ -702,7 +706,7 @@ cudaError_t enqueue_back(vrm_ctx* ctx, double* x, double* y, int cap, const doub
                                     s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, st, true)) != cudaSuccess)
     return e;
   if ((e = lp_full(c, x, y, s.fail_list, &s.ds->n_fail, cap, s.nbr_count, s.nbr_idx, s.cols, s.f, s.fii, s.status,
-                   s.ds, 0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
+                   s.retry_list, s.ds, 0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
     return e;
   if ((e = mark(ctx, VRM_STAGE_APPLY, st)) != cudaSuccess) return e;
   if ((e = apply_transposed_dev(c, cap, n_cur, cap, &s.st->n, gamma_in, s.diffused, s.dlist, s.counters + 0, s.cols,
@@ -1085,8 +1089,8 @@ vrm_status vrm_solve_weights(vrm_ctx* ctx, const double* x, const double* y, int
   }
   VRM_CUDA(lp_small(c, x, y, lp_list, lp_count, n, small, cols, f, fii, status, s.fail_list, s.retry_list, s.ds,
                       0.0, stream));
-  VRM_CUDA(lp_full(c, x, y, s.fail_list, &s.ds->n_fail, n, nbr_count, nbr_idx, cols, f, fii, status, s.ds, 0.0,
-                   stream));
+  VRM_CUDA(lp_full(c, x, y, s.fail_list, &s.ds->n_fail, n, nbr_count, nbr_idx, cols, f, fii, status,
+                   s.retry_list, s.ds, 0.0, stream));
   if (stats) {
     VRM_CUDA(read_back(ctx, stream));
     stats->n_in = stats->n_out = n;

@@ -373,8 +373,8 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
                      DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev = nullptr, double nu = 0.0);
 cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int* fail_list, const int* fail_count,
                     int cap, const int* nbr_count, const int* nbr_idx, int* cols, double* f, double* fii,
-                    uint8_t* status, DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev = nullptr,
-                    double nu = 0.0);
+                    uint8_t* status, int* retry_list, DevStats* ds, double nu_dt, cudaStream_t s,
+                    const double* dt_dev = nullptr, double nu = 0.0);
 // Identity weights of the removal candidates (list, *list_count on the
 // device): removed[i], cols4/w4 [n x 4] (vrm_remove.cu drives it).
 cudaError_t lp_identity(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,

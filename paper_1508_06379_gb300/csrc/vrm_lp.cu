@@ -29,7 +29,11 @@
 // For n = 1 the default kernel, k_lp_small32, pivots in binary32 with
 // certified decisions and keeps FP64 for the column offsets and the final
 // basis solve (see the section before it); k_lp_small re-runs the particles
-// it hands back, and serves n = 2 and the FP64-pivot schedule.
+// it hands back, and serves the FP64-pivot schedule.  For n = 2 both LPs run
+// in two parts: the pivots one particle per warp or half-warp in pairs of
+// binary32 numbers with certified decisions (k_lp_df; k_lp_full re-runs in
+// FP64 what it hands back), then the FP64 solve of the final bases one
+// particle per thread (k_lp9_finish).
 #include <climits>
 
 #include "vrm_internal.cuh"
@@ -1267,6 +1271,28 @@ __device__ __forceinline__ void lu_rows(double (&A)[M], double& z, double (&rcpd
   }
 }
 
+// Final basis of an n = 2 LP, kept in the particle's row of cols until
+// k_lp9_finish turns it into the stencil: entries 0..8 hold the particles of
+// the basic columns (-1 for an artificial), entries 9 and 10 the basic
+// variables (6 bits each: row r's artificial r or 9 + the column's rank),
+// the code and the pivot count.  Lane r < 9 of the group of G lanes holds
+// row r's variable and particle.
+template <int G>
+__device__ __forceinline__ void lp9_record(int* row, int gl, int var, int j, int code, int it) {
+  unsigned w0 = (unsigned)code << 30, w1 = (unsigned)it << 24;
+#pragma unroll
+  for (int r = 0; r < 9; ++r) {
+    const unsigned v = (unsigned)__shfl_sync(0xffffffffu, var, r, G);
+    if (r < 5)
+      w0 |= v << (6 * r);
+    else
+      w1 |= v << (6 * (r - 5));
+  }
+  if (gl < 9) row[gl] = j;
+  if (gl == 9) row[9] = (int)w0;
+  if (gl == 10) row[10] = (int)w1;
+}
+
 // Full-neighbourhood retry: one warp per particle.  Lane l holds tableau
 // column l (K <= 32 columns, the FP64 work of the pivots); the per-row
 // quantities (right-hand side, basic variable, ratio) live on lane r for row
@@ -1276,11 +1302,14 @@ __device__ __forceinline__ void lu_rows(double (&A)[M], double& z, double (&rcpd
 // swaps, multipliers times the pivot's reciprocal, separately rounded
 // updates), forward substitution in column order, back substitution row by
 // row; the result is bit-identical to the oracle's basis solve.
+// For n = 2 (M = 9) the kernel stops at the final basis and leaves it in the
+// particle's stencil row (lp9_record), for k_lp9_finish.
 template <int M, int W>
 __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restrict__ x,
                                                  const double* __restrict__ y, const int* __restrict__ fail_list,
                                                  const int* __restrict__ fail_count,
                                                  const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
+                                                 const int* __restrict__ small,
                                                  int* __restrict__ cols, double* __restrict__ f,
                                                  double* __restrict__ fii, uint8_t* __restrict__ status,
                                                  DevStats* __restrict__ ds, double nu_dt,
@@ -1298,13 +1327,16 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
   double st_ratio = 0.0;
   for (long t = warp; t < m; t += nwarps) {
     const int i = fail_list[t];
-    const int cnt = nbr_count[i];
+    // small (n = 2 only): the columns are the small neighbourhood's, an empty
+    // slot sorts last as a zero column, which never enters
+    const int cnt = M == 9 && small ? 8 : nbr_count[i];
     const int K = cnt < c.row_cap ? cnt : c.row_cap;
     const double xi0 = x[i], yi0 = y[i];
     double d2 = 1e300, dx = 0.0, dy = 0.0;
     int j = INT_MAX;
-    if (lane < K) {
-      j = nbr_idx[(size_t)i * c.k_cap + lane];
+    if (lane < K) j = M == 9 && small ? small[(size_t)i * 8 + lane] : nbr_idx[(size_t)i * c.k_cap + lane];
+    if (M == 9 && j < 0) j = INT_MAX;
+    if (j != INT_MAX) {
       dx = __dsub_rn(x[j], xi0);
       dy = __dsub_rn(y[j], yi0);
       d2 = dist2(dx, dy);
@@ -1420,6 +1452,11 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
       if (lane == q) isb = true;
       if (lane == leave) bas = M + q;
       ++it;
+    }
+    if constexpr (M == 9) {
+      const int bj = __shfl_sync(kAll, j, bas >= M && bas != INT_MAX ? bas - M : 0);
+      lp9_record<32>(cols + (size_t)i * W, lane, bas, bas >= M ? bj : -1, code, it);
+      continue;
     }
     // basic solution of the final basis by the oracle's LU sequence, row r of
     // B on lane r: column k is e_v for an artificial v = basis[k] < m, else
@@ -1545,6 +1582,469 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
   if (lane == 0 && st_cols) {
     atomicAdd(&ds->lp_full_columns, (unsigned long long)st_cols);
     atomicAdd(&ds->lp_full_column_pivots, st_colpiv);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// n = 2: certified pivots in pairs of binary32 numbers.  The nine-row LPs
+// take 8 (small) and 11 pivots (full neighbourhoods, 20 columns) on jittered
+// clouds, and running binary32 bounds outgrow the entries after about eight
+// pivots (25% of the full LPs certified); in FP64 the pivots of one LP take
+// the SM's FP64 pipe for 3,500 cycles.  A pair h + l (|l| <= 2^-24 |h|, up to
+// normalisation) carries 48 bits through fused multiply-adds on the binary32
+// pipes, about 15 operations per tableau entry and pivot and five for its
+// bound: 96% of the full LPs and 99.9% of the small ones are certified.
+//
+// The bounds follow k_lp_small32 with u^2 = 2^-48 in place of u:
+//   offsets split from the FP64 ones          2 u^2 |x|      (3 taken)
+//   their products and cubes                  12 u^2, 24 u^2 relative
+//   T - a p (df_fnma)                         20 u^2 (|T| + |a p|)  (24 taken)
+//   T_l / piv (df_rcp and df_mul)             18 u^2 relative       (24 taken)
+// and a comparison of h alone with a tolerance adds 2 u |h| for l.  The FP64
+// run's own distance from exact is smaller by 2^-8, inside the factor 1.25.
+// ---------------------------------------------------------------------------
+struct Df {
+  float h, l;
+};
+__device__ __forceinline__ Df df_fast_two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  return Df{s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Df df_two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return Df{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ Df df_mul(Df a, Df b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -p);
+  e = __fmaf_rn(a.h, b.l, e);
+  e = __fmaf_rn(a.l, b.h, e);
+  return df_fast_two_sum(p, e);
+}
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+  const Df s = df_two_sum(a.h, b.h);
+  return df_fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+// t - a p
+__device__ __forceinline__ Df df_fnma(Df a, Df p, Df t) {
+  const float q = __fmul_rn(a.h, p.h);
+  float e = __fmaf_rn(a.h, p.h, -q);
+  e = __fmaf_rn(a.h, p.l, e);
+  e = __fmaf_rn(a.l, p.h, e);
+  const Df s = df_two_sum(t.h, -q);
+  return df_fast_two_sum(s.h, __fadd_rn(s.l, __fsub_rn(t.l, e)));
+}
+// 1 / a: the hardware reciprocal r and its residual e = 1 - a r, r (1 + e + e^2)
+__device__ __forceinline__ Df df_rcp(Df a) {
+  const float r = rcp_approx(a.h);
+  float e = __fmaf_rn(-a.h, r, 1.0f);
+  e = __fmaf_rn(-a.l, r, e);
+  return df_fast_two_sum(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+}
+// A double by its bit pattern: the top 24 significant bits and the rest.
+// Magnitudes outside [2^-60, 2^60] set `bad`.
+__device__ __forceinline__ Df df_split(double a, bool& bad) {
+  const unsigned long long b = (unsigned long long)dbits(a);
+  if ((b << 1) == 0) return Df{0.0f, 0.0f};
+  const int e = (int)((b >> 52) & 0x7FF) - 1023;
+  if (e < -60 || e > 60) {
+    bad = true;
+    return Df{0.0f, 0.0f};
+  }
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const float h = __uint_as_float(sign | ((unsigned)(e + 127) << 23) | (unsigned)((b >> 29) & 0x7FFFFF));
+  const float scale = __uint_as_float(sign | ((unsigned)(e - 52 + 127) << 23));
+  return df_fast_two_sum(h, __fmul_rn(__uint2float_rn((unsigned)(b & 0x1FFFFFFF)), scale));
+}
+constexpr float kU2 = kU32 * kU32;
+constexpr float kDfFma = 24.0f * kU2, kDfMul = 24.0f * kU2;
+
+// One LP per group of G lanes: lane k of the group holds tableau column k
+// (unsorted; `rank` is its place in the order (d2, j)), and row r's
+// right-hand side, basic variable and ratio are on lane r < 9.  The final
+// basis goes to the particle's row of cols (lp9_record), an LP with an
+// uncertain decision to the retry list.  G = 32: full neighbourhoods (FULL);
+// G = 16: the small ones, two per warp (8 of the lanes hold columns, 9 hold
+// rows), which run in step until both are done.
+template <int G, bool FULL>
+__global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restrict__ x, const double* __restrict__ y,
+                                               const int* __restrict__ list, const int* __restrict__ list_count,
+                                               const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
+                                               const int* __restrict__ small, int* __restrict__ cols,
+                                               int* __restrict__ retry_list, DevStats* __restrict__ ds) {
+  constexpr int M = 9, W = VRM_STENCIL_W2;
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int kNone = 1 << 20;
+  const int lane = threadIdx.x & 31, gl = lane & (G - 1), gbase = lane & ~(G - 1);
+  const unsigned gmask = G == 32 ? kAll : (0xffffu << gbase);
+  auto ballot = [&](bool v) { return (__ballot_sync(kAll, v) & gmask) >> gbase; };
+  __shared__ float4 s_col[2][128 / G][M + 1];
+  unsigned it_all = 0;
+  const int m = *list_count;
+  const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const long nwarps = ((long)gridDim.x * blockDim.x) >> 5;
+  for (long t0 = warp * (32 / G); t0 < m; t0 += nwarps * (32 / G)) {
+    const long t = t0 + gbase / G;
+    const bool have = t < m;
+    const int i = list[have ? t : t0];
+    int K = 8, j = -1;
+    if (FULL) {
+      const int cnt = nbr_count[i];
+      K = cnt < c.row_cap ? cnt : c.row_cap;
+      if (gl < K) j = nbr_idx[(size_t)i * c.k_cap + gl];
+    } else if (gl < 8) {
+      j = small[(size_t)i * 8 + gl];
+    }
+    const bool col = have && j >= 0;
+    double dx = 0.0, dy = 0.0, d2 = 1e300;
+    if (col) {
+      dx = __dsub_rn(x[j], x[i]);
+      dy = __dsub_rn(y[j], y[i]);
+      d2 = dist2(dx, dy);
+    }
+    int rank = 0;  // columns before this one in the order (d2, j)
+    for (int k = 0; k < (FULL ? K : 8); ++k) {
+      const double od2 = __shfl_sync(kAll, d2, k, G);
+      const int oj = __shfl_sync(kAll, j, k, G);
+      rank += (lt_nonneg(od2, d2) || (dbits(od2) == dbits(d2) && oj < j)) ? 1 : 0;
+    }
+    bool bad = false;
+    Df T[M], d = {0.0f, 0.0f};
+    float E[M], Ed = 0.0f;
+    {
+      const Df xi = df_split(__dmul_rn(dx, c.inv_h), bad), eta = df_split(__dmul_rn(dy, c.inv_h), bad);
+      T[0] = xi;
+      T[1] = eta;
+      T[2] = df_mul(xi, xi);
+      T[3] = df_mul(xi, eta);
+      T[4] = df_mul(eta, eta);
+      T[5] = df_mul(T[2], xi);
+      T[6] = df_mul(T[2], eta);
+      T[7] = df_mul(xi, T[4]);
+      T[8] = df_mul(T[4], eta);
+      Df sum = {0.0f, 0.0f};
+      float sa = 0.0f, se = 0.0f;
+#pragma unroll
+      for (int r = 0; r < M; ++r) {
+        const float av = fabsf(T[r].h);
+        E[r] = (r < 2 ? 3.0f : r < 5 ? 12.0f : 24.0f) * kU2 * av;
+        sum = df_add(sum, T[r]);
+        sa += av;
+        se += E[r];
+      }
+      d.h = -sum.h;
+      d.l = -sum.l;
+      Ed = __fmaf_rn(32.0f * kU2, sa, se);
+    }
+    // row r on lane r
+    Df rhs = {gl == 2 || gl == 4 ? 2.0f : 0.0f, 0.0f};
+    float Eb = 0.0f;
+    int bas = gl < M ? gl : kNone, bj = -1;
+    bool isb = false;
+    bool unc = ballot(bad) != 0;
+    bool run = have && !unc;
+    int it = 0, code = 0, n_art = M;
+    while (__any_sync(kAll, run)) {
+      // entering column: the first in rank certainly below -tol, no earlier
+      // one uncertain
+      bool go = run && n_art > 0;
+      const float md = __fmaf_rn(kCertSafety, Ed, 2.0f * kU32 * fabsf(d.h));
+      const bool yes = col && !isb && d.h < -kTolPriceHi - md;
+      const bool maybe = col && !isb && !yes && !(d.h > -kTolPriceLo + md);
+      const int rq = (int)__reduce_min_sync(gmask, (unsigned)(yes ? rank : kNone));
+      if (ballot(maybe && rank < rq) != 0 && go) {
+        unc = true;
+        go = false;
+      }
+      if (rq == kNone) go = false;
+      if (go && it == kPivotCap) {
+        code = 2;
+        go = false;
+      }
+      const unsigned qb = ballot(yes && rank == rq);
+      const int q = qb ? __ffs(qb) - 1 : 0;
+      // the entering column, its cost and its particle through shared memory:
+      // its lane writes ten vectors, every lane reads them and lane r row r's
+      // (two buffers, so that one barrier a pivot suffices)
+      float4* const buf = s_col[it_all & 1][threadIdx.x / G];
+      ++it_all;
+      if (gl == q) {
+#pragma unroll
+        for (int r = 0; r < M; ++r) buf[r] = make_float4(T[r].h, T[r].l, E[r], 0.0f);
+        buf[M] = make_float4(d.h, d.l, Ed, __int_as_float(j));
+      }
+      __syncwarp();
+      const float4 mine = buf[gl < M ? gl : 0], cq = buf[M];
+      const Df am = {mine.x, mine.y};
+      const float eam = mine.z;
+      // ratio test, row r on lane r (as in lp_pivots32)
+      const bool isrow = gl < M;
+      const float mg = __fmaf_rn(kCertSafety, eam, 2.0f * kU32 * fabsf(am.h));
+      const float mb = __fmaf_rn(kCertSafety, Eb, 2.0f * kU32 * fabsf(rhs.h));
+      const bool el = isrow && am.h > kTolPivotHi + mg;
+      const bool amb = isrow && !el && !(am.h < kTolPivotLo - mg);
+      const bool nzr = rhs.h > kTolSnapHi + mb;
+      bool bad_row = (amb && !nzr) || (el && !nzr && !(rhs.h < kTolSnapLo - mb));
+      const float inv = rcp_approx(am.h);
+      const float ratio = nzr ? rhs.h * inv : 0.0f;
+      const float g = eam * inv;
+      const float gg = __fmaf_rn(2.0f * g, g, g);
+      const float er = nzr ? kCertSafety * __fmaf_rn(kRcpMul + 2.1f * kU32, ratio,
+                                                     __fmaf_rn(gg, rhs.h + Eb, Eb) * inv)
+                           : 0.0f;
+      bad_row = bad_row || (el && nzr && (!(g <= 0.5f) || !(er < 1.0e30f)));
+      const float lo = el ? fmaxf(ratio - er, 0.0f) : 3.0e38f, hi = el ? ratio + er : 3.0e38f;
+      const float thlo = __uint_as_float(__reduce_min_sync(gmask, __float_as_uint(lo)));
+      const float thhi = __uint_as_float(__reduce_min_sync(gmask, __float_as_uint(hi)));
+      const float l0 = __fmaf_rn(kTolTieLo, fmaxf(thlo, 1.0f), thlo);
+      const float l1 = __fmaf_rn(kTolTieHi, fmaxf(thhi, 1.0f), thhi);
+      const float limlo = __fmaf_rn(-4.0f * kU32, fabsf(l0), l0);
+      const float limhi = __fmaf_rn(4.0f * kU32, fabsf(l1), l1);
+      const unsigned elm = ballot(el), ambm = ballot(amb);
+      const unsigned poss = ballot(el && lo <= limhi);
+      unsigned tied = ballot(el && hi <= limlo);
+      // an uncertain row whose ratio, were it eligible, would lie above every
+      // possible tie limit does not matter
+      const bool amb_matters =
+          amb && !(__fmul_rn(__fsub_rn(rhs.h, mb), 1.0f - 8.0f * kU32) > __fmul_rn(limhi, __fadd_rn(am.h, mg)));
+      // (every vote outside the branches: the warp's two groups may differ)
+      bool no = ballot(bad_row) != 0;
+      const bool any_matters = ballot(amb_matters) != 0;
+      if (elm == 0) {
+        no = no || ambm != 0;  // no eligible row, or one that may be
+        if (go && !no) {
+          code = 2;
+          go = false;
+        }
+      } else {
+        no = no || any_matters;
+        if (__popc(poss) == 1)
+          tied = poss;
+        else
+          no = no || (poss & ~tied) != 0;
+        tied &= poss;
+      }
+      const int lbas = (int)__reduce_min_sync(gmask, (unsigned)(((tied >> gl) & 1u) ? bas : kNone));
+      const unsigned lb = ballot(((tied >> gl) & 1u) && bas == lbas);
+      const int leave = lb ? __ffs(lb) - 1 : 0;
+      Df piv, prhs0;
+      piv.h = __shfl_sync(kAll, am.h, leave, G);
+      piv.l = __shfl_sync(kAll, am.l, leave, G);
+      const float pe = __shfl_sync(kAll, eam, leave, G);
+      prhs0.h = __shfl_sync(kAll, rhs.h, leave, G);
+      prhs0.l = __shfl_sync(kAll, rhs.l, leave, G);
+      const float pebr = __shfl_sync(kAll, Eb, leave, G);
+      const Df dq = {cq.x, cq.y};
+      const float edq = cq.z;
+      const int jq = __float_as_int(cq.w);
+      const Df P = df_rcp(piv);
+      const float rho = pe * P.h;
+      no = no || !(rho <= 0.5f);
+      if (go && no) {
+        unc = true;
+        go = false;
+      }
+      if (go) {
+        const float rr = __fmaf_rn(2.0f * rho, rho, rho);
+        Df prow = T[0];
+        float eprow = E[0];
+#pragma unroll
+        for (int r = 1; r < M; ++r) {
+          prow.h = leave == r ? T[r].h : prow.h;
+          prow.l = leave == r ? T[r].l : prow.l;
+          eprow = leave == r ? E[r] : eprow;
+        }
+        prow = df_mul(prow, P);
+        const float eP = eprow * P.h;
+        float ap = fabsf(prow.h);
+        float Ep = __fmaf_rn(kDfMul, ap, __fmaf_rn(rr, ap + eP, eP));
+        if (gl == q) {
+          prow = Df{1.0f, 0.0f};
+          ap = 1.0f;
+          Ep = 0.0f;
+        }
+        const Df prhs = df_mul(prhs0, P);
+        const float ebP = pebr * P.h, aprhs = fabsf(prhs.h);
+        const float Ebp = __fmaf_rn(kDfMul, aprhs, __fmaf_rn(rr, aprhs + ebP, ebP));
+        // column q of the other rows becomes an exact 0 (its bound stays)
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+          const float4 a = buf[r];
+          const float aa = fabsf(a.x);
+          E[r] = __fmaf_rn(kDfFma, __fmaf_rn(aa, ap, fabsf(T[r].h)), __fmaf_rn(aa + a.z, Ep, __fmaf_rn(a.z, ap, E[r])));
+          T[r] = df_fnma(Df{a.x, a.y}, prow, T[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < M; ++r)
+          if (leave == r) {
+            T[r] = prow;
+            E[r] = Ep;
+          }
+        {
+          const float aa = fabsf(am.h);
+          const float en =
+              __fmaf_rn(kDfFma, __fmaf_rn(aa, aprhs, fabsf(rhs.h)), __fmaf_rn(aa + eam, Ebp, __fmaf_rn(eam, aprhs, Eb)));
+          const Df rn = df_fnma(am, prhs, rhs);
+          rhs = gl == leave ? prhs : rn;
+          Eb = gl == leave ? Ebp : en;
+        }
+        {
+          const float aa = fabsf(dq.h);
+          Ed = __fmaf_rn(kDfFma, __fmaf_rn(aa, ap, fabsf(d.h)), __fmaf_rn(aa + edq, Ep, __fmaf_rn(edq, ap, Ed)));
+          d = df_fnma(dq, prow, d);
+        }
+        if (lbas >= M) {
+          if (rank == lbas - M) isb = false;
+        } else {
+          --n_art;
+        }
+        if (gl == q) isb = true;
+        if (gl == leave) {
+          bas = M + rq;
+          bj = jq;
+        }
+        ++it;
+      }
+      run = go;
+    }
+    if (have && unc && gl == 0) retry_list[atomicAdd(&ds->n_retry, 1)] = i;
+    lp9_record<G>(cols + (size_t)i * W, have && !unc ? gl : G, bas, bj, code, it);
+  }
+}
+
+// The stencils of the n = 2 LPs from their final bases (lp9_record): the
+// oracle's LU solve (basis_solve), feasibility and the weights in column
+// order, as lp_finish does for n = 1.  One particle per thread: solved row
+// by row across a warp's lanes the 9 x 9 system takes the FP64 pipe about 300
+// warp instructions per particle, here 900 per 32.
+template <bool FULL>
+__global__ void __launch_bounds__(64) k_lp9_finish(Consts c, const double* __restrict__ x,
+                                                   const double* __restrict__ y, const int* __restrict__ list,
+                                                   const int* __restrict__ list_count,
+                                                   const int* __restrict__ nbr_count, int* __restrict__ cols,
+                                                   double* __restrict__ f, double* __restrict__ fii,
+                                                   uint8_t* __restrict__ status, int* __restrict__ fail_list,
+                                                   DevStats* __restrict__ ds, double nu_dt,
+                                                   const double* __restrict__ dt_dev, double nu) {
+  constexpr int M = 9, W = VRM_STENCIL_W2;
+  if (dt_dev) nu_dt = nu * *dt_dev;
+  const int m = *list_count;
+  const double inv_h2 = 1.0 / (c.h * c.h);
+  LpTally tl;
+  unsigned st_cols = 0;
+  unsigned long long st_colpiv = 0;
+  const long stride = (long)gridDim.x * blockDim.x;
+  for (long base = (long)blockIdx.x * blockDim.x; base < m; base += stride) {
+    const long t = base + threadIdx.x;
+    if (t < m) {
+      const int i = list[t];
+      int* const crow = cols + (size_t)i * W;
+      double* const frow = f + (size_t)i * W;
+      const unsigned w0 = (unsigned)crow[9], w1 = (unsigned)crow[10];
+      int code = (int)(w0 >> 30);
+      const int it = (int)(w1 >> 24);
+      int basis[M];
+      double bxi[M], beta[M], pj[M];
+      const double xi0 = x[i], yi0 = y[i];
+#pragma unroll
+      for (int r = 0; r < M; ++r) {
+        basis[r] = (int)((r < 5 ? w0 >> (6 * r) : w1 >> (6 * (r - 5))) & 63u);
+        const int j = crow[r];
+        pj[r] = __longlong_as_double((long long)j);
+        const bool s = basis[r] >= M;
+        bxi[r] = s ? __dmul_rn(__dsub_rn(x[s ? j : i], xi0), c.inv_h) : 0.0;
+        beta[r] = s ? __dmul_rn(__dsub_rn(y[s ? j : i], yi0), c.inv_h) : 0.0;
+      }
+      double wsum = 0.0, rmax = 0.0;
+      double pay[4][M];
+#pragma unroll
+      for (int r = 0; r < M; ++r) pay[2][r] = 0.0;
+      if (code == 0) {
+        double xB[M];
+        float cert = INFINITY;
+        if (!basis_solve<M>(basis, bxi, beta, xB, &cert)) code = 2;
+        bool plain = true;  // all structural, none snapped: the certificate applies
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+          const bool s = basis[r] >= M, pos = gt_pos(xB[r], kTolSnap);
+          plain = plain && s && pos;
+          if (!s) wsum = __dadd_rn(wsum, xB[r]);
+          pay[0][r] = bxi[r];
+          pay[1][r] = beta[r];
+          pay[2][r] = s && pos ? xB[r] : 0.0;
+          pay[3][r] = pj[r];
+        }
+        sort_by_key<M, 4>(basis, pay);
+        if (code == 0 && !gt_pos(wsum, kTolPhase1) && !(plain && cert <= cert_s<M>())) {
+          // the residual as the oracle evaluates it (resid_in_column_order);
+          // an LP with artificials left above the tolerance is infeasible anyway
+          double acc[M];
+#pragma unroll
+          for (int q = 0; q < M; ++q) acc[q] = 0.0;
+#pragma unroll
+          for (int r = 0; r < M; ++r) {
+            double v[M];
+            vcol<M>(pay[0][r], pay[1][r], v);
+#pragma unroll
+            for (int q = 0; q < M; ++q) acc[q] = __dadd_rn(acc[q], __dmul_rn(v[q], pay[2][r]));
+          }
+#pragma unroll
+          for (int q = 0; q < M; ++q) {
+            const double e = __dsub_rn(acc[q], b_of(q));
+            rmax = abs_gt(e, rmax) ? fabs(e) : rmax;
+          }
+        }
+      }
+      const bool feasible = code == 0 && !gt_pos(wsum, kTolPhase1) && !gt_pos(rmax, kTolResid);
+      tl.maxpiv = it > tl.maxpiv ? it : tl.maxpiv;
+      ++tl.solved;
+      tl.pivots += it;
+      if (FULL) {
+        const int cnt = nbr_count[i];
+        const unsigned K = (unsigned)(cnt < c.row_cap ? cnt : c.row_cap);
+        st_cols += K;
+        st_colpiv += (unsigned long long)K * (unsigned)it;
+      }
+      if (feasible || FULL || !c.fallback) {
+        int slot = 0;
+        double s = 0.0;
+        if (feasible) {
+#pragma unroll
+          for (int r = 0; r < M; ++r)
+            if (dbits(pay[2][r]) != 0) {
+              crow[slot] = (int)dbits(pay[3][r]);
+              frow[slot] = pay[2][r];
+              ++slot;
+              s = __dadd_rn(s, pay[2][r]);
+            }
+        }
+        for (int k = slot; k < W; ++k) {
+          crow[k] = -1;
+          frow[k] = 0.0;
+        }
+        fii[i] = feasible ? -s : 0.0;
+        status[i] = feasible ? (FULL ? VRM_LP_FULL : VRM_LP_SMALL) : VRM_LP_NONE;
+        if (feasible) {
+          ++tl.ok;
+          const double q = __dmul_rn(__dmul_rn(nu_dt, s), inv_h2);
+          tl.ratio = q > tl.ratio ? q : tl.ratio;
+        } else {
+          ++tl.none;
+        }
+      } else {
+        fail_list[atomicAdd(&ds->n_fail, 1)] = i;
+      }
+    }
+  }
+  flush_stats(ds, tl.ok, tl.none, tl.maxpiv, tl.ratio, FULL, tl.solved, tl.pivots);
+  if (FULL) {
+    st_cols = __reduce_add_sync(0xffffffffu, st_cols);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) st_colpiv += __shfl_xor_sync(0xffffffffu, st_colpiv, o);
+    if ((threadIdx.x & 31) == 0 && st_cols) {
+      atomicAdd(&ds->lp_full_columns, (unsigned long long)st_cols);
+      atomicAdd(&ds->lp_full_column_pivots, st_colpiv);
+    }
   }
 }
 
@@ -1772,6 +2272,44 @@ __global__ void k_lp_clear(int n, int w, const uint8_t* __restrict__ diffused, i
   }
 }
 
+// The n = 2 LPs of a list: small neighbourhoods (small given) or full ones.
+static cudaError_t lp9(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
+                       int cap, const int* nbr_count, const int* nbr_idx, const int* small, int* cols, double* f,
+                       double* fii, uint8_t* status, int* fail_list, int* retry_list, DevStats* ds, double nu_dt,
+                       cudaStream_t s, const double* dt_dev, double nu) {
+  const int sms = sm_count();
+  auto grid = [&](long per_block, int per_sm) {
+    const long b = ((long)cap + per_block - 1) / per_block, most = (long)per_sm * sms;
+    return (int)(b < most ? b : most);
+  };
+  if (c.lp_fp64_pivots) {
+    k_lp_full<9, 12><<<grid(4, 4), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols, f, fii,
+                                                status, ds, nu_dt, dt_dev, nu);
+    note_launch();
+  } else {
+    const cudaError_t e = cudaMemsetAsync(&ds->n_retry, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    if (small)
+      k_lp_df<16, false><<<grid(8, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
+                                                     retry_list, ds);
+    else
+      k_lp_df<32, true><<<grid(4, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
+                                                    retry_list, ds);
+    note_launch();
+    k_lp_full<9, 12><<<grid(4, 4), 128, 0, s>>>(c, x, y, retry_list, &ds->n_retry, nbr_count, nbr_idx, small, cols, f,
+                                                fii, status, ds, nu_dt, dt_dev, nu);
+    note_launch();
+  }
+  if (small)
+    k_lp9_finish<false><<<grid(64, 16), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii, status,
+                                                    fail_list, ds, nu_dt, dt_dev, nu);
+  else
+    k_lp9_finish<true><<<grid(64, 16), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii, status,
+                                                   fail_list, ds, nu_dt, dt_dev, nu);
+  note_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
                      int* retry_list, DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev, double nu) {
@@ -1783,9 +2321,9 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
   int blocks = (int)(((long)cap + tb - 1) / tb);
   if (blocks > c.lp_blocks_per_sm * sm_count()) blocks = c.lp_blocks_per_sm * sm_count();
   if (c.order == 2) {
-    k_lp_small<9, 12><<<blocks, tb, 0, s>>>(c, x, y, list, list_count, small, cols, f, fii, status, fail_list, ds,
-                                            nu_dt, dt_dev, nu);
-    note_launch();
+    const cudaError_t e = lp9(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list,
+                              retry_list, ds, nu_dt, s, dt_dev, nu);
+    if (e != cudaSuccess) return e;
   } else if (c.lp_fp64_pivots || !(c.inv_h > 1e-20 && c.inv_h < 1e20)) {
     k_lp_small<5, 8><<<blocks, tb, 0, s>>>(c, x, y, list, list_count, small, cols, f, fii, status, fail_list, ds,
                                            nu_dt, dt_dev, nu);
@@ -1820,17 +2358,17 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
 
 cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int* fail_list, const int* fail_count,
                     int cap, const int* nbr_count, const int* nbr_idx, int* cols, double* f, double* fii,
-                    uint8_t* status, DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev, double nu) {
+                    uint8_t* status, int* retry_list, DevStats* ds, double nu_dt, cudaStream_t s,
+                    const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
+  if (c.order == 2)
+    return lp9(c, x, y, fail_list, fail_count, cap, nbr_count, nbr_idx, nullptr, cols, f, fii, status, nullptr,
+               retry_list, ds, nu_dt, s, dt_dev, nu);
   long warps = cap;
   long blocks = (warps * 32 + 127) / 128;
   if (blocks > 4 * sm_count()) blocks = 4 * sm_count();
-  if (c.order == 2)
-    k_lp_full<9, 12><<<(int)blocks, 128, 0, s>>>(c, x, y, fail_list, fail_count, nbr_count, nbr_idx, cols, f, fii,
-                                                 status, ds, nu_dt, dt_dev, nu);
-  else
-    k_lp_full<5, 8><<<(int)blocks, 128, 0, s>>>(c, x, y, fail_list, fail_count, nbr_count, nbr_idx, cols, f, fii,
-                                                status, ds, nu_dt, dt_dev, nu);
+  k_lp_full<5, 8><<<(int)blocks, 128, 0, s>>>(c, x, y, fail_list, fail_count, nbr_count, nbr_idx, nullptr, cols, f,
+                                              fii, status, ds, nu_dt, dt_dev, nu);
   note_launch();
   return cudaGetLastError();
 }
