@@ -1594,6 +1594,11 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
 // normalisation) carries 48 bits through fused multiply-adds on the binary32
 // pipes, about 15 operations per tableau entry and pivot and five for its
 // bound: 96% of the full LPs and 99.9% of the small ones are certified.
+// Bound by issue (66% of the slots, the integer pipe half busy with selects
+// and votes).  175,000 LPs of 251,001 particles: full 1.71 ms + 0.27 ms of
+// FP64 re-runs + 0.42 ms of final solves, 7.87 ms when a warp did pivots and
+// solve in FP64; small 0.78 + 0.03 + 0.41 ms, 1.15 ms with one FP64 LP per
+// thread (9 x 8 tableau, spilled).
 //
 // The bounds follow k_lp_small32 with u^2 = 2^-48 in place of u:
 //   offsets split from the FP64 ones          2 u^2 |x|      (3 taken)

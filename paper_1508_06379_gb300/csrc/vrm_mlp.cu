@@ -8,15 +8,20 @@
 // GEMMs read bf16 copies (W1 padded to 256x128) and, for the backward pass,
 // transposed bf16 copies.
 //
-// Every product is one kernel, k_gemm<NT>: C[M x N] = A[M x K] B[N x K]^T with
-// A and B K-major bf16 in global memory.  A CTA of 4 warps owns a 128-row
-// tile of C and NT columns: thread 0 streams 64-column slabs of A and B into
-// a 4-stage shared-memory ring with TMA and issues the MMAs (M = 128, N = NT,
-// K = 16) into a TMEM accumulator; all four warps then read the accumulator
-// (one TMEM lane = one row per thread) and run the fused epilogue (bias,
-// GELU, GELU derivative, bf16 rounding, transposed copies for the next
-// product).  Weight gradients split K (the batch) across CTAs and sum the
-// partials in a fixed order, so training is deterministic.
+// Inference is one kernel (k_mlp_fused), a training step four:
+//   k_gather     the batch's rows, their transposes and the mask sums
+//   k_chain      per 128-row tile the forward pass, the loss gradient and the
+//                backward pass down to the first layer, with the tile's
+//                activations in shared memory
+//   k_weight_grad  the weight gradients of every layer, split over the batch
+//   k_update     the splits and the biases summed in a fixed order (training is
+//                deterministic), AdamW, and the bf16 copies of the weights
+// A batch of 4096 rows takes 95 us (540 us with a kernel per product, whose 32
+// CTAs stored row by row, a one-block loss and separate sums: 23 launches),
+// 512 rows 81 us (366), 16,384 rows 134 us (1123).
+// The products are tcgen05 MMAs (M = 128, K = 16) on K-major bf16 tiles that
+// TMA or the epilogues leave in shared memory in the 128-byte swizzle, with
+// fp32 accumulators in TMEM.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -40,7 +45,6 @@ constexpr int kOut = 32;
 constexpr int kOutPad = 64;   // dY row stride (one K slab)
 constexpr int kBM = 128;      // rows per tile
 constexpr int kBK = 64;       // K per slab
-constexpr int kStages = 4;
 constexpr long long kWaitCycles = 2000000000LL;  // about one second
 
 constexpr long kOffW1 = 0, kOffB1 = kOffW1 + (long)kHid * kIn;
@@ -49,28 +53,6 @@ constexpr long kOffW3 = kOffB2 + kHid, kOffB3 = kOffW3 + (long)kHid * kHid;
 constexpr long kOffW4 = kOffB3 + kHid, kOffB4 = kOffW4 + (long)kOut * kHid;
 constexpr long kParams = kOffB4 + kOut;
 static_assert(kParams == VRM_MLP_PARAMS, "parameter count");
-
-enum EpiMode { EPI_BIAS_GELU = 0, EPI_BIAS_F32 = 1, EPI_F32 = 2, EPI_GELU_BWD = 3 };
-
-struct Epi {
-  int mode;
-  int M, N;              // logical output rows and columns (stores are guarded)
-  const int* m_dev;      // optional device row count (< M)
-  int k_slabs;           // K slabs of 64 per CTA
-  const float* bias;     // [N]
-  const float* z_in;     // EPI_GELU_BWD: pre-activations, ld_zin
-  int ld_zin;
-  float* out_f32;        // EPI_BIAS_F32 / EPI_F32 (+ blockIdx.z * split_stride)
-  int ld_f32;
-  long long split_stride;
-  bf16* out_bf16;        // row-major, ld_bf16
-  int ld_bf16;
-  bf16* out_t;           // transposed copy out_t[col * ld_t + row], optional
-  int ld_t;
-  float* out_z;          // EPI_BIAS_GELU: pre-activation store, optional
-  int ld_z;
-  int* error;            // set on a wait that gave up
-};
 
 // GELU in its tanh form, 0.5 z (1 + tanh(c (z + a z^3))) with c = sqrt(2/pi),
 // a = 0.044715, on the hardware tanh (tanh.approx.f32, relative error about
@@ -94,153 +76,6 @@ __device__ __forceinline__ float gelu_grad(float z) {
   const float t = tanh_hw(kGeluC * fmaf(kGeluA * z, z2, z));
   const float du = kGeluC * fmaf(3.0f * kGeluA, z2, 1.0f);
   return fmaf(0.5f * z * du, fmaf(-t, t, 1.0f), 0.5f * (1.0f + t));
-}
-
-template <int NT>
-constexpr size_t gemm_smem_bytes() {
-  return 1024 + (size_t)kStages * (kBM * kBK * 2 + NT * kBK * 2) + 256;
-}
-
-template <int NT>
-__global__ void __launch_bounds__(128, 1) k_gemm(const __grid_constant__ CUtensorMap tma_a,
-                                                 const __grid_constant__ CUtensorMap tma_b, Epi e) {
-  static_assert(NT == 32 || NT == 64 || NT == 128 || NT == 256, "tile width");
-  extern __shared__ uint8_t smem_raw[];
-  const int m0 = blockIdx.x * kBM;
-  const int n0 = blockIdx.y * NT;
-  int m_limit = e.M;
-  if (e.m_dev) {
-    const int md = *e.m_dev;
-    m_limit = md < m_limit ? md : m_limit;
-  }
-  if (m0 >= m_limit) return;  // the whole CTA leaves before any barrier or TMEM use
-
-  uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sa = base;                                   // kStages x 16 KB
-  uint8_t* sb = base + (size_t)kStages * kBM * kBK * 2;  // kStages x NT*128 B
-  uint64_t* bars = (uint64_t*)(sb + (size_t)kStages * NT * kBK * 2);
-  uint64_t* full = bars;                // TMA -> MMA
-  uint64_t* empty = bars + kStages;     // MMA -> TMA
-  uint64_t* done = bars + 2 * kStages;  // MMA -> epilogue
-  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * kStages + 1);
-  __shared__ int s_fail;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) {
-    s_fail = 0;
-    for (int s = 0; s < kStages; ++s) {
-      umma::mbar_init(&full[s], 1);
-      umma::mbar_init(&empty[s], 1);
-    }
-    umma::mbar_init(done, 1);
-    umma::fence_barrier_init();
-  }
-  if (warp == 0) umma::tmem_alloc(tmem_slot, NT);
-  umma::fence_before_sync();
-  __syncthreads();
-  umma::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-
-  const int nk = e.k_slabs;
-  const int kslab0 = blockIdx.z * nk;
-  constexpr uint32_t kStageBytes = kBM * kBK * 2 + NT * kBK * 2;
-  if (threadIdx.x == 0) {
-    bool ok = true;
-    const uint32_t idesc = umma::idesc_bf16(kBM, NT);
-    auto load = [&](int stage, int kb) {
-      umma::mbar_arrive_expect_tx(&full[stage], kStageBytes);
-      umma::tma_load_2d(sa + (size_t)stage * kBM * kBK * 2, &tma_a, &full[stage], (kslab0 + kb) * kBK, m0);
-      umma::tma_load_2d(sb + (size_t)stage * NT * kBK * 2, &tma_b, &full[stage], (kslab0 + kb) * kBK, n0);
-    };
-    for (int s = 0; s < kStages && s < nk; ++s) load(s, s);
-    for (int kb = 0; kb < nk && ok; ++kb) {
-      const int s = kb % kStages;
-      if (!umma::mbar_wait(&full[s], (uint32_t)(kb / kStages) & 1u, kWaitCycles)) {
-        ok = false;
-        break;
-      }
-      umma::fence_after_sync();
-      const uint64_t da = umma::desc_sw128(umma::smem_u32(sa + (size_t)s * kBM * kBK * 2));
-      const uint64_t db = umma::desc_sw128(umma::smem_u32(sb + (size_t)s * NT * kBK * 2));
-#pragma unroll
-      for (int k = 0; k < kBK / 16; ++k)  // +32 bytes per K step (encoded >> 4)
-        umma::mma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
-      umma::mma_commit(&empty[s]);
-      const int kp = kb - 1;  // refill the slot read one slab earlier
-      if (kp >= 0 && kp + kStages < nk) {
-        const int sp = kp % kStages;
-        if (!umma::mbar_wait(&empty[sp], (uint32_t)(kp / kStages) & 1u, kWaitCycles)) {
-          ok = false;
-          break;
-        }
-        load(sp, kp + kStages);
-      }
-    }
-    umma::mma_commit(done);
-    if (!ok) s_fail = 1;
-  }
-  const bool got = umma::mbar_wait(done, 0, 2 * kWaitCycles);
-  umma::fence_after_sync();
-  const bool failed = __syncthreads_or(!got || s_fail) != 0;  // uniform: the TMEM loads below are warp-wide
-  if (failed) {
-    if (threadIdx.x == 0 && e.error) atomicExch(e.error, 1);
-  } else {
-    // epilogue: this thread's TMEM lane is row m0 + 32 warp + lane
-    const int row = m0 + warp * 32 + lane;
-    const bool row_ok = row < m_limit;
-    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-    for (int c0 = 0; c0 < NT; c0 += 16) {
-      float v[16];
-      umma::tmem_ld16(trow + (uint32_t)c0, v);
-      const int col0 = n0 + c0;
-      if (!row_ok || col0 >= e.N) continue;
-      if (e.mode == EPI_BIAS_GELU) {
-        __align__(16) bf16 hv[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float z = v[i] + e.bias[col0 + i];
-          if (e.out_z) e.out_z[(size_t)row * e.ld_z + col0 + i] = z;
-          hv[i] = __float2bfloat16_rn(gelu(z));
-        }
-        uint4* dst = reinterpret_cast<uint4*>(e.out_bf16 + (size_t)row * e.ld_bf16 + col0);
-        dst[0] = *reinterpret_cast<uint4*>(&hv[0]);
-        dst[1] = *reinterpret_cast<uint4*>(&hv[8]);
-        if (e.out_t) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) e.out_t[(size_t)(col0 + i) * e.ld_t + row] = hv[i];
-        }
-      } else if (e.mode == EPI_BIAS_F32) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (col0 + i < e.N) e.out_f32[(size_t)row * e.ld_f32 + col0 + i] = v[i] + e.bias[col0 + i];
-      } else if (e.mode == EPI_F32) {
-        float* dst = e.out_f32 + (size_t)blockIdx.z * e.split_stride + (size_t)row * e.ld_f32 + col0;
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (col0 + i < e.N) dst[i] = v[i];
-      } else {  // EPI_GELU_BWD
-        __align__(16) bf16 hv[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float z = e.z_in[(size_t)row * e.ld_zin + col0 + i];
-          hv[i] = __float2bfloat16_rn(v[i] * gelu_grad(z));
-        }
-        uint4* dst = reinterpret_cast<uint4*>(e.out_bf16 + (size_t)row * e.ld_bf16 + col0);
-        dst[0] = *reinterpret_cast<uint4*>(&hv[0]);
-        dst[1] = *reinterpret_cast<uint4*>(&hv[8]);
-        if (e.out_t) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) e.out_t[(size_t)(col0 + i) * e.ld_t + row] = hv[i];
-        }
-      }
-    }
-  }
-  umma::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    umma::fence_after_sync();
-    umma::tmem_dealloc(tmem, NT);
-  }
 }
 
 // ---- fused inference ------------------------------------------------------------------
@@ -528,117 +363,545 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
 
 // ---- small kernels -----------------------------------------------------------------
 
+// ---- training -------------------------------------------------------------------
+//
 // Batch assembly: rows idx[r] (or r) of the data set into X [B x 128],
-// X^T [128 x B] and T [B x 32]; rows >= rows are zero (their mask is 0, so
-// they add nothing to the loss or the gradients).
-__global__ void k_gather(const bf16* __restrict__ X_all, const float* __restrict__ T_all,
-                         const int* __restrict__ idx, int rows, int B, bf16* __restrict__ Xb, bf16* __restrict__ Xbt,
-                         float* __restrict__ Tb) {
-  const long total = (long)B * kInPad;
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-    const int r = (int)(t / kInPad), c = (int)(t % kInPad);
-    bf16 v = __float2bfloat16_rn(0.0f);
-    if (r < rows) {
-      const long src = idx ? idx[r] : r;
-      v = X_all[src * kInPad + c];
-      if (c < kOut) Tb[(size_t)r * kOut + c] = T_all[src * kOut + c];
-    } else if (c < kOut) {
-      Tb[(size_t)r * kOut + c] = 0.0f;
+// X^T [128 x B] and T [B x 32], and the sum of each 32-row block's mask; rows
+// >= rows are zero (their mask is 0, so they add nothing to the loss or the
+// gradients).  One block per 32 rows, transposed through shared memory, so
+// that every store is coalesced (aligned: X_all starts on a 4-byte boundary).
+constexpr int kGatherRows = 32;
+__global__ void __launch_bounds__(256) k_gather(const bf16* __restrict__ X_all, const float* __restrict__ T_all,
+                                                const int* __restrict__ idx, int rows, int B, bf16* __restrict__ Xb,
+                                                bf16* __restrict__ Xbt, float* __restrict__ Tb,
+                                                float* __restrict__ cnt, bool aligned) {
+  __shared__ uint32_t tile[kGatherRows][kInPad / 2 + 1];
+  __shared__ float part[8];
+  const int tid = threadIdx.x, r0 = blockIdx.x * kGatherRows;
+  float m = 0.0f;
+  for (int t = tid; t < kGatherRows * (kInPad / 2); t += 256) {  // pairs of columns
+    const int r = t / (kInPad / 2), c = t % (kInPad / 2), row = r0 + r;
+    uint32_t v = 0;
+    if (row < rows) {
+      const bf16* src = X_all + (size_t)(idx ? idx[row] : row) * kInPad + 2 * c;
+      if (aligned) {
+        v = *reinterpret_cast<const uint32_t*>(src);
+      } else {
+        const uint16_t* h = reinterpret_cast<const uint16_t*>(src);
+        v = (uint32_t)h[0] | (uint32_t)h[1] << 16;
+      }
     }
-    Xb[(size_t)r * kInPad + c] = v;
-    Xbt[(size_t)c * B + r] = v;
-  }
-}
-
-// Masked mean squared error and its gradient, one block, fixed summation
-// order: dY = 2 M (Y - T) / sum(M), written as bf16 [B x 64] (columns >= 32
-// zero) and transposed [128 x B] (rows >= 32 zero).
-__global__ void __launch_bounds__(1024) k_loss(const float* __restrict__ Y, const float* __restrict__ T,
-                                               const bf16* __restrict__ Xb, int B, bf16* __restrict__ dY,
-                                               bf16* __restrict__ dYt, float* __restrict__ loss) {
-  __shared__ float red[32];
-  const int tid = threadIdx.x;
-  const long total = (long)B * kOut;
-  auto block_sum = [&](float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    float s = 0.0f;
-    if (tid < 32) {
-      s = tid < (int)(blockDim.x >> 5) ? red[tid] : 0.0f;
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    reinterpret_cast<uint32_t*>(Xb)[(size_t)row * (kInPad / 2) + c] = v;
+    tile[r][c] = v;
+    if (c >= kOut && c < 3 * kOut / 2) {  // columns 64..95
+      const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&v);
+      m += __bfloat162float(b.x) + __bfloat162float(b.y);
     }
-    __syncthreads();
-    if (tid == 0) red[0] = s;
-    __syncthreads();
-    const float r = red[0];
-    __syncthreads();
-    return r;
-  };
-  float cnt = 0.0f;
-  for (long t = tid; t < total; t += blockDim.x) {
-    const int r = (int)(t / kOut), k = (int)(t % kOut);
-    cnt += __bfloat162float(Xb[(size_t)r * kInPad + 2 * kOut + k]);
   }
-  cnt = block_sum(cnt);
-  const float inv = 1.0f / fmaxf(cnt, 1.0f);
-  float l = 0.0f;
-  for (long t = tid; t < total; t += blockDim.x) {
-    const int r = (int)(t / kOut), k = (int)(t % kOut);
-    const float m = __bfloat162float(Xb[(size_t)r * kInPad + 2 * kOut + k]);
-    const float d = m * (Y[t] - T[t]);
-    l += d * d;
-    const bf16 g = __float2bfloat16_rn(2.0f * d * inv);
-    dY[(size_t)r * kOutPad + k] = g;
-    dY[(size_t)r * kOutPad + kOut + k] = __float2bfloat16_rn(0.0f);
-    dYt[(size_t)k * B + r] = g;
+  for (int t = tid; t < kGatherRows * kOut; t += 256) {
+    const int row = r0 + t / kOut;
+    Tb[(size_t)r0 * kOut + t] =
+        row < rows ? T_all[(size_t)(idx ? idx[row] : row) * kOut + t % kOut] : 0.0f;
   }
-  l = block_sum(l);
+  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+  if ((tid & 31) == 0) part[tid >> 5] = m;
+  __syncthreads();
+  for (int t = tid; t < kInPad * (kGatherRows / 2); t += 256) {  // pairs of rows of X^T
+    const int c = t / (kGatherRows / 2), r = 2 * (t % (kGatherRows / 2));
+    const uint32_t a = tile[r][c / 2], b = tile[r + 1][c / 2];
+    const uint32_t v = c & 1 ? (a >> 16) | (b & 0xFFFF0000u) : (a & 0xFFFFu) | (b << 16);
+    reinterpret_cast<uint32_t*>(Xbt + (size_t)c * B + r0)[r / 2] = v;
+  }
   if (tid == 0) {
-    loss[0] = l * inv;
-    loss[1] = cnt;
+    float sum = 0.0f;
+    for (int w = 0; w < 8; ++w) sum += part[w];
+    cnt[blockIdx.x] = sum;
   }
 }
 
-// out[n] = sum over the B entries of row n of a bf16 [N x B] matrix (one
-// warp per row, fixed order).
-__global__ void k_rowsum(const bf16* __restrict__ m, int N, int B, float* __restrict__ out) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (w >= N) return;
-  float s = 0.0f;
-  for (int r = lane; r < B; r += 32) s += __bfloat162float(m[(size_t)w * B + r]);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[w] = s;
+// Forward and backward pass of 128-row tiles, seven products in a row:
+//   0-2  Z = A W^T + b, A = GELU(Z)         (A in shared memory, in place)
+//   3    Y = A W4^T + b4, dY = 2 M (Y - T) / sum(M) and the tile's loss
+//   4    dZ3 = (dY W4) GELU'(Z3)
+//   5, 6 dZ2 = (dZ3 W3) GELU'(Z2), dZ1 = (dZ2 W2) GELU'(Z1)
+// One thread of warp 16 streams the weight slabs through a ring with TMA and
+// issues the MMAs; warps 0-15 run each product's epilogue (warp w: TMEM lanes
+// 32 (w mod 4), columns 64 (w div 4)) and write the next operand in the
+// swizzled layout.  Pre-activations go to global memory and come back to the
+// same thread, tile by tile with the rows contiguous; what k_weight_grad reads
+// (A^T, dZ^T, dY^T) goes out transposed, 64 bytes of a row per warp.  The
+// chain is bound by its own latency: about 3 us per product.
+// Barriers: xfull (input tile loaded), wfull / wempty (ring), accf (a
+// product's MMAs are complete), actr (its epilogue is done: 16 warps).  Every
+// wait is bounded, as in k_mlp_fused.
+constexpr int kChainRing = 4;
+constexpr int kChainSlabs = 23;  // W1: 2, W2, W3, W4: 4 each, W4^T: 1, W3^T, W2^T: 4 each
+constexpr size_t kChainSmem = 1024 + 4 * (size_t)kSlabBytes + (size_t)kChainRing * kRingBytes + 256;
+
+struct ChainMaps {
+  CUtensorMap w[7];  // W1, W2, W3, W4, W4^T, W3^T, W2^T
+};
+struct ChainArgs {
+  const float* theta;
+  const bf16* Xb;
+  const float* Tb;
+  const float* cnt;   // mask sums of the batch's 32-row blocks
+  float* Z[3];        // [tile][256][128]
+  bf16* At[3];        // A1^T, A2^T, A3^T [256 x B]
+  bf16* dZt[3];       // dZ1^T, dZ2^T, dZ3^T [256 x B]
+  bf16* dYt;          // [128 x B], rows >= 32 stay 0
+  float* lossp;       // [tiles][8]
+  int B;
+  int* error;
+};
+
+__device__ __forceinline__ int chain_k(int p) { return p == 0 ? 2 : p == 4 ? 1 : 4; }  // K slabs of product p
+
+__global__ void __launch_bounds__(kFusedThreads, 1)
+    k_chain(const __grid_constant__ CUtensorMap tx, const __grid_constant__ ChainMaps maps,
+            const __grid_constant__ ChainArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  const int ntiles = a.B / kBM;
+  const int my_tiles = (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+  uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* H = base;                              // 4 slabs x 16 KB
+  uint8_t* ring = base + 4 * (size_t)kSlabBytes;  // kChainRing x 32 KB
+  uint64_t* bars = (uint64_t*)(ring + (size_t)kChainRing * kRingBytes);
+  uint64_t *xfull = bars, *accf = bars + 1, *actr = bars + 2, *drain = bars + 3;
+  uint64_t *wfull = bars + 4, *wempty = bars + 4 + kChainRing;
+  uint32_t* tmem_slot = (uint32_t*)(bars + 4 + 2 * kChainRing);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    umma::mbar_init(xfull, 1);
+    umma::mbar_init(accf, 1);
+    umma::mbar_init(actr, kEpiWarps);
+    umma::mbar_init(drain, 1);
+    for (int s = 0; s < kChainRing; ++s) {
+      umma::mbar_init(&wfull[s], 1);
+      umma::mbar_init(&wempty[s], 1);
+    }
+    *abort_flag = 0;
+    umma::fence_barrier_init();
+  }
+  if (warp == 0) umma::tmem_alloc(tmem_slot, 256);
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == kEpiWarps) {
+    if (lane == 0) {
+      const int total = my_tiles * kChainSlabs;
+      int lp = 0, lk = 0;  // product and slab of the next load
+      auto load_w = [&](int gl) {
+        const int st = gl % kChainRing;
+        umma::mbar_arrive_expect_tx(&wfull[st], lp == 3 ? (uint32_t)kOut * kBK * 2 : kRingBytes);
+        umma::tma_load_2d(ring + (size_t)st * kRingBytes, &maps.w[lp], &wfull[st], lk * kBK, 0);
+        if (++lk == chain_k(lp)) {
+          lk = 0;
+          lp = lp == 6 ? 0 : lp + 1;
+        }
+      };
+      auto load_x = [&](int tile) {
+        umma::mbar_arrive_expect_tx(xfull, 2u * kSlabBytes);
+        umma::tma_load_2d(H, &tx, xfull, 0, tile * kBM);
+        umma::tma_load_2d(H + kSlabBytes, &tx, xfull, kBK, tile * kBM);
+      };
+      load_x(blockIdx.x);
+      int g_load = 0, g = 0;
+      for (; g_load < kChainRing && g_load < total; ++g_load) load_w(g_load);
+      bool fail = false;
+      for (int i = 0; i < my_tiles && !fail; ++i) {
+        for (int p = 0; p < 7 && !fail; ++p) {
+          const int e = 7 * i + p;  // epilogues that must be done
+          if (*abort_flag || (e > 0 && !umma::mbar_wait(actr, (uint32_t)(e - 1) & 1u, kWaitCycles))) {
+            fail = true;
+            break;
+          }
+          if (p == 0) {
+            // the last product of the tile before has read its operand (its
+            // epilogue is done): the next input may replace it
+            if (i > 0) load_x(blockIdx.x + i * gridDim.x);
+            if (!umma::mbar_wait(xfull, (uint32_t)i & 1u, kWaitCycles)) {
+              fail = true;
+              break;
+            }
+          }
+          umma::fence_after_sync();
+          const uint32_t idesc = umma::idesc_bf16(kBM, p == 3 ? kOut : kHid);
+          const int nk = chain_k(p);
+          for (int kb = 0; kb < nk; ++kb, ++g) {
+            const int st = g % kChainRing;
+            if (!umma::mbar_wait(&wfull[st], (uint32_t)(g / kChainRing) & 1u, kWaitCycles)) {
+              fail = true;
+              break;
+            }
+            umma::fence_after_sync();
+            const uint64_t da = umma::desc_sw128(umma::smem_u32(H + (size_t)kb * kSlabBytes));
+            const uint64_t db = umma::desc_sw128(umma::smem_u32(ring + (size_t)st * kRingBytes));
+#pragma unroll
+            for (int k = 0; k < kBK / 16; ++k) umma::mma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+            umma::mma_commit(&wempty[st]);
+            const int gp = g - 1;  // refill the slot of the slab before
+            if (gp >= 0 && gp + kChainRing < total) {
+              if (!umma::mbar_wait(&wempty[gp % kChainRing], (uint32_t)(gp / kChainRing) & 1u, kWaitCycles)) {
+                fail = true;
+                break;
+              }
+              load_w(g_load++);
+            }
+          }
+          if (!fail) umma::mma_commit(accf);
+        }
+      }
+      if (fail) *abort_flag = 1;
+      umma::mma_commit(drain);
+      if (!umma::mbar_wait(drain, 0u, kWaitCycles)) *abort_flag = 1;
+    }
+  } else {
+    const int q = warp & 3, cg = warp >> 2;
+    const int r = q * 32 + lane;  // row within the tile
+    float inv = 0.0f;
+    if (cg < 2) {  // sum of the batch's mask (whole numbers: exact in any order below 2^24)
+      float c = 0.0f;
+      for (int k = lane; k < a.B / kGatherRows; k += 32) c += a.cnt[k];
+      for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      inv = 1.0f / fmaxf(c, 1.0f);
+    }
+    const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+    uint8_t* const hrow = H + (size_t)cg * kSlabBytes + (size_t)r * 128;  // this thread's 64 columns
+    bool stop = false;
+    for (int i = 0; i < my_tiles && !stop; ++i) {
+      const int tile = blockIdx.x + i * gridDim.x;
+      const int row = tile * kBM + r;
+      for (int p = 0; p < 7; ++p) {
+        if (*abort_flag) {
+          stop = true;
+          break;
+        }
+        if (!umma::mbar_wait(accf, (uint32_t)(7 * i + p) & 1u, 2 * kWaitCycles)) {
+          *abort_flag = 1;
+          stop = true;
+          break;
+        }
+        umma::fence_after_sync();
+        if (p == 3) {
+          __align__(16) bf16 gv[16];
+          if (cg < 2) {
+            const int c0 = cg * 16;
+            float v[16];
+            umma::tmem_ld16(trow + (uint32_t)c0, v);
+            __align__(16) bf16 mk[16];
+            const uint4* xm = reinterpret_cast<const uint4*>(a.Xb + (size_t)row * kInPad + 2 * kOut + c0);
+            reinterpret_cast<uint4*>(mk)[0] = xm[0];
+            reinterpret_cast<uint4*>(mk)[1] = xm[1];
+            const float4* tt = reinterpret_cast<const float4*>(a.Tb + (size_t)row * kOut + c0);
+            float l = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float4 t4 = tt[k];
+              const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int n = 4 * k + u;
+                const float y = v[n] + __ldg(a.theta + kOffB4 + c0 + n);
+                const float d = __bfloat162float(mk[n]) * (y - tv[u]);
+                l += d * d;
+                gv[n] = __float2bfloat16_rn(2.0f * d * inv);
+                a.dYt[(size_t)(c0 + n) * a.B + row] = gv[n];
+              }
+            }
+            for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            if (lane == 0) a.lossp[(size_t)tile * 8 + warp] = l;
+          } else {
+#pragma unroll
+            for (int n = 0; n < 16; ++n) gv[n] = __float2bfloat16_rn(0.0f);
+          }
+          // dY: columns 16 cg .. 16 cg + 15 of the first slab (zeros from 32 on)
+          uint8_t* const drow = H + (size_t)r * 128;
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            *reinterpret_cast<uint4*>(drow + (((2 * cg + u) ^ (r & 7)) << 4)) = reinterpret_cast<uint4*>(gv)[u];
+        } else {
+          const bool fwd = p < 3;
+          const int l = fwd ? p : 6 - p;  // layer whose Z this is
+          float* const zt = a.Z[l] + ((size_t)tile * kHid + cg * 64) * kBM + r;
+          bf16* const ot = (fwd ? a.At[l] : a.dZt[l]) + (size_t)(cg * 64) * a.B + row;
+          const float* const b = a.theta + (l == 0 ? kOffB1 : l == 1 ? kOffB2 : kOffB3) + cg * 64;
+#pragma unroll 1
+          for (int c0 = 0; c0 < 64; c0 += 32) {
+            float v[32];
+            float z[32];
+            if (!fwd) {
+#pragma unroll
+              for (int k = 0; k < 32; ++k) z[k] = zt[(size_t)(c0 + k) * kBM];
+            }
+            umma::tmem_ld32(trow + (uint32_t)(cg * 64 + c0), v);
+            __align__(16) bf16 hv[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+              if (fwd) {
+                const float zz = v[k] + __ldg(b + c0 + k);
+                zt[(size_t)(c0 + k) * kBM] = zz;
+                hv[k] = __float2bfloat16_rn(gelu(zz));
+              } else {
+                hv[k] = __float2bfloat16_rn(v[k] * gelu_grad(z[k]));
+              }
+              ot[(size_t)(c0 + k) * a.B] = hv[k];
+            }
+            if (p < 6) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                *reinterpret_cast<uint4*>(hrow + ((((c0 >> 3) + u) ^ (r & 7)) << 4)) =
+                    reinterpret_cast<uint4*>(hv)[u];
+            }
+          }
+        }
+        umma::fence_proxy_async_smem();
+        umma::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) umma::mbar_arrive(actr);
+      }
+    }
+  }
+  umma::fence_before_sync();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag && a.error) atomicExch(a.error, 1);
+  if (warp == 0) {
+    umma::fence_after_sync();
+    umma::tmem_dealloc(tmem, 256);
+  }
 }
 
-// g[r * cols + c] = sum_s part[s][r * ld + c] for r < rows, c < cols.
-__global__ void k_split_sum(const float* __restrict__ part, int splits, long long stride, int rows, int cols, int ld,
-                            float* __restrict__ g) {
-  const long total = (long)rows * cols;
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-    const int r = (int)(t / cols), c = (int)(t % cols);
-    float s = 0.0f;
-    for (int k = 0; k < splits; ++k) s += part[(size_t)k * stride + (size_t)r * ld + c];
-    g[t] = s;
+// Weight gradients: dW[M x N] = dZ^T A with the batch as K, split over
+// blockIdx.x; blockIdx.y is one 128-row piece of a layer's gradient:
+//   0, 1 W1 (N = 128, the padded inputs), 2, 3 W2, 4, 5 W3, 6 W4 (32 rows)
+// One thread loads both operands' slabs with TMA through a two-stage ring (two
+// CTAs per SM) and issues the MMAs; the four warps write the accumulator
+// transposed, part[split][piece][column][row], so that a warp's store is 128
+// contiguous bytes.
+constexpr int kPieces = 7;
+constexpr int kWgStages = 2;
+constexpr uint32_t kWgStageBytes = kSlabBytes + kRingBytes;
+constexpr size_t kWgSmem = 1024 + (size_t)kWgStages * kWgStageBytes + 128;
+constexpr long long kPartSplit = (long long)kPieces * kHid * kBM;  // floats of one split
+
+struct WgMaps {
+  CUtensorMap a[4], b[4];  // per layer: dZ^T (dY^T), activations^T
+};
+
+__global__ void __launch_bounds__(128, 2)
+    k_weight_grad(const __grid_constant__ WgMaps maps, int k_slabs, float* __restrict__ part, int* __restrict__ error) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = (uint64_t*)(base + (size_t)kWgStages * kWgStageBytes);
+  uint64_t *full = bars, *empty = bars + kWgStages, *done = bars + 2 * kWgStages;
+  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * kWgStages + 1);
+  __shared__ int s_fail;
+  const int piece = blockIdx.y, layer = piece >> 1, m0 = (piece & 1) * kBM;
+  const int N = layer == 0 ? kInPad : kHid;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    for (int s = 0; s < kWgStages; ++s) {
+      umma::mbar_init(&full[s], 1);
+      umma::mbar_init(&empty[s], 1);
+    }
+    umma::mbar_init(done, 1);
+    umma::fence_barrier_init();
+  }
+  if (warp == 0) umma::tmem_alloc(tmem_slot, 256);
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  if (threadIdx.x == 0) {
+    bool ok = true;
+    const int k0 = blockIdx.x * k_slabs;
+    const uint32_t idesc = umma::idesc_bf16(kBM, N);
+    auto load = [&](int kb) {
+      const int s = kb % kWgStages;
+      uint8_t* sa = base + (size_t)s * kWgStageBytes;
+      umma::mbar_arrive_expect_tx(&full[s], kSlabBytes + (uint32_t)N * kBK * 2);
+      umma::tma_load_2d(sa, &maps.a[layer], &full[s], (k0 + kb) * kBK, m0);
+      umma::tma_load_2d(sa + kSlabBytes, &maps.b[layer], &full[s], (k0 + kb) * kBK, 0);
+    };
+    for (int s = 0; s < kWgStages && s < k_slabs; ++s) load(s);
+    for (int kb = 0; kb < k_slabs && ok; ++kb) {
+      const int s = kb % kWgStages;
+      const uint32_t par = (uint32_t)(kb / kWgStages) & 1u;
+      if (!umma::mbar_wait(&full[s], par, kWaitCycles)) {
+        ok = false;
+        break;
+      }
+      umma::fence_after_sync();
+      uint8_t* sa = base + (size_t)s * kWgStageBytes;
+      const uint64_t da = umma::desc_sw128(umma::smem_u32(sa)), db = umma::desc_sw128(umma::smem_u32(sa + kSlabBytes));
+#pragma unroll
+      for (int k = 0; k < kBK / 16; ++k) umma::mma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+      umma::mma_commit(&empty[s]);
+      if (kb + kWgStages < k_slabs) {
+        if (!umma::mbar_wait(&empty[s], par, kWaitCycles)) {
+          ok = false;
+          break;
+        }
+        load(kb + kWgStages);
+      }
+    }
+    umma::mma_commit(done);
+    if (!ok) s_fail = 1;
+  }
+  const bool got = umma::mbar_wait(done, 0, 2 * kWaitCycles);
+  umma::fence_after_sync();
+  const bool failed = __syncthreads_or(!got || s_fail) != 0;  // uniform: the TMEM loads below are warp-wide
+  if (failed) {
+    if (threadIdx.x == 0 && error) atomicExch(error, 1);
+  } else if (layer < 3 || warp == 0) {
+    float* const out = part + (size_t)blockIdx.x * kPartSplit + (size_t)piece * kHid * kBM + warp * 32 + lane;
+    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+    for (int c0 = 0; c0 < N; c0 += 32) {
+      float v[32];
+      umma::tmem_ld32(trow + (uint32_t)c0, v);
+#pragma unroll
+      for (int k = 0; k < 32; ++k) out[(size_t)(c0 + k) * kBM] = v[k];
+    }
+  }
+  umma::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) {
+    umma::fence_after_sync();
+    umma::tmem_dealloc(tmem, 256);
   }
 }
 
 // AdamW (decoupled weight decay): c1 = 1 - beta1^t, c2 = 1 - beta2^t.
+struct AdamwArgs {
+  float lr, b1, b2, eps, wd, c1, c2;
+};
+__device__ __forceinline__ float adamw_one(const AdamwArgs& o, float* theta, float* m, float* v, float gi) {
+  const float mi = o.b1 * *m + (1.0f - o.b1) * gi;
+  const float vi = o.b2 * *v + (1.0f - o.b2) * gi * gi;
+  *m = mi;
+  *v = vi;
+  const float mh = mi / o.c1, vh = vi / o.c2;
+  const float th = *theta - o.lr * (mh / (sqrtf(vh) + o.eps) + o.wd * *theta);
+  *theta = th;
+  return th;
+}
 __global__ void k_adamw(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
-                        const float* __restrict__ g, long n, float lr, float b1, float b2, float eps, float wd,
-                        float c1, float c2) {
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float mh = mi / c1, vh = vi / c2;
-    theta[i] = theta[i] - lr * (mh / (sqrtf(vh) + eps) + wd * theta[i]);
+                        const float* __restrict__ g, long n, AdamwArgs o) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
+    adamw_one(o, theta + i, m + i, v + i, g[i]);
+}
+
+// The last kernel of a gradient or training step.  Blocks 0..159 take one
+// 32 x 32 tile of a weight matrix each: the splits' partial sums (rows
+// contiguous) added in split order, transposed through shared memory, then
+// the gradient written (grad given) or AdamW applied and the bf16 copies of
+// the weight and of its transpose written.  The next blocks take eight bias
+// entries each, a warp summing a row of dZ^T lane by lane, and the last one
+// sums the tiles' losses.
+constexpr int kUpdTiles = 24 + 64 + 64 + 8;
+constexpr int kUpdBias = (3 * kHid + kOut) / 8;
+struct UpdArgs {
+  const float* part;
+  int splits;
+  const bf16* dZt[3];
+  const bf16* dYt;
+  const float* lossp;
+  const float* cnt;
+  int B;
+  float *theta, *m, *v, *grad, *loss;
+  bf16 *W[4], *Wt[4];  // Wt[0] null: W1 has no transposed copy
+  AdamwArgs opt;
+};
+
+__global__ void __launch_bounds__(256) k_update(const __grid_constant__ UpdArgs a) {
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int b = blockIdx.x;
+  if (b < kUpdTiles) {
+    __shared__ float tile[32][33];
+    const int layer = b < 24 ? 0 : b < 88 ? 1 : b < 152 ? 2 : 3;
+    const int t = b - (layer == 0 ? 0 : layer == 1 ? 24 : layer == 2 ? 88 : 152);
+    const int tc = layer == 0 ? 3 : 8;  // tiles across
+    const int r0 = 32 * (t / tc), c0 = 32 * (t % tc);
+    const long off = layer == 0 ? kOffW1 : layer == 1 ? kOffW2 : layer == 2 ? kOffW3 : kOffW4;
+    const int cols = layer == 0 ? kIn : kHid;
+    const float* p = a.part + ((size_t)(2 * layer + r0 / kBM) * kHid + c0 + ty) * kBM + r0 % kBM + tx;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+    for (int k = 0; k < a.splits; ++k, p += kPartSplit)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] += p[(size_t)(8 * u) * kBM];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) tile[ty + 8 * u][tx] = s[u];  // [column][row]
+    __syncthreads();
+    if (a.grad) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a.grad[off + (long)(r0 + ty + 8 * u) * cols + c0 + tx] = tile[tx][ty + 8 * u];
+      return;
+    }
+    float th[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + ty + 8 * u;
+      const long i = off + (long)r * cols + c0 + tx;
+      th[u] = adamw_one(a.opt, a.theta + i, a.m + i, a.v + i, tile[tx][ty + 8 * u]);
+      a.W[layer][(long)r * (layer == 0 ? kInPad : kHid) + c0 + tx] = __float2bfloat16_rn(th[u]);
+    }
+    if (layer == 0) return;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) tile[tx][ty + 8 * u] = th[u];
+    __syncthreads();
+    const int ld = layer == 3 ? kOutPad : kHid;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      a.Wt[layer][(long)(c0 + ty + 8 * u) * ld + r0 + tx] = __float2bfloat16_rn(tile[ty + 8 * u][tx]);
+  } else if (b < kUpdTiles + kUpdBias) {
+    const int w = (b - kUpdTiles) * 8 + ty;  // b1, b2, b3, b4
+    const int layer = w / kHid, n = w % kHid;
+    const bf16* row = (layer < 3 ? a.dZt[layer] : a.dYt) + (size_t)n * a.B;
+    float s = 0.0f;
+#pragma unroll 8
+    for (int r = tx; r < a.B; r += 32) s += __bfloat162float(row[r]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (tx == 0) {
+      const long i = (layer == 0 ? kOffB1 : layer == 1 ? kOffB2 : layer == 2 ? kOffB3 : kOffB4) + n;
+      if (a.grad)
+        a.grad[i] = s;
+      else
+        adamw_one(a.opt, a.theta + i, a.m + i, a.v + i, s);
+    }
+  } else {
+    __shared__ float red[2][8];
+    float l = 0.0f, c = 0.0f;
+    for (int k = threadIdx.x; k < a.B / kBM * 8; k += 256) l += a.lossp[k];
+    for (int k = threadIdx.x; k < a.B / kGatherRows; k += 256) c += a.cnt[k];
+    for (int o = 16; o > 0; o >>= 1) {
+      l += __shfl_xor_sync(0xffffffffu, l, o);
+      c += __shfl_xor_sync(0xffffffffu, c, o);
+    }
+    if (tx == 0) {
+      red[0][ty] = l;
+      red[1][ty] = c;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) {
+        l += red[0][w];
+        c += red[1][w];
+      }
+      a.loss[0] = l * (1.0f / fmaxf(c, 1.0f));
+      a.loss[1] = c;
+    }
   }
 }
 
-// bf16 weights for the GEMMs from the fp32 parameters: W1 padded to 256 x 128,
+// bf16 weights for the products from the fp32 parameters: W1 padded to 256 x 128,
 // W2, W3, W4, and transposed copies W2^T, W3^T (256 x 256), W4^T (256 x 64).
 __global__ void k_refresh(const float* __restrict__ th, bf16* __restrict__ W1, bf16* __restrict__ W2,
                           bf16* __restrict__ W3, bf16* __restrict__ W4, bf16* __restrict__ W2t,
@@ -705,47 +968,6 @@ bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uin
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NT>
-cudaError_t launch_gemm_nt(const CUtensorMap& a, const CUtensorMap& b, int m_tiles, int n_tiles, int splits,
-                           const Epi& e, cudaStream_t s) {
-  static bool attr_set = false;
-  const size_t smem = gemm_smem_bytes<NT>();
-  if (!attr_set) {
-    cudaError_t r = cudaFuncSetAttribute(k_gemm<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (r != cudaSuccess) return r;
-    attr_set = true;
-  }
-  dim3 grid(m_tiles, n_tiles, splits);
-  k_gemm<NT><<<grid, 128, smem, s>>>(a, b, e);
-  note_launch();
-  return cudaGetLastError();
-}
-
-// C[M x N] = A[M x K] B[N x K]^T with K split `splits` ways (K / 64 divisible).
-cudaError_t gemm(const CUtensorMap& a, const CUtensorMap& b, int nt, int m_bound, int N, int K, int splits, Epi e,
-                 cudaStream_t s) {
-  if (K % kBK || (K / kBK) % splits) return cudaErrorInvalidValue;
-  e.k_slabs = K / kBK / splits;
-  const int m_tiles = (m_bound + kBM - 1) / kBM;
-  const int n_tiles = (N + nt - 1) / nt;
-  switch (nt) {
-    case 32: return launch_gemm_nt<32>(a, b, m_tiles, n_tiles, splits, e, s);
-    case 64: return launch_gemm_nt<64>(a, b, m_tiles, n_tiles, splits, e, s);
-    case 128: return launch_gemm_nt<128>(a, b, m_tiles, n_tiles, splits, e, s);
-    case 256: return launch_gemm_nt<256>(a, b, m_tiles, n_tiles, splits, e, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-Epi epi(int mode, int M, int N) {
-  Epi e;
-  memset(&e, 0, sizeof(e));
-  e.mode = mode;
-  e.M = M;
-  e.N = N;
-  return e;
-}
-
 int blocks_for_n(long n, int threads) {
   long b = (n + threads - 1) / threads;
   const long cap = 8L * sm_count();
@@ -761,13 +983,13 @@ struct vrm_mlp {
   float *theta = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr, *part = nullptr, *loss = nullptr;
   bf16 *W1 = nullptr, *W2 = nullptr, *W3 = nullptr, *W4 = nullptr, *W2t = nullptr, *W3t = nullptr, *W4t = nullptr;
   bf16 *Xb = nullptr, *Xbt = nullptr;
-  float* Tb = nullptr;
-  float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *Y = nullptr;
-  bf16 *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *H1t = nullptr, *H2t = nullptr, *H3t = nullptr;
-  bf16 *dY = nullptr, *dYt = nullptr;
-  bf16 *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr, *dZ1t = nullptr, *dZ2t = nullptr, *dZ3t = nullptr;
-  CUtensorMap mW1, mW2, mW3, mW4, mW2t, mW3t, mW4t;  // weights as B operands
-  CUtensorMap mX, mXt, mH1, mH2, mH3, mH1t, mH2t, mH3t, mdY, mdYt, mdZ1t, mdZ2, mdZ2t, mdZ3, mdZ3t;
+  float *Tb = nullptr, *cnt = nullptr, *lossp = nullptr;
+  float* Z[3] = {};
+  bf16 *At[3] = {}, *dZt[3] = {}, *dYt = nullptr;
+  CUtensorMap mW1, mW2, mW3, mW4;  // weights as B operands
+  CUtensorMap mX;
+  ChainMaps chain;
+  WgMaps wg;
 };
 
 namespace vrm {
@@ -825,8 +1047,8 @@ namespace {
 
 void free_mlp(vrm_mlp* n) {
   void* ptrs[] = {n->err, n->theta, n->m, n->v, n->grad, n->part, n->loss, n->W1, n->W2, n->W3, n->W4, n->W2t,
-                  n->W3t, n->W4t, n->Xb, n->Xbt, n->Tb, n->Z1, n->Z2, n->Z3, n->Y, n->H1, n->H2, n->H3, n->H1t,
-                  n->H2t, n->H3t, n->dY, n->dYt, n->dZ1, n->dZ2, n->dZ3, n->dZ1t, n->dZ2t, n->dZ3t};
+                  n->W3t, n->W4t, n->Xb, n->Xbt, n->Tb, n->cnt, n->lossp, n->Z[0], n->Z[1], n->Z[2], n->At[0],
+                  n->At[1], n->At[2], n->dZt[0], n->dZt[1], n->dZt[2], n->dYt};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -838,72 +1060,65 @@ cudaError_t zalloc(T** p, size_t count) {
   return e;
 }
 
-// Forward and backward of the current batch (Xb, Xbt, Tb): loss -> net->loss,
-// gradient -> net->grad.
+// Forward and backward pass of the current batch (Xb, Xbt, Tb) up to the
+// partial weight gradients.
 cudaError_t forward_backward(vrm_mlp* n, cudaStream_t s) {
-  const int B = n->B;
-  cudaError_t r;
-  // forward, keeping pre-activations and transposed activations
-  Epi e = epi(EPI_BIAS_GELU, B, kHid);
-  e.error = n->err;
-  e.ld_bf16 = kHid;
-  e.ld_t = B;
-  e.ld_z = kHid;
-  e.bias = n->theta + kOffB1, e.out_bf16 = n->H1, e.out_t = n->H1t, e.out_z = n->Z1;
-  if ((r = gemm(n->mX, n->mW1, 256, B, kHid, kInPad, 1, e, s)) != cudaSuccess) return r;
-  e.bias = n->theta + kOffB2, e.out_bf16 = n->H2, e.out_t = n->H2t, e.out_z = n->Z2;
-  if ((r = gemm(n->mH1, n->mW2, 256, B, kHid, kHid, 1, e, s)) != cudaSuccess) return r;
-  e.bias = n->theta + kOffB3, e.out_bf16 = n->H3, e.out_t = n->H3t, e.out_z = n->Z3;
-  if ((r = gemm(n->mH2, n->mW3, 256, B, kHid, kHid, 1, e, s)) != cudaSuccess) return r;
-  Epi f = epi(EPI_BIAS_F32, B, kOut);
-  f.error = n->err;
-  f.bias = n->theta + kOffB4, f.out_f32 = n->Y, f.ld_f32 = kOut;
-  if ((r = gemm(n->mH3, n->mW4, 32, B, kOut, kHid, 1, f, s)) != cudaSuccess) return r;
-  k_loss<<<1, 1024, 0, s>>>(n->Y, n->Tb, n->Xb, B, n->dY, n->dYt, n->loss);
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t r = cudaFuncSetAttribute(k_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(k_weight_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
+    if (r != cudaSuccess) return r;
+    attr_set = true;
+  }
+  ChainArgs a;
+  a.theta = n->theta;
+  a.Xb = n->Xb;
+  a.Tb = n->Tb;
+  a.cnt = n->cnt;
+  for (int l = 0; l < 3; ++l) {
+    a.Z[l] = n->Z[l];
+    a.At[l] = n->At[l];
+    a.dZt[l] = n->dZt[l];
+  }
+  a.dYt = n->dYt;
+  a.lossp = n->lossp;
+  a.B = n->B;
+  a.error = n->err;
+  const int tiles = n->B / kBM;
+  k_chain<<<tiles < sm_count() ? tiles : sm_count(), kFusedThreads, kChainSmem, s>>>(n->mX, n->chain, a);
   note_launch();
-  // backward
-  const long long pstride = (long long)kHid * kHid;
-  Epi w = epi(EPI_F32, kOut, kHid);  // dW4 = dY^T H3
-  w.error = n->err;
-  w.out_f32 = n->part, w.ld_f32 = kHid, w.split_stride = pstride;
-  if ((r = gemm(n->mdYt, n->mH3t, 256, kOut, kHid, B, n->splits, w, s)) != cudaSuccess) return r;
-  k_split_sum<<<blocks_for_n((long)kOut * kHid, 256), 256, 0, s>>>(n->part, n->splits, pstride, kOut, kHid, kHid,
-                                                                    n->grad + kOffW4);
+  k_weight_grad<<<dim3(n->splits, kPieces), 128, kWgSmem, s>>>(n->wg, n->B / kBK / n->splits, n->part, n->err);
   note_launch();
-  k_rowsum<<<(kOut * 32 + 255) / 256, 256, 0, s>>>(n->dYt, kOut, B, n->grad + kOffB4);
-  note_launch();
-  Epi d = epi(EPI_GELU_BWD, B, kHid);  // dZ3 = (dY W4) * gelu'(Z3)
-  d.error = n->err;
-  d.ld_bf16 = kHid, d.ld_t = B, d.ld_zin = kHid;
-  d.z_in = n->Z3, d.out_bf16 = n->dZ3, d.out_t = n->dZ3t;
-  if ((r = gemm(n->mdY, n->mW4t, 256, B, kHid, kOutPad, 1, d, s)) != cudaSuccess) return r;
-  w = epi(EPI_F32, kHid, kHid);  // dW3 = dZ3^T H2
-  w.error = n->err;
-  w.out_f32 = n->part, w.ld_f32 = kHid, w.split_stride = pstride;
-  if ((r = gemm(n->mdZ3t, n->mH2t, 256, kHid, kHid, B, n->splits, w, s)) != cudaSuccess) return r;
-  k_split_sum<<<blocks_for_n(pstride, 256), 256, 0, s>>>(n->part, n->splits, pstride, kHid, kHid, kHid,
-                                                          n->grad + kOffW3);
-  note_launch();
-  k_rowsum<<<(kHid * 32 + 255) / 256, 256, 0, s>>>(n->dZ3t, kHid, B, n->grad + kOffB3);
-  note_launch();
-  d.z_in = n->Z2, d.out_bf16 = n->dZ2, d.out_t = n->dZ2t;  // dZ2 = (dZ3 W3) * gelu'(Z2)
-  if ((r = gemm(n->mdZ3, n->mW3t, 256, B, kHid, kHid, 1, d, s)) != cudaSuccess) return r;
-  if ((r = gemm(n->mdZ2t, n->mH1t, 256, kHid, kHid, B, n->splits, w, s)) != cudaSuccess) return r;  // dW2
-  k_split_sum<<<blocks_for_n(pstride, 256), 256, 0, s>>>(n->part, n->splits, pstride, kHid, kHid, kHid,
-                                                          n->grad + kOffW2);
-  note_launch();
-  k_rowsum<<<(kHid * 32 + 255) / 256, 256, 0, s>>>(n->dZ2t, kHid, B, n->grad + kOffB2);
-  note_launch();
-  d.z_in = n->Z1, d.out_bf16 = n->dZ1, d.out_t = n->dZ1t;  // dZ1 = (dZ2 W2) * gelu'(Z1)
-  if ((r = gemm(n->mdZ2, n->mW2t, 256, B, kHid, kHid, 1, d, s)) != cudaSuccess) return r;
-  w = epi(EPI_F32, kHid, kInPad);  // dW1 = dZ1^T X (padded input columns dropped in the sum)
-  w.error = n->err;
-  w.out_f32 = n->part, w.ld_f32 = kInPad, w.split_stride = pstride;
-  if ((r = gemm(n->mdZ1t, n->mXt, 128, kHid, kInPad, B, n->splits, w, s)) != cudaSuccess) return r;
-  k_split_sum<<<blocks_for_n((long)kHid * kIn, 256), 256, 0, s>>>(n->part, n->splits, pstride, kHid, kIn, kInPad,
-                                                                    n->grad + kOffW1);
-  note_launch();
-  k_rowsum<<<(kHid * 32 + 255) / 256, 256, 0, s>>>(n->dZ1t, kHid, B, n->grad + kOffB1);
+  return cudaGetLastError();
+}
+
+// The gradient of the batch into n->grad (opt null), or one AdamW step with it.
+cudaError_t update(vrm_mlp* n, const AdamwArgs* opt, cudaStream_t s) {
+  UpdArgs a;
+  memset(&a, 0, sizeof(a));
+  a.part = n->part;
+  a.splits = n->splits;
+  for (int l = 0; l < 3; ++l) a.dZt[l] = n->dZt[l];
+  a.dYt = n->dYt;
+  a.lossp = n->lossp;
+  a.cnt = n->cnt;
+  a.B = n->B;
+  a.theta = n->theta;
+  a.m = n->m;
+  a.v = n->v;
+  a.loss = n->loss;
+  bf16* w[4] = {n->W1, n->W2, n->W3, n->W4};
+  bf16* wt[4] = {nullptr, n->W2t, n->W3t, n->W4t};
+  for (int l = 0; l < 4; ++l) {
+    a.W[l] = w[l];
+    a.Wt[l] = wt[l];
+  }
+  if (opt)
+    a.opt = *opt;
+  else
+    a.grad = n->grad;
+  k_update<<<kUpdTiles + kUpdBias + 1, 256, 0, s>>>(a);
   note_launch();
   return cudaGetLastError();
 }
@@ -916,7 +1131,8 @@ cudaError_t refresh(vrm_mlp* n, cudaStream_t s) {
 }
 
 cudaError_t gather(vrm_mlp* n, const bf16* X, const float* T, const int* idx, int rows, cudaStream_t s) {
-  k_gather<<<blocks_for_n((long)n->B * kInPad, 256), 256, 0, s>>>(X, T, idx, rows, n->B, n->Xb, n->Xbt, n->Tb);
+  k_gather<<<n->B / kGatherRows, 256, 0, s>>>(X, T, idx, rows, n->B, n->Xb, n->Xbt, n->Tb, n->cnt,
+                                                   ((uintptr_t)X & 3u) == 0);
   note_launch();
   return cudaGetLastError();
 }
@@ -933,14 +1149,10 @@ bool adamw_ok(const vrm_adamw* a) {
          a->weight_decay >= 0 && std::isfinite(a->lr);
 }
 
-vrm_status run_adamw(vrm_mlp* n, const float* grad, const vrm_adamw* a, int32_t t, cudaStream_t s) {
+AdamwArgs adamw_args(const vrm_adamw* a, int32_t t) {
   const double c1 = 1.0 - std::pow((double)a->beta1, (double)t);
   const double c2 = 1.0 - std::pow((double)a->beta2, (double)t);
-  k_adamw<<<blocks_for_n(kParams, 256), 256, 0, s>>>(n->theta, n->m, n->v, grad, kParams, a->lr, a->beta1, a->beta2,
-                                                      a->eps, a->weight_decay, (float)c1, (float)c2);
-  note_launch();
-  if (refresh(n, s) != cudaSuccess) return VRM_ERR_CUDA;
-  return cudaGetLastError() == cudaSuccess ? VRM_OK : VRM_ERR_CUDA;
+  return AdamwArgs{a->lr, a->beta1, a->beta2, a->eps, a->weight_decay, (float)c1, (float)c2};
 }
 
 }  // namespace
@@ -973,7 +1185,7 @@ vrm_status vrm_mlp_create(int32_t batch_rows, vrm_mlp** out) {
   MLP_ALLOC(m, kParams);
   MLP_ALLOC(v, kParams);
   MLP_ALLOC(grad, kParams);
-  MLP_ALLOC(part, (size_t)splits * kHid * kHid);
+  MLP_ALLOC(part, (size_t)splits * kPartSplit);
   MLP_ALLOC(loss, 2);
   MLP_ALLOC(W1, (size_t)kHid * kInPad);
   MLP_ALLOC(W2, (size_t)kHid * kHid);
@@ -985,39 +1197,27 @@ vrm_status vrm_mlp_create(int32_t batch_rows, vrm_mlp** out) {
   MLP_ALLOC(Xb, (size_t)B * kInPad);
   MLP_ALLOC(Xbt, (size_t)kInPad * B);
   MLP_ALLOC(Tb, (size_t)B * kOut);
-  MLP_ALLOC(Z1, (size_t)B * kHid);
-  MLP_ALLOC(Z2, (size_t)B * kHid);
-  MLP_ALLOC(Z3, (size_t)B * kHid);
-  MLP_ALLOC(Y, (size_t)B * kOut);
-  MLP_ALLOC(H1, (size_t)B * kHid);
-  MLP_ALLOC(H2, (size_t)B * kHid);
-  MLP_ALLOC(H3, (size_t)B * kHid);
-  MLP_ALLOC(H1t, (size_t)kHid * B);
-  MLP_ALLOC(H2t, (size_t)kHid * B);
-  MLP_ALLOC(H3t, (size_t)kHid * B);
-  MLP_ALLOC(dY, (size_t)B * kOutPad);
+  MLP_ALLOC(cnt, B / kGatherRows);
+  MLP_ALLOC(lossp, (size_t)B / kBM * 8);
+  for (int l = 0; l < 3; ++l) {
+    MLP_ALLOC(Z[l], (size_t)B * kHid);
+    MLP_ALLOC(At[l], (size_t)kHid * B);
+    MLP_ALLOC(dZt[l], (size_t)kHid * B);
+  }
   MLP_ALLOC(dYt, (size_t)kBM * B);
-  MLP_ALLOC(dZ1, (size_t)B * kHid);
-  MLP_ALLOC(dZ2, (size_t)B * kHid);
-  MLP_ALLOC(dZ3, (size_t)B * kHid);
-  MLP_ALLOC(dZ1t, (size_t)kHid * B);
-  MLP_ALLOC(dZ2t, (size_t)kHid * B);
-  MLP_ALLOC(dZ3t, (size_t)kHid * B);
 #undef MLP_ALLOC
   bool ok = e == cudaSuccess;
-  // B operands (weights): boxes of NT rows; A operands: 128-row boxes
+  // B operands: boxes of N rows; A operands: 128-row boxes
   ok = ok && make_map(&n->mW1, n->W1, kHid, kInPad, 256) && make_map(&n->mW2, n->W2, kHid, kHid, 256) &&
        make_map(&n->mW3, n->W3, kHid, kHid, 256) && make_map(&n->mW4, n->W4, kOut, kHid, 32) &&
-       make_map(&n->mW2t, n->W2t, kHid, kHid, 256) && make_map(&n->mW3t, n->W3t, kHid, kHid, 256) &&
-       make_map(&n->mW4t, n->W4t, kHid, kOutPad, 256);
-  ok = ok && make_map(&n->mX, n->Xb, B, kInPad, kBM) && make_map(&n->mXt, n->Xbt, kInPad, B, 128) &&
-       make_map(&n->mH1, n->H1, B, kHid, kBM) && make_map(&n->mH2, n->H2, B, kHid, kBM) &&
-       make_map(&n->mH3, n->H3, B, kHid, kBM) && make_map(&n->mH1t, n->H1t, kHid, B, 256) &&
-       make_map(&n->mH2t, n->H2t, kHid, B, 256) && make_map(&n->mH3t, n->H3t, kHid, B, 256) &&
-       make_map(&n->mdY, n->dY, B, kOutPad, kBM) && make_map(&n->mdYt, n->dYt, kBM, B, kBM) &&
-       make_map(&n->mdZ1t, n->dZ1t, kHid, B, kBM) && make_map(&n->mdZ2, n->dZ2, B, kHid, kBM) &&
-       make_map(&n->mdZ2t, n->dZ2t, kHid, B, kBM) && make_map(&n->mdZ3, n->dZ3, B, kHid, kBM) &&
-       make_map(&n->mdZ3t, n->dZ3t, kHid, B, kBM);
+       make_map(&n->mX, n->Xb, B, kInPad, kBM);
+  CUtensorMap* cw = n->chain.w;
+  ok = ok && make_map(&cw[4], n->W4t, kHid, kOutPad, 256) && make_map(&cw[5], n->W3t, kHid, kHid, 256) &&
+       make_map(&cw[6], n->W2t, kHid, kHid, 256);
+  cw[0] = n->mW1, cw[1] = n->mW2, cw[2] = n->mW3, cw[3] = n->mW4;
+  for (int l = 0; l < 3; ++l)
+    ok = ok && make_map(&n->wg.a[l], n->dZt[l], kHid, B, kBM) && make_map(&n->wg.b[l + 1], n->At[l], kHid, B, 256);
+  ok = ok && make_map(&n->wg.a[3], n->dYt, kBM, B, kBM) && make_map(&n->wg.b[0], n->Xbt, kInPad, B, 128);
   if (!ok) {
     free_mlp(n);
     delete n;
@@ -1065,7 +1265,7 @@ vrm_status vrm_mlp_grads(vrm_mlp* n, const uint16_t* X, const float* T, int32_t 
                          cudaStream_t s) {
   if (!n || !X || !T || rows < 1 || rows > n->B) return VRM_ERR_ARG;
   if (gather(n, reinterpret_cast<const bf16*>(X), T, nullptr, rows, s) != cudaSuccess) return VRM_ERR_CUDA;
-  if (forward_backward(n, s) != cudaSuccess) return VRM_ERR_CUDA;
+  if (forward_backward(n, s) != cudaSuccess || update(n, nullptr, s) != cudaSuccess) return VRM_ERR_CUDA;
   if (grad && cudaMemcpyAsync(grad, n->grad, sizeof(float) * kParams, cudaMemcpyDefault, s) != cudaSuccess)
     return VRM_ERR_CUDA;
   if (loss && cudaMemcpyAsync(loss, n->loss, sizeof(float) * 2, cudaMemcpyDefault, s) != cudaSuccess)
@@ -1077,15 +1277,19 @@ vrm_status vrm_mlp_train_step(vrm_mlp* n, const uint16_t* X_all, const float* T_
                               int32_t rows, const vrm_adamw* hp, int32_t t, float* loss, cudaStream_t s) {
   if (!n || !X_all || !T_all || rows < 1 || rows > n->B || t < 1 || !adamw_ok(hp)) return VRM_ERR_ARG;
   if (gather(n, reinterpret_cast<const bf16*>(X_all), T_all, batch_idx, rows, s) != cudaSuccess) return VRM_ERR_CUDA;
-  if (forward_backward(n, s) != cudaSuccess) return VRM_ERR_CUDA;
+  const AdamwArgs o = adamw_args(hp, t);
+  if (forward_backward(n, s) != cudaSuccess || update(n, &o, s) != cudaSuccess) return VRM_ERR_CUDA;
   if (loss && cudaMemcpyAsync(loss, n->loss, sizeof(float) * 2, cudaMemcpyDefault, s) != cudaSuccess)
     return VRM_ERR_CUDA;
-  return run_adamw(n, n->grad, hp, t, s);
+  return VRM_OK;
 }
 
 vrm_status vrm_mlp_adamw(vrm_mlp* n, const float* grad, const vrm_adamw* hp, int32_t t, cudaStream_t s) {
   if (!n || !grad || t < 1 || !adamw_ok(hp)) return VRM_ERR_ARG;
-  return run_adamw(n, grad, hp, t, s);
+  k_adamw<<<blocks_for_n(kParams, 256), 256, 0, s>>>(n->theta, n->m, n->v, grad, kParams, adamw_args(hp, t));
+  note_launch();
+  if (refresh(n, s) != cudaSuccess) return VRM_ERR_CUDA;
+  return cudaGetLastError() == cudaSuccess ? VRM_OK : VRM_ERR_CUDA;
 }
 
 vrm_status vrm_mlp_error(vrm_mlp* n, cudaStream_t s) {
