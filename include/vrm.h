@@ -125,7 +125,8 @@ typedef struct vrm_stats {
   int64_t lp_full_column_pivots; /* columns x pivots summed over them (their algorithmic work) */
   int64_t learned_screens; /* five-slot supports screened by the learned path (binary32 solves) */
   int64_t remove_candidates; /* vrm_remove_close: particles closer than r h to one of larger key */
-  int64_t lp_small_rechecked; /* of lp_small_solved: LPs whose binary32 pivot decisions were not all
+  int64_t lp_small_rechecked; /* of lp_small_solved: LPs whose binary32 pivot decisions (of pairs of
+                                 binary32 numbers in calls of at most 65,536 capacity) were not all
                                  certain and that were re-run with FP64 pivots (same result either way) */
 } vrm_stats;
 

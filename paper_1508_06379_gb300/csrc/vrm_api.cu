@@ -9,6 +9,7 @@
 // replayed on later calls; n and dt travel in a host-to-device copy at the
 // head of the graph.  When graph capture is unavailable the same kernels run
 // eagerly, rounds unrolled with a host check between them.
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -58,7 +59,8 @@ struct vrm::Scratch {
   RoundBufs rb = {};
   // neighbourhoods and weights of vrm_step
   int *nbr_count = nullptr, *nbr_idx = nullptr, *small = nullptr, *cols = nullptr, *fail_list = nullptr;
-  int* retry_list = nullptr;  // small LPs re-run in FP64
+  int* retry_list = nullptr;   // small LPs that the binary32 pivots hand back
+  int* retry_list2 = nullptr;  // LPs that the pairs of binary32 numbers hand back
   uint8_t *seg_mask = nullptr, *status = nullptr;
   double *f = nullptr, *fii = nullptr;
   // the stencils transposed per target (the application's lists, a CSR)
@@ -180,7 +182,7 @@ void free_scratch(Scratch& s) {
                   r.cy, r.keep, r.keep_s, r.apos,
                   r.cg.grid, r.cg.cell_key, r.cg.cell_rank, r.cg.cell_count, r.cg.cell_start, r.cg.sorted_idx,
                   r.cg.sorted_xy, r.cg.sorted_loc, r.cg.bbox, r.scan_tmp, s.nbr_count, s.nbr_idx, s.small, s.cols,
-                  s.fail_list, s.retry_list, s.seg_mask, s.status, s.f, s.fii, s.tcount, s.toff, s.tent, s.ds,
+                  s.fail_list, s.retry_list, s.retry_list2, s.seg_mask, s.status, s.f, s.fii, s.tcount, s.toff, s.tent, s.ds,
                   s.counters, s.st};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -391,7 +393,7 @@ cudaError_t enqueue_stage_weights(vrm_ctx* ctx, const double* x, const double* y
     lp_list = ctx->L.rlist;
     lp_count = s.counters + 2;
   }
-  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list, s.ds,
+  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list, s.retry_list2, s.ds,
                     0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
     return e;
   if (!rows && (e = search_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key,
@@ -399,7 +401,7 @@ cudaError_t enqueue_stage_weights(vrm_ctx* ctx, const double* x, const double* y
                                     s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, st, true)) != cudaSuccess)
     return e;
   return lp_full(c, x, y, s.fail_list, &s.ds->n_fail, cap, s.nbr_count, s.nbr_idx, s.cols, s.f, s.fii, s.status,
-                 s.retry_list, s.ds, 0.0, st, &s.st->dt, ctx->p.nu);
+                 s.retry_list2, s.ds, 0.0, st, &s.st->dt, ctx->p.nu);
 }
 
 // Scratch for `cap` particles (grown by 25% steps, never shrunk).
@@ -475,6 +477,7 @@ cudaError_t ensure_scratch(vrm_ctx* ctx, int cap, cudaStream_t st) {
   VRM_ALLOC(s.cols, (long)n * ctx->c.w);
   VRM_ALLOC(s.fail_list, n);
   VRM_ALLOC(s.retry_list, n);
+  VRM_ALLOC(s.retry_list2, n);
   VRM_ALLOC(s.seg_mask, n);
   VRM_ALLOC(s.status, n);
   VRM_ALLOC(s.f, (long)n * ctx->c.w);
@@ -697,7 +700,7 @@ cudaError_t enqueue_back(vrm_ctx* ctx, double* x, double* y, int cap, const doub
     lp_list = ctx->L.rlist;
     lp_count = s.counters + 2;
   }
-  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list, s.ds,
+  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list, s.retry_list2, s.ds,
                     0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
     return e;
   if ((e = mark(ctx, VRM_STAGE_LP_FULL, st)) != cudaSuccess) return e;
@@ -706,7 +709,7 @@ cudaError_t enqueue_back(vrm_ctx* ctx, double* x, double* y, int cap, const doub
                                     s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, st, true)) != cudaSuccess)
     return e;
   if ((e = lp_full(c, x, y, s.fail_list, &s.ds->n_fail, cap, s.nbr_count, s.nbr_idx, s.cols, s.f, s.fii, s.status,
-                   s.retry_list, s.ds, 0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
+                   s.retry_list2, s.ds, 0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
     return e;
   if ((e = mark(ctx, VRM_STAGE_APPLY, st)) != cudaSuccess) return e;
   if ((e = apply_transposed_dev(c, cap, n_cur, cap, &s.st->n, gamma_in, s.diffused, s.dlist, s.counters + 0, s.cols,
@@ -1087,10 +1090,10 @@ vrm_status vrm_solve_weights(vrm_ctx* ctx, const double* x, const double* y, int
     lp_list = ctx->L.rlist;
     lp_count = s.counters + 2;
   }
-  VRM_CUDA(lp_small(c, x, y, lp_list, lp_count, n, small, cols, f, fii, status, s.fail_list, s.retry_list, s.ds,
+  VRM_CUDA(lp_small(c, x, y, lp_list, lp_count, n, small, cols, f, fii, status, s.fail_list, s.retry_list, s.retry_list2, s.ds,
                       0.0, stream));
   VRM_CUDA(lp_full(c, x, y, s.fail_list, &s.ds->n_fail, n, nbr_count, nbr_idx, cols, f, fii, status,
-                   s.retry_list, s.ds, 0.0, stream));
+                   s.retry_list2, s.ds, 0.0, stream));
   if (stats) {
     VRM_CUDA(read_back(ctx, stream));
     stats->n_in = stats->n_out = n;
@@ -1665,6 +1668,8 @@ extern "C" vrm_status vrm_step_batched(vrm_batch* b, vrm_cloud* clouds, int32_t 
   if (!active) return VRM_ERR_CUDA;
   vrm_status result = VRM_OK;
   bool hit = b->exec != nullptr;
+  long load = 0;  // the clouds run at the same time
+  for (int c = 0; c < n_clouds; ++c) load += clouds[c].n > 0 ? clouds[c].capacity : 0;
   VRM_CUDA(cudaStreamSynchronize(stream));
   for (int c = 0; c < n_clouds && result == VRM_OK; ++c) {
     vrm_cloud& C = clouds[c];
@@ -1699,6 +1704,7 @@ extern "C" vrm_status vrm_step_batched(vrm_batch* b, vrm_cloud* clouds, int32_t 
     P.dt = C.dt;
     P.max_rounds = ctx->p.max_rounds;
     *ctx->s.h_params = P;
+    ctx->c.lp_load = (int)(load < INT_MAX ? load : INT_MAX);
     const BatchKey& K = b->key[c];
     hit = hit && K.x == C.x && K.y == C.y && K.gi == C.gamma_in && K.go == C.gamma_out && K.cap == C.capacity &&
           K.h == C.h && K.scratch_gen == ctx->scratch_gen;

@@ -41,6 +41,8 @@ struct Consts {
   int lp_blocks_per_sm;  // grid cap of k_lp_small
   int lp_fp64_pivots;    // 1: small LPs pivot in FP64; 0: certified binary32 pivots, FP64 re-runs
   int apply_block;       // threads per block of k_apply
+  // capacity of all clouds that run at the same time (a batch), 0: this one's
+  int lp_load;
 };
 
 // The schedule every context starts with.
@@ -88,8 +90,9 @@ struct DevStats {
   unsigned long long learned_screens;        // supports screened by the learned path
   unsigned long long lp_full_columns;        // columns summed over the full-neighbourhood LPs
   unsigned long long lp_full_column_pivots;  // columns x pivots summed over them
-  int n_retry;                               // retry list of the current small-LP pass (FP64 re-runs)
-  unsigned long long lp_small_retries;       // small LPs re-run in FP64 (uncertain binary32 decision)
+  int n_retry;                               // LPs of the current pass that the binary32 pivots handed back
+  int n_retry_pairs;                         // ... and that the pairs handed back (FP64 re-runs)
+  unsigned long long lp_small_retries;       // small LPs handed back by the first certified pivots (n = 1)
 };
 
 // Growth-control selection state (device resident).
@@ -369,11 +372,11 @@ cudaError_t rounds_finish(StepState* st, const RoundBufs& rb, int cap, cudaStrea
 // nu_dt = nu * dt for the stability statistic; with dt_dev it is nu * *dt_dev.
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
-                     int* retry_list,
+                     int* retry_list, int* retry_list2,
                      DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev = nullptr, double nu = 0.0);
 cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int* fail_list, const int* fail_count,
                     int cap, const int* nbr_count, const int* nbr_idx, int* cols, double* f, double* fii,
-                    uint8_t* status, int* retry_list, DevStats* ds, double nu_dt, cudaStream_t s,
+                    uint8_t* status, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,
                     const double* dt_dev = nullptr, double nu = 0.0);
 // Identity weights of the removal candidates (list, *list_count on the
 // device): removed[i], cols4/w4 [n x 4] (vrm_remove.cu drives it).

@@ -29,11 +29,12 @@
 // For n = 1 the default kernel, k_lp_small32, pivots in binary32 with
 // certified decisions and keeps FP64 for the column offsets and the final
 // basis solve (see the section before it); k_lp_small re-runs the particles
-// it hands back, and serves the FP64-pivot schedule.  For n = 2 both LPs run
+// it hands back, and serves the FP64-pivot schedule.  Small clouds' LPs and,
+// for n = 2, both LPs run
 // in two parts: the pivots one particle per warp or half-warp in pairs of
 // binary32 numbers with certified decisions (k_lp_df; k_lp_full re-runs in
 // FP64 what it hands back), then the FP64 solve of the final bases one
-// particle per thread (k_lp9_finish).
+// particle per thread (k_lp_finish).
 #include <climits>
 
 #include "vrm_internal.cuh"
@@ -1271,26 +1272,38 @@ __device__ __forceinline__ void lu_rows(double (&A)[M], double& z, double (&rcpd
   }
 }
 
-// Final basis of an n = 2 LP, kept in the particle's row of cols until
-// k_lp9_finish turns it into the stencil: entries 0..8 hold the particles of
-// the basic columns (-1 for an artificial), entries 9 and 10 the basic
-// variables (6 bits each: row r's artificial r or 9 + the column's rank),
-// the code and the pivot count.  Lane r < 9 of the group of G lanes holds
-// row r's variable and particle.
-template <int G>
-__device__ __forceinline__ void lp9_record(int* row, int gl, int var, int j, int code, int it) {
-  unsigned w0 = (unsigned)code << 30, w1 = (unsigned)it << 24;
+// Final basis of an LP, kept in the particle's row of cols until k_lp_finish
+// turns it into the stencil: entries 0..m-1 hold the particles of the basic
+// columns (-1 for an artificial), the next ones the basic variables (row r's
+// artificial r or m + the column's rank), the code and the pivot count: two
+// entries of 6-bit variables for m = 9, one of 4-bit ones for m = 5.  Lane
+// r < m of the group of G lanes holds row r's variable and particle.
+template <int M, int G>
+__device__ __forceinline__ void lp_record(int* row, int gl, int var, int j, int code, int it) {
+  unsigned w0 = M == 9 ? (unsigned)code << 30 : (unsigned)code << 30 | (unsigned)it << 20;
+  unsigned w1 = (unsigned)it << 24;
 #pragma unroll
-  for (int r = 0; r < 9; ++r) {
+  for (int r = 0; r < M; ++r) {
     const unsigned v = (unsigned)__shfl_sync(0xffffffffu, var, r, G);
-    if (r < 5)
+    if (M == 5)
+      w0 |= v << (4 * r);
+    else if (r < 5)
       w0 |= v << (6 * r);
     else
       w1 |= v << (6 * (r - 5));
   }
-  if (gl < 9) row[gl] = j;
-  if (gl == 9) row[9] = (int)w0;
-  if (gl == 10) row[10] = (int)w1;
+  if (gl < M) row[gl] = j;
+  if (gl == M) row[M] = (int)w0;
+  if (M == 9 && gl == M + 1) row[M + 1] = (int)w1;
+}
+template <int M>
+__device__ __forceinline__ void lp_recorded(const int* row, int (&basis)[M], int& code, int& it) {
+  const unsigned w0 = (unsigned)row[M], w1 = M == 9 ? (unsigned)row[M == 9 ? M + 1 : M] : w0;
+  code = (int)(w0 >> 30);
+  it = M == 9 ? (int)(w1 >> 24) : (int)(w0 >> 20 & 127u);
+#pragma unroll
+  for (int r = 0; r < M; ++r)
+    basis[r] = M == 5 ? (int)(w0 >> (4 * r) & 15u) : (int)((r < 5 ? w0 >> (6 * r) : w1 >> (6 * (r - 5))) & 63u);
 }
 
 // Full-neighbourhood retry: one warp per particle.  Lane l holds tableau
@@ -1302,8 +1315,9 @@ __device__ __forceinline__ void lp9_record(int* row, int gl, int var, int j, int
 // swaps, multipliers times the pivot's reciprocal, separately rounded
 // updates), forward substitution in column order, back substitution row by
 // row; the result is bit-identical to the oracle's basis solve.
-// For n = 2 (M = 9) the kernel stops at the final basis and leaves it in the
-// particle's stencil row (lp9_record), for k_lp9_finish.
+// For n = 2 (M = 9) and for the columns of small neighbourhoods (small given)
+// the kernel stops at the final basis and leaves it in the particle's stencil
+// row (lp_record), for k_lp_finish.
 template <int M, int W>
 __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restrict__ x,
                                                  const double* __restrict__ y, const int* __restrict__ fail_list,
@@ -1327,15 +1341,15 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
   double st_ratio = 0.0;
   for (long t = warp; t < m; t += nwarps) {
     const int i = fail_list[t];
-    // small (n = 2 only): the columns are the small neighbourhood's, an empty
-    // slot sorts last as a zero column, which never enters
-    const int cnt = M == 9 && small ? 8 : nbr_count[i];
+    // small: the columns are the small neighbourhood's, an empty slot sorts
+    // last as a zero column, which never enters
+    const int cnt = small ? 8 : nbr_count[i];
     const int K = cnt < c.row_cap ? cnt : c.row_cap;
     const double xi0 = x[i], yi0 = y[i];
     double d2 = 1e300, dx = 0.0, dy = 0.0;
     int j = INT_MAX;
-    if (lane < K) j = M == 9 && small ? small[(size_t)i * 8 + lane] : nbr_idx[(size_t)i * c.k_cap + lane];
-    if (M == 9 && j < 0) j = INT_MAX;
+    if (lane < K) j = small ? small[(size_t)i * 8 + lane] : nbr_idx[(size_t)i * c.k_cap + lane];
+    if (j < 0) j = INT_MAX;
     if (j != INT_MAX) {
       dx = __dsub_rn(x[j], xi0);
       dy = __dsub_rn(y[j], yi0);
@@ -1453,9 +1467,9 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
       if (lane == leave) bas = M + q;
       ++it;
     }
-    if constexpr (M == 9) {
+    if (M == 9 || small) {
       const int bj = __shfl_sync(kAll, j, bas >= M && bas != INT_MAX ? bas - M : 0);
-      lp9_record<32>(cols + (size_t)i * W, lane, bas, bas >= M ? bj : -1, code, it);
+      lp_record<M, 32>(cols + (size_t)i * W, lane, bas, bas >= M ? bj : -1, code, it);
       continue;
     }
     // basic solution of the final basis by the oracle's LU sequence, row r of
@@ -1586,7 +1600,7 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
 }
 
 // ---------------------------------------------------------------------------
-// n = 2: certified pivots in pairs of binary32 numbers.  The nine-row LPs
+// Certified pivots in pairs of binary32 numbers.  The nine-row LPs
 // take 8 (small) and 11 pivots (full neighbourhoods, 20 columns) on jittered
 // clouds, and running binary32 bounds outgrow the entries after about eight
 // pivots (25% of the full LPs certified); in FP64 the pivots of one LP take
@@ -1667,21 +1681,23 @@ constexpr float kDfFma = 24.0f * kU2, kDfMul = 24.0f * kU2;
 // One LP per group of G lanes: lane k of the group holds tableau column k
 // (unsorted; `rank` is its place in the order (d2, j)), and row r's
 // right-hand side, basic variable and ratio are on lane r < 9.  The final
-// basis goes to the particle's row of cols (lp9_record), an LP with an
-// uncertain decision to the retry list.  G = 32: full neighbourhoods (FULL);
-// G = 16: the small ones, two per warp (8 of the lanes hold columns, 9 hold
-// rows), which run in step until both are done.
-template <int G, bool FULL>
+// basis goes to the particle's row of cols (lp_record), an LP with an
+// uncertain decision to the retry list.  n = 2: G = 32 for the full
+// neighbourhoods (FULL), G = 16 for the small ones, two per warp (8 of the
+// lanes hold columns, 9 hold rows); n = 1: G = 8, four small LPs per warp, for
+// the LPs of small clouds, where the latency of one LP counts (lp_small).  The
+// LPs of a warp run in step until all are done.
+template <int M, int G, bool FULL>
 __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restrict__ x, const double* __restrict__ y,
                                                const int* __restrict__ list, const int* __restrict__ list_count,
                                                const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
                                                const int* __restrict__ small, int* __restrict__ cols,
-                                               int* __restrict__ retry_list, DevStats* __restrict__ ds) {
-  constexpr int M = 9, W = VRM_STENCIL_W2;
+                                               int* __restrict__ retry_list, DevStats* __restrict__ ds, bool count_retries) {
+  constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int kNone = 1 << 20;
   const int lane = threadIdx.x & 31, gl = lane & (G - 1), gbase = lane & ~(G - 1);
-  const unsigned gmask = G == 32 ? kAll : (0xffffu << gbase);
+  const unsigned gmask = (kAll >> (32 - G)) << gbase;
   auto ballot = [&](bool v) { return (__ballot_sync(kAll, v) & gmask) >> gbase; };
   __shared__ float4 s_col[2][128 / G][M + 1];
   unsigned it_all = 0;
@@ -1723,10 +1739,12 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       T[2] = df_mul(xi, xi);
       T[3] = df_mul(xi, eta);
       T[4] = df_mul(eta, eta);
-      T[5] = df_mul(T[2], xi);
-      T[6] = df_mul(T[2], eta);
-      T[7] = df_mul(xi, T[4]);
-      T[8] = df_mul(T[4], eta);
+      if constexpr (M == 9) {
+        T[5] = df_mul(T[2], xi);
+        T[6] = df_mul(T[2], eta);
+        T[7] = df_mul(xi, T[4]);
+        T[8] = df_mul(T[4], eta);
+      }
       Df sum = {0.0f, 0.0f};
       float sa = 0.0f, se = 0.0f;
 #pragma unroll
@@ -1812,7 +1830,7 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       // possible tie limit does not matter
       const bool amb_matters =
           amb && !(__fmul_rn(__fsub_rn(rhs.h, mb), 1.0f - 8.0f * kU32) > __fmul_rn(limhi, __fadd_rn(am.h, mg)));
-      // (every vote outside the branches: the warp's two groups may differ)
+      // (every vote outside the branches: the warp's groups may differ)
       bool no = ballot(bad_row) != 0;
       const bool any_matters = ballot(amb_matters) != 0;
       if (elm == 0) {
@@ -1912,18 +1930,21 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       }
       run = go;
     }
-    if (have && unc && gl == 0) retry_list[atomicAdd(&ds->n_retry, 1)] = i;
-    lp9_record<G>(cols + (size_t)i * W, have && !unc ? gl : G, bas, bj, code, it);
+    if (have && unc && gl == 0) {
+      retry_list[atomicAdd(&ds->n_retry_pairs, 1)] = i;
+      if (count_retries) atomicAdd(&ds->lp_small_retries, 1ull);
+    }
+    lp_record<M, G>(cols + (size_t)i * W, have && !unc ? gl : G, bas, bj, code, it);
   }
 }
 
-// The stencils of the n = 2 LPs from their final bases (lp9_record): the
+// The stencils of recorded LPs from their final bases (lp_record): the
 // oracle's LU solve (basis_solve), feasibility and the weights in column
-// order, as lp_finish does for n = 1.  One particle per thread: solved row
-// by row across a warp's lanes the 9 x 9 system takes the FP64 pipe about 300
-// warp instructions per particle, here 900 per 32.
-template <bool FULL>
-__global__ void __launch_bounds__(64) k_lp9_finish(Consts c, const double* __restrict__ x,
+// order, as lp_finish does.  One particle per thread: solved row by row across
+// a warp's lanes the 9 x 9 system takes the FP64 pipe about 300 warp
+// instructions per particle, here 900 per 32.
+template <int M, bool FULL>
+__global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __restrict__ x,
                                                    const double* __restrict__ y, const int* __restrict__ list,
                                                    const int* __restrict__ list_count,
                                                    const int* __restrict__ nbr_count, int* __restrict__ cols,
@@ -1931,7 +1952,7 @@ __global__ void __launch_bounds__(64) k_lp9_finish(Consts c, const double* __res
                                                    uint8_t* __restrict__ status, int* __restrict__ fail_list,
                                                    DevStats* __restrict__ ds, double nu_dt,
                                                    const double* __restrict__ dt_dev, double nu) {
-  constexpr int M = 9, W = VRM_STENCIL_W2;
+  constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W;
   if (dt_dev) nu_dt = nu * *dt_dev;
   const int m = *list_count;
   const double inv_h2 = 1.0 / (c.h * c.h);
@@ -1945,15 +1966,12 @@ __global__ void __launch_bounds__(64) k_lp9_finish(Consts c, const double* __res
       const int i = list[t];
       int* const crow = cols + (size_t)i * W;
       double* const frow = f + (size_t)i * W;
-      const unsigned w0 = (unsigned)crow[9], w1 = (unsigned)crow[10];
-      int code = (int)(w0 >> 30);
-      const int it = (int)(w1 >> 24);
-      int basis[M];
+      int basis[M], code, it;
+      lp_recorded<M>(crow, basis, code, it);
       double bxi[M], beta[M], pj[M];
       const double xi0 = x[i], yi0 = y[i];
 #pragma unroll
       for (int r = 0; r < M; ++r) {
-        basis[r] = (int)((r < 5 ? w0 >> (6 * r) : w1 >> (6 * (r - 5))) & 63u);
         const int j = crow[r];
         pj[r] = __longlong_as_double((long long)j);
         const bool s = basis[r] >= M;
@@ -2277,66 +2295,92 @@ __global__ void k_lp_clear(int n, int w, const uint8_t* __restrict__ diffused, i
   }
 }
 
-// The n = 2 LPs of a list: small neighbourhoods (small given) or full ones.
-static cudaError_t lp9(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
-                       int cap, const int* nbr_count, const int* nbr_idx, const int* small, int* cols, double* f,
-                       double* fii, uint8_t* status, int* fail_list, int* retry_list, DevStats* ds, double nu_dt,
-                       cudaStream_t s, const double* dt_dev, double nu) {
+// The LPs of a list in pairs of binary32 numbers (small neighbourhoods, or
+// for n = 2 full ones: small null), the uncertain ones in FP64, then the final
+// solves.  fp64: every LP in FP64.  ds->n_retry_pairs is 0 on entry.
+template <int M>
+static cudaError_t lp_pairs(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
+                            int cap, const int* nbr_count, const int* nbr_idx, const int* small, int* cols, double* f,
+                            double* fii, uint8_t* status, int* fail_list, int* retry_list, DevStats* ds, double nu_dt,
+                            cudaStream_t s, const double* dt_dev, double nu, bool fp64, bool count_retries) {
+  constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W, G = M == 9 ? 16 : 8;
   const int sms = sm_count();
   auto grid = [&](long per_block, int per_sm) {
     const long b = ((long)cap + per_block - 1) / per_block, most = (long)per_sm * sms;
     return (int)(b < most ? b : most);
   };
-  if (c.lp_fp64_pivots) {
-    k_lp_full<9, 12><<<grid(4, 4), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols, f, fii,
-                                                status, ds, nu_dt, dt_dev, nu);
-    note_launch();
-  } else {
-    const cudaError_t e = cudaMemsetAsync(&ds->n_retry, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    if (small)
-      k_lp_df<16, false><<<grid(8, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
-                                                     retry_list, ds);
+  if (!fp64) {
+    if (M == 5 || small)
+      k_lp_df<M, G, false><<<grid(128 / G, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small,
+                                                             cols, retry_list, ds, count_retries);
     else
-      k_lp_df<32, true><<<grid(4, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
-                                                    retry_list, ds);
+      k_lp_df<9, 32, true><<<grid(4, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
+                                                       retry_list, ds, false);
     note_launch();
-    k_lp_full<9, 12><<<grid(4, 4), 128, 0, s>>>(c, x, y, retry_list, &ds->n_retry, nbr_count, nbr_idx, small, cols, f,
-                                                fii, status, ds, nu_dt, dt_dev, nu);
-    note_launch();
+    list = retry_list;
   }
-  if (small)
-    k_lp9_finish<false><<<grid(64, 16), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii, status,
-                                                    fail_list, ds, nu_dt, dt_dev, nu);
-  else
-    k_lp9_finish<true><<<grid(64, 16), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii, status,
-                                                   fail_list, ds, nu_dt, dt_dev, nu);
+  const int* const all = list_count;
+  k_lp_full<M, W><<<grid(4, 4), 128, 0, s>>>(c, x, y, list, fp64 ? all : &ds->n_retry_pairs, nbr_count, nbr_idx, small,
+                                             cols, f, fii, status, ds, nu_dt, dt_dev, nu);
+  note_launch();
+  return cudaGetLastError();
+}
+template <int M, bool FULL>
+static cudaError_t lp_finish_list(const Consts& c, const double* x, const double* y, const int* list,
+                                  const int* list_count, int cap, const int* nbr_count, int* cols, double* f,
+                                  double* fii, uint8_t* status, int* fail_list, DevStats* ds, double nu_dt,
+                                  cudaStream_t s, const double* dt_dev, double nu) {
+  const long b = ((long)cap + 63) / 64, most = 16L * sm_count();
+  k_lp_finish<M, FULL><<<(int)(b < most ? b : most), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii,
+                                                                 status, fail_list, ds, nu_dt, dt_dev, nu);
   note_launch();
   return cudaGetLastError();
 }
 
+// Largest particle capacities whose n = 1 LPs all go to the pairs kernel, eight
+// lanes per LP, and whose hand-backs do.  One LP per thread takes 32 us in
+// binary32 and 43 for the re-run of a few in FP64 however few they are, the
+// pairs and their solves 35 for all; but they take seven times the
+// instructions.  Steps of 3,600, 20,449 and 32,400 particles: 290, 323 and 386
+// us with all LPs in pairs, 346, 371 and 409 with binary32 and FP64 (65,536:
+// 435 and 446, 90,000: 511 and 483).  Hand-backs in pairs: 423, 474, 509 and
+// 578 us at 65,536, 90,000, 129,600 and 184,900 particles against 446, 483,
+// 531 and 582, but 1,675 against 1,664 at a million.  The capacity is what the
+// host knows; twice the particles is usual.  The clouds of a batch run at the
+// same time, so the sum of their capacities counts there (32 clouds of 10,000
+// to 300,000 particles: 4.49 ms, 4.60 when each went by its own).
+constexpr int kPairsCap = 65536;
+constexpr int kPairsRetryCap = 6 * 65536;
+
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
-                     int* retry_list, DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev, double nu) {
+                     int* retry_list, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,
+                     const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(&ds->n_retry, 0, 2 * sizeof(int), s);  // n_retry and n_retry_pairs
+  if (e != cudaSuccess) return e;
+  if (c.order == 2) {
+    e = lp_pairs<9>(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list,
+                    retry_list2, ds, nu_dt, s, dt_dev, nu, c.lp_fp64_pivots != 0, false);
+    if (e != cudaSuccess) return e;
+    return lp_finish_list<9, false>(c, x, y, list, list_count, cap, nullptr, cols, f, fii, status, fail_list, ds,
+                                    nu_dt, s, dt_dev, nu);
+  }
   // lp_block = kLpWsThreads or kLpWsThreadsWide selects the warp-specialised
   // binary32 LP; the other LP kernels then run with 128 threads per block
   const bool ws = c.lp_block == kLpWsThreads || c.lp_block == kLpWsThreadsWide;
   const int tb = ws ? 128 : c.lp_block;
   int blocks = (int)(((long)cap + tb - 1) / tb);
   if (blocks > c.lp_blocks_per_sm * sm_count()) blocks = c.lp_blocks_per_sm * sm_count();
-  if (c.order == 2) {
-    const cudaError_t e = lp9(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list,
-                              retry_list, ds, nu_dt, s, dt_dev, nu);
-    if (e != cudaSuccess) return e;
-  } else if (c.lp_fp64_pivots || !(c.inv_h > 1e-20 && c.inv_h < 1e20)) {
+  if (c.lp_fp64_pivots || !(c.inv_h > 1e-20 && c.inv_h < 1e20)) {
     k_lp_small<5, 8><<<blocks, tb, 0, s>>>(c, x, y, list, list_count, small, cols, f, fii, status, fail_list, ds,
                                            nu_dt, dt_dev, nu);
     note_launch();
-  } else {
-    // certified binary32 pivots, then the uncertain particles in FP64
-    cudaError_t e = cudaMemsetAsync(&ds->n_retry, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+  }
+  const int load = c.lp_load > cap ? c.lp_load : cap;
+  if (load > kPairsCap) {
+    // certified binary32 pivots, then the uncertain particles in pairs or in FP64
     if (c.lp_block == kLpWsThreads) {
       // warp-specialised form, 4 + 2 warps: two resident blocks per SM
       k_lp_small32_ws<5, 8, 4, 2, 2><<<2 * sm_count(), kLpWsThreads, 0, s>>>(
@@ -2350,25 +2394,40 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
                                                retry_list, ds, nu_dt, dt_dev, nu);
     }
     note_launch();
-    // the re-run list is a few percent of the LPs: one-warp blocks spread it
-    // over every SM instead of over the first few hundred blocks
-    int rblocks = (int)(((long)cap + 31) / 32);
-    if (rblocks > 32 * sm_count()) rblocks = 32 * sm_count();
-    k_lp_small<5, 8><<<rblocks, 32, 0, s>>>(c, x, y, retry_list, &ds->n_retry, small, cols, f, fii, status,
-                                           fail_list, ds, nu_dt, dt_dev, nu);
-    note_launch();
+    if (load > kPairsRetryCap) {
+      // the re-run list is a few percent of the LPs: one-warp blocks spread it
+      // over every SM instead of over the first few hundred blocks
+      int rblocks = (int)(((long)cap + 31) / 32);
+      if (rblocks > 32 * sm_count()) rblocks = 32 * sm_count();
+      k_lp_small<5, 8><<<rblocks, 32, 0, s>>>(c, x, y, retry_list, &ds->n_retry, small, cols, f, fii, status,
+                                              fail_list, ds, nu_dt, dt_dev, nu);
+      note_launch();
+      return cudaGetLastError();
+    }
+    list = retry_list;
+    list_count = &ds->n_retry;
   }
-  return cudaGetLastError();
+  e = lp_pairs<5>(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list, retry_list2,
+                  ds, nu_dt, s, dt_dev, nu, false, load <= kPairsCap);
+  if (e != cudaSuccess) return e;
+  return lp_finish_list<5, false>(c, x, y, list, list_count, cap, nullptr, cols, f, fii, status, fail_list, ds, nu_dt,
+                                  s, dt_dev, nu);
 }
 
 cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int* fail_list, const int* fail_count,
                     int cap, const int* nbr_count, const int* nbr_idx, int* cols, double* f, double* fii,
-                    uint8_t* status, int* retry_list, DevStats* ds, double nu_dt, cudaStream_t s,
+                    uint8_t* status, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,
                     const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
-  if (c.order == 2)
-    return lp9(c, x, y, fail_list, fail_count, cap, nbr_count, nbr_idx, nullptr, cols, f, fii, status, nullptr,
-               retry_list, ds, nu_dt, s, dt_dev, nu);
+  if (c.order == 2) {
+    cudaError_t e = cudaMemsetAsync(&ds->n_retry_pairs, 0, sizeof(int), s);
+    if (e == cudaSuccess)
+      e = lp_pairs<9>(c, x, y, fail_list, fail_count, cap, nbr_count, nbr_idx, nullptr, cols, f, fii, status, nullptr,
+                      retry_list2, ds, nu_dt, s, dt_dev, nu, c.lp_fp64_pivots != 0, false);
+    if (e != cudaSuccess) return e;
+    return lp_finish_list<9, true>(c, x, y, fail_list, fail_count, cap, nbr_count, cols, f, fii, status, nullptr, ds,
+                                   nu_dt, s, dt_dev, nu);
+  }
   long warps = cap;
   long blocks = (warps * 32 + 127) / 128;
   if (blocks > 4 * sm_count()) blocks = 4 * sm_count();
