@@ -640,26 +640,46 @@ cudaError_t enqueue_front(vrm_ctx* ctx, double* x, double* y, int cap, const dou
   const int* n_dev = &s.st->n;
   cudaError_t e;
   if ((e = mark(ctx, VRM_STAGE_REDUCE, st)) != cudaSuccess) return e;
-  // the growth control's first pass also takes the bounding box of the
-  // particles for the grid build below
-  if ((e = reduce_select_dev(gamma, cap, n_dev, c.c_bound, diffused, s.rstate, s.tie_flag, s.tie_rank, s.scan_tmp,
-                             s.ds, st, s.dflag_ts, s.tie_ts, x, y, s.bbox)) != cudaSuccess)
-    return e;
-  if ((e = compact_flags_dev(diffused, cap, n_dev, s.dlist, s.counters + 0, s.pos, s.scan_tmp, st, s.dflag_ts)) !=
-      cudaSuccess)
-    return e;
-  if ((e = mark(ctx, VRM_STAGE_GRID, st)) != cudaSuccess) return e;
-  if ((e = grid_build_dev(x, y, cap, n_dev, c.Rh, c.lo2, c.hi2, s.ncell_cap, s.grid, s.cell_key, s.cell_rank,
-                          s.cell_count, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.bbox, s.scan_tmp,
-                          st, s.cell_ts, true, true)) != cudaSuccess)
-    return e;
+  if (cap <= kSmallCap) {
+    if ((e = front_small(gamma, x, y, cap, n_dev, c.c_bound, c.Rh, c.lo2, c.hi2, s.ncell_cap, diffused, s.dlist,
+                         s.counters + 0, s.ds, s.grid, s.cell_count, s.cell_ts, st)) != cudaSuccess)
+      return e;
+    if ((e = mark(ctx, VRM_STAGE_GRID, st)) != cudaSuccess) return e;
+    if ((e = grid_bin_dev(x, y, cap, n_dev, s.ncell_cap, s.grid, s.cell_key, s.cell_rank, s.cell_count, s.cell_start,
+                          s.sorted_xy, s.sorted_loc, s.sorted_idx, s.scan_tmp, st, s.cell_ts, true)) != cudaSuccess)
+      return e;
+  } else {
+    // the growth control's first pass also takes the bounding box of the
+    // particles for the grid build below
+    if ((e = reduce_select_dev(gamma, cap, n_dev, c.c_bound, diffused, s.rstate, s.tie_flag, s.tie_rank, s.scan_tmp,
+                               s.ds, st, s.dflag_ts, s.tie_ts, x, y, s.bbox)) != cudaSuccess)
+      return e;
+    if ((e = compact_flags_dev(diffused, cap, n_dev, s.dlist, s.counters + 0, s.pos, s.scan_tmp, st, s.dflag_ts)) !=
+        cudaSuccess)
+      return e;
+    if ((e = mark(ctx, VRM_STAGE_GRID, st)) != cudaSuccess) return e;
+    if ((e = grid_build_dev(x, y, cap, n_dev, c.Rh, c.lo2, c.hi2, s.ncell_cap, s.grid, s.cell_key, s.cell_rank,
+                            s.cell_count, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.bbox, s.scan_tmp,
+                            st, s.cell_ts, true, true)) != cudaSuccess)
+      return e;
+  }
   if ((e = search_masks_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key,
                                  s.cell_rank, s.dlist, s.counters + 0, cap, s.mask, st)) != cudaSuccess)
     return e;
-  if ((e = open_list(s.dlist, s.counters + 0, cap, s.mask, s.rb.keep_flag, s.pos, s.rb.open, s.counters + 1,
-                     s.rb.keep_ts, st)) != cudaSuccess)
+  // (small clouds: with the state of the rounds, enqueue_rounds_init)
+  if (cap > kSmallCap && (e = open_list(s.dlist, s.counters + 0, cap, s.mask, s.rb.keep_flag, s.pos, s.rb.open,
+                                        s.counters + 1, s.rb.keep_ts, st)) != cudaSuccess)
     return e;
   return mark(ctx, VRM_STAGE_INSERT, st);
+}
+
+// State of the insertion rounds (enqueue_front has run).
+cudaError_t enqueue_rounds_init(vrm_ctx* ctx, int cap, cudaGraphConditionalHandle handle, bool graph,
+                                cudaStream_t st) {
+  Scratch& s = ctx->s;
+  if (cap <= kSmallCap)
+    return open_small(s.dlist, s.counters + 0, s.mask, s.counters + 1, s.rb, s.st, handle, graph, st);
+  return rounds_init(s.st, s.counters + 1, s.rb, s.mask, cap, handle, graph, st);
 }
 
 // Final grid, neighbourhoods, weights, application + Euler, statistics copy.
@@ -749,7 +769,7 @@ bool record_step(vrm_ctx* ctx, cudaStream_t cs, cudaStream_t body_stream, double
     ok = cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, nullptr, nullptr, nullptr) == cudaSuccess;
     ok = ok && cudaGraphConditionalHandleCreate(&handle, cg, 0, cudaGraphCondAssignDefault) == cudaSuccess;
   }
-  ok = ok && rounds_init(s.st, s.counters + 1, s.rb, s.mask, cap, handle, true, cs) == cudaSuccess;
+  ok = ok && enqueue_rounds_init(ctx, cap, handle, true, cs) == cudaSuccess;
   if (ok) {
     cudaStreamCaptureStatus status;
     cudaGraph_t cg = nullptr;
@@ -833,7 +853,7 @@ vrm_status run_step_eager(vrm_ctx* ctx, double* x, double* y, int cap, const dou
   Scratch& s = ctx->s;
   VRM_CUDA(enqueue_head(ctx, st));
   VRM_CUDA(enqueue_front(ctx, x, y, cap, gamma_in, diffused, st));
-  VRM_CUDA(rounds_init(s.st, s.counters + 1, s.rb, s.mask, cap, 0, false, st));
+  VRM_CUDA(enqueue_rounds_init(ctx, cap, 0, false, st));
   for (int r = 0; r < ctx->p.max_rounds; ++r) {
     VRM_CUDA(cudaMemcpyAsync(s.h_state, s.st, sizeof(StepState), cudaMemcpyDeviceToHost, st));
     VRM_CUDA(cudaStreamSynchronize(st));
@@ -1704,7 +1724,7 @@ extern "C" vrm_status vrm_step_batched(vrm_batch* b, vrm_cloud* clouds, int32_t 
     P.dt = C.dt;
     P.max_rounds = ctx->p.max_rounds;
     *ctx->s.h_params = P;
-    ctx->c.lp_load = (int)(load < INT_MAX ? load : INT_MAX);
+    ctx->c.load = (int)(load < INT_MAX ? load : INT_MAX);
     const BatchKey& K = b->key[c];
     hit = hit && K.x == C.x && K.y == C.y && K.gi == C.gamma_in && K.go == C.gamma_out && K.cap == C.capacity &&
           K.h == C.h && K.scratch_gen == ctx->scratch_gen;

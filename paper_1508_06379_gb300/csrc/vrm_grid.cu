@@ -286,38 +286,7 @@ __global__ void k_bbox(const double* __restrict__ x, const double* __restrict__ 
 __global__ void k_grid_finalize(unsigned long long* __restrict__ bb, int n, const int* __restrict__ n_dev,
                                 double Rh, double lo2, double hi2, int ncell_cap, Grid* __restrict__ g) {
   if (n_dev) n = *n_dev;
-  Grid G;
-  G.nonfinite = (int)bb[4];
-  double x0 = 0, x1 = 0, y0 = 0, y1 = 0;
-  if (n > 0 && bb[0] != ~0ull) {
-    x0 = from_ordered_bits(bb[0]);
-    x1 = from_ordered_bits(bb[1]);
-    y0 = from_ordered_bits(bb[2]);
-    y1 = from_ordered_bits(bb[3]);
-  }
-  double cs = Rh * (1.0 + 1e-6);
-  double w = x1 - x0, hgt = y1 - y0;
-  // keep nx * ny within the cell capacity for very sparse clouds
-  while ((floor(w / cs) + 1.0) * (floor(hgt / cs) + 1.0) > (double)ncell_cap) cs *= 2.0;
-  G.x0 = x0;
-  G.y0 = y0;
-  G.inv_cs = 1.0 / cs;
-  G.nx = (int)floor(w * G.inv_cs) + 1;
-  G.ny = (int)floor(hgt * G.inv_cs) + 1;
-  if ((long)G.nx * G.ny > ncell_cap) {  // rounding at the limit: enlarge once more
-    G.inv_cs *= 0.5;
-    G.nx = (int)floor(w * G.inv_cs) + 1;
-    G.ny = (int)floor(hgt * G.inv_cs) + 1;
-  }
-  G.ncell = G.nx * G.ny;
-  const double s2 = G.inv_cs * G.inv_cs;
-  const float lo2c = (float)(lo2 * s2), hi2c = (float)(hi2 * s2);
-  G.lo_out = lo2c - kBand;
-  G.lo_in = lo2c + kBand;
-  G.hi_in = hi2c - kBand;
-  G.hi_out = hi2c + kBand;
-  G.seg_eps = kSegEps;
-  *g = G;
+  *g = grid_geometry(bb[0], bb[1], bb[2], bb[3], bb[4] != 0, n, Rh, lo2, hi2, ncell_cap);
   bb[0] = ~0ull;
   bb[1] = 0ull;
   bb[2] = ~0ull;
@@ -407,12 +376,16 @@ __global__ void k_zero_cells(const Grid* __restrict__ g, int* __restrict__ cell_
 
 cudaError_t grid_bin_dev(const double* x, const double* y, int n_bound, const int* n_dev, int ncell_cap, const Grid* g,
                          int* cell_key, int* cell_rank, int* cell_count, int* cell_start, double2* sorted_xy,
-                         float2* sorted_loc, int* sorted_idx, int* scan_tmp, cudaStream_t s, int* cell_ts) {
+                         float2* sorted_loc, int* sorted_idx, int* scan_tmp, cudaStream_t s, int* cell_ts,
+                         bool cells_empty) {
   // only the grid's own cells (g->ncell, known on the device) are counted
   // and scanned, not the whole capacity: a cloud of spacing h has about
   // (extent / 2h)^2 cells, far fewer than the capacity's 2 per particle
   const int* ncell_dev = reinterpret_cast<const int*>(reinterpret_cast<const char*>(g) + offsetof(Grid, ncell));
-  k_zero_cells<<<stream_grid(ncell_cap, 4), kBlock, 0, s>>>(g, cell_count, cell_ts); note_launch();
+  if (!cells_empty) {
+    k_zero_cells<<<stream_grid(ncell_cap, 4), kBlock, 0, s>>>(g, cell_count, cell_ts);
+    note_launch();
+  }
   const int b = stream_grid(n_bound, 8);
   k_bin<<<b, kBlock, 0, s>>>(x, y, n_bound, n_dev, g, cell_key, cell_rank, cell_count, cell_ts); note_launch();
   cudaError_t e = cell_ts ? scan_presummed_i32_dev(cell_count, cell_start, ncell_cap, ncell_dev, cell_ts, s)

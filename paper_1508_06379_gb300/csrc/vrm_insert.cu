@@ -18,6 +18,8 @@
 //      of its annulus, found in the same 3 x 3 cells.
 // All threads of a warp do the same kind of work on nearby proposals, and
 // every distance is the FP64 definition, so the result is the oracle's.
+#include <algorithm>
+
 #include "vrm_internal.cuh"
 
 namespace vrm {
@@ -91,6 +93,48 @@ __global__ void __launch_bounds__(kBlock) k_conflict(Consts c, const Grid* __res
   }
 }
 
+// Small clouds: the same, a warp per proposal.
+__global__ void __launch_bounds__(128) k_conflict_warp(Consts c, const Grid* __restrict__ gp,
+                                                       const int* __restrict__ cell_start,
+                                                       const double2* __restrict__ sxy,
+                                                       const float2* __restrict__ sloc, const int* __restrict__ sidx,
+                                                       const int* __restrict__ cell_key,
+                                                       const int* __restrict__ n_cand_dev, uint8_t* __restrict__ keep,
+                                                       uint8_t* __restrict__ keep_s, int* __restrict__ keep_ts) {
+  const int n_cand = *n_cand_dev;
+  const Grid g = *gp;
+  const int lane = threadIdx.x & 31;
+  for (long p = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < n_cand;
+       p += ((long)gridDim.x * blockDim.x) >> 5) {
+    const int ci = sidx[p], key = cell_key[ci];
+    const double2 pc = sxy[p];
+    const float2 lc = sloc[p];
+    const int gy = key / g.nx, gx = key - gy * g.nx;
+    const WarpCells wc = warp_cells(cell_start, g, gx, gy);
+    bool close = false;
+    for (int k = lane; k < wc.total; k += 32) {
+      int ox, oy;
+      const int q = warp_candidate(wc, k, &ox, &oy);
+      const float2 lo = sloc[q];
+      const float du = ((float)ox - lc.x) + lo.x, dv = ((float)oy - lc.y) + lo.y;
+      const float d2f = __fmaf_rn(du, du, dv * dv);
+      if (d2f > g.lo_in || sidx[q] >= ci) continue;
+      if (d2f < g.lo_out) {
+        close = true;
+      } else {
+        const double2 o = sxy[q];
+        close = close || dist2(__dsub_rn(pc.x, o.x), __dsub_rn(pc.y, o.y)) < c.lo2;
+      }
+    }
+    const bool ok = !__any_sync(0xffffffffu, close);
+    if (lane == 0) {
+      keep[ci] = ok;
+      keep_s[p] = ok;
+      if (ok) atomicAdd(&keep_ts[ci >> kScanTileLog], 1);
+    }
+  }
+}
+
 // Segment bits of the accepted proposals in the annulus of open particle i,
 // ORed into mask[i]; returns true if the mask is still not full.  FP32
 // filter on cell-local coordinates as in the neighbour search.  The open
@@ -136,6 +180,40 @@ __device__ __forceinline__ bool mask_update_one(const Consts& c, const Grid& g, 
   }
   mask[i] = (uint8_t)mk;
   return mk != 0xFFu;
+}
+
+// The same by a whole warp; returns the new mask.
+__device__ __forceinline__ unsigned mask_update_warp(const Consts& c, const Grid& g,
+                                                     const int* __restrict__ cell_start,
+                                                     const double2* __restrict__ sxy, const float2* __restrict__ sloc,
+                                                     const uint8_t* __restrict__ keep_s, const double* __restrict__ x,
+                                                     const double* __restrict__ y, const PartCells& pcells, int i,
+                                                     const uint8_t* __restrict__ mask) {
+  const int lane = threadIdx.x & 31;
+  const int key = pcells.cell_key[i];
+  const float2 li = pcells.sorted_loc[pcells.cell_start[key] + pcells.cell_rank[i]];
+  const int gy = key / g.nx, gx = key - gy * g.nx;
+  const WarpCells wc = warp_cells(cell_start, g, gx, gy);
+  unsigned mk = mask[i];
+  for (int k = lane; k < wc.total; k += 32) {
+    int ox, oy;
+    const int q = warp_candidate(wc, k, &ox, &oy);
+    const float2 lo = sloc[q];
+    const float du = ((float)ox - li.x) + lo.x, dv = ((float)oy - li.y) + lo.y;
+    const float d2f = __fmaf_rn(du, du, dv * dv);
+    if (d2f < g.lo_out || d2f > g.hi_out || !keep_s[q]) continue;
+    int s = -1;
+    if (d2f > g.lo_in && d2f < g.hi_in) s = segment_or_ambiguous(du, dv, g.seg_eps);
+    if (s < 0) {
+      const double2 o = sxy[q];
+      const double dx = __dsub_rn(o.x, x[i]), dy = __dsub_rn(o.y, y[i]);
+      const double d2 = dist2(dx, dy);
+      if (d2 < c.lo2 || d2 > c.hi2) continue;
+      s = segment_of(dx, dy);
+    }
+    mk |= 1u << s;
+  }
+  return __reduce_or_sync(0xffffffffu, mk);
 }
 
 // out[k] = list[t] for the k-th flagged t (order kept); *count = total.
@@ -209,22 +287,7 @@ cudaError_t open_list(const int* dlist, const int* dcount, int cap, const uint8_
 
 __global__ void k_rounds_init(StepState* st, const int* __restrict__ n_open_src, cudaGraphConditionalHandle h,
                               int graph) {
-  st->n_open = *n_open_src;
-  st->n_list = st->n_open;
-  st->round = 0;
-  st->rounds_appended = 0;
-  st->overflow = 0;
-  st->n_needed = 0;
-  st->open_segments = 0;
-  st->n_next = 0;
-  st->n_act[0] = st->n_open;
-  st->n_act[1] = 0;
-  st->blocks_done = 0;
-  st->n_cur = st->n;
-  // with max_rounds = 0 no round runs and the open list stays as it is: its
-  // empty segments are the ones reported
-  const int go = st->n_open > 0 && st->max_rounds > 0;
-  if (graph) cudaGraphSetConditional(h, go);
+  rounds_start(st, *n_open_src, h, graph);
 }
 
 // cnt[t] of the first round (every position active) and its tile sums:
@@ -384,6 +447,8 @@ __global__ void k_append_dev(const double* __restrict__ cx, const double* __rest
 // append), its count for the next round set (0 once the mask is full) and,
 // if still open, its position appended to the next active list; the last
 // block to finish records the round's counters and the loop condition.
+// WARP (small clouds): a warp per open particle.
+template <bool WARP>
 __global__ void __launch_bounds__(kBlock) k_round_update(
     Consts c, const Grid* __restrict__ gp, const int* __restrict__ cell_start, const double2* __restrict__ sxy,
     const float2* __restrict__ sloc, const uint8_t* __restrict__ keep_s, const int* __restrict__ apos,
@@ -402,7 +467,45 @@ __global__ void __launch_bounds__(kBlock) k_round_update(
   int* act_next = par ? act0 : act1;
   const int n_act = st->n_act[par];
   const int lane = threadIdx.x & 31;
-  for (long base = (long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_act; base += stride) {
+  if constexpr (WARP) {
+    // the block's eight particles meet for one append and their tile sums
+    // (an atomic per particle on the list's length would take 2 ns each)
+    __shared__ int s_t[kBlock / 32], s_dc[kBlock / 32];
+    __shared__ bool s_open[kBlock / 32];
+    const int w = threadIdx.x >> 5;
+    for (long k0 = (long)blockIdx.x * (kBlock / 32); k0 < n_act; k0 += stride >> 5) {
+      const long k = k0 + w;
+      if (k < n_act) {
+        const int t = act[k], i = open[t];
+        const unsigned mk = mask_update_warp(c, g, cell_start, sxy, sloc, keep_s, x, y, pcells, i, mask);
+        if (lane == 0) {
+          mask[i] = (uint8_t)mk;
+          const int cn = __popc(~mk & 0xFFu);
+          s_t[w] = t;
+          s_dc[w] = cn - cnt[t];
+          s_open[w] = cn != 0;
+          cnt[t] = cn;
+        }
+      } else if (lane == 0) {
+        s_dc[w] = 0;
+        s_open[w] = false;
+      }
+      __syncthreads();
+      if (w == 0) {
+        const bool in = lane < kBlock / 32;
+        const int t = in ? s_t[lane] : 0, dc = in ? s_dc[lane] : 0;
+        const bool still = in && s_open[lane];
+        tile_sum_add(cnt_ts, dc ? t : -1, dc);
+        const unsigned sb = __ballot_sync(0xffffffffu, still);
+        int slot0 = 0;
+        if (lane == 0 && sb) slot0 = atomicAdd(&st->n_act[par ^ 1], __popc(sb));
+        slot0 = __shfl_sync(0xffffffffu, slot0, 0);
+        if (still) act_next[slot0 + __popc(sb & ((1u << lane) - 1u))] = t;
+      }
+      __syncthreads();
+    }
+  }
+  for (long base = (long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); !WARP && base < n_act; base += stride) {
     const long k = base + lane;
     bool still = false;
     int t = 0, dc = 0;
@@ -497,15 +600,28 @@ cudaError_t round_body(const Consts& c, StepState* st, const Grid* pgrid, const 
                                        cg.cell_count, cg.sorted_xy, cg.sorted_loc, cg.sorted_idx, rb.cell_ts,
                                        rb.keep_ts);
   note_launch();
-  k_conflict<<<bc, kBlock, 0, s>>>(c, pgrid, cg.cell_start, cg.sorted_xy, cg.sorted_loc, cg.sorted_idx, cg.cell_key,
-                                   &st->n_cand, rb.keep, rb.keep_s, rb.keep_ts);
+  const bool warps = warp_scans(c, cap);
+  // 4 blocks of 8 warps per SM: 20,449 particles take 21 us per mask update
+  // (27 and 37 with 2 and 1: a particle's chain of loads is 4 us)
+  const int wblocks = std::min((cap + kBlock / 32 - 1) / (kBlock / 32), 4 * sm_count());
+  if (warps)
+    k_conflict_warp<<<2 * wblocks, 128, 0, s>>>(c, pgrid, cg.cell_start, cg.sorted_xy, cg.sorted_loc, cg.sorted_idx,
+                                                cg.cell_key, &st->n_cand, rb.keep, rb.keep_s, rb.keep_ts);
+  else
+    k_conflict<<<bc, kBlock, 0, s>>>(c, pgrid, cg.cell_start, cg.sorted_xy, cg.sorted_loc, cg.sorted_idx, cg.cell_key,
+                                     &st->n_cand, rb.keep, rb.keep_s, rb.keep_ts);
   note_launch();
   e = scan_presummed_u8_dev(rb.keep, rb.apos, (int)cand_cap, &st->n_cand, rb.keep_ts, s);
   if (e != cudaSuccess) return e;
   k_append_dev<<<bc, kBlock, 0, s>>>(rb.cx, rb.cy, rb.keep, rb.apos, st, x, y); note_launch();
-  k_round_update<<<bo, kBlock, 0, s>>>(c, pgrid, cg.cell_start, cg.sorted_xy, cg.sorted_loc, rb.keep_s, rb.apos,
-                                       rb.open, rb.cnt, rb.cnt_ts, rb.act0, rb.act1, pcells, st, x, y, mask,
-                                       handle, graph ? 1 : 0);
+  if (warps)
+    k_round_update<true><<<wblocks, kBlock, 0, s>>>(c, pgrid, cg.cell_start, cg.sorted_xy, cg.sorted_loc, rb.keep_s,
+                                                    rb.apos, rb.open, rb.cnt, rb.cnt_ts, rb.act0, rb.act1, pcells, st,
+                                                    x, y, mask, handle, graph ? 1 : 0);
+  else
+    k_round_update<false><<<bo, kBlock, 0, s>>>(c, pgrid, cg.cell_start, cg.sorted_xy, cg.sorted_loc, rb.keep_s,
+                                                rb.apos, rb.open, rb.cnt, rb.cnt_ts, rb.act0, rb.act1, pcells, st, x,
+                                                y, mask, handle, graph ? 1 : 0);
   note_launch();
   return cudaGetLastError();
 }

@@ -3,6 +3,7 @@
 // Layout of the work (one context, one stream):
 //   vrm_grid.cu    bounding box, cell binning, scans and compaction
 //   vrm_reduce.cu  growth control (Sec. 3.5): exact radix select on |Gamma|
+//   vrm_small.cu   the step's first kernels for small clouds
 //   vrm_search.cu  annulus neighbourhoods, segment masks, small neighbourhoods
 //   vrm_insert.cu  insertion rounds (Sec. 4.2)
 //   vrm_lp.cu      phase-I simplex per particle (Sec. 4.1, 4.3)
@@ -42,8 +43,17 @@ struct Consts {
   int lp_fp64_pivots;    // 1: small LPs pivot in FP64; 0: certified binary32 pivots, FP64 re-runs
   int apply_block;       // threads per block of k_apply
   // capacity of all clouds that run at the same time (a batch), 0: this one's
-  int lp_load;
+  int load;
 };
+
+// Largest capacity (of all clouds that run at the same time) whose cell scans
+// give a warp to each particle or proposal instead of a thread: at 870
+// particles a thread's chain of dependent loads over nine cells takes 33 us in
+// the neighbourhood search and in the masks (7 and 9 by warps), 17 in the mask
+// update (10) and 8 in the conflict test (5); at 20,449 34, 14, 21 and 11
+// against 20, 11, 21 and 7.
+constexpr int kWarpScanCap = 65536;
+inline bool warp_scans(const Consts& c, int cap) { return (c.load > cap ? c.load : cap) <= kWarpScanCap; }
 
 // The schedule every context starts with.
 inline void default_schedule(Consts& c) {
@@ -188,6 +198,137 @@ __device__ __forceinline__ int segment_or_ambiguous(float du, float dv, float ep
   return segment_of(du, dv);
 }
 
+__device__ __forceinline__ u128 dbl_floor_to_u128(double t) {
+  const double two64 = 18446744073709551616.0;
+  unsigned long long hi = __double2ull_rz(__dmul_rn(t, 5.421010862427522170e-20));  // t * 2^-64, exact
+  double rem = __dsub_rn(t, __dmul_rn(__ull2double_rn(hi), two64));
+  unsigned long long lo = __double2ull_rz(rem);
+  return ((u128)hi << 64) | (u128)lo;
+}
+
+__device__ __forceinline__ double u128_to_dbl(u128 s) {
+  const double two64 = 18446744073709551616.0;
+  unsigned long long hi = (unsigned long long)(s >> 64), lo = (unsigned long long)s;
+  return __dadd_rn(__dmul_rn(__ull2double_rn(hi), two64), __ull2double_rn(lo));
+}
+
+// floor(|a| 2^(96-E)) from the bit pattern key of |a| (a finite, |a| < 2^E):
+// |a| = M 2^(e-1075) for a normal (M with the hidden bit), M 2^-1074 for a
+// subnormal; the product by 2^(96-E) is a shift, floor a right shift.
+__device__ __forceinline__ u128 q_of_key(unsigned long long key, int E) {
+  const int ebits = (int)(key >> 52);
+  const unsigned long long frac = key & 0xFFFFFFFFFFFFFull;
+  const unsigned long long M = ebits ? (frac | 0x10000000000000ull) : frac;
+  const int sh = (ebits ? ebits - 1075 : -1074) + 96 - E;
+  if (sh >= 0) return (u128)M << sh;  // sh <= 43 because |a| < 2^E
+  if (sh <= -64) return 0;
+  return (u128)(M >> (-sh));
+}
+
+// E with max|Gamma| < 2^E (frexp exponent) from the bit pattern, no FP64.
+__device__ __forceinline__ int exponent_of_key(unsigned long long key) {
+  const int ebits = (int)(key >> 52);
+  if (ebits) return ebits - 1022;
+  const unsigned long long frac = key & 0xFFFFFFFFFFFFFull;
+  return (64 - __clzll((long long)frac)) - 1074;  // bit length of frac - 1074
+}
+
+// Cell grid of n particles whose bounding box is given as ordered bit patterns
+// (an empty one as left by k_bbox_init).
+__device__ __forceinline__ Grid grid_geometry(unsigned long long mnx, unsigned long long mxx, unsigned long long mny,
+                                              unsigned long long mxy, bool nonfinite, int n, double Rh, double lo2,
+                                              double hi2, int ncell_cap) {
+  Grid G;
+  G.nonfinite = nonfinite ? 1 : 0;
+  double x0 = 0, x1 = 0, y0 = 0, y1 = 0;
+  if (n > 0 && mnx != ~0ull) {
+    x0 = from_ordered_bits(mnx);
+    x1 = from_ordered_bits(mxx);
+    y0 = from_ordered_bits(mny);
+    y1 = from_ordered_bits(mxy);
+  }
+  double cs = Rh * (1.0 + 1e-6);
+  double w = x1 - x0, hgt = y1 - y0;
+  // keep nx * ny within the cell capacity for very sparse clouds
+  while ((floor(w / cs) + 1.0) * (floor(hgt / cs) + 1.0) > (double)ncell_cap) cs *= 2.0;
+  G.x0 = x0;
+  G.y0 = y0;
+  G.inv_cs = 1.0 / cs;
+  G.nx = (int)floor(w * G.inv_cs) + 1;
+  G.ny = (int)floor(hgt * G.inv_cs) + 1;
+  if ((long)G.nx * G.ny > ncell_cap) {  // rounding at the limit: enlarge once more
+    G.inv_cs *= 0.5;
+    G.nx = (int)floor(w * G.inv_cs) + 1;
+    G.ny = (int)floor(hgt * G.inv_cs) + 1;
+  }
+  G.ncell = G.nx * G.ny;
+  const double s2 = G.inv_cs * G.inv_cs;
+  const float lo2c = (float)(lo2 * s2), hi2c = (float)(hi2 * s2);
+  G.lo_out = lo2c - kBand;
+  G.lo_in = lo2c + kBand;
+  G.hi_in = hi2c - kBand;
+  G.hi_out = hi2c + kBand;
+  G.seg_eps = kSegEps;
+  return G;
+}
+
+// The 3 x 3 cells around cell (cx, cy), read by a whole warp: per row the cells
+// are one range of the sorted arrays, so the candidates are numbered 0..total-1
+// over the three rows and handed to the lanes.
+struct WarpCells {
+  int s[3][4];  // starts of the row's three cells and the end of the last
+  int total;
+};
+__device__ __forceinline__ WarpCells warp_cells(const int* __restrict__ cell_start, const Grid& g, int cx, int cy) {
+  const int lane = threadIdx.x & 31;
+  int v = 0;
+  if (lane < 12) {
+    const int by = cy - 1 + (lane >> 2);
+    int bx = cx - 1 + (lane & 3);
+    bx = bx < 0 ? 0 : (bx > g.nx ? g.nx : bx);
+    if (by >= 0 && by < g.ny) v = cell_start[by * g.nx + bx];
+  }
+  WarpCells c;
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c.s[r][k] = __shfl_sync(0xffffffffu, v, 4 * r + k);
+  c.total = (c.s[0][3] - c.s[0][0]) + (c.s[1][3] - c.s[1][0]) + (c.s[2][3] - c.s[2][0]);
+  return c;
+}
+// Sorted position of candidate k < total, and its cell's offset from (cx, cy).
+__device__ __forceinline__ int warp_candidate(const WarpCells& c, int k, int* ox, int* oy) {
+  const int n0 = c.s[0][3] - c.s[0][0], n01 = n0 + c.s[1][3] - c.s[1][0];
+  const int r = (k >= n0) + (k >= n01);
+  const int q = r == 0 ? c.s[0][0] + k : r == 1 ? c.s[1][0] + k - n0 : c.s[2][0] + k - n01;
+  const int s1 = r == 0 ? c.s[0][1] : r == 1 ? c.s[1][1] : c.s[2][1];
+  const int s2 = r == 0 ? c.s[0][2] : r == 1 ? c.s[1][2] : c.s[2][2];
+  *ox = (q >= s1) + (q >= s2) - 1;
+  *oy = r - 1;
+  return q;
+}
+
+// State of the insertion rounds with n_open open particles, and the loop
+// condition (one thread).
+__device__ __forceinline__ void rounds_start(StepState* st, int n_open, cudaGraphConditionalHandle h, int graph) {
+  st->n_open = n_open;
+  st->n_list = n_open;
+  st->round = 0;
+  st->rounds_appended = 0;
+  st->overflow = 0;
+  st->n_needed = 0;
+  st->open_segments = 0;
+  st->n_next = 0;
+  st->n_act[0] = n_open;
+  st->n_act[1] = 0;
+  st->blocks_done = 0;
+  st->n_cur = st->n;
+  // with max_rounds = 0 no round runs and the open list stays as it is: its
+  // empty segments are the ones reported
+  const int go = n_open > 0 && st->max_rounds > 0;
+  if (graph) cudaGraphSetConditional(h, go);
+}
+
 // Analytic velocity of the RK3 step (vrm_velocity).
 struct Velocity {
   int kind;
@@ -229,7 +370,8 @@ cudaError_t grid_bbox_reset(unsigned long long* bbox_tmp, cudaStream_t s);
 // counts is one launch.
 cudaError_t grid_bin_dev(const double* x, const double* y, int n_bound, const int* n_dev, int ncell_cap, const Grid* g,
                          int* cell_key, int* cell_rank, int* cell_count, int* cell_start, double2* sorted_xy,
-                         float2* sorted_loc, int* sorted_idx, int* scan_tmp, cudaStream_t s, int* cell_ts = nullptr);
+                         float2* sorted_loc, int* sorted_idx, int* scan_tmp, cudaStream_t s, int* cell_ts = nullptr,
+                         bool cells_empty = false);
 // Grid g, built over [0, *n0_dev), extended to [0, *n1_dev) with the same
 // geometry: the new particles are binned onto the existing counts (points
 // outside the grid clamp into its edge cells; cells are >= R h, so the 3 x 3
@@ -367,6 +509,18 @@ cudaError_t round_body(const Consts& c, StepState* st, const Grid* pgrid, const 
                        int cap, uint8_t* mask, double* x, double* y, cudaGraphConditionalHandle handle, bool graph,
                        cudaStream_t s);
 cudaError_t rounds_finish(StepState* st, const RoundBufs& rb, int cap, cudaStream_t s);
+
+// vrm_small.cu: a step's first kernels for clouds of at most kSmallCap capacity.
+constexpr int kSmallCap = 65536;
+// Growth control, diffused list, cell grid geometry and cleared cell counts
+// (the bounding-box accumulators and the reduce state are not used).
+cudaError_t front_small(const double* gamma, const double* x, const double* y, int cap, const int* n_dev,
+                        double c_bound, double Rh, double lo2, double hi2, int ncell_cap, uint8_t* diffused,
+                        int* dlist, int* dcount, DevStats* ds, Grid* g, int* cell_count, int* cell_ts,
+                        cudaStream_t s);
+// open_list and rounds_init in one.
+cudaError_t open_small(const int* dlist, const int* dcount, const uint8_t* mask, int* n_open, const RoundBufs& rb,
+                       StepState* st, cudaGraphConditionalHandle handle, bool graph, cudaStream_t s);
 
 // vrm_lp.cu
 // nu_dt = nu * dt for the stability statistic; with dt_dev it is nu * *dt_dev.

@@ -2378,7 +2378,7 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
     note_launch();
     return cudaGetLastError();
   }
-  const int load = c.lp_load > cap ? c.lp_load : cap;
+  const int load = c.load > cap ? c.load : cap;
   if (load > kPairsCap) {
     // certified binary32 pivots, then the uncertain particles in pairs or in FP64
     if (c.lp_block == kLpWsThreads) {

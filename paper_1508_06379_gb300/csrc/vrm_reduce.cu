@@ -21,41 +21,6 @@
 
 namespace vrm {
 
-__device__ __forceinline__ u128 dbl_floor_to_u128(double t) {
-  const double two64 = 18446744073709551616.0;
-  unsigned long long hi = __double2ull_rz(__dmul_rn(t, 5.421010862427522170e-20));  // t * 2^-64, exact
-  double rem = __dsub_rn(t, __dmul_rn(__ull2double_rn(hi), two64));
-  unsigned long long lo = __double2ull_rz(rem);
-  return ((u128)hi << 64) | (u128)lo;
-}
-
-__device__ __forceinline__ double u128_to_dbl(u128 s) {
-  const double two64 = 18446744073709551616.0;
-  unsigned long long hi = (unsigned long long)(s >> 64), lo = (unsigned long long)s;
-  return __dadd_rn(__dmul_rn(__ull2double_rn(hi), two64), __ull2double_rn(lo));
-}
-
-// floor(|a| 2^(96-E)) from the bit pattern key of |a| (a finite, |a| < 2^E):
-// |a| = M 2^(e-1075) for a normal (M with the hidden bit), M 2^-1074 for a
-// subnormal; the product by 2^(96-E) is a shift, floor a right shift.
-__device__ __forceinline__ u128 q_of_key(unsigned long long key, int E) {
-  const int ebits = (int)(key >> 52);
-  const unsigned long long frac = key & 0xFFFFFFFFFFFFFull;
-  const unsigned long long M = ebits ? (frac | 0x10000000000000ull) : frac;
-  const int sh = (ebits ? ebits - 1075 : -1074) + 96 - E;
-  if (sh >= 0) return (u128)M << sh;  // sh <= 43 because |a| < 2^E
-  if (sh <= -64) return 0;
-  return (u128)(M >> (-sh));
-}
-
-// E with max|Gamma| < 2^E (frexp exponent) from the bit pattern, no FP64.
-__device__ __forceinline__ int exponent_of_key(unsigned long long key) {
-  const int ebits = (int)(key >> 52);
-  if (ebits) return ebits - 1022;
-  const unsigned long long frac = key & 0xFFFFFFFFFFFFFull;
-  return (64 - __clzll((long long)frac)) - 1074;  // bit length of frac - 1074
-}
-
 // Bucket value from its limbs; read past L1 (other blocks wrote them by atomics).
 __device__ __forceinline__ u128 limbs_value(const unsigned long long* h) {
   return (u128)__ldcg(h) + ((u128)__ldcg(h + 1) << 32) + ((u128)__ldcg(h + 2) << 64);

@@ -258,6 +258,163 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
   }
 }
 
+// Small clouds: counts, masks and small neighbourhoods of the listed particles
+// (k_search_all<., false, true, false>), a warp per particle: the lanes test
+// the candidates, lane s < 8 keeps segment s's closest.  A segment whose two
+// closest members are within two bands of each other in FP32 is decided by
+// the FP64 order in a second pass.
+__global__ void __launch_bounds__(128) k_search_warp(Consts c, const Grid* __restrict__ gp,
+                                                     const int* __restrict__ cell_start,
+                                                     const double2* __restrict__ sxy,
+                                                     const float2* __restrict__ sloc, const int* __restrict__ sidx,
+                                                     const int* __restrict__ list, const int* __restrict__ list_count,
+                                                     const int* __restrict__ cell_key,
+                                                     const int* __restrict__ cell_rank, int* __restrict__ nbr_count,
+                                                     uint8_t* __restrict__ seg_mask, int* __restrict__ small,
+                                                     DevStats* __restrict__ ds) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int m = *list_count;
+  const Grid g = *gp;
+  const float tie = 2.f * kBand;
+  const int lane = threadIdx.x & 31;
+  int local_max = 0;
+  for (long t = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < m; t += ((long)gridDim.x * blockDim.x) >> 5) {
+    const int i = list[t];
+    const int key = cell_key[i];
+    const int p = cell_start[key] + cell_rank[i];
+    const double2 pi = sxy[p];
+    const float2 li = sloc[p];
+    const int cy = key / g.nx, cx = key - cy * g.nx;
+    const WarpCells wc = warp_cells(cell_start, g, cx, cy);
+    // candidate k: its segment, or -1 if it is not a neighbour
+    auto member = [&](int k, int* j, float* d2f, double* d2) {
+      int ox, oy;
+      const int q = warp_candidate(wc, k, &ox, &oy);
+      const float2 lj = sloc[q];
+      *j = sidx[q];
+      const float du = ((float)ox - li.x) + lj.x, dv = ((float)oy - li.y) + lj.y;
+      *d2f = __fmaf_rn(du, du, dv * dv);
+      if (*d2f < g.lo_out || *d2f > g.hi_out || *j == i) return -1;
+      const bool certain_in = *d2f > g.lo_in && *d2f < g.hi_in;
+      int s = certain_in && !d2 ? segment_or_ambiguous(du, dv, g.seg_eps) : -1;
+      double e;
+      if (s < 0) s = exact_member(c, pi, sxy[q], certain_in, d2 ? d2 : &e);
+      return s;
+    };
+    int cnt = 0, bj = -1;  // lane s: segment s's closest so far
+    float bf = 3e38f;
+    unsigned mask = 0, amb = 0;
+    for (int k0 = 0; k0 < wc.total; k0 += 32) {
+      int j = 0, s = -1;
+      float d2f = 3e38f;
+      if (k0 + lane < wc.total) s = member(k0 + lane, &j, &d2f, nullptr);
+      cnt += __popc(__ballot_sync(kAll, s >= 0));
+#pragma unroll 1
+      for (int sg = 0; sg < 8; ++sg) {
+        const bool mine = s == sg;
+        if (!__any_sync(kAll, mine)) continue;
+        mask |= 1u << sg;
+        const float dmin = __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(mine ? d2f : 3e38f)));
+        const unsigned near = __ballot_sync(kAll, mine && d2f - dmin <= tie);
+        const int jmin = (int)__reduce_min_sync(kAll, mine && d2f == dmin ? (unsigned)j : 0x7FFFFFFFu);
+        const float pb = __shfl_sync(kAll, bf, sg);
+        const int pj = __shfl_sync(kAll, bj, sg);
+        if (__popc(near) > 1 || (pj >= 0 && fabsf(dmin - pb) <= tie)) amb |= 1u << sg;
+        if (lane == sg && (pj < 0 || dmin < pb || (dmin == pb && jmin < pj))) {
+          bf = dmin;
+          bj = jmin;
+        }
+      }
+    }
+    while (amb) {
+      // exact FP64 order (ties to the smaller index)
+      const int sg = __ffs(amb) - 1;
+      amb &= amb - 1;
+      unsigned long long bd = ~0ull;
+      int jd = 0x7FFFFFFF;
+      for (int k = lane; k < wc.total; k += 32) {
+        int j;
+        float d2f;
+        double d2 = 0.0;
+        if (member(k, &j, &d2f, &d2) != sg) continue;
+        const unsigned long long b = (unsigned long long)__double_as_longlong(d2);  // d2 >= +0
+        if (b < bd || (b == bd && j < jd)) {
+          bd = b;
+          jd = j;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long od = __shfl_xor_sync(kAll, bd, o);
+        const int oj = __shfl_xor_sync(kAll, jd, o);
+        if (od < bd || (od == bd && oj < jd)) {
+          bd = od;
+          jd = oj;
+        }
+      }
+      if (lane == sg) bj = jd;
+    }
+    if (lane < 8) small[(size_t)i * 8 + lane] = bj;
+    if (lane == 0) {
+      nbr_count[i] = cnt;
+      seg_mask[i] = (uint8_t)mask;
+    }
+    local_max = cnt > local_max ? cnt : local_max;
+  }
+  __shared__ int w_max[4];
+  if (lane == 0) w_max[threadIdx.x >> 5] = local_max;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 4; ++w) local_max = w_max[w] > local_max ? w_max[w] : local_max;
+    if (local_max > 0) atomicMax(&ds->max_count, local_max);
+  }
+}
+
+// Small clouds: segment masks, a warp per particle (k_search_masks_list).
+__global__ void __launch_bounds__(128) k_masks_warp(Consts c, const Grid* __restrict__ gp,
+                                                    const int* __restrict__ cell_start,
+                                                    const double2* __restrict__ sxy, const float2* __restrict__ sloc,
+                                                    const int* __restrict__ sidx, const int* __restrict__ cell_key,
+                                                    const int* __restrict__ cell_rank, const int* __restrict__ list,
+                                                    const int* __restrict__ list_count, uint8_t* __restrict__ mask) {
+  const int m = *list_count;
+  const Grid g = *gp;
+  const int lane = threadIdx.x & 31;
+  for (long t = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < m; t += ((long)gridDim.x * blockDim.x) >> 5) {
+    const int i = list[t];
+    const int key = cell_key[i];
+    const int p = cell_start[key] + cell_rank[i];
+    const double2 pi = sxy[p];
+    const float2 li = sloc[p];
+    const int cy = key / g.nx, cx = key - cy * g.nx;
+    const WarpCells wc = warp_cells(cell_start, g, cx, cy);
+    unsigned mk = 0;
+    for (int k = lane; k < wc.total; k += 32) {
+      int ox, oy;
+      const int q = warp_candidate(wc, k, &ox, &oy);
+      const float2 lj = sloc[q];
+      const float du = ((float)ox - li.x) + lj.x, dv = ((float)oy - li.y) + lj.y;
+      const float d2f = __fmaf_rn(du, du, dv * dv);
+      if (d2f < g.lo_out || d2f > g.hi_out) continue;
+      const bool certain_in = d2f > g.lo_in && d2f < g.hi_in;
+      int s = certain_in ? segment_or_ambiguous(du, dv, g.seg_eps) : -1;
+      if (s < 0) {
+        double d2;
+        if (sidx[q] != i) s = exact_member(c, pi, sxy[q], false, &d2);
+      }
+      if (s >= 0) mk |= 1u << s;
+    }
+    mk = __reduce_or_sync(0xffffffffu, mk);
+    if (lane == 0) mask[i] = (uint8_t)mk;
+  }
+}
+
+// Grid of the warp-per-particle kernels.
+static int warp_grid(int m_bound) {
+  const long b = ((long)m_bound + 3) / 4, most = 16L * sm_count();
+  return (int)(b < most ? b : most);
+}
+
 // Segment masks of the listed particles (the diffused list, in index order:
 // lattice order keeps a warp's particles neighbours), each located in the
 // sorted arrays through its cell key and rank: FP32 distances on the
@@ -320,6 +477,12 @@ cudaError_t search_masks_list_dev(const Consts& c, const Grid* g, const int* cel
                                   const int* cell_rank, const int* list, const int* list_count, int m_bound,
                                   uint8_t* mask, cudaStream_t s) {
   if (m_bound <= 0) return cudaSuccess;
+  if (warp_scans(c, m_bound)) {
+    k_masks_warp<<<warp_grid(m_bound), 128, 0, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, cell_key,
+                                                    cell_rank, list, list_count, mask);
+    note_launch();
+    return cudaGetLastError();
+  }
   const int blocks = (m_bound + kBlock - 1) / kBlock;
   k_search_masks_list<<<blocks, kBlock, 0, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, cell_key,
                                                 cell_rank, list, list_count, mask);
@@ -359,6 +522,12 @@ cudaError_t search_list_dev(const Consts& c, const Grid* g, const int* cell_star
                             int* nbr_count, int* nbr_idx, uint8_t* seg_mask, int* small, DevStats* ds,
                             cudaStream_t s, bool rows) {
   if (m_bound <= 0) return cudaSuccess;
+  if (!rows && warp_scans(c, m_bound)) {
+    k_search_warp<<<warp_grid(m_bound), 128, 0, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, list,
+                                                     list_count, cell_key, cell_rank, nbr_count, seg_mask, small, ds);
+    note_launch();
+    return cudaGetLastError();
+  }
   const int tb = c.search_block;
   const int blocks = (int)(((long)m_bound + tb - 1) / tb);
 #define VRM_SEARCH_LAUNCH(K, R)                                                                                    \
