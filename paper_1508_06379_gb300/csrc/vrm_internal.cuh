@@ -39,6 +39,7 @@ struct Consts {
   int row_cap;           // neighbour entries kept per row (<= k_cap)
   int search_block;      // threads per block of k_search_all
   int lp_block;          // threads per block of k_lp_small
+  int lp_auto;           // 1: no schedule was set, the LP's form follows the capacity
   int lp_blocks_per_sm;  // grid cap of k_lp_small
   int lp_fp64_pivots;    // 1: small LPs pivot in FP64; 0: certified binary32 pivots, FP64 re-runs
   int apply_block;       // threads per block of k_apply
@@ -60,6 +61,7 @@ inline void default_schedule(Consts& c) {
   c.row_cap = c.k_cap;
   c.search_block = 256;
   c.lp_block = 128;
+  c.lp_auto = 1;
   c.lp_blocks_per_sm = 16;
   c.lp_fp64_pivots = 0;
   c.apply_block = 256;

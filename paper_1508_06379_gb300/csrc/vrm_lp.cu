@@ -2351,6 +2351,13 @@ static cudaError_t lp_finish_list(const Consts& c, const double* x, const double
 // to 300,000 particles: 4.49 ms, 4.60 when each went by its own).
 constexpr int kPairsCap = 65536;
 constexpr int kPairsRetryCap = 6 * 65536;
+// Smallest capacity that takes the 8 + 4-warp form where no schedule was set:
+// steps of 640,000 particles 1,075 us against 1,114 with one kind of warp, of a
+// million 1,469 against 1,581; 787 and 797 at 360,000.  The form fills every SM,
+// so batches, whose clouds run beside each other, keep the other (4.54 ms
+// against 4.66), as do capacities that may hold fewer LPs than this (an RK3
+// step of 500,000 in 730,000: 2.41 against 2.47 ms).
+constexpr int kWsCap = 18 * 65536;
 
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
@@ -2381,11 +2388,12 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
   const int load = c.load > cap ? c.load : cap;
   if (load > kPairsCap) {
     // certified binary32 pivots, then the uncertain particles in pairs or in FP64
-    if (c.lp_block == kLpWsThreads) {
+    const int form = c.lp_auto && c.load == 0 && cap >= kWsCap ? kLpWsThreadsWide : c.lp_block;
+    if (form == kLpWsThreads) {
       // warp-specialised form, 4 + 2 warps: two resident blocks per SM
       k_lp_small32_ws<5, 8, 4, 2, 2><<<2 * sm_count(), kLpWsThreads, 0, s>>>(
           c, x, y, list, list_count, small, cols, f, fii, status, fail_list, retry_list, ds, nu_dt, dt_dev, nu);
-    } else if (c.lp_block == kLpWsThreadsWide) {
+    } else if (form == kLpWsThreadsWide) {
       // 8 + 4 warps: one resident block per SM
       k_lp_small32_ws<5, 8, 8, 4, 1><<<sm_count(), kLpWsThreadsWide, 0, s>>>(
           c, x, y, list, list_count, small, cols, f, fii, status, fail_list, retry_list, ds, nu_dt, dt_dev, nu);
