@@ -969,16 +969,19 @@ vrm_status vrm_remove_close(vrm_ctx* ctx, const double* x, const double* y, cons
   VRM_CUDA(cudaMemsetAsync(s.ds, 0, sizeof(DevStats), stream));
   VRM_CUDA(grid_build(x, y, n, c.Rh, c.lo2, c.hi2, s.ncell_cap, s.grid, s.cell_key, s.cell_rank, s.cell_count,
                       s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.bbox, s.scan_tmp, stream));
-  VRM_CUDA(search_all(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, n, s.nbr_count, s.nbr_idx,
-                      s.seg_mask, s.small, s.ds, stream));
   VRM_CUDA(remove_close_flags(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, n, gamma,
-                              ctx->rm_close, stream));
+                              ctx->rm_close, s.ds, stream));
   VRM_CUDA(compact_flags(ctx->rm_close, n, ctx->rm_clist, s.counters + 3, s.pos, s.scan_tmp, stream));
   VRM_CUDA(cudaMemsetAsync(ctx->rm_removed, 0, (size_t)n, stream));
-  VRM_CUDA(lp_identity(c, x, y, ctx->rm_clist, s.counters + 3, n, s.nbr_count, s.nbr_idx, ctx->rm_close,
-                       ctx->rm_removed, ctx->rm_cols4, ctx->rm_w4, stream));
-  VRM_CUDA(remove_gather(c, n, gamma, ctx->rm_removed, s.nbr_count, s.nbr_idx, ctx->rm_cols4, ctx->rm_w4,
-                         ctx->rm_gnew, ctx->rm_keep, s.ds, stream));
+  // the candidates' closest non-candidates per segment
+  VRM_CUDA(search_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key, s.cell_rank,
+                           ctx->rm_clist, s.counters + 3, n, s.nbr_count, s.nbr_idx, s.seg_mask, s.small, s.ds, stream,
+                           false, ctx->rm_close));
+  VRM_CUDA(lp_identity(c, x, y, ctx->rm_clist, s.counters + 3, n, s.small, ctx->rm_removed, ctx->rm_cols4, ctx->rm_w4,
+                       stream));
+  // (the rows are not needed here: their buffers hold the lists)
+  VRM_CUDA(remove_apply(ctx->rm_clist, s.counters + 3, n, gamma, ctx->rm_removed, ctx->rm_cols4, ctx->rm_w4, s.pos,
+                        s.nbr_idx, ctx->rm_gnew, ctx->rm_keep, s.ds, stream));
   VRM_CUDA(compact_flags(ctx->rm_keep, n, ctx->rm_klist, s.counters + 4, s.pos, s.scan_tmp, stream));
   VRM_CUDA(remove_out(n, s.counters + 4, ctx->rm_klist, x, y, ctx->rm_gnew, x_out, y_out, gamma_out, stream));
   VRM_CUDA(read_back(ctx, stream));

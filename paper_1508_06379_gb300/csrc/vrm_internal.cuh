@@ -439,18 +439,15 @@ cudaError_t reduce_select_dev(const double* gamma, int n_bound, const int* n_dev
 cudaError_t search_all(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
                        const float2* sorted_loc, const int* sorted_idx, int n, int* nbr_count, int* nbr_idx,
                        uint8_t* seg_mask, int* small, DevStats* ds, cudaStream_t s);
-cudaError_t search_all_dev(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
-                           const float2* sorted_loc, const int* sorted_idx, int n_bound, const int* n_dev,
-                           int* nbr_count, int* nbr_idx, uint8_t* seg_mask, int* small, DevStats* ds,
-                           cudaStream_t s, bool sorted = true);
 // Rows, masks and small neighbourhoods of the listed particles only (rows in
 // visiting order, padded to whole 32-byte sectors); rows = false leaves the
-// rows unwritten (counts, masks and small neighbourhoods still are).
+// rows unwritten (counts, masks and small neighbourhoods still are); skip
+// (with rows = false, optional): flagged particles are left out of them.
 cudaError_t search_list_dev(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
                             const float2* sorted_loc, const int* sorted_idx, const int* cell_key,
                             const int* cell_rank, const int* list, const int* list_count, int m_bound,
                             int* nbr_count, int* nbr_idx, uint8_t* seg_mask, int* small, DevStats* ds,
-                            cudaStream_t s, bool rows = true);
+                            cudaStream_t s, bool rows = true, const uint8_t* skip = nullptr);
 cudaError_t search_masks_list_dev(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
                                   const float2* sorted_loc, const int* sorted_idx, const int* cell_key,
                                   const int* cell_rank, const int* list, const int* list_count, int m_bound,
@@ -535,10 +532,9 @@ cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int
                     uint8_t* status, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,
                     const double* dt_dev = nullptr, double nu = 0.0);
 // Identity weights of the removal candidates (list, *list_count on the
-// device): removed[i], cols4/w4 [n x 4] (vrm_remove.cu drives it).
+// device) on the columns of small: removed[i], cols4/w4 [n x 4].
 cudaError_t lp_identity(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
-                        int cap, const int* nbr_count, const int* nbr_idx, const uint8_t* close, uint8_t* removed,
-                        int* cols4, double* w4, cudaStream_t s);
+                        int cap, const int* small, uint8_t* removed, int* cols4, double* w4, cudaStream_t s);
 cudaError_t lp_clear(int n, int w, const uint8_t* diffused, int* cols, double* f, double* fii, uint8_t* status,
                      cudaStream_t s);
 
@@ -561,12 +557,15 @@ cudaError_t apply_gather_dev(const Consts& c, int n_bound, const int* n_dev, int
                              double* gamma_out, double dt, const double* dt_dev, cudaStream_t s);
 
 // vrm_remove.cu: particle removal (candidates, gather, compaction).
+// Candidate flags, and the largest neighbour count in ds->max_count.
 cudaError_t remove_close_flags(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
                                const float2* sorted_loc, const int* sorted_idx, int n, const double* gamma,
-                               uint8_t* close, cudaStream_t s);
-cudaError_t remove_gather(const Consts& c, int n, const double* gamma, const uint8_t* removed, const int* nbr_count,
-                          const int* nbr_idx, const int* cols4, const double* w4, double* gnew, uint8_t* keep,
-                          DevStats* ds, cudaStream_t s);
+                               uint8_t* close, DevStats* ds, cudaStream_t s);
+// The removed particles' circulation moved to their targets through lists of
+// entries (head[n], next[4 n]: scratch).
+cudaError_t remove_apply(const int* clist, const int* n_cand, int n, const double* gamma, const uint8_t* removed,
+                         const int* cols4, const double* w4, int* head, int* next, double* gnew, uint8_t* keep,
+                         DevStats* ds, cudaStream_t s);
 cudaError_t remove_out(int n, const int* n_keep, const int* klist, const double* x, const double* y,
                        const double* gnew, double* x_out, double* y_out, double* g_out, cudaStream_t s);
 

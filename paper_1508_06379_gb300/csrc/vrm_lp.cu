@@ -2074,8 +2074,8 @@ __global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __rest
 // Identity weights of the removal candidates (particle removal, the outlook
 // of Sec. 6.2): the phase-I simplex of k_lp_small with rows (0,0) (1,0) (0,1)
 // of r_ij / h and b = (1, 0, 0), i.e. sum g = 1 and sum g r = 0 with g >= 0,
-// on the closest kept particle (close[j] == 0) of every 45-degree segment of
-// the candidate's annulus row (ties to the smaller index), columns ordered by
+// on the closest non-candidate of every 45-degree segment of the candidate's
+// annulus (small, from the search that skips candidates), columns ordered by
 // (d2, j).  The same entering, leaving, snapping and feasibility rules; the
 // final basis solved by the oracle's LU sequence.  One candidate per thread.
 // removed[i] = 1 and the nonzero weights (at most 3 of the 4 slots, column
@@ -2083,57 +2083,19 @@ __global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __rest
 __global__ void __launch_bounds__(128) k_lp_identity(Consts c, const double* __restrict__ x,
                                                      const double* __restrict__ y, const int* __restrict__ list,
                                                      const int* __restrict__ list_count,
-                                                     const int* __restrict__ nbr_count,
-                                                     const int* __restrict__ nbr_idx,
-                                                     const uint8_t* __restrict__ close, uint8_t* __restrict__ removed,
+                                                     const int* __restrict__ small, uint8_t* __restrict__ removed,
                                                      int* __restrict__ cols4, double* __restrict__ w4) {
   constexpr int M = 3;
   const int m = *list_count;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < m; t += (long)gridDim.x * blockDim.x) {
     const int i = list[t];
-    const double xi0 = x[i], yi0 = y[i];
-    const int cnt0 = nbr_count[i];
-    const int K = cnt0 < c.row_cap ? cnt0 : c.row_cap;
-    const int* row = nbr_idx + (size_t)i * c.k_cap;
-    // closest kept member of every segment
-    double cd2[8], cxi[8], ceta[8];
     int cj[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      cd2[s] = 1e300;
-      cj[s] = INT_MAX;
-      cxi[s] = ceta[s] = 0.0;
-    }
-    for (int e = 0; e < K; ++e) {
-      const int j = row[e];
-      if (close[j]) continue;
-      const double dx = __dsub_rn(x[j], xi0), dy = __dsub_rn(y[j], yi0);
-      const double d2 = dist2(dx, dy);
-      const int sg = segment_of(dx, dy);
-      double cb = cd2[0];
-      int cjb = cj[0];
-#pragma unroll
-      for (int s = 1; s < 8; ++s) {
-        cb = (sg == s) ? cd2[s] : cb;
-        cjb = (sg == s) ? cj[s] : cjb;
-      }
-      const bool take = lt_nonneg(d2, cb) || (dbits(d2) == dbits(cb) && j < cjb);
-#pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        const bool here = take && sg == s;
-        cd2[s] = here ? d2 : cd2[s];
-        cj[s] = here ? j : cj[s];
-        cxi[s] = here ? dx : cxi[s];
-        ceta[s] = here ? dy : ceta[s];
-      }
-    }
-    sort8(cd2, cj, cxi, ceta);
+    double cxi[8], ceta[8];
+    lp_columns(c, x, y, small, i, cj, cxi, ceta);
     unsigned basic = 0;  // empty columns never enter
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       if (cj[k] == INT_MAX) basic |= 1u << k;
-      cxi[k] = __dmul_rn(cxi[k], c.inv_h);
-      ceta[k] = __dmul_rn(ceta[k], c.inv_h);
     }
     double T[M][8], rhs[M], d[8];
 #pragma unroll
@@ -2282,13 +2244,21 @@ __global__ void __launch_bounds__(128) k_lp_identity(Consts c, const double* __r
   }
 }
 
-__global__ void k_lp_clear(int n, int w, const uint8_t* __restrict__ diffused, int* __restrict__ cols,
+__global__ void k_lp_clear(int n, int w, bool vec, const uint8_t* __restrict__ diffused, int* __restrict__ cols,
                            double* __restrict__ f, double* __restrict__ fii, uint8_t* __restrict__ status) {
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     if (diffused[i]) continue;
-    for (int k = 0; k < w; ++k) {
-      cols[i * w + k] = -1;
-      f[i * w + k] = 0.0;
+    if (vec) {  // rows of a multiple of 4, on 16-byte boundaries
+      for (int k = 0; k < w; k += 4) {
+        *reinterpret_cast<int4*>(cols + i * w + k) = make_int4(-1, -1, -1, -1);
+        *reinterpret_cast<double2*>(f + i * w + k) = make_double2(0.0, 0.0);
+        *reinterpret_cast<double2*>(f + i * w + k + 2) = make_double2(0.0, 0.0);
+      }
+    } else {
+      for (int k = 0; k < w; ++k) {
+        cols[i * w + k] = -1;
+        f[i * w + k] = 0.0;
+      }
     }
     fii[i] = 0.0;
     status[i] = VRM_LP_NOT_DIFFUSED;
@@ -2450,17 +2420,17 @@ cudaError_t lp_clear(int n, int w, const uint8_t* diffused, int* cols, double* f
   if (n <= 0) return cudaSuccess;
   int blocks = (n + kBlock - 1) / kBlock;
   if (blocks > 8 * sm_count()) blocks = 8 * sm_count();
-  k_lp_clear<<<blocks, kBlock, 0, s>>>(n, w, diffused, cols, f, fii, status); note_launch();
+  const bool vec = (((uintptr_t)cols | (uintptr_t)f) & 15u) == 0 && w % 4 == 0;
+  k_lp_clear<<<blocks, kBlock, 0, s>>>(n, w, vec, diffused, cols, f, fii, status); note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t lp_identity(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
-                        int cap, const int* nbr_count, const int* nbr_idx, const uint8_t* close, uint8_t* removed,
-                        int* cols4, double* w4, cudaStream_t s) {
+                        int cap, const int* small, uint8_t* removed, int* cols4, double* w4, cudaStream_t s) {
   if (cap <= 0) return cudaSuccess;
   int blocks = (cap + 127) / 128;
   if (blocks > 16 * sm_count()) blocks = 16 * sm_count();
-  k_lp_identity<<<blocks, 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, close, removed, cols4, w4);
+  k_lp_identity<<<blocks, 128, 0, s>>>(c, x, y, list, list_count, small, removed, cols4, w4);
   note_launch();
   return cudaGetLastError();
 }

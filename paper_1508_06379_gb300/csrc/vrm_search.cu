@@ -14,15 +14,18 @@
 // undecided cases (rare on jittered clouds, frequent on exact lattices) take
 // the FP64 definition, so the result is bit-identical to it.
 //
-// The row is kept in a per-thread buffer of KCAP entries (rows are k_cap
-// apart): sorted by index for the library's neighbourhood calls, in visiting
-// order inside a step (SORTED = false: the application orders the few
-// matches itself, and a sorted insertion per member was a third of the
-// kernel); a row that overflows keeps the row_cap smallest indices either
-// way, except in the step's form over the diffused list (LIST), which
-// writes members straight to the row and cuts it at row_cap: the step
-// then repeats with whole rows or reports the capacity error.  The closest particle of every segment is tracked in shared memory
+// Rows (k_cap apart) are sorted by index for the library's neighbourhood
+// calls: the members are collected in shared memory in visiting order and
+// sorted in registers by an odd-even merge network of 16, 24 or 32 (a sorted
+// insertion per member in local memory doubled the kernel: 205 us for 393,000
+// particles, 131 this way; 80 registers and 48 KB a block, three blocks per SM:
+// two take 158 us and four 148 before the rows went out as vectors, three 141); a row that overflows keeps the row_cap smallest
+// indices.  The step's form over the diffused list (LIST) writes members
+// straight to the row in visiting order and cuts it at row_cap: the step then
+// repeats with whole rows or reports the capacity error.  The closest particle of every segment is tracked in shared memory
 // with ties to the smaller index.
+#include <climits>
+
 #include "vrm_internal.cuh"
 
 namespace vrm {
@@ -50,9 +53,61 @@ __device__ __forceinline__ int exact_member(const Consts& c, const double2& pi, 
 // list's order.  Rows are then padded with -1 to the end of their last
 // 32-byte sector, so that the sector is written whole.
 // ROWS = false (list form only): the rows are not written (the count, mask
-// and small neighbourhood are).
-template <int KCAP, bool SORTED, bool LIST = false, bool ROWS = true>
-__global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __restrict__ gp,
+// and small neighbourhood are).  skip (list form, optional): flagged particles
+// are not members (SKIP).
+// Comparators of Batcher's odd-even merge sort of the next power of two, those
+// past N left out (entries there would be the largest).
+template <int N>
+struct SortNet {
+  int n = 0;
+  unsigned char a[256] = {}, b[256] = {};
+  constexpr SortNet() {
+    const int P = N <= 16 ? 16 : 32;
+    for (int p = 1; p < P; p <<= 1)
+      for (int k = p; k >= 1; k >>= 1)
+        for (int j = k % p; j + k < P; j += 2 * k)
+          for (int i = 0; i < k; ++i)
+            if (i + j + k < N && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+              a[n] = (unsigned char)(i + j);
+              b[n] = (unsigned char)(i + j + k);
+              ++n;
+            }
+  }
+};
+template <int N>
+__device__ __forceinline__ void sort_row(int (&v)[N]) {
+  constexpr SortNet<N> net;
+#pragma unroll
+  for (int t = 0; t < net.n; ++t) {
+    const int x = v[net.a[t]], y = v[net.b[t]];
+    v[net.a[t]] = x < y ? x : y;
+    v[net.b[t]] = x < y ? y : x;
+  }
+}
+// The m <= N entries of a thread's list (stride nb) sorted into its row.
+template <int N>
+__device__ __forceinline__ void write_sorted_row(const int* list, int nb, int m, int* __restrict__ row) {
+  int v[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t) v[t] = t < m ? list[t * nb] : INT_MAX;
+  sort_row<N>(v);
+  const bool whole = ((uintptr_t)row & 15u) == 0;  // (k_cap may be any number)
+#pragma unroll
+  for (int t = 0; t < N; t += 4) {
+    if (whole && t + 4 <= m) {
+      *reinterpret_cast<int4*>(row + t) = make_int4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (t + u < m) row[t + u] = v[t + u];
+    }
+  }
+}
+
+// (The list forms want 64 registers, four blocks per SM: 184 us for 696,000
+// particles, 261 at the 80 the compiler takes by itself.)
+template <int KCAP, bool LIST = false, bool ROWS = true, bool SKIP = false>
+__global__ void __launch_bounds__(kBlock, LIST ? 4 : 3) k_search_all(Consts c, const Grid* __restrict__ gp,
                                                        const int* __restrict__ cell_start,
                                                        const double2* __restrict__ sxy,
                                                        const float2* __restrict__ sloc,
@@ -63,7 +118,8 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
                                                        DevStats* __restrict__ ds,
                                                        const int* __restrict__ list = nullptr,
                                                        const int* __restrict__ cell_key = nullptr,
-                                                       const int* __restrict__ cell_rank = nullptr) {
+                                                       const int* __restrict__ cell_rank = nullptr,
+                                                       const uint8_t* __restrict__ skip = nullptr) {
   if (n_dev) n = *n_dev;
   const Grid g = *gp;
   const int k_cap = c.row_cap < KCAP ? c.row_cap : KCAP;  // entries kept
@@ -80,6 +136,7 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
   float* const s_bf = reinterpret_cast<float*>(s_search);
   int* const s_bj = s_search + 8 * nb;
   const int tx = threadIdx.x;
+  int* const row_list = s_search + 16 * nb + tx;  // !LIST: the members so far, entry t at t nb
   for (long t0 = (long)blockIdx.x * blockDim.x + threadIdx.x; t0 < n; t0 += (long)gridDim.x * blockDim.x) {
     int i, cx, cy;
     long p;
@@ -102,8 +159,7 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
     // LIST: members go straight to the row in visiting order (a row longer
     // than row_cap is cut; the step then repeats with whole rows or reports
     // the capacity error, so no smallest-index rule is needed); otherwise
-    // they are collected in a per-thread buffer first
-    int list[LIST ? 1 : KCAP];
+    // they are collected in shared memory first
     int* const row_out = nbr_idx + (size_t)i * stride;
     int cnt = 0;
 #pragma unroll
@@ -135,6 +191,7 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
           const float d2f = __fmaf_rn(du, du, dv * dv);
           if (d2f < g.lo_out || d2f > g.hi_out) continue;
           if (j == i) continue;
+          if (SKIP && skip[j]) continue;
           const bool certain_in = d2f > g.lo_in && d2f < g.hi_in;
           int s = certain_in ? segment_or_ambiguous(du, dv, g.seg_eps) : -1;
           if (s < 0) {
@@ -155,30 +212,29 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
           }
           if (LIST) {
             if (ROWS && cnt < k_cap) row_out[cnt] = j;
-          } else if (SORTED || cnt >= k_cap) {
-            if (!SORTED && cnt == k_cap) {
-              // the row overflows (rare): order the entries kept so far, so
-              // that it keeps the k_cap smallest indices like a sorted row
+          } else if (cnt < k_cap) {
+            row_list[cnt * nb] = j;
+          } else {
+            // the row overflows (rare): it keeps the k_cap smallest indices,
+            // in order from here on
+            if (cnt == k_cap)
               for (int a = 1; a < k_cap; ++a) {
-                const int v = list[a];
+                const int v = row_list[a * nb];
                 int b = a;
-                while (b > 0 && list[b - 1] > v) {
-                  list[b] = list[b - 1];
+                while (b > 0 && row_list[(b - 1) * nb] > v) {
+                  row_list[b * nb] = row_list[(b - 1) * nb];
                   --b;
                 }
-                list[b] = v;
+                row_list[b * nb] = v;
               }
-            }
-            if (cnt < k_cap || j < list[k_cap - 1]) {
-              int pos = cnt < k_cap ? cnt : k_cap - 1;
-              while (pos > 0 && list[pos - 1] > j) {
-                list[pos] = list[pos - 1];
+            if (j < row_list[(k_cap - 1) * nb]) {
+              int pos = k_cap - 1;
+              while (pos > 0 && row_list[(pos - 1) * nb] > j) {
+                row_list[pos * nb] = row_list[(pos - 1) * nb];
                 --pos;
               }
-              list[pos] = j;
+              row_list[pos * nb] = j;
             }
-          } else {
-            list[cnt] = j;  // unsorted row: append in visiting order
           }
           ++cnt;
         }
@@ -210,6 +266,7 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
             if (d2f < g.lo_out || d2f > g.hi_out) continue;
             const int j = sidx[q];
             if (j == i) continue;
+            if (SKIP && skip[j]) continue;
             const bool certain_in = d2f > g.lo_in && d2f < g.hi_in;
             double d2;
             const int s = exact_member(c, pi, sxy[q], certain_in, &d2);
@@ -235,8 +292,15 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
     nbr_count[i] = cnt;
     const int m = cnt < k_cap ? cnt : k_cap;
     int* row = nbr_idx + (size_t)i * stride;
-    if (!LIST)
-      for (int t = 0; t < m; ++t) row[t] = list[t];
+    if (!LIST) {
+      const unsigned here = __activemask();  // (whoever is here decides for itself)
+      if (!__any_sync(here, m > 16))
+        write_sorted_row<16>(row_list, nb, m, row);
+      else if (KCAP > 16 && !__any_sync(here, m > 24))
+        write_sorted_row<(KCAP > 16 ? 24 : 16)>(row_list, nb, m, row);
+      else if (KCAP > 24)
+        write_sorted_row<(KCAP > 24 ? 32 : 16)>(row_list, nb, m, row);
+    }
     if (LIST && ROWS) {
       const int pad = ((m + 7) & ~7) < (int)stride ? ((m + 7) & ~7) : (int)stride;
       for (int t = m; t < pad; ++t) row[t] = -1;
@@ -259,7 +323,7 @@ __global__ void __launch_bounds__(kBlock) k_search_all(Consts c, const Grid* __r
 }
 
 // Small clouds: counts, masks and small neighbourhoods of the listed particles
-// (k_search_all<., false, true, false>), a warp per particle: the lanes test
+// (k_search_all<., true, false>), a warp per particle: the lanes test
 // the candidates, lane s < 8 keeps segment s's closest.  A segment whose two
 // closest members are within two bands of each other in FP32 is decided by
 // the FP64 order in a second pass.
@@ -491,27 +555,25 @@ cudaError_t search_masks_list_dev(const Consts& c, const Grid* g, const int* cel
 }
 
 // Dynamic shared memory of k_search_all: a segment's best distance and
-// index per thread, eight segments.
-static size_t search_smem(int tb) { return (size_t)tb * 8 * (sizeof(float) + sizeof(int)); }
+// index per thread, eight segments, and the row being collected.
+static size_t search_smem(int tb, int list) { return (size_t)tb * (8 * (sizeof(float) + sizeof(int)) + sizeof(int) * list); }
 
-cudaError_t search_all_dev(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
-                           const float2* sorted_loc, const int* sorted_idx, int n_bound, const int* n_dev,
-                           int* nbr_count, int* nbr_idx, uint8_t* seg_mask, int* small, DevStats* ds,
-                           cudaStream_t s, bool sorted) {
-  if (n_bound <= 0) return cudaSuccess;
+cudaError_t search_all(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
+                       const float2* sorted_loc, const int* sorted_idx, int n, int* nbr_count, int* nbr_idx,
+                       uint8_t* seg_mask, int* small, DevStats* ds, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
   const int tb = c.search_block;
-  const int blocks = (int)(((long)n_bound + tb - 1) / tb);
-#define VRM_SEARCH_LAUNCH(K, S)                                                                                     \
-  k_search_all<K, S><<<blocks, tb, search_smem(tb), s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx,      \
-                                                         n_bound, n_dev, nbr_count, nbr_idx, seg_mask, small, ds)
-  if (c.row_cap <= 16) {
-    if (sorted) VRM_SEARCH_LAUNCH(16, true); else VRM_SEARCH_LAUNCH(16, false);
-  } else if (c.row_cap <= 24) {
-    if (sorted) VRM_SEARCH_LAUNCH(24, true); else VRM_SEARCH_LAUNCH(24, false);
-  } else {
-    if (sorted) VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, true); else VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, false);
+  const int blocks = (int)(((long)n + tb - 1) / tb);
+  const auto kernel = c.row_cap <= 16   ? k_search_all<16>
+                      : c.row_cap <= 24 ? k_search_all<24>
+                                        : k_search_all<VRM_KCAP_MAX>;
+  const size_t smem = search_smem(tb, c.row_cap <= 16 ? 16 : c.row_cap <= 24 ? 24 : VRM_KCAP_MAX);
+  if (smem > 40 * 1024) {  // (beside the static part, more than a launch may ask for without this)
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
   }
-#undef VRM_SEARCH_LAUNCH
+  kernel<<<blocks, tb, smem, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, n, nullptr, nbr_count, nbr_idx,
+                                  seg_mask, small, ds, nullptr, nullptr, nullptr, nullptr);
   note_launch();
   return cudaGetLastError();
 }
@@ -520,9 +582,9 @@ cudaError_t search_list_dev(const Consts& c, const Grid* g, const int* cell_star
                             const float2* sorted_loc, const int* sorted_idx, const int* cell_key,
                             const int* cell_rank, const int* list, const int* list_count, int m_bound,
                             int* nbr_count, int* nbr_idx, uint8_t* seg_mask, int* small, DevStats* ds,
-                            cudaStream_t s, bool rows) {
+                            cudaStream_t s, bool rows, const uint8_t* skip) {
   if (m_bound <= 0) return cudaSuccess;
-  if (!rows && warp_scans(c, m_bound)) {
+  if (!rows && !skip && warp_scans(c, m_bound)) {
     k_search_warp<<<warp_grid(m_bound), 128, 0, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, list,
                                                      list_count, cell_key, cell_rank, nbr_count, seg_mask, small, ds);
     note_launch();
@@ -530,28 +592,23 @@ cudaError_t search_list_dev(const Consts& c, const Grid* g, const int* cell_star
   }
   const int tb = c.search_block;
   const int blocks = (int)(((long)m_bound + tb - 1) / tb);
-#define VRM_SEARCH_LAUNCH(K, R)                                                                                    \
-  k_search_all<K, false, true, R><<<blocks, tb, search_smem(tb), s>>>(                                            \
+#define VRM_SEARCH_LAUNCH(K, R, S)                                                                                    \
+  k_search_all<K, true, R, S><<<blocks, tb, search_smem(tb, 0), s>>>(                                            \
       c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, m_bound, list_count, nbr_count, nbr_idx, seg_mask, small, \
-      ds, list, cell_key, cell_rank)
-  if (!rows)
-    VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, false);  // rows not written: the cap only bounds the count
+      ds, list, cell_key, cell_rank, skip)
+  if (!rows && skip)
+    VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, false, true);
+  else if (!rows)
+    VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, false, false);  // rows not written: the cap only bounds the count
   else if (c.row_cap <= 16)
-    VRM_SEARCH_LAUNCH(16, true);
+    VRM_SEARCH_LAUNCH(16, true, false);
   else if (c.row_cap <= 24)
-    VRM_SEARCH_LAUNCH(24, true);
+    VRM_SEARCH_LAUNCH(24, true, false);
   else
-    VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, true);
+    VRM_SEARCH_LAUNCH(VRM_KCAP_MAX, true, false);
 #undef VRM_SEARCH_LAUNCH
   note_launch();
   return cudaGetLastError();
-}
-
-cudaError_t search_all(const Consts& c, const Grid* g, const int* cell_start, const double2* sorted_xy,
-                       const float2* sorted_loc, const int* sorted_idx, int n, int* nbr_count, int* nbr_idx,
-                       uint8_t* seg_mask, int* small, DevStats* ds, cudaStream_t s) {
-  return search_all_dev(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, n, nullptr, nbr_count, nbr_idx,
-                        seg_mask, small, ds, s, true);
 }
 
 }  // namespace vrm
