@@ -70,6 +70,17 @@ __device__ __forceinline__ float gelu(float z) {
   const float hz = 0.5f * z;
   return fmaf(hz, tanh_hw(u), hz);
 }
+// GELU of a pair z0, z1, rounded to bf16 (z0 in the low half): the operations
+// of gelu on packed pairs, half the instructions.
+__device__ __forceinline__ uint32_t gelu_bf16x2(f32x2 z) {
+  const f32x2 t = fma2(pack2(kGeluCA, kGeluCA), mul2(z, z), pack2(kGeluC, kGeluC));
+  const f32x2 hz = mul2(pack2(0.5f, 0.5f), z);
+  float u0, u1;
+  unpack2(mul2(z, t), u0, u1);
+  unpack2(fma2(hz, pack2(tanh_hw(u0), tanh_hw(u1)), hz), u0, u1);
+  const __nv_bfloat162 r = __floats2bfloat162_rn(u0, u1);
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
 // d/dz of the same: 0.5 (1 + t) + 0.5 z (1 - t^2) c (1 + 3 a z^2).
 __device__ __forceinline__ float gelu_grad(float z) {
   const float z2 = z * z;
@@ -84,25 +95,32 @@ __device__ __forceinline__ float gelu_grad(float z) {
 // activations never leave shared memory.  Two tiles are in flight per CTA
 // (slots 0 and 1: activation tiles H[0], H[1], TMEM columns 0-255 and
 // 256-511) so that the MMAs of one overlap the epilogue of the other:
-//   warp 16 (one thread): streams the weight slabs (64 input columns of one
+//   warp 17 (one thread): streams the weight slabs (64 input columns of one
 //     layer: W1, W2, W3 with 256 rows, W4 with 32) through a 3-stage ring
-//     with TMA, loads the input tiles, and issues the MMAs layer by layer,
-//     alternating the slots (a weight slab is loaded once per slot);
+//     with TMA as stages come free, ahead of the MMAs (a weight slab is loaded
+//     once per slot);
+//   warp 16 (one thread): issues the MMAs layer by layer, alternating the
+//     slots;
 //   warps 0-15: the epilogue of each (slot, layer) as its accumulator
 //     completes: warp w reads TMEM lanes 32 (w mod 4), columns 64 (w div 4),
 //     adds the bias, applies GELU and writes bf16 back into the slot's
 //     activation tile in the MMA operand layout (128-byte swizzle), which the
-//     next layer reads as A; the last layer writes the 32 proposals.
+//     next layer reads as A; the last layer writes the 32 proposals, and one
+//     thread loads the slot's next input (its MMAs have read the tile).
 // Barriers per slot: xfull (input tile loaded), accf (the layer's MMAs are
 // complete: commit), actr (the layer's epilogue is done: 16 warp arrivals,
-// so the next layer may overwrite TMEM and read the activations), hfree (the
-// last layer's MMAs are complete: the next input may replace the tile).
+// so the next layer may overwrite TMEM and read the activations).
+// 500,000 rows take 243 us (314 us with one thread for both the weights and
+// the MMAs, whose loads waited behind its issue, a scalar load per bias and
+// GELU a value at a time).  Of a tile's 14,300 clocks the MMA thread spends
+// 10,300 issuing and the epilogues 11,300: shared memory carries both
+// operands, the weight slabs and the activations.
 // Every wait is bounded; one that gives up raises a shared abort flag that
 // every role checks before its next wait, and the error flag in global
 // memory.
 
 constexpr int kEpiWarps = 16;
-constexpr int kFusedThreads = (kEpiWarps + 1) * 32;
+constexpr int kFusedThreads = (kEpiWarps + 2) * 32;
 constexpr int kRing = 3;
 constexpr int kSlabsPerTile = 14;  // W1: 2, W2: 4, W3: 4, W4: 4
 constexpr int kSlabsPerPair = 2 * kSlabsPerTile;
@@ -175,10 +193,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   uint64_t* xfull = bars;
   uint64_t* accf = bars + 2;
   uint64_t* actr = bars + 4;
-  uint64_t* hfree = bars + 6;
-  uint64_t* wfull = bars + 8;
-  uint64_t* wempty = bars + 8 + kRing;
-  uint64_t* drain = bars + 8 + 2 * kRing;
+  uint64_t* wfull = bars + 6;
+  uint64_t* wempty = bars + 6 + kRing;
+  uint64_t* drain = bars + 6 + 2 * kRing;
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
@@ -188,7 +205,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
       umma::mbar_init(&xfull[s], 1);
       umma::mbar_init(&accf[s], 1);
       umma::mbar_init(&actr[s], kEpiWarps);
-      umma::mbar_init(&hfree[s], 1);
     }
     for (int s = 0; s < kRing; ++s) {
       umma::mbar_init(&wfull[s], 1);
@@ -204,27 +220,36 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   umma::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == kEpiWarps) {
-    // ---- producer / MMA issue (one thread) ----
+  auto load_x = [&](int s, int tile) {  // the slot's input tile, over its activations
+    uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
+    umma::mbar_arrive_expect_tx(&xfull[s], 2u * kSlabBytes);
+    umma::tma_load_2d(h, &tx, &xfull[s], 0, tile * kBM);
+    umma::tma_load_2d(h + kSlabBytes, &tx, &xfull[s], kBK, tile * kBM);
+  };
+  if (warp == kEpiWarps + 1) {
+    // ---- weight slabs (one thread) ----
     if (lane == 0) {
       const CUtensorMap* wmap[4] = {&tw1, &tw2, &tw3, &tw4};
-      auto load_w = [&](int gl) {
+      bool fail = false;
+      for (int g = 0; g < total; ++g) {
         int layer, kb;
-        slab_at(gl, pairs_full, &layer, &kb);
-        const int st = gl % kRing;
+        slab_at(g, pairs_full, &layer, &kb);
+        const int st = g % kRing;
+        if (g >= kRing &&
+            (*abort_flag || !umma::mbar_wait(&wempty[st], (uint32_t)(g / kRing - 1) & 1u, 2 * kWaitCycles))) {
+          fail = true;
+          break;
+        }
         umma::mbar_arrive_expect_tx(&wfull[st], layer == 3 ? (uint32_t)kOut * kBK * 2 : kRingBytes);
         umma::tma_load_2d(ring + (size_t)st * kRingBytes, wmap[layer], &wfull[st], kb * kBK, 0);
-      };
-      auto load_x = [&](int s, int tile) {
-        uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
-        umma::mbar_arrive_expect_tx(&xfull[s], 2u * kSlabBytes);
-        umma::tma_load_2d(h, &tx, &xfull[s], 0, tile * kBM);
-        umma::tma_load_2d(h + kSlabBytes, &tx, &xfull[s], kBK, tile * kBM);
-      };
+      }
+      if (fail) *abort_flag = 1;
+    }
+  } else if (warp == kEpiWarps) {
+    // ---- MMA issue (one thread) ----
+    if (lane == 0) {
       load_x(0, blockIdx.x);
       if (my_tiles > 1) load_x(1, blockIdx.x + gridDim.x);
-      int g_load = 0;
-      for (; g_load < kRing && g_load < total; ++g_load) load_w(g_load);
       bool fail = false;
       int g = 0;
       for (int p = 0; p < npairs && !fail; ++p) {
@@ -235,12 +260,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
               fail = true;
               break;
             }
-            if (l == 0 && !umma::mbar_wait(&xfull[s], (uint32_t)p & 1u, kWaitCycles)) {
+            const int e = 4 * p + l;  // epilogues of this slot that must be done
+            if (e > 0 && !umma::mbar_wait(&actr[s], (uint32_t)(e - 1) & 1u, kWaitCycles)) {
               fail = true;
               break;
             }
-            const int e = 4 * p + l;  // epilogues of this slot that must be done
-            if (e > 0 && !umma::mbar_wait(&actr[s], (uint32_t)(e - 1) & 1u, kWaitCycles)) {
+            if (l == 0 && !umma::mbar_wait(&xfull[s], (uint32_t)p & 1u, kWaitCycles)) {
               fail = true;
               break;
             }
@@ -261,30 +286,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
               for (int k = 0; k < kBK / 16; ++k)
                 umma::mma_bf16(tmem + (uint32_t)(s * 256), da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
               umma::mma_commit(&wempty[st]);
-              // refill the slot of the previous slab (its MMAs were issued earlier)
-              const int gp = g - 1;
-              if (gp >= 0 && gp + kRing < total && g_load == gp + kRing) {
-                if (!umma::mbar_wait(&wempty[gp % kRing], (uint32_t)(gp / kRing) & 1u, kWaitCycles)) {
-                  fail = true;
-                  break;
-                }
-                load_w(g_load++);
-              }
             }
-            if (fail) break;
-            umma::mma_commit(&accf[s]);
-            if (l == 3) umma::mma_commit(&hfree[s]);
+            if (!fail) umma::mma_commit(&accf[s]);
           }
-        }
-        // the next inputs, once the last layer's MMAs of a slot have read its tile
-        for (int s = 0; s < nslot && !fail; ++s) {
-          const int nt = 2 * (p + 1) + s;
-          if (nt >= my_tiles) continue;
-          if (!umma::mbar_wait(&hfree[s], (uint32_t)p & 1u, kWaitCycles)) {
-            fail = true;
-            break;
-          }
-          load_x(s, blockIdx.x + nt * gridDim.x);
         }
       }
       if (fail) *abort_flag = 1;
@@ -311,24 +315,37 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             break;
           }
           umma::fence_after_sync();
+          // the last layer's MMAs have read the slot's tile: its next input
+          if (l == 3 && threadIdx.x == 0 && 2 * (p + 1) + s < my_tiles)
+            load_x(s, blockIdx.x + (2 * (p + 1) + s) * gridDim.x);
           const uint32_t trow = tmem + (uint32_t)(s * 256) + ((uint32_t)(q * 32) << 16);
           uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
           if (l < 3) {
-            const float* b = a.bias + (l == 0 ? kOffB1 : l == 1 ? kOffB2 : kOffB3);
+            // 32 columns at a time: the biases four to a load, bias and GELU on
+            // pairs of columns
+            const ulonglong2* b =
+                reinterpret_cast<const ulonglong2*>(a.bias + (l == 0 ? kOffB1 : l == 1 ? kOffB2 : kOffB3) + cg * 64);
+            uint8_t* slab = h + (size_t)cg * kSlabBytes + (size_t)r * 128;
 #pragma unroll 1
-            for (int c0 = cg * 64; c0 < cg * 64 + 64; c0 += 32) {
-              float v[32];
-              umma::tmem_ld32(trow + (uint32_t)c0, v);
-              __align__(16) __nv_bfloat162 hv[16];
+            for (int half = 0; half < 2; ++half) {
+              uint32_t v[32];
+              umma::tmem_request32(trow + (uint32_t)(cg * 64 + half * 32), v);
+              ulonglong2 bb[8];
 #pragma unroll
-              for (int i = 0; i < 16; ++i)
-                hv[i] = __floats2bfloat162_rn(gelu(v[2 * i] + __ldg(b + c0 + 2 * i)),
-                                              gelu(v[2 * i + 1] + __ldg(b + c0 + 2 * i + 1)));
-              uint8_t* slab = h + (size_t)(c0 >> 6) * kSlabBytes + (size_t)r * 128;
-              const int ch = (c0 & 63) >> 3;
+              for (int k = 0; k < 8; ++k) bb[k] = __ldg(b + half * 8 + k);
+              umma::tmem_wait32(v);
 #pragma unroll
-              for (int u = 0; u < 4; ++u)
-                *reinterpret_cast<uint4*>(slab + (((ch + u) ^ (r & 7)) << 4)) = *reinterpret_cast<uint4*>(&hv[4 * u]);
+              for (int u = 0; u < 4; ++u) {  // eight columns: one 16-byte chunk of the operand
+                uint32_t hv[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  const uint32_t* vv = &v[8 * u + 2 * k];
+                  const f32x2 b2 = k & 1 ? bb[2 * u + (k >> 1)].y : bb[2 * u + (k >> 1)].x;
+                  hv[k] = gelu_bf16x2(add2(pack2(__uint_as_float(vv[0]), __uint_as_float(vv[1])), b2));
+                }
+                *reinterpret_cast<uint4*>(slab + (((half * 4 + u) ^ (r & 7)) << 4)) =
+                    make_uint4(hv[0], hv[1], hv[2], hv[3]);
+              }
             }
           } else if (cg < 2) {
             const int c0 = cg * 16;
@@ -434,6 +451,7 @@ __global__ void __launch_bounds__(256) k_gather(const bf16* __restrict__ X_all, 
 // Barriers: xfull (input tile loaded), wfull / wempty (ring), accf (a
 // product's MMAs are complete), actr (its epilogue is done: 16 warps).  Every
 // wait is bounded, as in k_mlp_fused.
+constexpr int kChainThreads = (kEpiWarps + 1) * 32;
 constexpr int kChainRing = 4;
 constexpr int kChainSlabs = 23;  // W1: 2, W2, W3, W4: 4 each, W4^T: 1, W3^T, W2^T: 4 each
 constexpr size_t kChainSmem = 1024 + 4 * (size_t)kSlabBytes + (size_t)kChainRing * kRingBytes + 256;
@@ -457,7 +475,7 @@ struct ChainArgs {
 
 __device__ __forceinline__ int chain_k(int p) { return p == 0 ? 2 : p == 4 ? 1 : 4; }  // K slabs of product p
 
-__global__ void __launch_bounds__(kFusedThreads, 1)
+__global__ void __launch_bounds__(kChainThreads, 1)
     k_chain(const __grid_constant__ CUtensorMap tx, const __grid_constant__ ChainMaps maps,
             const __grid_constant__ ChainArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -1086,7 +1104,7 @@ cudaError_t forward_backward(vrm_mlp* n, cudaStream_t s) {
   a.B = n->B;
   a.error = n->err;
   const int tiles = n->B / kBM;
-  k_chain<<<tiles < sm_count() ? tiles : sm_count(), kFusedThreads, kChainSmem, s>>>(n->mX, n->chain, a);
+  k_chain<<<tiles < sm_count() ? tiles : sm_count(), kChainThreads, kChainSmem, s>>>(n->mX, n->chain, a);
   note_launch();
   k_weight_grad<<<dim3(n->splits, kPieces), 128, kWgSmem, s>>>(n->wg, n->B / kBK / n->splits, n->part, n->err);
   note_launch();
