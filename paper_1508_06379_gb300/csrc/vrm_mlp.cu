@@ -46,6 +46,7 @@ constexpr int kOutPad = 64;   // dY row stride (one K slab)
 constexpr int kBM = 128;      // rows per tile
 constexpr int kBK = 64;       // K per slab
 constexpr long long kWaitCycles = 2000000000LL;  // about one second
+constexpr long long kDrainCycles = 4000000LL;    // about 2 ms
 
 constexpr long kOffW1 = 0, kOffB1 = kOffW1 + (long)kHid * kIn;
 constexpr long kOffW2 = kOffB1 + kHid, kOffB2 = kOffW2 + (long)kHid * kHid;
@@ -91,42 +92,58 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 // ---- fused inference ------------------------------------------------------------------
 //
-// The whole network for 128-row tiles in one persistent kernel; a tile's
-// activations never leave shared memory.  Two tiles are in flight per CTA
-// (slots 0 and 1: activation tiles H[0], H[1], TMEM columns 0-255 and
-// 256-511) so that the MMAs of one overlap the epilogue of the other:
-//   warp 17 (one thread): streams the weight slabs (64 input columns of one
-//     layer: W1, W2, W3 with 256 rows, W4 with 32) through a 3-stage ring
-//     with TMA as stages come free, ahead of the MMAs (a weight slab is loaded
-//     once per slot);
-//   warp 16 (one thread): issues the MMAs layer by layer, alternating the
-//     slots;
+// The whole network for 256-row tiles in one persistent kernel of CTA pairs; a
+// tile's activations never leave shared memory.  A CTA holds 128 of the rows
+// and half of every weight slab; one MMA of the pair covers both.  Two tiles
+// are in flight per pair (slots 0 and 1: activation tiles H[0], H[1], TMEM
+// columns 0-255 and 256-511) so that the MMAs of one overlap the epilogue of
+// the other:
+//   warp 17 (one thread): streams the CTA's halves of the weight slabs (64
+//     input columns of one layer: 128 rows of W1, W2, W3, 16 of W4) through a
+//     5-stage ring with TMA as stages come free, ahead of the MMAs (a weight
+//     slab is loaded once per slot);
+//   warp 16 of the leading CTA (one thread): issues the MMAs layer by layer,
+//     alternating the slots;
+//   warp 18 (one thread): loads a slot's next input as its last layer's MMAs
+//     complete;
 //   warps 0-15: the epilogue of each (slot, layer) as its accumulator
 //     completes: warp w reads TMEM lanes 32 (w mod 4), columns 64 (w div 4),
 //     adds the bias, applies GELU and writes bf16 back into the slot's
 //     activation tile in the MMA operand layout (128-byte swizzle), which the
-//     next layer reads as A; the last layer writes the 32 proposals, and one
-//     thread loads the slot's next input (its MMAs have read the tile).
-// Barriers per slot: xfull (input tile loaded), accf (the layer's MMAs are
-// complete: commit), actr (the layer's epilogue is done: 16 warp arrivals,
-// so the next layer may overwrite TMEM and read the activations).
-// 500,000 rows take 243 us (314 us with one thread for both the weights and
-// the MMAs, whose loads waited behind its issue, a scalar load per bias and
-// GELU a value at a time).  Of a tile's 14,300 clocks the MMA thread spends
-// 10,300 issuing and the epilogues 11,300: shared memory carries both
-// operands, the weight slabs and the activations.
-// Every wait is bounded; one that gives up raises a shared abort flag that
-// every role checks before its next wait, and the error flag in global
-// memory.
+//     next layer reads as A; the last layer writes the 32 proposals.
+// Barriers (xfull, actr and wfull count in the leading CTA for both, accf and
+// wempty are signalled in both): xfull (a slot's input tiles loaded), accf (the
+// layer's MMAs are complete: commit), actr (the layer's epilogue is done: 32
+// warp arrivals, so the next layer may overwrite TMEM and read the
+// activations), hfree (the last layer's MMAs are complete: the next input may
+// replace the tile; both CTAs), wfull and wempty (ring).  Every wait is bounded;
+// one that gives up raises its CTA's abort flag, which every role checks before
+// its next wait, and the error flag in global memory.
+//
+// 500,000 rows take 207 us (314 us with a 128-row tile per CTA and one thread
+// for weights, inputs and MMAs; 243 us with a thread for the weights, biases by
+// vector and GELU on pairs).  What the rest gave, in clocks of the MMA thread
+// per 128-row tile: issue 4,600 -> 1,100 with an elected thread (a branch on
+// the lane makes every MMA wait for its operands to move to uniform
+// registers); the pair halves what shared memory takes in and L2 gives out per
+// MMA, 448 KB a tile before.  The arrivals keep their default scope: the
+// activations cross to the async proxy by the proxy fence before them, and an
+// arrival released at cluster scope waits for all the CTA's stores (300 us).
+// What bounds it now: of a tile's 11,000 clocks the epilogues take 9,000, three
+// times about 3,000, at 1,600 of the FMA pipe (six operations a value) and
+// 2,400 of shared memory (64 KB of A, 64 KB of the half weight slabs read, 64 KB
+// of them and 64 KB of activations written).  Epilogue warps split between the
+// slots instead took 250 us: two warps a scheduler do not cover the latencies.
 
 constexpr int kEpiWarps = 16;
-constexpr int kFusedThreads = (kEpiWarps + 2) * 32;
-constexpr int kRing = 3;
+constexpr int kFusedThreads = (kEpiWarps + 3) * 32;
+constexpr int kRing = 5;
 constexpr int kSlabsPerTile = 14;  // W1: 2, W2: 4, W3: 4, W4: 4
 constexpr int kSlabsPerPair = 2 * kSlabsPerTile;
-constexpr uint32_t kSlabBytes = kBM * kBK * 2;  // one 128-row activation slab
+constexpr uint32_t kSlabBytes = kBM * kBK * 2;  // one 128-row activation slab, or half a weight slab
 constexpr uint32_t kRingBytes = 256 * kBK * 2;  // one 256-row weight slab
-constexpr size_t kFusedSmem = 1024 + 2 * 4 * (size_t)kSlabBytes + (size_t)kRing * kRingBytes + 256;
+constexpr int kBiases = 3 * kHid + kOut;
+constexpr size_t kFusedSmem = 1024 + (2 * 4 + kRing) * (size_t)kSlabBytes + kBiases * sizeof(float) + 256;
 
 // Layer and K slab of the g-th weight slab a single tile consumes.
 __device__ __forceinline__ void slab_of(int s, int* layer, int* kb) {
@@ -169,7 +186,7 @@ struct FusedArgs {
   int* error;
 };
 
-__global__ void __launch_bounds__(kFusedThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFusedThreads, 1)
     k_mlp_fused(const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap tw1,
                 const __grid_constant__ CUtensorMap tw2, const __grid_constant__ CUtensorMap tw3,
                 const __grid_constant__ CUtensorMap tw4, FusedArgs a) {
@@ -179,23 +196,27 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     const int r = *a.rows_dev;
     rows = r < rows ? r : rows;
   }
-  const int ntiles = (rows + kBM - 1) / kBM;
-  if ((int)blockIdx.x >= ntiles) return;
-  const int my_tiles = (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+  const int ntiles = (rows + 2 * kBM - 1) / (2 * kBM);
+  const int pair = (int)blockIdx.x >> 1, npair = (int)gridDim.x >> 1;
+  const int rank = (int)umma::cluster_rank();
+  if (pair >= ntiles) return;  // both CTAs
+  const int my_tiles = (ntiles - 1 - pair) / npair + 1;
   const int pairs_full = my_tiles / 2;
   const int npairs = (my_tiles + 1) / 2;
   const int total = pairs_full * kSlabsPerPair + (my_tiles & 1) * kSlabsPerTile;
 
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* H = base;                         // 2 slots x 4 slabs x 16 KB
-  uint8_t* ring = base + 8 * (size_t)kSlabBytes;  // kRing x 32 KB
-  uint64_t* bars = (uint64_t*)(ring + (size_t)kRing * kRingBytes);
+  uint8_t* H = base;                              // 2 slots x 4 slabs x 16 KB
+  uint8_t* ring = base + 8 * (size_t)kSlabBytes;  // kRing x 16 KB
+  float* s_bias = (float*)(ring + (size_t)kRing * kSlabBytes);  // b1, b2, b3, b4
+  uint64_t* bars = (uint64_t*)(s_bias + kBiases);
   uint64_t* xfull = bars;
   uint64_t* accf = bars + 2;
   uint64_t* actr = bars + 4;
-  uint64_t* wfull = bars + 6;
-  uint64_t* wempty = bars + 6 + kRing;
-  uint64_t* drain = bars + 6 + 2 * kRing;
+  uint64_t* hfree = bars + 6;
+  uint64_t* wfull = bars + 8;
+  uint64_t* wempty = bars + 8 + kRing;
+  uint64_t* drain = bars + 8 + 2 * kRing;
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
@@ -204,7 +225,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     for (int s = 0; s < 2; ++s) {
       umma::mbar_init(&xfull[s], 1);
       umma::mbar_init(&accf[s], 1);
-      umma::mbar_init(&actr[s], kEpiWarps);
+      umma::mbar_init(&actr[s], 2 * kEpiWarps);
+      umma::mbar_init(&hfree[s], 1);
     }
     for (int s = 0; s < kRing; ++s) {
       umma::mbar_init(&wfull[s], 1);
@@ -214,42 +236,59 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     *abort_flag = 0;
     umma::fence_barrier_init();
   }
-  if (warp == 0) umma::tmem_alloc(tmem_slot, 512);
+  for (int k = threadIdx.x; k < kBiases; k += kFusedThreads)
+    s_bias[k] = a.bias[(k < kHid ? kOffB1 : k < 2 * kHid ? kOffB2 : k < 3 * kHid ? kOffB3 : kOffB4) + k % kHid];
+  __syncwarp();
+  if (warp == 0) umma::tmem_alloc_pair(tmem_slot, 512);
   umma::fence_before_sync();
   __syncthreads();
+  umma::cluster_sync();
   umma::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  const int last_tile = (rows - 1) / kBM;  // 128-row tiles of the input
 
-  auto load_x = [&](int s, int tile) {  // the slot's input tile, over its activations
-    uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
-    umma::mbar_arrive_expect_tx(&xfull[s], 2u * kSlabBytes);
-    umma::tma_load_2d(h, &tx, &xfull[s], 0, tile * kBM);
-    umma::tma_load_2d(h + kSlabBytes, &tx, &xfull[s], kBK, tile * kBM);
-  };
   if (warp == kEpiWarps + 1) {
     // ---- weight slabs (one thread) ----
-    if (lane == 0) {
+    if (umma::elect_one()) {
       const CUtensorMap* wmap[4] = {&tw1, &tw2, &tw3, &tw4};
-      bool fail = false;
       for (int g = 0; g < total; ++g) {
         int layer, kb;
         slab_at(g, pairs_full, &layer, &kb);
         const int st = g % kRing;
-        if (g >= kRing &&
-            (*abort_flag || !umma::mbar_wait(&wempty[st], (uint32_t)(g / kRing - 1) & 1u, 2 * kWaitCycles))) {
-          fail = true;
+        if (g >= kRing && (*abort_flag || !umma::mbar_wait(&wempty[st], (uint32_t)(g / kRing - 1) & 1u,
+                                                                   2 * kWaitCycles))) {
+          *abort_flag = 1;
           break;
         }
-        umma::mbar_arrive_expect_tx(&wfull[st], layer == 3 ? (uint32_t)kOut * kBK * 2 : kRingBytes);
-        umma::tma_load_2d(ring + (size_t)st * kRingBytes, wmap[layer], &wfull[st], kb * kBK, 0);
+        const int half = layer == 3 ? kOut / 2 : kBM;  // rows of this CTA
+        if (rank == 0) umma::mbar_arrive_expect_tx(&wfull[st], 2u * (uint32_t)half * kBK * 2);
+        umma::tma_load_2d_pair(ring + (size_t)st * kSlabBytes, wmap[layer], umma::lead_addr(&wfull[st]), kb * kBK,
+                               rank * half);
       }
-      if (fail) *abort_flag = 1;
+    }
+  } else if (warp == kEpiWarps + 2) {
+    // ---- input tiles (one thread) ----
+    if (umma::elect_one()) {
+      for (int i = 0; i < my_tiles; ++i) {
+        const int s = i & 1;
+        if (i >= 2 && (*abort_flag || !umma::mbar_wait(&hfree[s], (uint32_t)(i / 2 - 1) & 1u, 2 * kWaitCycles))) {
+          *abort_flag = 1;
+          break;
+        }
+        // over the slot's activations; a half beyond the last row loads the
+        // last rows again and stores nothing
+        uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
+        const int t = 2 * (pair + i * npair) + rank;
+        const int row0 = (t < last_tile ? t : last_tile) * kBM;
+        const uint32_t bar = umma::lead_addr(&xfull[s]);
+        if (rank == 0) umma::mbar_arrive_expect_tx(&xfull[s], 4u * kSlabBytes);
+        umma::tma_load_2d_pair(h, &tx, bar, 0, row0);
+        umma::tma_load_2d_pair(h + kSlabBytes, &tx, bar, kBK, row0);
+      }
     }
   } else if (warp == kEpiWarps) {
-    // ---- MMA issue (one thread) ----
-    if (lane == 0) {
-      load_x(0, blockIdx.x);
-      if (my_tiles > 1) load_x(1, blockIdx.x + gridDim.x);
+    // ---- MMA issue (one thread of the pair) ----
+    if (rank == 0 && umma::elect_one()) {
       bool fail = false;
       int g = 0;
       for (int p = 0; p < npairs && !fail; ++p) {
@@ -270,7 +309,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
               break;
             }
             umma::fence_after_sync();
-            const uint32_t idesc = umma::idesc_bf16(kBM, l == 3 ? kOut : kHid);
+            const uint32_t idesc = umma::idesc_bf16(2 * kBM, l == 3 ? kOut : kHid);
             const int nk = l == 0 ? 2 : 4;
             uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
             for (int kb = 0; kb < nk; ++kb, ++g) {
@@ -281,25 +320,27 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
               }
               umma::fence_after_sync();
               const uint64_t da = umma::desc_sw128(umma::smem_u32(h + (size_t)kb * kSlabBytes));
-              const uint64_t db = umma::desc_sw128(umma::smem_u32(ring + (size_t)st * kRingBytes));
+              const uint64_t db = umma::desc_sw128(umma::smem_u32(ring + (size_t)st * kSlabBytes));
 #pragma unroll
               for (int k = 0; k < kBK / 16; ++k)
-                umma::mma_bf16(tmem + (uint32_t)(s * 256), da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
-              umma::mma_commit(&wempty[st]);
+                umma::mma_bf16_pair(tmem + (uint32_t)(s * 256), da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+              umma::mma_commit_pair(&wempty[st]);
             }
-            if (!fail) umma::mma_commit(&accf[s]);
+            if (fail) break;
+            umma::mma_commit_pair(&accf[s]);
+            if (l == 3) umma::mma_commit_pair(&hfree[s]);
           }
         }
       }
       if (fail) *abort_flag = 1;
       // every MMA issued completes before the TMEM is released
-      umma::mma_commit(drain);
+      umma::mma_commit_pair(drain);
       if (!umma::mbar_wait(drain, 0u, kWaitCycles)) *abort_flag = 1;
     }
   } else {
     // ---- epilogue warps ----
     const int q = warp & 3, cg = warp >> 2;
-    const int r = q * 32 + lane;  // row within the tile
+    const int r = q * 32 + lane;  // row within the CTA's half of the tile
     bool stop = false;
     for (int p = 0; p < npairs && !stop; ++p) {
       const int nslot = (2 * p + 1 < my_tiles) ? 2 : 1;
@@ -315,66 +356,74 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             break;
           }
           umma::fence_after_sync();
-          // the last layer's MMAs have read the slot's tile: its next input
-          if (l == 3 && threadIdx.x == 0 && 2 * (p + 1) + s < my_tiles)
-            load_x(s, blockIdx.x + (2 * (p + 1) + s) * gridDim.x);
           const uint32_t trow = tmem + (uint32_t)(s * 256) + ((uint32_t)(q * 32) << 16);
-          uint8_t* h = H + (size_t)s * 4 * kSlabBytes;
+          const uint32_t done = umma::lead_addr(&actr[s]);
           if (l < 3) {
-            // 32 columns at a time: the biases four to a load, bias and GELU on
-            // pairs of columns
-            const ulonglong2* b =
-                reinterpret_cast<const ulonglong2*>(a.bias + (l == 0 ? kOffB1 : l == 1 ? kOffB2 : kOffB3) + cg * 64);
-            uint8_t* slab = h + (size_t)cg * kSlabBytes + (size_t)r * 128;
-#pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-              uint32_t v[32];
-              umma::tmem_request32(trow + (uint32_t)(cg * 64 + half * 32), v);
-              ulonglong2 bb[8];
+            // 32 columns at a time, bias and GELU on pairs of columns
+            const ulonglong2* b = reinterpret_cast<const ulonglong2*>(s_bias + l * kHid + cg * 64);
+            uint8_t* slab = H + ((size_t)s * 4 + cg) * kSlabBytes + (size_t)r * 128;
+            uint32_t va[32], vb[32];
+            umma::tmem_request32(trow + (uint32_t)(cg * 64), va);
+            umma::tmem_wait32(va);
+            umma::tmem_request32(trow + (uint32_t)(cg * 64 + 32), vb);
 #pragma unroll
-              for (int k = 0; k < 8; ++k) bb[k] = __ldg(b + half * 8 + k);
-              umma::tmem_wait32(v);
+            for (int half = 0; half < 2; ++half) {
+              if (half == 1) umma::tmem_wait32(vb);
+              const uint32_t* v = half == 0 ? va : vb;
 #pragma unroll
               for (int u = 0; u < 4; ++u) {  // eight columns: one 16-byte chunk of the operand
                 uint32_t hv[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const uint32_t* vv = &v[8 * u + 2 * k];
-                  const f32x2 b2 = k & 1 ? bb[2 * u + (k >> 1)].y : bb[2 * u + (k >> 1)].x;
-                  hv[k] = gelu_bf16x2(add2(pack2(__uint_as_float(vv[0]), __uint_as_float(vv[1])), b2));
+                for (int k = 0; k < 2; ++k) {
+                  const ulonglong2 b4 = b[half * 8 + 2 * u + k];
+                  const uint32_t* vv = &v[8 * u + 4 * k];
+                  hv[2 * k] = gelu_bf16x2(add2(pack2(__uint_as_float(vv[0]), __uint_as_float(vv[1])), b4.x));
+                  hv[2 * k + 1] = gelu_bf16x2(add2(pack2(__uint_as_float(vv[2]), __uint_as_float(vv[3])), b4.y));
                 }
                 *reinterpret_cast<uint4*>(slab + (((half * 4 + u) ^ (r & 7)) << 4)) =
                     make_uint4(hv[0], hv[1], hv[2], hv[3]);
               }
             }
-          } else if (cg < 2) {
-            const int c0 = cg * 16;
+            umma::fence_proxy_async_smem();  // the activation writes feed the next MMAs (async proxy)
+            umma::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive_cluster(done);
+          } else {
+            // the accumulator is free once it is read; the proposals are stored after that
             float v[16];
-            umma::tmem_ld16(trow + (uint32_t)c0, v);
-            const int row = (blockIdx.x + (2 * p + s) * gridDim.x) * kBM + r;
-            if (row < rows) {
-              const float* b = a.bias + kOffB4 + c0;
+            const int c0 = (cg & 1) * 16;
+            if (cg < 2) umma::tmem_ld16(trow + (uint32_t)c0, v);
+            umma::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive_cluster(done);
+            const int row = ((pair + (2 * p + s) * npair) * 2 + rank) * kBM + r;
+            if (cg < 2 && row < rows) {
+              const float* b = s_bias + 3 * kHid + c0;
               float4* dst = reinterpret_cast<float4*>(a.Y + (size_t)row * kOut + c0);
 #pragma unroll
               for (int i = 0; i < 4; ++i)
-                dst[i] = make_float4(v[4 * i] + __ldg(b + 4 * i), v[4 * i + 1] + __ldg(b + 4 * i + 1),
-                                     v[4 * i + 2] + __ldg(b + 4 * i + 2), v[4 * i + 3] + __ldg(b + 4 * i + 3));
+                dst[i] = make_float4(v[4 * i] + b[4 * i], v[4 * i + 1] + b[4 * i + 1], v[4 * i + 2] + b[4 * i + 2],
+                                     v[4 * i + 3] + b[4 * i + 3]);
             }
           }
-          umma::fence_proxy_async_smem();  // the activation writes feed the next MMAs (async proxy)
-          umma::fence_before_sync();
-          __syncwarp();
-          if (lane == 0) umma::mbar_arrive(&actr[s]);
         }
       }
     }
   }
+  __syncwarp();
   umma::fence_before_sync();
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag && a.error) atomicExch(a.error, 1);
+  if (*abort_flag) {
+    if (threadIdx.x == 0 && a.error) atomicExch(a.error, 1);
+    // copies that nothing waited for arrive before the CTA ends
+    const long long t0 = clock64();
+    while (clock64() - t0 < kDrainCycles) {
+    }
+  }
+  umma::cluster_sync();  // no MMA, copy or arrival of the peer is under way
   if (warp == 0) {
     umma::fence_after_sync();
-    umma::tmem_dealloc(tmem, 512);
+    umma::tmem_dealloc_pair(tmem, 512);
   }
 }
 
@@ -1005,6 +1054,7 @@ struct vrm_mlp {
   float* Z[3] = {};
   bf16 *At[3] = {}, *dZt[3] = {}, *dYt = nullptr;
   CUtensorMap mW1, mW2, mW3, mW4;  // weights as B operands
+  CUtensorMap half[4];             // the same, half of the rows at a time (CTA pairs)
   CUtensorMap mX;
   ChainMaps chain;
   WgMaps wg;
@@ -1046,15 +1096,16 @@ cudaError_t mlp_forward(vrm_mlp* net, const CUtensorMap& mX, int rows, const int
     if (r != cudaSuccess) return r;
     attr_set = true;
   }
-  const int ntiles = (rows + kBM - 1) / kBM;
-  const int grid = ntiles < sm_count() ? ntiles : sm_count();
+  const int ntiles = (rows + 2 * kBM - 1) / (2 * kBM), npair = sm_count() / 2;
+  const int grid = 2 * (ntiles < npair ? ntiles : npair);
   FusedArgs fa;
   fa.bias = net->theta;
   fa.Y = Y;
   fa.rows = rows;
   fa.rows_dev = rows_dev;
   fa.error = net->err;
-  k_mlp_fused<<<grid, kFusedThreads, kFusedSmem, s>>>(mX, net->mW1, net->mW2, net->mW3, net->mW4, fa);
+  k_mlp_fused<<<grid, kFusedThreads, kFusedSmem, s>>>(mX, net->half[0], net->half[1], net->half[2], net->half[3],
+                                                      fa);
   note_launch();
   return cudaGetLastError();
 }
@@ -1226,6 +1277,8 @@ vrm_status vrm_mlp_create(int32_t batch_rows, vrm_mlp** out) {
 #undef MLP_ALLOC
   bool ok = e == cudaSuccess;
   // B operands: boxes of N rows; A operands: 128-row boxes
+  ok = ok && make_map(&n->half[0], n->W1, kHid, kInPad, kBM) && make_map(&n->half[1], n->W2, kHid, kHid, kBM) &&
+       make_map(&n->half[2], n->W3, kHid, kHid, kBM) && make_map(&n->half[3], n->W4, kOut, kHid, kOut / 2);
   ok = ok && make_map(&n->mW1, n->W1, kHid, kInPad, 256) && make_map(&n->mW2, n->W2, kHid, kHid, 256) &&
        make_map(&n->mW3, n->W3, kHid, kHid, 256) && make_map(&n->mW4, n->W4, kOut, kHid, 32) &&
        make_map(&n->mX, n->Xb, B, kInPad, kBM);
