@@ -16,9 +16,9 @@
 //   k_weight_grad  the weight gradients of every layer, split over the batch
 //   k_update     the splits and the biases summed in a fixed order (training is
 //                deterministic), AdamW, and the bf16 copies of the weights
-// A batch of 4096 rows takes 95 us (540 us with a kernel per product, whose 32
+// A batch of 4096 rows takes 81 us (540 us with a kernel per product, whose 32
 // CTAs stored row by row, a one-block loss and separate sums: 23 launches),
-// 512 rows 81 us (366), 16,384 rows 134 us (1123).
+// 512 rows 69 us (369), 16,384 rows 119 us (1119).
 // The products are tcgen05 MMAs (M = 128, K = 16) on K-major bf16 tiles that
 // TMA or the epilogues leave in shared memory in the 128-byte swizzle, with
 // fp32 accumulators in TMEM.
@@ -66,13 +66,7 @@ __device__ __forceinline__ float tanh_hw(float u) {
 }
 // c (z + a z^3) as z (c + (c a) z^2): five fp32 operations and the tanh.
 constexpr float kGeluCA = kGeluC * kGeluA;
-__device__ __forceinline__ float gelu(float z) {
-  const float u = z * fmaf(kGeluCA, z * z, kGeluC);
-  const float hz = 0.5f * z;
-  return fmaf(hz, tanh_hw(u), hz);
-}
-// GELU of a pair z0, z1, rounded to bf16 (z0 in the low half): the operations
-// of gelu on packed pairs, half the instructions.
+// Of a pair z0, z1 (half the instructions), rounded to bf16 with z0 in the low half.
 __device__ __forceinline__ uint32_t gelu_bf16x2(f32x2 z) {
   const f32x2 t = fma2(pack2(kGeluCA, kGeluCA), mul2(z, z), pack2(kGeluC, kGeluC));
   const f32x2 hz = mul2(pack2(0.5f, 0.5f), z);
@@ -82,12 +76,16 @@ __device__ __forceinline__ uint32_t gelu_bf16x2(f32x2 z) {
   const __nv_bfloat162 r = __floats2bfloat162_rn(u0, u1);
   return *reinterpret_cast<const uint32_t*>(&r);
 }
-// d/dz of the same: 0.5 (1 + t) + 0.5 z (1 - t^2) c (1 + 3 a z^2).
-__device__ __forceinline__ float gelu_grad(float z) {
-  const float z2 = z * z;
-  const float t = tanh_hw(kGeluC * fmaf(kGeluA * z, z2, z));
-  const float du = kGeluC * fmaf(3.0f * kGeluA, z2, 1.0f);
-  return fmaf(0.5f * z * du, fmaf(-t, t, 1.0f), 0.5f * (1.0f + t));
+// d/dz of the same, of a pair: 0.5 (1 + t) + 0.5 z (1 - t^2) c (1 + 3 a z^2).
+__device__ __forceinline__ f32x2 gelu_grad2(f32x2 z) {
+  const f32x2 one = pack2(1.0f, 1.0f), half = pack2(0.5f, 0.5f), cc = pack2(kGeluC, kGeluC);
+  const f32x2 z2 = mul2(z, z);
+  float u0, u1;
+  unpack2(mul2(cc, fma2(mul2(pack2(kGeluA, kGeluA), z), z2, z)), u0, u1);
+  const float t0 = tanh_hw(u0), t1 = tanh_hw(u1);
+  const f32x2 t = pack2(t0, t1);
+  const f32x2 du = mul2(cc, fma2(pack2(3.0f * kGeluA, 3.0f * kGeluA), z2, one));
+  return fma2(mul2(mul2(half, z), du), fma2(pack2(-t0, -t1), t, one), mul2(half, add2(one, t)));
 }
 
 // ---- fused inference ------------------------------------------------------------------
@@ -490,20 +488,28 @@ __global__ void __launch_bounds__(256) k_gather(const bf16* __restrict__ X_all, 
 //   3    Y = A W4^T + b4, dY = 2 M (Y - T) / sum(M) and the tile's loss
 //   4    dZ3 = (dY W4) GELU'(Z3)
 //   5, 6 dZ2 = (dZ3 W3) GELU'(Z2), dZ1 = (dZ2 W2) GELU'(Z1)
-// One thread of warp 16 streams the weight slabs through a ring with TMA and
-// issues the MMAs; warps 0-15 run each product's epilogue (warp w: TMEM lanes
-// 32 (w mod 4), columns 64 (w div 4)) and write the next operand in the
-// swizzled layout.  Pre-activations go to global memory and come back to the
-// same thread, tile by tile with the rows contiguous; what k_weight_grad reads
-// (A^T, dZ^T, dY^T) goes out transposed, 64 bytes of a row per warp.  The
-// chain is bound by its own latency: about 3 us per product.
+// One thread of warp 17 streams the weight slabs through a ring with TMA, one of
+// warp 16 loads the inputs and issues the MMAs; warps 0-15 run each product's
+// epilogue (warp w: TMEM lanes 32 (w mod 4), columns 64 (w div 4)) and write the
+// next operand in the swizzled layout.  Products accumulate in alternating
+// halves of the TMEM (chain_half), so that what an epilogue stores goes out
+// after the operand is handed over, under the next product: pre-activations Z1
+// and Z2, which come back to the same thread, tile by tile with the rows
+// contiguous (Z3 stays in its half until product 4), and what k_weight_grad
+// reads (A^T, dZ^T, dY^T), transposed, 64 bytes of a row per warp.
+// The chain is bound by its epilogues: of 63,000 clocks for a tile those up to
+// the hand-over take 4,000 (forward) and 6,500 (backward) a product, the MMAs
+// 2,000, and the stores 5,000 beside them (192 KB a product from one SM).  A step
+// of 4096 rows went from 95 to 81 us with the stores after the hand-over, elected
+// threads, a thread for the weights, biases in shared memory (each is used once
+// by a tile: a load from L2 every time) and Z3 kept.
 // Barriers: xfull (input tile loaded), wfull / wempty (ring), accf (a
 // product's MMAs are complete), actr (its epilogue is done: 16 warps).  Every
 // wait is bounded, as in k_mlp_fused.
-constexpr int kChainThreads = (kEpiWarps + 1) * 32;
+constexpr int kChainThreads = (kEpiWarps + 2) * 32;
 constexpr int kChainRing = 4;
-constexpr int kChainSlabs = 23;  // W1: 2, W2, W3, W4: 4 each, W4^T: 1, W3^T, W2^T: 4 each
-constexpr size_t kChainSmem = 1024 + 4 * (size_t)kSlabBytes + (size_t)kChainRing * kRingBytes + 256;
+constexpr size_t kChainSmem =
+    1024 + 4 * (size_t)kSlabBytes + (size_t)kChainRing * kRingBytes + kBiases * sizeof(float) + 256;
 
 struct ChainMaps {
   CUtensorMap w[7];  // W1, W2, W3, W4, W4^T, W3^T, W2^T
@@ -513,7 +519,7 @@ struct ChainArgs {
   const bf16* Xb;
   const float* Tb;
   const float* cnt;   // mask sums of the batch's 32-row blocks
-  float* Z[3];        // [tile][256][128]
+  float* Z[2];        // [tile][256][128]
   bf16* At[3];        // A1^T, A2^T, A3^T [256 x B]
   bf16* dZt[3];       // dZ1^T, dZ2^T, dZ3^T [256 x B]
   bf16* dYt;          // [128 x B], rows >= 32 stay 0
@@ -522,6 +528,8 @@ struct ChainArgs {
   int* error;
 };
 
+// Half of the TMEM that product p accumulates in.
+__device__ __forceinline__ uint32_t chain_half(int p) { return p == 1 || p == 3 || p == 4 || p == 6 ? 256u : 0u; }
 __device__ __forceinline__ int chain_k(int p) { return p == 0 ? 2 : p == 4 ? 1 : 4; }  // K slabs of product p
 
 __global__ void __launch_bounds__(kChainThreads, 1)
@@ -533,7 +541,8 @@ __global__ void __launch_bounds__(kChainThreads, 1)
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* H = base;                              // 4 slabs x 16 KB
   uint8_t* ring = base + 4 * (size_t)kSlabBytes;  // kChainRing x 32 KB
-  uint64_t* bars = (uint64_t*)(ring + (size_t)kChainRing * kRingBytes);
+  float* s_bias = (float*)(ring + (size_t)kChainRing * kRingBytes);  // b1, b2, b3, b4
+  uint64_t* bars = (uint64_t*)(s_bias + kBiases);
   uint64_t *xfull = bars, *accf = bars + 1, *actr = bars + 2, *drain = bars + 3;
   uint64_t *wfull = bars + 4, *wempty = bars + 4 + kChainRing;
   uint32_t* tmem_slot = (uint32_t*)(bars + 4 + 2 * kChainRing);
@@ -552,33 +561,47 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     *abort_flag = 0;
     umma::fence_barrier_init();
   }
-  if (warp == 0) umma::tmem_alloc(tmem_slot, 256);
+  for (int k = threadIdx.x; k < kBiases; k += kChainThreads)
+    s_bias[k] = a.theta[(k < kHid ? kOffB1 : k < 2 * kHid ? kOffB2 : k < 3 * kHid ? kOffB3 : kOffB4) + k % kHid];
+  __syncwarp();
+  if (warp == 0) umma::tmem_alloc(tmem_slot, 512);
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == kEpiWarps) {
-    if (lane == 0) {
-      const int total = my_tiles * kChainSlabs;
-      int lp = 0, lk = 0;  // product and slab of the next load
-      auto load_w = [&](int gl) {
-        const int st = gl % kChainRing;
-        umma::mbar_arrive_expect_tx(&wfull[st], lp == 3 ? (uint32_t)kOut * kBK * 2 : kRingBytes);
-        umma::tma_load_2d(ring + (size_t)st * kRingBytes, &maps.w[lp], &wfull[st], lk * kBK, 0);
-        if (++lk == chain_k(lp)) {
-          lk = 0;
-          lp = lp == 6 ? 0 : lp + 1;
+  if (warp == kEpiWarps + 1) {
+    // ---- weight slabs (one thread) ----
+    if (umma::elect_one()) {
+      int g = 0;
+      bool fail = false;
+      for (int i = 0; i < my_tiles && !fail; ++i) {
+        for (int p = 0; p < 7 && !fail; ++p) {
+          const int nk = chain_k(p);
+          for (int kb = 0; kb < nk; ++kb, ++g) {
+            const int st = g % kChainRing;
+            if (g >= kChainRing && (*abort_flag || !umma::mbar_wait(&wempty[st], (uint32_t)(g / kChainRing - 1) & 1u,
+                                                                    2 * kWaitCycles))) {
+              *abort_flag = 1;
+              fail = true;
+              break;
+            }
+            umma::mbar_arrive_expect_tx(&wfull[st], p == 3 ? (uint32_t)kOut * kBK * 2 : kRingBytes);
+            umma::tma_load_2d(ring + (size_t)st * kRingBytes, &maps.w[p], &wfull[st], kb * kBK, 0);
+          }
         }
-      };
+      }
+    }
+  } else if (warp == kEpiWarps) {
+    // ---- inputs and MMA issue (one thread) ----
+    if (umma::elect_one()) {
       auto load_x = [&](int tile) {
         umma::mbar_arrive_expect_tx(xfull, 2u * kSlabBytes);
         umma::tma_load_2d(H, &tx, xfull, 0, tile * kBM);
         umma::tma_load_2d(H + kSlabBytes, &tx, xfull, kBK, tile * kBM);
       };
       load_x(blockIdx.x);
-      int g_load = 0, g = 0;
-      for (; g_load < kChainRing && g_load < total; ++g_load) load_w(g_load);
+      int g = 0;
       bool fail = false;
       for (int i = 0; i < my_tiles && !fail; ++i) {
         for (int p = 0; p < 7 && !fail; ++p) {
@@ -609,16 +632,9 @@ __global__ void __launch_bounds__(kChainThreads, 1)
             const uint64_t da = umma::desc_sw128(umma::smem_u32(H + (size_t)kb * kSlabBytes));
             const uint64_t db = umma::desc_sw128(umma::smem_u32(ring + (size_t)st * kRingBytes));
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) umma::mma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+            for (int k = 0; k < kBK / 16; ++k) 
+              umma::mma_bf16(tmem + chain_half(p), da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
             umma::mma_commit(&wempty[st]);
-            const int gp = g - 1;  // refill the slot of the slab before
-            if (gp >= 0 && gp + kChainRing < total) {
-              if (!umma::mbar_wait(&wempty[gp % kChainRing], (uint32_t)(gp / kChainRing) & 1u, kWaitCycles)) {
-                fail = true;
-                break;
-              }
-              load_w(g_load++);
-            }
           }
           if (!fail) umma::mma_commit(accf);
         }
@@ -637,99 +653,156 @@ __global__ void __launch_bounds__(kChainThreads, 1)
       for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
       inv = 1.0f / fmaxf(c, 1.0f);
     }
-    const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
     uint8_t* const hrow = H + (size_t)cg * kSlabBytes + (size_t)r * 128;  // this thread's 64 columns
+    // the next operand is written: its MMAs may start
+    auto handed = [&]() {
+      umma::fence_proxy_async_smem();
+      umma::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) umma::mbar_arrive(actr);
+    };
     bool stop = false;
     for (int i = 0; i < my_tiles && !stop; ++i) {
       const int tile = blockIdx.x + i * gridDim.x;
       const int row = tile * kBM + r;
       for (int p = 0; p < 7; ++p) {
+        const int e = 7 * i + p;
+        const uint32_t trow = tmem + chain_half(p) + ((uint32_t)(q * 32) << 16);
+        const bool fwd = p < 3;
+        const int l = fwd ? p : 6 - p;  // layer whose Z this is (p != 3)
+        float* const zt = a.Z[p < 2 || p > 4 ? l : 0] + ((size_t)tile * kHid + cg * 64) * kBM + r;
+        bf16* const ot = (fwd ? a.At[l] : a.dZt[p == 3 ? 0 : l]) + (size_t)(cg * 64) * a.B + row;
+        // what the epilogue reads from memory is requested ahead of the MMAs' end
+        float z[32];  // Z's first 32 columns; p == 3: 16 targets and, as bits, the mask
+        if (p > 4) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) z[k] = zt[(size_t)k * kBM];
+        } else if (p == 3 && cg < 2) {
+          const float4* tt = reinterpret_cast<const float4*>(a.Tb + (size_t)row * kOut + cg * 16);
+          const float4* xm = reinterpret_cast<const float4*>(a.Xb + (size_t)row * kInPad + 2 * kOut + cg * 16);
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const float4 t4 = k < 4 ? tt[k] : xm[k - 4];
+            z[4 * k] = t4.x, z[4 * k + 1] = t4.y, z[4 * k + 2] = t4.z, z[4 * k + 3] = t4.w;
+          }
+        }
         if (*abort_flag) {
           stop = true;
           break;
         }
-        if (!umma::mbar_wait(accf, (uint32_t)(7 * i + p) & 1u, 2 * kWaitCycles)) {
+        if (!umma::mbar_wait(accf, (uint32_t)e & 1u, 2 * kWaitCycles)) {
           *abort_flag = 1;
           stop = true;
           break;
         }
         umma::fence_after_sync();
         if (p == 3) {
-          __align__(16) bf16 gv[16];
+          uint32_t gv[8];
+          float loss = 0.0f;
+          const int c0 = cg * 16;
           if (cg < 2) {
-            const int c0 = cg * 16;
             float v[16];
             umma::tmem_ld16(trow + (uint32_t)c0, v);
-            __align__(16) bf16 mk[16];
-            const uint4* xm = reinterpret_cast<const uint4*>(a.Xb + (size_t)row * kInPad + 2 * kOut + c0);
-            reinterpret_cast<uint4*>(mk)[0] = xm[0];
-            reinterpret_cast<uint4*>(mk)[1] = xm[1];
-            const float4* tt = reinterpret_cast<const float4*>(a.Tb + (size_t)row * kOut + c0);
-            float l = 0.0f;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float4 t4 = tt[k];
-              const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int n = 4 * k + u;
-                const float y = v[n] + __ldg(a.theta + kOffB4 + c0 + n);
-                const float d = __bfloat162float(mk[n]) * (y - tv[u]);
-                l += d * d;
-                gv[n] = __float2bfloat16_rn(2.0f * d * inv);
-                a.dYt[(size_t)(c0 + n) * a.B + row] = gv[n];
-              }
+            for (int n = 0; n < 16; n += 2) {
+              const uint32_t mk = __float_as_uint(z[16 + n / 2]);  // two mask entries
+              const float y0 = v[n] + s_bias[3 * kHid + c0 + n];
+              const float y1 = v[n + 1] + s_bias[3 * kHid + c0 + n + 1];
+              const float d0 = __uint_as_float(mk << 16) * (y0 - z[n]);
+              const float d1 = __uint_as_float(mk & 0xFFFF0000u) * (y1 - z[n + 1]);
+              loss += d0 * d0;
+              loss += d1 * d1;
+              const __nv_bfloat162 g = __floats2bfloat162_rn(2.0f * d0 * inv, 2.0f * d1 * inv);
+              gv[n / 2] = *reinterpret_cast<const uint32_t*>(&g);
             }
-            for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-            if (lane == 0) a.lossp[(size_t)tile * 8 + warp] = l;
           } else {
 #pragma unroll
-            for (int n = 0; n < 16; ++n) gv[n] = __float2bfloat16_rn(0.0f);
+            for (int n = 0; n < 8; ++n) gv[n] = 0u;
           }
           // dY: columns 16 cg .. 16 cg + 15 of the first slab (zeros from 32 on)
           uint8_t* const drow = H + (size_t)r * 128;
 #pragma unroll
           for (int u = 0; u < 2; ++u)
-            *reinterpret_cast<uint4*>(drow + (((2 * cg + u) ^ (r & 7)) << 4)) = reinterpret_cast<uint4*>(gv)[u];
+            *reinterpret_cast<uint4*>(drow + (((2 * cg + u) ^ (r & 7)) << 4)) =
+                make_uint4(gv[4 * u], gv[4 * u + 1], gv[4 * u + 2], gv[4 * u + 3]);
+          handed();
+          if (cg < 2) {
+            uint16_t* const dy = reinterpret_cast<uint16_t*>(a.dYt) + (size_t)c0 * a.B + row;
+#pragma unroll
+            for (int n = 0; n < 16; ++n) dy[(size_t)n * a.B] = (uint16_t)(gv[n / 2] >> (16 * (n & 1)));
+            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+            if (lane == 0) a.lossp[(size_t)tile * 8 + warp] = loss;
+          }
         } else {
-          const bool fwd = p < 3;
-          const int l = fwd ? p : 6 - p;  // layer whose Z this is
-          float* const zt = a.Z[l] + ((size_t)tile * kHid + cg * 64) * kBM + r;
-          bf16* const ot = (fwd ? a.At[l] : a.dZt[l]) + (size_t)(cg * 64) * a.B + row;
-          const float* const b = a.theta + (l == 0 ? kOffB1 : l == 1 ? kOffB2 : kOffB3) + cg * 64;
-#pragma unroll 1
-          for (int c0 = 0; c0 < 64; c0 += 32) {
-            float v[32];
-            float z[32];
-            if (!fwd) {
+          const ulonglong2* const b = reinterpret_cast<const ulonglong2*>(s_bias + l * kHid + cg * 64);
+          uint32_t hv[32];  // the operand's 64 columns
 #pragma unroll
-              for (int k = 0; k < 32; ++k) z[k] = zt[(size_t)(c0 + k) * kBM];
-            }
-            umma::tmem_ld32(trow + (uint32_t)(cg * 64 + c0), v);
-            __align__(16) bf16 hv[32];
+          for (int half = 0; half < 2; ++half) {
+            uint32_t v[32];
+            umma::tmem_request32(trow + (uint32_t)(cg * 64 + 32 * half), v);
+            if (p == 4) {  // Z3 is still where product 2 left it, without the bias
+              uint32_t zv[32];
+              umma::tmem_request32(tmem + chain_half(2) + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * 64 + 32 * half),
+                                   zv);
+              umma::tmem_wait32(zv);
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-              if (fwd) {
-                const float zz = v[k] + __ldg(b + c0 + k);
-                zt[(size_t)(c0 + k) * kBM] = zz;
-                hv[k] = __float2bfloat16_rn(gelu(zz));
-              } else {
-                hv[k] = __float2bfloat16_rn(v[k] * gelu_grad(z[k]));
+              for (int k = 0; k < 16; ++k) {
+                const ulonglong2 b4 = b[8 * half + (k >> 1)];
+                unpack2(add2(pack2(__uint_as_float(zv[2 * k]), __uint_as_float(zv[2 * k + 1])), k & 1 ? b4.y : b4.x),
+                        z[2 * k], z[2 * k + 1]);
               }
-              ot[(size_t)(c0 + k) * a.B] = hv[k];
+            } else if (!fwd && half == 1) {
+#pragma unroll
+              for (int k = 0; k < 32; ++k) z[k] = zt[(size_t)(32 + k) * kBM];
+            }
+            umma::tmem_wait32(v);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              if (fwd) {
+                const ulonglong2 b4 = b[8 * half + (k >> 1)];
+                hv[16 * half + k] = gelu_bf16x2(
+                    add2(pack2(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1])), k & 1 ? b4.y : b4.x));
+              } else {
+                float g0, g1;
+                unpack2(mul2(pack2(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1])),
+                             gelu_grad2(pack2(z[2 * k], z[2 * k + 1]))),
+                        g0, g1);
+                const __nv_bfloat162 g = __floats2bfloat162_rn(g0, g1);
+                hv[16 * half + k] = *reinterpret_cast<const uint32_t*>(&g);
+              }
             }
             if (p < 6) {
 #pragma unroll
               for (int u = 0; u < 4; ++u)
-                *reinterpret_cast<uint4*>(hrow + ((((c0 >> 3) + u) ^ (r & 7)) << 4)) =
-                    reinterpret_cast<uint4*>(hv)[u];
+                *reinterpret_cast<uint4*>(hrow + (((4 * half + u) ^ (r & 7)) << 4)) =
+                    make_uint4(hv[16 * half + 4 * u], hv[16 * half + 4 * u + 1], hv[16 * half + 4 * u + 2],
+                               hv[16 * half + 4 * u + 3]);
+            }
+          }
+          handed();
+          // the stores run under the next product (which accumulates in the
+          // other half of the TMEM)
+          uint16_t* const o16 = reinterpret_cast<uint16_t*>(ot);
+#pragma unroll
+          for (int k = 0; k < 64; ++k) o16[(size_t)k * a.B] = (uint16_t)(hv[k >> 1] >> (16 * (k & 1)));
+          if (p < 2) {
+#pragma unroll 1
+            for (int c0 = 0; c0 < 64; c0 += 32) {
+              uint32_t v[32];
+              umma::tmem_request32(trow + (uint32_t)(cg * 64 + c0), v);
+              umma::tmem_wait32(v);
+#pragma unroll
+              for (int k = 0; k < 16; ++k) {
+                const ulonglong2 b4 = b[c0 / 4 + (k >> 1)];
+                float z0, z1;
+                unpack2(add2(pack2(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1])), k & 1 ? b4.y : b4.x), z0,
+                        z1);
+                zt[(size_t)(c0 + 2 * k) * kBM] = z0;
+                zt[(size_t)(c0 + 2 * k + 1) * kBM] = z1;
+              }
             }
           }
         }
-        umma::fence_proxy_async_smem();
-        umma::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) umma::mbar_arrive(actr);
       }
     }
   }
@@ -738,7 +811,7 @@ __global__ void __launch_bounds__(kChainThreads, 1)
   if (threadIdx.x == 0 && *abort_flag && a.error) atomicExch(a.error, 1);
   if (warp == 0) {
     umma::fence_after_sync();
-    umma::tmem_dealloc(tmem, 256);
+    umma::tmem_dealloc(tmem, 512);
   }
 }
 
@@ -784,7 +857,7 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   umma::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if (threadIdx.x == 0) {
+  if (warp == 0 && umma::elect_one()) {
     bool ok = true;
     const int k0 = blockIdx.x * k_slabs;
     const uint32_t idesc = umma::idesc_bf16(kBM, N);
@@ -1051,7 +1124,7 @@ struct vrm_mlp {
   bf16 *W1 = nullptr, *W2 = nullptr, *W3 = nullptr, *W4 = nullptr, *W2t = nullptr, *W3t = nullptr, *W4t = nullptr;
   bf16 *Xb = nullptr, *Xbt = nullptr;
   float *Tb = nullptr, *cnt = nullptr, *lossp = nullptr;
-  float* Z[3] = {};
+  float* Z[2] = {};
   bf16 *At[3] = {}, *dZt[3] = {}, *dYt = nullptr;
   CUtensorMap mW1, mW2, mW3, mW4;  // weights as B operands
   CUtensorMap half[4];             // the same, half of the rows at a time (CTA pairs)
@@ -1116,7 +1189,7 @@ namespace {
 
 void free_mlp(vrm_mlp* n) {
   void* ptrs[] = {n->err, n->theta, n->m, n->v, n->grad, n->part, n->loss, n->W1, n->W2, n->W3, n->W4, n->W2t,
-                  n->W3t, n->W4t, n->Xb, n->Xbt, n->Tb, n->cnt, n->lossp, n->Z[0], n->Z[1], n->Z[2], n->At[0],
+                  n->W3t, n->W4t, n->Xb, n->Xbt, n->Tb, n->cnt, n->lossp, n->Z[0], n->Z[1], n->At[0],
                   n->At[1], n->At[2], n->dZt[0], n->dZt[1], n->dZt[2], n->dYt};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1146,7 +1219,7 @@ cudaError_t forward_backward(vrm_mlp* n, cudaStream_t s) {
   a.Tb = n->Tb;
   a.cnt = n->cnt;
   for (int l = 0; l < 3; ++l) {
-    a.Z[l] = n->Z[l];
+    if (l < 2) a.Z[l] = n->Z[l];
     a.At[l] = n->At[l];
     a.dZt[l] = n->dZt[l];
   }
@@ -1269,7 +1342,7 @@ vrm_status vrm_mlp_create(int32_t batch_rows, vrm_mlp** out) {
   MLP_ALLOC(cnt, B / kGatherRows);
   MLP_ALLOC(lossp, (size_t)B / kBM * 8);
   for (int l = 0; l < 3; ++l) {
-    MLP_ALLOC(Z[l], (size_t)B * kHid);
+    if (l < 2) MLP_ALLOC(Z[l], (size_t)B * kHid);
     MLP_ALLOC(At[l], (size_t)kHid * B);
     MLP_ALLOC(dZt[l], (size_t)kHid * B);
   }
