@@ -113,6 +113,9 @@ struct vrm_ctx {
   int rk_cap = 0;
   double *rk_x1 = nullptr, *rk_y1 = nullptr, *rk_x2 = nullptr, *rk_y2 = nullptr;
   double *rk_g1 = nullptr, *rk_g2 = nullptr, *rk_dg = nullptr, *rk_u = nullptr, *rk_v = nullptr;
+  // the stream of the stages' analytic velocities, its fork and its join
+  cudaStream_t vel_stream = nullptr;
+  cudaEvent_t vel_fork = nullptr, vel_join = nullptr;
   // direct-sum velocity: fp32-split sources and targets
   int bs_src_cap = 0, bs_tgt_cap = 0;
   float4 *bs_src = nullptr, *bs_tgt = nullptr;
@@ -356,6 +359,26 @@ cudaError_t ensure_rk(vrm_ctx* ctx, int cap, cudaStream_t st) {
   ctx->rk_cap = cap;
   return cudaSuccess;
 }
+
+cudaError_t ensure_vel_stream(vrm_ctx* ctx) {
+  cudaError_t e = cudaSuccess;
+  if (!ctx->vel_fork) e = cudaEventCreateWithFlags(&ctx->vel_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess && !ctx->vel_join) e = cudaEventCreateWithFlags(&ctx->vel_join, cudaEventDisableTiming);
+  if (e != cudaSuccess || ctx->vel_stream) return e;
+  int least = 0, greatest = 0;
+  if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess) return e;
+  return cudaStreamCreateWithPriority(&ctx->vel_stream, cudaStreamNonBlocking, least);
+}
+
+// Waits for a velocity still under way where vrm_rk3_step returns early: it
+// reads the caller's positions.
+struct VelGuard {
+  cudaStream_t s;
+  bool pending = false;
+  ~VelGuard() {
+    if (pending) cudaStreamSynchronize(s);
+  }
+};
 
 // Neighbourhoods and weights of every diffused particle (list s.dlist) at
 // positions (x, y) of the n_cur particles: cell grid, search, learned
@@ -949,6 +972,9 @@ void vrm_destroy(vrm_ctx* ctx) {
     for (int k = 0; k <= VRM_STAGE_COUNT; ++k) cudaEventDestroy(ctx->ev[k]);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   if (ctx->body_stream) cudaStreamDestroy(ctx->body_stream);
+  if (ctx->vel_stream) cudaStreamDestroy(ctx->vel_stream);
+  if (ctx->vel_fork) cudaEventDestroy(ctx->vel_fork);
+  if (ctx->vel_join) cudaEventDestroy(ctx->vel_join);
   delete ctx;
 }
 
@@ -1190,12 +1216,26 @@ vrm_status vrm_rk3_step(vrm_ctx* ctx, double* x, double* y, int32_t n, int32_t c
   vrm_status r = run_step_eager(ctx, x, y, capacity, gamma_in, nullptr, s.diffused, false, stream);
   ctx->timing = timing;
   if (r != VRM_OK) return r;
+  // an analytic velocity runs beside its stage's cell grid and search on a
+  // stream of its own, the first one from here on (beside the read-back too)
+  const int* n_cur = &s.st->n_cur;  // particles of every stage
+  const bool aside = V.kind == VRM_VEL_LAMB_OSEEN;
+  if (aside) VRM_CUDA(ensure_vel_stream(ctx));
+  VelGuard vel_guard{ctx->vel_stream};
+  auto start_velocity = [&](const double* px, const double* py, double t_s) {
+    cudaError_t e = cudaEventRecord(ctx->vel_fork, stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->vel_stream, ctx->vel_fork, 0);
+    if (e != cudaSuccess) return e;
+    vel_guard.pending = true;
+    e = rk3_velocity(capacity, n_cur, t_s, V, px, py, ctx->rk_u, ctx->rk_v, ctx->vel_stream);
+    return e == cudaSuccess ? cudaEventRecord(ctx->vel_join, ctx->vel_stream) : e;
+  };
+  if (aside) VRM_CUDA(start_velocity(x, y, t));
   VRM_CUDA(read_back(ctx, stream));
   if (s.h_grid->nonfinite || s.h_ds->nonfinite) return VRM_ERR_ARG;
   fill_front_stats(ctx, n, st);
   if (s.h_state->overflow) return VRM_ERR_CAPACITY;
-  const int n1 = s.h_state->n_cur;  // particles of every stage
-  const int* n_cur = &s.st->n_cur;
+  const int n1 = s.h_state->n_cur;
   double* Xs[3] = {x, ctx->rk_x1, ctx->rk_x2};
   double* Ys[3] = {y, ctx->rk_y1, ctx->rk_y2};
   const double* Gs[3] = {gamma_in, ctx->rk_g1, ctx->rk_g2};
@@ -1208,6 +1248,8 @@ vrm_status vrm_rk3_step(vrm_ctx* ctx, double* x, double* y, int32_t n, int32_t c
     // without a velocity every stage sits at the initial positions
     const double* px = move ? Xs[k] : x;
     const double* py = move ? Ys[k] : y;
+    // the stage before has read rk_u, rk_v and written the positions
+    if (aside && k > 0) VRM_CUDA(start_velocity(px, py, ts[k]));
     VRM_CUDA(enqueue_stage_weights(ctx, px, py, capacity, stream));
     VRM_CUDA(apply_transposed_dev(ctx->c, capacity, n_cur, k == 0 ? n : capacity, k == 0 ? nullptr : n_cur, Gs[k],
                                   s.diffused, s.dlist, s.counters + 0, s.cols, s.f, s.fii, s.tcount, s.toff,
@@ -1229,7 +1271,13 @@ vrm_status vrm_rk3_step(vrm_ctx* ctx, double* x, double* y, int32_t n, int32_t c
       us = ctx->rk_u;
       vs = ctx->rk_v;
     }
-    VRM_CUDA(rk3_stage(k, capacity, n_cur, dt, ts[k], V, x, y, gamma_in, n, px, py, Gs[k], ctx->rk_dg, us, vs, Xo[k],
+    if (aside) {
+      VRM_CUDA(cudaStreamWaitEvent(stream, ctx->vel_join, 0));
+      vel_guard.pending = false;  // this stream's own synchronisation now covers it
+      us = ctx->rk_u;
+      vs = ctx->rk_v;
+    }
+    VRM_CUDA(rk3_stage(k, capacity, n_cur, dt, x, y, gamma_in, n, px, py, Gs[k], ctx->rk_dg, us, vs, Xo[k],
                        Yo[k], Go[k], stream));
   }
   VRM_CUDA(read_back(ctx, stream));

@@ -597,11 +597,15 @@ cudaError_t remove_out(int n, const int* n_keep, const int* klist, const double*
 // vrm_rk3.cu
 // One stage update of the SSP-RK3 step (positions by the velocity, circulations
 // by the stage's dGamma), for n particles (*n_dev if given).
-// us, vs: precomputed stage velocities (or null: the analytic field of vel).
-cudaError_t rk3_stage(int stage, int n_bound, const int* n_dev, double dt, double t_s, const Velocity& vel,
-                      const double* X0, const double* Y0, const double* G0, int n_g0, const double* Xs,
-                      const double* Ys, const double* Gs, const double* dg, const double* us, const double* vs,
-                      double* Xo, double* Yo, double* Go, cudaStream_t s);
+// us, vs: the stage's velocities (null: the particles stay).
+cudaError_t rk3_stage(int stage, int n_bound, const int* n_dev, double dt, const double* X0, const double* Y0,
+                      const double* G0, int n_g0, const double* Xs, const double* Ys, const double* Gs,
+                      const double* dg, const double* us, const double* vs, double* Xo, double* Yo, double* Go,
+                      cudaStream_t s);
+
+// The Lamb-Oseen velocity of the particles (*n_dev if given) into us, vs.
+cudaError_t rk3_velocity(int n_bound, const int* n_dev, double t_s, const Velocity& vel, const double* X,
+                         const double* Y, double* us, double* vs, cudaStream_t s);
 
 // vrm_bs.cu: smoothed Biot-Savart velocity by direct summation.
 // Splits FP64 positions into fp32 hi/lo pairs (and circulations to fp32).

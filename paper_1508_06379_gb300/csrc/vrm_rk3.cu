@@ -60,9 +60,31 @@ __device__ __forceinline__ void lamb_oseen_uv(const Velocity& v, double x, doubl
   *w = __dmul_rn(dx, k);
 }
 
-__global__ void k_rk3_stage(int stage, int n_bound, const int* __restrict__ n_dev, double dt, double t_s, Velocity vel,
-                            const double* X0, const double* Y0, const double* __restrict__ G0, int n_g0,
-                            const double* Xs, const double* Ys, const double* Gs, const double* __restrict__ dg,
+// The Lamb-Oseen velocity of every particle.  Bound by the FP64 pipe (about 100
+// operations a particle: 80 us for 406,000).  vrm_rk3_step runs it on a stream
+// of its own beside the stage's cell grid and search, which leave that pipe
+// idle: one block per SM keeps it busy and leaves the search its warps.  An RK3
+// step of 403,000 particles 2.35 -> 2.25 ms against the velocity taken in the
+// stage update (2 blocks per SM 2.32, 8 2.37, 128 threads 2.28, 64 2.44), of
+// 69,000 1,045 -> 1,014 us, of 2,500 608 -> 596.
+constexpr int kVelThreads = 256;
+__global__ void __launch_bounds__(kVelThreads) k_lamb_oseen(int n_bound, const int* __restrict__ n_dev, double t_s,
+                                                            Velocity vel, const double* __restrict__ X,
+                                                            const double* __restrict__ Y, double* __restrict__ us,
+                                                            double* __restrict__ vs) {
+  const int n = n_dev ? min(*n_dev, n_bound) : n_bound;
+  for (long j = (long)blockIdx.x * kVelThreads + threadIdx.x; j < n; j += (long)gridDim.x * kVelThreads) {
+    double u, w;
+    lamb_oseen_uv(vel, X[j], Y[j], t_s, &u, &w);
+    us[j] = u;
+    vs[j] = w;
+  }
+}
+
+// us, vs: the stage's velocity, or null where the particles stay.
+__global__ void k_rk3_stage(int stage, int n_bound, const int* __restrict__ n_dev, double dt, const double* X0,
+                            const double* Y0, const double* __restrict__ G0, int n_g0, const double* Xs,
+                            const double* Ys, const double* Gs, const double* __restrict__ dg,
                             const double* __restrict__ us, const double* __restrict__ vs, double* Xo, double* Yo,
                             double* Go) {
   const int n = n_dev ? *n_dev : n_bound;
@@ -72,17 +94,10 @@ __global__ void k_rk3_stage(int stage, int n_bound, const int* __restrict__ n_de
     const double gs = stage == 0 ? g0 : Gs[j];
     const double ge = __dadd_rn(gs, __dmul_rn(dt, dg[j]));
     double xe = 0.0, ye = 0.0;
-    const bool move = vel.kind != VRM_VEL_NONE;
+    const bool move = us != nullptr;
     if (move) {
-      double u, w;
-      if (us) {
-        u = us[j];
-        w = vs[j];
-      } else {
-        lamb_oseen_uv(vel, Xs[j], Ys[j], t_s, &u, &w);
-      }
-      xe = __dadd_rn(Xs[j], __dmul_rn(dt, u));
-      ye = __dadd_rn(Ys[j], __dmul_rn(dt, w));
+      xe = __dadd_rn(Xs[j], __dmul_rn(dt, us[j]));
+      ye = __dadd_rn(Ys[j], __dmul_rn(dt, vs[j]));
     }
     if (stage == 0) {
       Go[j] = ge;
@@ -102,15 +117,25 @@ __global__ void k_rk3_stage(int stage, int n_bound, const int* __restrict__ n_de
   }
 }
 
-cudaError_t rk3_stage(int stage, int n_bound, const int* n_dev, double dt, double t_s, const Velocity& vel,
-                      const double* X0, const double* Y0, const double* G0, int n_g0, const double* Xs,
-                      const double* Ys, const double* Gs, const double* dg, const double* us, const double* vs,
-                      double* Xo, double* Yo, double* Go, cudaStream_t s) {
+cudaError_t rk3_velocity(int n_bound, const int* n_dev, double t_s, const Velocity& vel, const double* X,
+                         const double* Y, double* us, double* vs, cudaStream_t s) {
+  if (n_bound <= 0) return cudaSuccess;
+  int blocks = (n_bound + kVelThreads - 1) / kVelThreads;
+  if (blocks > sm_count()) blocks = sm_count();
+  k_lamb_oseen<<<blocks, kVelThreads, 0, s>>>(n_bound, n_dev, t_s, vel, X, Y, us, vs);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t rk3_stage(int stage, int n_bound, const int* n_dev, double dt, const double* X0, const double* Y0,
+                      const double* G0, int n_g0, const double* Xs, const double* Ys, const double* Gs,
+                      const double* dg, const double* us, const double* vs, double* Xo, double* Yo, double* Go,
+                      cudaStream_t s) {
   if (n_bound <= 0) return cudaSuccess;
   int blocks = (n_bound + kBlock - 1) / kBlock;
   if (blocks > 8 * sm_count()) blocks = 8 * sm_count();
-  k_rk3_stage<<<blocks, kBlock, 0, s>>>(stage, n_bound, n_dev, dt, t_s, vel, X0, Y0, G0, n_g0, Xs, Ys, Gs, dg, us, vs,
-                                        Xo, Yo, Go);
+  k_rk3_stage<<<blocks, kBlock, 0, s>>>(stage, n_bound, n_dev, dt, X0, Y0, G0, n_g0, Xs, Ys, Gs, dg, us, vs, Xo, Yo,
+                                        Go);
   note_launch();
   return cudaGetLastError();
 }
