@@ -1675,6 +1675,23 @@ __device__ __forceinline__ Df df_split(double a, bool& bad) {
   const float scale = __uint_as_float(sign | ((unsigned)(e - 52 + 127) << 23));
   return df_fast_two_sum(h, __fmul_rn(__uint2float_rn((unsigned)(b & 0x1FFFFFFF)), scale));
 }
+// Two rows' t - a p at once with the packed instructions, each with the
+// roundings of df_fnma (a difference x - y as x + (-1) y): ah, al the rows'
+// values of the entering column, (ph, pl) the pivot row's entry and nph, npl
+// its negative, twice each.
+__device__ __forceinline__ void df_fnma2(f32x2 ah, f32x2 al, f32x2 ph, f32x2 nph, f32x2 npl, f32x2 m1, f32x2& th,
+                                         f32x2& tl) {
+  const f32x2 q = mul2(ah, ph);
+  f32x2 ne = fma2(ah, nph, q);
+  ne = fma2(ah, npl, ne);
+  ne = fma2(al, nph, ne);
+  const f32x2 s = fma2(q, m1, th), bb = fma2(th, m1, s);
+  const f32x2 v = fma2(fma2(bb, m1, s), m1, th);  // th - (s - bb)
+  const f32x2 e = fma2(add2(q, bb), m1, v);       // ... + (-q - bb)
+  const f32x2 x = add2(e, add2(tl, ne));
+  th = add2(s, x);
+  tl = fma2(fma2(s, m1, th), m1, x);
+}
 constexpr float kU2 = kU32 * kU32;
 constexpr float kDfFma = 24.0f * kU2, kDfMul = 24.0f * kU2;
 
@@ -1687,6 +1704,21 @@ constexpr float kDfFma = 24.0f * kU2, kDfMul = 24.0f * kU2;
 // lanes hold columns, 9 hold rows); n = 1: G = 8, four small LPs per warp, for
 // the LPs of small clouds, where the latency of one LP counts (lp_small).  The
 // LPs of a warp run in step until all are done.
+// An update's rows go two by two through the packed instructions (full LPs of
+// 229,000 particles 1,780 -> 1,570 us, small ones 800 -> 725).
+//
+// A small LP of n = 2 has nine equations for eight columns: nearly all end
+// with artificials in the basis, and their FP64 solves (404 us for 229,000)
+// would only find the residual too large.  Their other eight lanes therefore
+// carry the columns of the artificials of rows 0, 1, 3, ..., 8, whose reduced
+// costs are 1 - y_r for the dual y of the final basis.  With d_j = -y V_j and
+// the phase-I sum w = y b > 0, every f >= 0 has y (b - V f) = w + sum_j f_j d_j,
+// so max_r |b - V f|_r >= (w - sum_j f_j max(0, -d_j)) / |y|_1, where f_j <=
+// 4.1 / (xi_j^2 + eta_j^2) wherever rows 2 and 4 hold to 0.05, and |y_2| <= w / 2
+// + |y_4|.  Where that is above 2e-11 (all quantities with their bounds, twice
+// the slack taken), no weights the final solve could give pass its residual
+// test at 1e-12, whose own rounding is below 1e-11 for offsets of 0.01 to 100
+// spacings: the LP is recorded as infeasible (code 2) and not solved.
 template <int M, int G, bool FULL>
 __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restrict__ x, const double* __restrict__ y,
                                                const int* __restrict__ list, const int* __restrict__ list_count,
@@ -1699,7 +1731,13 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
   const int lane = threadIdx.x & 31, gl = lane & (G - 1), gbase = lane & ~(G - 1);
   const unsigned gmask = (kAll >> (32 - G)) << gbase;
   auto ballot = [&](bool v) { return (__ballot_sync(kAll, v) & gmask) >> gbase; };
-  __shared__ float4 s_col[2][128 / G][M + 1];
+  // rows in pairs, the cost row after the last one
+  constexpr int R = M + 1, P2 = R / 2;
+  constexpr bool kDual = M == 9 && !FULL;
+  static_assert(!kDual || G == 16, "eight lanes for the dual's columns");
+  static_assert(R % 2 == 0, "the rows and the cost row in pairs");
+  __shared__ float4 s_col[2][128 / G][2 * P2];
+  const f32x2 m1 = pack2(-1.0f, -1.0f), fma_u = pack2(kDfFma, kDfFma);
   unsigned it_all = 0;
   const int m = *list_count;
   const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1730,10 +1768,10 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       rank += (lt_nonneg(od2, d2) || (dbits(od2) == dbits(d2) && oj < j)) ? 1 : 0;
     }
     bool bad = false;
-    Df T[M], d = {0.0f, 0.0f};
-    float E[M], Ed = 0.0f;
+    float Th[R], Tl[R], E[R];
     {
       const Df xi = df_split(__dmul_rn(dx, c.inv_h), bad), eta = df_split(__dmul_rn(dy, c.inv_h), bad);
+      Df T[M];
       T[0] = xi;
       T[1] = eta;
       T[2] = df_mul(xi, xi);
@@ -1750,14 +1788,25 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
 #pragma unroll
       for (int r = 0; r < M; ++r) {
         const float av = fabsf(T[r].h);
+        Th[r] = T[r].h;
+        Tl[r] = T[r].l;
         E[r] = (r < 2 ? 3.0f : r < 5 ? 12.0f : 24.0f) * kU2 * av;
         sum = df_add(sum, T[r]);
         sa += av;
         se += E[r];
       }
-      d.h = -sum.h;
-      d.l = -sum.l;
-      Ed = __fmaf_rn(32.0f * kU2, sa, se);
+      Th[M] = -sum.h;
+      Tl[M] = -sum.l;
+      E[M] = __fmaf_rn(32.0f * kU2, sa, se);
+    }
+    float norm2 = 0.0f;  // xi^2 + eta^2 of the column
+    const bool art = kDual && gl >= 8;
+    if (kDual) {
+      norm2 = Th[2] + Th[4];
+      const int row = gl < 10 ? gl - 8 : gl - 7;
+#pragma unroll
+      for (int r = 0; r < M; ++r)
+        if (art) Th[r] = r == row ? 1.0f : 0.0f;
     }
     // row r on lane r
     Df rhs = {gl == 2 || gl == 4 ? 2.0f : 0.0f, 0.0f};
@@ -1771,9 +1820,9 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       // entering column: the first in rank certainly below -tol, no earlier
       // one uncertain
       bool go = run && n_art > 0;
-      const float md = __fmaf_rn(kCertSafety, Ed, 2.0f * kU32 * fabsf(d.h));
-      const bool yes = col && !isb && d.h < -kTolPriceHi - md;
-      const bool maybe = col && !isb && !yes && !(d.h > -kTolPriceLo + md);
+      const float md = __fmaf_rn(kCertSafety, E[M], 2.0f * kU32 * fabsf(Th[M]));
+      const bool yes = col && !isb && Th[M] < -kTolPriceHi - md;
+      const bool maybe = col && !isb && !yes && !(Th[M] > -kTolPriceLo + md);
       const int rq = (int)__reduce_min_sync(gmask, (unsigned)(yes ? rank : kNone));
       if (ballot(maybe && rank < rq) != 0 && go) {
         unc = true;
@@ -1786,20 +1835,25 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       }
       const unsigned qb = ballot(yes && rank == rq);
       const int q = qb ? __ffs(qb) - 1 : 0;
-      // the entering column, its cost and its particle through shared memory:
-      // its lane writes ten vectors, every lane reads them and lane r row r's
-      // (two buffers, so that one barrier a pivot suffices)
+      // the entering column with its cost, and its particle through shared
+      // memory: its lane writes a pair of rows as (h, h, l, l) and (E, E, |h| +
+      // E, |h| + E), every lane reads them and lane r row r's (two buffers, so
+      // that one barrier a pivot suffices)
       float4* const buf = s_col[it_all & 1][threadIdx.x / G];
       ++it_all;
       if (gl == q) {
 #pragma unroll
-        for (int r = 0; r < M; ++r) buf[r] = make_float4(T[r].h, T[r].l, E[r], 0.0f);
-        buf[M] = make_float4(d.h, d.l, Ed, __int_as_float(j));
+        for (int p = 0; p < P2; ++p) {
+          buf[2 * p] = make_float4(Th[2 * p], Th[2 * p + 1], Tl[2 * p], Tl[2 * p + 1]);
+          buf[2 * p + 1] = make_float4(E[2 * p], E[2 * p + 1], __fadd_rn(fabsf(Th[2 * p]), E[2 * p]),
+                                       __fadd_rn(fabsf(Th[2 * p + 1]), E[2 * p + 1]));
+        }
       }
+      const int jq = __shfl_sync(kAll, j, q, G);
       __syncwarp();
-      const float4 mine = buf[gl < M ? gl : 0], cq = buf[M];
-      const Df am = {mine.x, mine.y};
-      const float eam = mine.z;
+      const float* const mine = reinterpret_cast<const float*>(buf + (gl < M ? gl & ~1 : 0)) + (gl < M ? gl & 1 : 0);
+      const Df am = {mine[0], mine[2]};
+      const float eam = mine[4];
       // ratio test, row r on lane r (as in lp_pivots32)
       const bool isrow = gl < M;
       const float mg = __fmaf_rn(kCertSafety, eam, 2.0f * kU32 * fabsf(am.h));
@@ -1857,9 +1911,6 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       prhs0.h = __shfl_sync(kAll, rhs.h, leave, G);
       prhs0.l = __shfl_sync(kAll, rhs.l, leave, G);
       const float pebr = __shfl_sync(kAll, Eb, leave, G);
-      const Df dq = {cq.x, cq.y};
-      const float edq = cq.z;
-      const int jq = __float_as_int(cq.w);
       const Df P = df_rcp(piv);
       const float rho = pe * P.h;
       no = no || !(rho <= 0.5f);
@@ -1869,12 +1920,12 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
       }
       if (go) {
         const float rr = __fmaf_rn(2.0f * rho, rho, rho);
-        Df prow = T[0];
+        Df prow = {Th[0], Tl[0]};
         float eprow = E[0];
 #pragma unroll
         for (int r = 1; r < M; ++r) {
-          prow.h = leave == r ? T[r].h : prow.h;
-          prow.l = leave == r ? T[r].l : prow.l;
+          prow.h = leave == r ? Th[r] : prow.h;
+          prow.l = leave == r ? Tl[r] : prow.l;
           eprow = leave == r ? E[r] : eprow;
         }
         prow = df_mul(prow, P);
@@ -1890,17 +1941,28 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
         const float ebP = pebr * P.h, aprhs = fabsf(prhs.h);
         const float Ebp = __fmaf_rn(kDfMul, aprhs, __fmaf_rn(rr, aprhs + ebP, ebP));
         // column q of the other rows becomes an exact 0 (its bound stays)
+        {
+          const f32x2 ph = pack2(prow.h, prow.h), nph = pack2(-prow.h, -prow.h), npl = pack2(-prow.l, -prow.l);
+          const f32x2 ap2 = pack2(ap, ap), Ep2 = pack2(Ep, Ep);
 #pragma unroll
-        for (int r = 0; r < M; ++r) {
-          const float4 a = buf[r];
-          const float aa = fabsf(a.x);
-          E[r] = __fmaf_rn(kDfFma, __fmaf_rn(aa, ap, fabsf(T[r].h)), __fmaf_rn(aa + a.z, Ep, __fmaf_rn(a.z, ap, E[r])));
-          T[r] = df_fnma(Df{a.x, a.y}, prow, T[r]);
+          for (int p = 0; p < P2; ++p) {
+            const float4 a = buf[2 * p], b = buf[2 * p + 1];
+            f32x2 th = pack2(Th[2 * p], Th[2 * p + 1]), tl = pack2(Tl[2 * p], Tl[2 * p + 1]);
+            // kDfFma (|a| |p| + |T|) + (|a| + E_a) E_p + E_a |p| + E
+            const f32x2 mag = fma2(pack2(fabsf(a.x), fabsf(a.y)), ap2, pack2(fabsf(Th[2 * p]), fabsf(Th[2 * p + 1])));
+            f32x2 en = fma2(pack2(b.x, b.y), ap2, pack2(E[2 * p], E[2 * p + 1]));
+            en = fma2(fma_u, mag, fma2(pack2(b.z, b.w), Ep2, en));
+            df_fnma2(pack2(a.x, a.y), pack2(a.z, a.w), ph, nph, npl, m1, th, tl);
+            unpack2(en, E[2 * p], E[2 * p + 1]);
+            unpack2(th, Th[2 * p], Th[2 * p + 1]);
+            unpack2(tl, Tl[2 * p], Tl[2 * p + 1]);
+          }
         }
 #pragma unroll
         for (int r = 0; r < M; ++r)
           if (leave == r) {
-            T[r] = prow;
+            Th[r] = prow.h;
+            Tl[r] = prow.l;
             E[r] = Ep;
           }
         {
@@ -1910,11 +1972,6 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
           const Df rn = df_fnma(am, prhs, rhs);
           rhs = gl == leave ? prhs : rn;
           Eb = gl == leave ? Ebp : en;
-        }
-        {
-          const float aa = fabsf(dq.h);
-          Ed = __fmaf_rn(kDfFma, __fmaf_rn(aa, ap, fabsf(d.h)), __fmaf_rn(aa + edq, Ep, __fmaf_rn(edq, ap, Ed)));
-          d = df_fnma(dq, prow, d);
         }
         if (lbas >= M) {
           if (rank == lbas - M) isb = false;
@@ -1929,6 +1986,25 @@ __global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restric
         ++it;
       }
       run = go;
+    }
+    if (kDual) {
+      // infeasible for certain?  y: the exact dual of the final basis, wsum =
+      // y b, d_j = -y V_j; see above
+      const bool left = gl < M && bas < M;
+      const float mb = __fmaf_rn(kCertSafety, Eb, 2.0f * kU32 * fabsf(rhs.h));
+      const float md = __fmaf_rn(kCertSafety, E[M], 2.0f * kU32 * fabsf(Th[M]));
+      float lo = left ? rhs.h - mb : 0.0f, hi = left ? fabsf(rhs.h) + mb : 0.0f, yn = art ? fabsf(1.0f - Th[M]) + md : 0.0f;
+      float slack = 0.0f;
+      if (col)
+        slack = norm2 > 1e-4f && norm2 < 1e4f ? fmaxf(md - Th[M], 0.0f) * __fdividef(4.1f, norm2) : 3.0e38f;
+#pragma unroll
+      for (int o = G / 2; o > 0; o >>= 1) {
+        lo += __shfl_xor_sync(kAll, lo, o);
+        hi += __shfl_xor_sync(kAll, hi, o);
+        yn += __shfl_xor_sync(kAll, yn, o);
+        slack += __shfl_xor_sync(kAll, slack, o);
+      }
+      if (lo > __fmaf_rn(2.0f, slack, 1e-10f * (yn + hi))) code = 2;
     }
     if (have && unc && gl == 0) {
       retry_list[atomicAdd(&ds->n_retry_pairs, 1)] = i;
@@ -1968,21 +2044,21 @@ __global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __rest
       double* const frow = f + (size_t)i * W;
       int basis[M], code, it;
       lp_recorded<M>(crow, basis, code, it);
-      double bxi[M], beta[M], pj[M];
-      const double xi0 = x[i], yi0 = y[i];
-#pragma unroll
-      for (int r = 0; r < M; ++r) {
-        const int j = crow[r];
-        pj[r] = __longlong_as_double((long long)j);
-        const bool s = basis[r] >= M;
-        bxi[r] = s ? __dmul_rn(__dsub_rn(x[s ? j : i], xi0), c.inv_h) : 0.0;
-        beta[r] = s ? __dmul_rn(__dsub_rn(y[s ? j : i], yi0), c.inv_h) : 0.0;
-      }
       double wsum = 0.0, rmax = 0.0;
       double pay[4][M];
 #pragma unroll
       for (int r = 0; r < M; ++r) pay[2][r] = 0.0;
       if (code == 0) {
+        double bxi[M], beta[M], pj[M];
+        const double xi0 = x[i], yi0 = y[i];
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+          const int j = crow[r];
+          pj[r] = __longlong_as_double((long long)j);
+          const bool s = basis[r] >= M;
+          bxi[r] = s ? __dmul_rn(__dsub_rn(x[s ? j : i], xi0), c.inv_h) : 0.0;
+          beta[r] = s ? __dmul_rn(__dsub_rn(y[s ? j : i], yi0), c.inv_h) : 0.0;
+        }
         double xB[M];
         float cert = INFINITY;
         if (!basis_solve<M>(basis, bxi, beta, xB, &cert)) code = 2;
