@@ -1719,8 +1719,13 @@ constexpr float kDfFma = 24.0f * kU2, kDfMul = 24.0f * kU2;
 // the slack taken), no weights the final solve could give pass its residual
 // test at 1e-12, whose own rounding is below 1e-11 for offsets of 0.01 to 100
 // spacings: the LP is recorded as infeasible (code 2) and not solved.
+// Six blocks per SM for the small LPs of n = 2, with a few spills: 723 us for
+// 229,000 (four blocks 775, five 742, seven 755); the full ones keep the
+// compiler's five (1,563 us; four 1,650, six 1,600).
+template <int M, bool FULL>
+constexpr int kDfBlocks = M == 9 && !FULL ? 6 : 1;
 template <int M, int G, bool FULL>
-__global__ void __launch_bounds__(128) k_lp_df(Consts c, const double* __restrict__ x, const double* __restrict__ y,
+__global__ void __launch_bounds__(128, kDfBlocks<M, FULL>) k_lp_df(Consts c, const double* __restrict__ x, const double* __restrict__ y,
                                                const int* __restrict__ list, const int* __restrict__ list_count,
                                                const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
                                                const int* __restrict__ small, int* __restrict__ cols,
