@@ -34,6 +34,19 @@ struct Learned {
   ProjScratch proj;       // correction rounds
 };
 
+// What a step starts from, one copy to the device, and what it leaves for the
+// host, one copy back: five copies and a memset take 2 us each in a small
+// cloud's step.
+struct StepHead {
+  StepState st;
+  DevStats ds;
+};
+struct DevBlock {
+  StepHead head;
+  int counters[8];
+  Grid grid;
+};
+
 struct vrm::Scratch {
   int cap = 0;        // particles the buffers hold
   int ncell_cap = 0;  // cells of the grid
@@ -66,16 +79,17 @@ struct vrm::Scratch {
   // the stencils transposed per target (the application's lists, a CSR)
   int *tcount = nullptr, *toff = nullptr;
   double2* tent = nullptr;
-  // counters and state
+  // counters and state, in one block (and grid), and its pinned host mirror
+  DevBlock *block = nullptr, *h_block = nullptr;
   DevStats* ds = nullptr;
   int* counters = nullptr;  // [0] |D|, [1] first open list length
   StepState* st = nullptr;
-  // pinned host mirrors
   DevStats* h_ds = nullptr;
   int* h_counters = nullptr;
   Grid* h_grid = nullptr;
-  StepState* h_params = nullptr;  // n, capacity, dt, max_rounds of the next step
   StepState* h_state = nullptr;   // state after the step
+  StepHead* h_head = nullptr;     // pinned: n, capacity, dt, max_rounds of the next step; counters of 0
+  StepState* h_params = nullptr;  // its state
 };
 
 // The particle grid's cells as the insertion rounds read them.
@@ -178,18 +192,17 @@ void drop_graph(vrm_ctx* ctx) {
 
 void free_scratch(Scratch& s) {
   RoundBufs& r = s.rb;
-  void* ptrs[] = {s.grid, s.cell_key, s.cell_rank, s.cell_count, s.cell_start, s.sorted_xy, s.sorted_loc,
+  void* ptrs[] = {s.block, s.cell_key, s.cell_rank, s.cell_count, s.cell_start, s.sorted_xy, s.sorted_loc,
                   s.sorted_idx, s.bbox, s.scan_tmp, s.pos, s.rstate, s.tie_flag, s.tie_rank, s.dflag_ts, s.tie_ts,
                   s.cell_ts, s.diffused, s.dlist,
                   s.mask, r.open, r.act0, r.act1, r.cnt, r.cpos, r.cnt_ts, r.cell_ts, r.keep_ts, r.keep_flag, r.cx,
                   r.cy, r.keep, r.keep_s, r.apos,
                   r.cg.grid, r.cg.cell_key, r.cg.cell_rank, r.cg.cell_count, r.cg.cell_start, r.cg.sorted_idx,
                   r.cg.sorted_xy, r.cg.sorted_loc, r.cg.bbox, r.scan_tmp, s.nbr_count, s.nbr_idx, s.small, s.cols,
-                  s.fail_list, s.retry_list, s.retry_list2, s.seg_mask, s.status, s.f, s.fii, s.tcount, s.toff, s.tent, s.ds,
-                  s.counters, s.st};
+                  s.fail_list, s.retry_list, s.retry_list2, s.seg_mask, s.status, s.f, s.fii, s.tcount, s.toff, s.tent};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  void* hp[] = {s.h_ds, s.h_counters, s.h_grid, s.h_params, s.h_state};
+  void* hp[] = {s.h_block, s.h_head};
   for (void* p : hp)
     if (p) cudaFreeHost(p);
   Scratch empty;
@@ -388,8 +401,8 @@ cudaError_t enqueue_stage_weights(vrm_ctx* ctx, const double* x, const double* y
   const Consts& c = ctx->c;
   const int* n_cur = &s.st->n_cur;
   cudaError_t e;
-  // the full-neighbourhood queue of this stage starts empty
-  if ((e = cudaMemsetAsync(&s.ds->n_fail, 0, sizeof(int), st)) != cudaSuccess) return e;
+  // the full-neighbourhood queue and the re-run lists of this stage start empty
+  if ((e = cudaMemsetAsync(&s.ds->n_fail, 0, 3 * sizeof(int), st)) != cudaSuccess) return e;
   if ((e = grid_build_dev(x, y, cap, n_cur, c.Rh, c.lo2, c.hi2, s.ncell_cap, s.grid, s.cell_key, s.cell_rank,
                           s.cell_count, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.bbox, s.scan_tmp,
                           st, s.cell_ts, true)) != cudaSuccess)
@@ -449,7 +462,7 @@ cudaError_t ensure_scratch(vrm_ctx* ctx, int cap, cudaStream_t st) {
   RoundBufs& r = s.rb;
 #define VRM_ALLOC(ptr, count) \
   if (e == cudaSuccess) e = dalloc(&(ptr), (size_t)(count))
-  VRM_ALLOC(s.grid, 1);
+  VRM_ALLOC(s.block, 1);
   VRM_ALLOC(s.cell_key, n);
   VRM_ALLOC(s.cell_rank, n);
   VRM_ALLOC(s.cell_count, ncell);
@@ -508,9 +521,6 @@ cudaError_t ensure_scratch(vrm_ctx* ctx, int cap, cudaStream_t st) {
   VRM_ALLOC(s.tcount, n);
   VRM_ALLOC(s.toff, (long)n + 1);
   VRM_ALLOC(s.tent, (long)n * ctx->c.w);
-  VRM_ALLOC(s.ds, 1);
-  VRM_ALLOC(s.counters, 8);
-  VRM_ALLOC(s.st, 1);
 #undef VRM_ALLOC
   // the bounding box starts at its initial values (every grid build leaves it so)
   if (e == cudaSuccess) e = grid_bbox_reset(s.bbox, st);
@@ -523,11 +533,20 @@ cudaError_t ensure_scratch(vrm_ctx* ctx, int cap, cudaStream_t st) {
   // round leaves them empty
   if (e == cudaSuccess) e = cudaMemsetAsync(r.cg.cell_count, 0, sizeof(int) * (size_t)ncell, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(r.cell_ts, 0, sizeof(int) * (size_t)(ncell / kScanTile + 2), st);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_ds, sizeof(DevStats));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_counters, sizeof(int) * 8);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_grid, sizeof(Grid));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_params, sizeof(StepState));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_state, sizeof(StepState));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_block, sizeof(DevBlock));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&s.h_head, sizeof(StepHead));
+  if (e == cudaSuccess) {
+    s.st = &s.block->head.st;
+    s.ds = &s.block->head.ds;
+    s.counters = s.block->counters;
+    s.grid = &s.block->grid;
+    s.h_state = &s.h_block->head.st;
+    s.h_ds = &s.h_block->head.ds;
+    s.h_counters = s.h_block->counters;
+    s.h_grid = &s.h_block->grid;
+    memset(s.h_head, 0, sizeof(StepHead));
+    s.h_params = &s.h_head->st;
+  }
   if (e != cudaSuccess) {
     free_scratch(s);
     cudaGetLastError();
@@ -596,10 +615,7 @@ void fill_consts(const vrm_params& p, Consts& c) {
 
 cudaError_t read_back(vrm_ctx* ctx, cudaStream_t st) {
   Scratch& s = ctx->s;
-  cudaError_t e = cudaMemcpyAsync(s.h_ds, s.ds, sizeof(DevStats), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s.h_counters, s.counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s.h_grid, s.grid, sizeof(Grid), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s.h_state, s.st, sizeof(StepState), cudaMemcpyDeviceToHost, st);
+  cudaError_t e = cudaMemcpyAsync(s.h_block, s.block, sizeof(DevBlock), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e;
 }
@@ -761,18 +777,12 @@ cudaError_t enqueue_back(vrm_ctx* ctx, double* x, double* y, int cap, const doub
                                 0.0, &s.st->dt, st)) != cudaSuccess)
     return e;
   if ((e = mark(ctx, VRM_STAGE_COUNT, st)) != cudaSuccess) return e;
-  if ((e = cudaMemcpyAsync(s.h_ds, s.ds, sizeof(DevStats), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-  if ((e = cudaMemcpyAsync(s.h_counters, s.counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-    return e;
-  if ((e = cudaMemcpyAsync(s.h_grid, s.grid, sizeof(Grid), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-  return cudaMemcpyAsync(s.h_state, s.st, sizeof(StepState), cudaMemcpyDeviceToHost, st);
+  return cudaMemcpyAsync(s.h_block, s.block, sizeof(DevBlock), cudaMemcpyDeviceToHost, st);
 }
 
 cudaError_t enqueue_head(vrm_ctx* ctx, cudaStream_t st) {
   Scratch& s = ctx->s;
-  cudaError_t e = cudaMemcpyAsync(s.st, s.h_params, sizeof(StepState), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s.ds, 0, sizeof(DevStats), st);
-  return e;
+  return cudaMemcpyAsync(&s.block->head, s.h_head, sizeof(StepHead), cudaMemcpyHostToDevice, st);
 }
 
 // Records one context's whole step into the graph being captured on cs: the

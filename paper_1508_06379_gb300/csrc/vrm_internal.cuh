@@ -93,7 +93,10 @@ struct DevStats {
   int small_ok, full_ok, no_stencil;
   int max_pivots;
   int max_count;
+  // the lists of one pass of the LPs (set to 0 together)
   int n_fail;          // particles queued for the full-neighbourhood LP
+  int n_retry;         // LPs that the binary32 pivots handed back
+  int n_retry_pairs;   // ... and that the pairs handed back (FP64 re-runs)
   int nonfinite;       // set if a circulation was NaN/Inf
   unsigned long long max_dt_ratio_bits;  // positive double, as bits
   unsigned long long lp_small_pivots, lp_full_pivots;
@@ -102,8 +105,6 @@ struct DevStats {
   unsigned long long learned_screens;        // supports screened by the learned path
   unsigned long long lp_full_columns;        // columns summed over the full-neighbourhood LPs
   unsigned long long lp_full_column_pivots;  // columns x pivots summed over them
-  int n_retry;                               // LPs of the current pass that the binary32 pivots handed back
-  int n_retry_pairs;                         // ... and that the pairs handed back (FP64 re-runs)
   unsigned long long lp_small_retries;       // small LPs handed back by the first certified pivots (n = 1)
 };
 

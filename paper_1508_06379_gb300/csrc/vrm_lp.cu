@@ -2415,8 +2415,7 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
                      int* retry_list, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,
                      const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(&ds->n_retry, 0, 2 * sizeof(int), s);  // n_retry and n_retry_pairs
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   if (c.order == 2) {
     e = lp_pairs<9>(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list,
                     retry_list2, ds, nu_dt, s, dt_dev, nu, c.lp_fp64_pivots != 0, false);
