@@ -429,8 +429,8 @@ cudaError_t enqueue_stage_weights(vrm_ctx* ctx, const double* x, const double* y
     lp_list = ctx->L.rlist;
     lp_count = s.counters + 2;
   }
-  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list, s.retry_list2, s.ds,
-                    0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
+  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list,
+                    s.retry_list2, s.rb.keep_flag, s.ds, 0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
     return e;
   if (!rows && (e = search_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key,
                                     s.cell_rank, s.fail_list, &s.ds->n_fail, std::min(cap, 32 * sm_count()),
@@ -760,8 +760,8 @@ cudaError_t enqueue_back(vrm_ctx* ctx, double* x, double* y, int cap, const doub
     lp_list = ctx->L.rlist;
     lp_count = s.counters + 2;
   }
-  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list, s.retry_list2, s.ds,
-                    0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
+  if ((e = lp_small(c, x, y, lp_list, lp_count, cap, s.small, s.cols, s.f, s.fii, s.status, s.fail_list, s.retry_list,
+                    s.retry_list2, s.rb.keep_flag, s.ds, 0.0, st, &s.st->dt, ctx->p.nu)) != cudaSuccess)
     return e;
   if ((e = mark(ctx, VRM_STAGE_LP_FULL, st)) != cudaSuccess) return e;
   if (!rows && (e = search_list_dev(c, s.grid, s.cell_start, s.sorted_xy, s.sorted_loc, s.sorted_idx, s.cell_key,
@@ -1150,8 +1150,8 @@ vrm_status vrm_solve_weights(vrm_ctx* ctx, const double* x, const double* y, int
     lp_list = ctx->L.rlist;
     lp_count = s.counters + 2;
   }
-  VRM_CUDA(lp_small(c, x, y, lp_list, lp_count, n, small, cols, f, fii, status, s.fail_list, s.retry_list, s.retry_list2, s.ds,
-                      0.0, stream));
+  VRM_CUDA(lp_small(c, x, y, lp_list, lp_count, n, small, cols, f, fii, status, s.fail_list, s.retry_list,
+                    s.retry_list2, s.rb.keep_flag, s.ds, 0.0, stream));
   VRM_CUDA(lp_full(c, x, y, s.fail_list, &s.ds->n_fail, n, nbr_count, nbr_idx, cols, f, fii, status,
                    s.retry_list2, s.ds, 0.0, stream));
   if (stats) {

@@ -551,8 +551,8 @@ cudaError_t open_small(const int* dlist, const int* dcount, const uint8_t* mask,
 // nu_dt = nu * dt for the stability statistic; with dt_dev it is nu * *dt_dev.
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
-                     int* retry_list, int* retry_list2,
-                     DevStats* ds, double nu_dt, cudaStream_t s, const double* dt_dev = nullptr, double nu = 0.0);
+                     int* retry_list, int* retry_list2, uint8_t* pending, DevStats* ds, double nu_dt,
+                     cudaStream_t s, const double* dt_dev = nullptr, double nu = 0.0);
 cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int* fail_list, const int* fail_count,
                     int cap, const int* nbr_count, const int* nbr_idx, int* cols, double* f, double* fii,
                     uint8_t* status, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,

@@ -1318,21 +1318,19 @@ __device__ __forceinline__ void lp_recorded(const int* row, int (&basis)[M], int
 // For n = 2 (M = 9) and for the columns of small neighbourhoods (small given)
 // the kernel stops at the final basis and leaves it in the particle's stencil
 // row (lp_record), for k_lp_finish.
-template <int M, int W>
-__global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restrict__ x,
-                                                 const double* __restrict__ y, const int* __restrict__ fail_list,
-                                                 const int* __restrict__ fail_count,
-                                                 const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
-                                                 const int* __restrict__ small,
-                                                 int* __restrict__ cols, double* __restrict__ f,
-                                                 double* __restrict__ fii, uint8_t* __restrict__ status,
-                                                 DevStats* __restrict__ ds, double nu_dt,
-                                                 const double* __restrict__ dt_dev, double nu) {
+// SMALL_END: the columns of small neighbourhoods, solved here all the same,
+// an infeasible LP queued for the full neighbourhoods (next_list) as the small
+// LPs' other kernels do.  warp of nwarps warps.
+template <int M, int W, bool SMALL_END>
+__device__ __forceinline__ void lp_by_warps(const Consts& c, const double* __restrict__ x,
+                                            const double* __restrict__ y, const int* __restrict__ fail_list,
+                                            const int* __restrict__ fail_count, const int* __restrict__ nbr_count,
+                                            const int* __restrict__ nbr_idx, const int* __restrict__ small,
+                                            int* __restrict__ cols, double* __restrict__ f, double* __restrict__ fii,
+                                            uint8_t* __restrict__ status, int* __restrict__ next_list,
+                                            DevStats* __restrict__ ds, double nu_dt, long warp, long nwarps) {
   constexpr unsigned kAll = 0xffffffffu;
-  if (dt_dev) nu_dt = nu * *dt_dev;
   const int lane = threadIdx.x & 31;
-  const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long nwarps = ((long)gridDim.x * blockDim.x) >> 5;
   const int m = *fail_count;
   const double inv_h2 = 1.0 / (c.h * c.h);
   int st_ok = 0, st_none = 0, st_maxpiv = 0, st_solved = 0, st_pivots = 0;
@@ -1467,7 +1465,7 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
       if (lane == leave) bas = M + q;
       ++it;
     }
-    if (M == 9 || small) {
+    if (M == 9 || (!SMALL_END && small)) {
       const int bj = __shfl_sync(kAll, j, bas >= M && bas != INT_MAX ? bas - M : 0);
       lp_record<M, 32>(cols + (size_t)i * W, lane, bas, bas >= M ? bj : -1, code, it);
       continue;
@@ -1565,11 +1563,13 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
       }
       if (lane == 0) {
         fii[i] = -sacc;
-        status[i] = VRM_LP_FULL;
+        status[i] = SMALL_END ? VRM_LP_SMALL : VRM_LP_FULL;
         ++st_ok;
         const double qr = __dmul_rn(__dmul_rn(nu_dt, sacc), inv_h2);
         st_ratio = qr > st_ratio ? qr : st_ratio;
       }
+    } else if (SMALL_END && c.fallback) {
+      if (lane == 0) next_list[atomicAdd(&ds->n_fail, 1)] = i;
     } else {
       if (lane < W) {
         crow[lane] = -1;
@@ -1589,7 +1589,8 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
       st_colpiv += (unsigned long long)K * it;
     }
   }
-  flush_stats(ds, st_ok, st_none, st_maxpiv, st_ratio, true, st_solved, st_pivots);
+  flush_stats(ds, st_ok, st_none, st_maxpiv, st_ratio, !SMALL_END, st_solved, st_pivots);
+  if (SMALL_END) return;
   st_cols = __reduce_add_sync(kAll, (unsigned)st_cols);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) st_colpiv += __shfl_xor_sync(kAll, st_colpiv, o);
@@ -1597,6 +1598,21 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
     atomicAdd(&ds->lp_full_columns, (unsigned long long)st_cols);
     atomicAdd(&ds->lp_full_column_pivots, st_colpiv);
   }
+}
+template <int M, int W>
+__global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restrict__ x,
+                                                 const double* __restrict__ y, const int* __restrict__ fail_list,
+                                                 const int* __restrict__ fail_count,
+                                                 const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
+                                                 const int* __restrict__ small,
+                                                 int* __restrict__ cols, double* __restrict__ f,
+                                                 double* __restrict__ fii, uint8_t* __restrict__ status,
+                                                 DevStats* __restrict__ ds, double nu_dt,
+                                                 const double* __restrict__ dt_dev, double nu) {
+  if (dt_dev) nu_dt = nu * *dt_dev;
+  lp_by_warps<M, W, false>(c, x, y, fail_list, fail_count, nbr_count, nbr_idx, small, cols, f, fii, status, nullptr, ds,
+                           nu_dt, ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                           ((long)gridDim.x * blockDim.x) >> 5);
 }
 
 // ---------------------------------------------------------------------------
@@ -1699,7 +1715,8 @@ constexpr float kDfFma = 24.0f * kU2, kDfMul = 24.0f * kU2;
 // (unsorted; `rank` is its place in the order (d2, j)), and row r's
 // right-hand side, basic variable and ratio are on lane r < 9.  The final
 // basis goes to the particle's row of cols (lp_record), an LP with an
-// uncertain decision to the retry list.  n = 2: G = 32 for the full
+// uncertain decision to the retry list (n = 1: and marked in pending, by its
+// list position).  n = 2: G = 32 for the full
 // neighbourhoods (FULL), G = 16 for the small ones, two per warp (8 of the
 // lanes hold columns, 9 hold rows); n = 1: G = 8, four small LPs per warp, for
 // the LPs of small clouds, where the latency of one LP counts (lp_small).  The
@@ -1729,7 +1746,8 @@ __global__ void __launch_bounds__(128, kDfBlocks<M, FULL>) k_lp_df(Consts c, con
                                                const int* __restrict__ list, const int* __restrict__ list_count,
                                                const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
                                                const int* __restrict__ small, int* __restrict__ cols,
-                                               int* __restrict__ retry_list, DevStats* __restrict__ ds, bool count_retries) {
+                                               int* __restrict__ retry_list, uint8_t* __restrict__ pending,
+                                               DevStats* __restrict__ ds, bool count_retries) {
   constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int kNone = 1 << 20;
@@ -2015,6 +2033,7 @@ __global__ void __launch_bounds__(128, kDfBlocks<M, FULL>) k_lp_df(Consts c, con
       retry_list[atomicAdd(&ds->n_retry_pairs, 1)] = i;
       if (count_retries) atomicAdd(&ds->lp_small_retries, 1ull);
     }
+    if (M == 5 && have && gl == 0) pending[t] = unc;
     lp_record<M, G>(cols + (size_t)i * W, have && !unc ? gl : G, bas, bj, code, it);
   }
 }
@@ -2025,25 +2044,24 @@ __global__ void __launch_bounds__(128, kDfBlocks<M, FULL>) k_lp_df(Consts c, con
 // a warp's lanes the 9 x 9 system takes the FP64 pipe about 300 warp
 // instructions per particle, here 900 per 32.
 template <int M, bool FULL>
-__global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __restrict__ x,
+__device__ __forceinline__ void lp_finish_recorded(const Consts& c, const double* __restrict__ x,
                                                    const double* __restrict__ y, const int* __restrict__ list,
                                                    const int* __restrict__ list_count,
+                                                   const uint8_t* __restrict__ pending,
                                                    const int* __restrict__ nbr_count, int* __restrict__ cols,
                                                    double* __restrict__ f, double* __restrict__ fii,
                                                    uint8_t* __restrict__ status, int* __restrict__ fail_list,
-                                                   DevStats* __restrict__ ds, double nu_dt,
-                                                   const double* __restrict__ dt_dev, double nu) {
+                                                   DevStats* __restrict__ ds, double nu_dt, int block, int nblocks) {
   constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W;
-  if (dt_dev) nu_dt = nu * *dt_dev;
   const int m = *list_count;
   const double inv_h2 = 1.0 / (c.h * c.h);
   LpTally tl;
   unsigned st_cols = 0;
   unsigned long long st_colpiv = 0;
-  const long stride = (long)gridDim.x * blockDim.x;
-  for (long base = (long)blockIdx.x * blockDim.x; base < m; base += stride) {
+  const long stride = (long)nblocks * blockDim.x;
+  for (long base = (long)block * blockDim.x; base < m; base += stride) {
     const long t = base + threadIdx.x;
-    if (t < m) {
+    if (t < m && !(M == 5 && pending[t])) {
       const int i = list[t];
       int* const crow = cols + (size_t)i * W;
       double* const frow = f + (size_t)i * W;
@@ -2150,6 +2168,46 @@ __global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __rest
       atomicAdd(&ds->lp_full_column_pivots, st_colpiv);
     }
   }
+}
+template <int M, bool FULL>
+__global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __restrict__ x,
+                                                   const double* __restrict__ y, const int* __restrict__ list,
+                                                   const int* __restrict__ list_count,
+                                                   const int* __restrict__ nbr_count, int* __restrict__ cols,
+                                                   double* __restrict__ f, double* __restrict__ fii,
+                                                   uint8_t* __restrict__ status, int* __restrict__ fail_list,
+                                                   DevStats* __restrict__ ds, double nu_dt,
+                                                   const double* __restrict__ dt_dev, double nu) {
+  if (dt_dev) nu_dt = nu * *dt_dev;
+  lp_finish_recorded<M, FULL>(c, x, y, list, list_count, nullptr, nbr_count, cols, f, fii, status, fail_list, ds, nu_dt,
+                              blockIdx.x, gridDim.x);
+}
+
+// The end of the small LPs of n = 1 in pairs: the last blocks re-run the
+// uncertain ones in FP64, a warp each, while the others solve the final bases
+// of the rest (first, so that they spread evenly over the SMs; pending, by list position: the records cannot tell, a re-run
+// overwrites its own).  Both are short chains of FP64 latency: 28 us one after
+// the other, 19 together for 17,000 LPs, 25 and 17 for 345.
+template <int M, int W>
+__global__ void __launch_bounds__(64) k_lp_small_end(Consts c, const double* __restrict__ x,
+                                                      const double* __restrict__ y, const int* __restrict__ list,
+                                                      const int* __restrict__ list_count,
+                                                      const uint8_t* __restrict__ pending,
+                                                      const int* __restrict__ retry_list,
+                                                      const int* __restrict__ small, int retry_blocks,
+                                                      int* __restrict__ cols, double* __restrict__ f,
+                                                      double* __restrict__ fii, uint8_t* __restrict__ status,
+                                                      int* __restrict__ fail_list, DevStats* __restrict__ ds,
+                                                      double nu_dt, const double* __restrict__ dt_dev, double nu) {
+  if (dt_dev) nu_dt = nu * *dt_dev;
+  const int solve_blocks = (int)gridDim.x - retry_blocks;
+  if ((int)blockIdx.x < solve_blocks)
+    lp_finish_recorded<M, false>(c, x, y, list, list_count, pending, nullptr, cols, f, fii, status, fail_list, ds, nu_dt,
+                                 blockIdx.x, solve_blocks);
+  else
+    lp_by_warps<M, W, true>(c, x, y, retry_list, &ds->n_retry_pairs, nullptr, nullptr, small, cols, f, fii, status,
+                            fail_list, ds, nu_dt, ((long)(blockIdx.x - solve_blocks) * blockDim.x + threadIdx.x) >> 5,
+                            ((long)retry_blocks * blockDim.x) >> 5);
 }
 
 // Identity weights of the removal candidates (particle removal, the outlook
@@ -2363,10 +2421,10 @@ static cudaError_t lp_pairs(const Consts& c, const double* x, const double* y, c
   if (!fp64) {
     if (M == 5 || small)
       k_lp_df<M, G, false><<<grid(128 / G, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small,
-                                                             cols, retry_list, ds, count_retries);
+                                                             cols, retry_list, nullptr, ds, count_retries);
     else
       k_lp_df<9, 32, true><<<grid(4, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
-                                                       retry_list, ds, false);
+                                                       retry_list, nullptr, ds, false);
     note_launch();
     list = retry_list;
   }
@@ -2412,8 +2470,8 @@ constexpr int kWsCap = 18 * 65536;
 
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
-                     int* retry_list, int* retry_list2, DevStats* ds, double nu_dt, cudaStream_t s,
-                     const double* dt_dev, double nu) {
+                     int* retry_list, int* retry_list2, uint8_t* pending, DevStats* ds, double nu_dt,
+                     cudaStream_t s, const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
   cudaError_t e;
   if (c.order == 2) {
@@ -2465,11 +2523,20 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
     list = retry_list;
     list_count = &ds->n_retry;
   }
-  e = lp_pairs<5>(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list, retry_list2,
-                  ds, nu_dt, s, dt_dev, nu, false, load <= kPairsCap);
-  if (e != cudaSuccess) return e;
-  return lp_finish_list<5, false>(c, x, y, list, list_count, cap, nullptr, cols, f, fii, status, fail_list, ds, nu_dt,
-                                  s, dt_dev, nu);
+  const long sms = sm_count();
+  const auto blocks_of = [&](long per_block, long per_sm) {
+    const long b = ((long)cap + per_block - 1) / per_block;
+    return (int)(b < per_sm * sms ? b : per_sm * sms);
+  };
+  k_lp_df<5, 8, false><<<blocks_of(16, 16), 128, 0, s>>>(c, x, y, list, list_count, nullptr, nullptr, small, cols,
+                                                         retry_list2, pending, ds, load <= kPairsCap);
+  note_launch();
+  const int retry_blocks = blocks_of(2, 4);
+  k_lp_small_end<5, 8><<<retry_blocks + blocks_of(64, 16), 64, 0, s>>>(
+      c, x, y, list, list_count, pending, retry_list2, small, retry_blocks, cols, f, fii, status, fail_list, ds, nu_dt,
+      dt_dev, nu);
+  note_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int* fail_list, const int* fail_count,
