@@ -380,7 +380,9 @@ __global__ void __launch_bounds__(128) k_search_warp(Consts c, const Grid* __res
         mask |= 1u << sg;
         const float dmin = __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(mine ? d2f : 3e38f)));
         const unsigned near = __ballot_sync(kAll, mine && d2f - dmin <= tie);
-        const int jmin = (int)__reduce_min_sync(kAll, mine && d2f == dmin ? (unsigned)j : 0x7FFFFFFFu);
+        // (not above dmin rather than equal to it: a NaN offset, which the step
+        // refuses in the end, must leave an index too)
+        const int jmin = (int)__reduce_min_sync(kAll, mine && !(d2f > dmin) ? (unsigned)j : 0x7FFFFFFFu);
         const float pb = __shfl_sync(kAll, bf, sg);
         const int pj = __shfl_sync(kAll, bj, sg);
         if (__popc(near) > 1 || (pj >= 0 && fabsf(dmin - pb) <= tie)) amb |= 1u << sg;
@@ -416,7 +418,7 @@ __global__ void __launch_bounds__(128) k_search_warp(Consts c, const Grid* __res
           jd = oj;
         }
       }
-      if (lane == sg) bj = jd;
+      if (lane == sg && jd != 0x7FFFFFFF) bj = jd;
     }
     if (lane < 8) small[(size_t)i * 8 + lane] = bj;
     if (lane == 0) {
