@@ -7,10 +7,16 @@
 // separate kernels leave it, bit for bit.
 //
 // Bound by latency and, from some ten thousand particles on, by the one SM's
-// issue: 870 particles take 15 us and 20,449 48 us, the ten kernels of the
-// front 75 us either way; the open list and the rounds' state 5 and 11 us
-// against 17.  The line: at 65,536 of capacity (32,000 particles, usually) the
-// two are about equal.
+// issue: 870 particles take 13 us, 20,449 43 us and 32,041 80 us, the ten
+// kernels of the front 75 us either way.  k_front_small_cluster shares the
+// particles out to the eight blocks of a cluster: each takes
+// its own into its shared memory and sums their digits, the blocks exchange
+// digit sums, candidates and counts through distributed shared memory, and every
+// block takes the same decisions; its six cluster barriers make it slower for
+// few particles.  The open list and the rounds' state take 5 and 11 us against
+// 17.
+#include <cooperative_groups.h>
+
 #include "vrm_internal.cuh"
 
 namespace vrm {
@@ -19,14 +25,19 @@ namespace {
 
 constexpr int kFsThreads = 1024;
 constexpr int kFsWarps = kFsThreads / 32;
-constexpr int kFsKeys = 21504;  // keys kept in shared memory, as many as fit (further ones are read again)
+// keys kept in shared memory: as many as fit, further ones are read again; in
+// a cluster all of them
+template <int C>
+constexpr int kFsKeys = C == 1 ? 21504 : kSmallCap / C;
 // The first selection takes the keys' top 16 bits (sixteenths of a binade)
 // below those of the largest key: q is 0 more than 96 binades below it.
 constexpr int kFsBins = 97 * 16;
 constexpr int kFsPieces = 7;  // 16-bit pieces of a sum of q (at most 96 + 16 bits)
+constexpr int kFsCluster = 8;  // blocks of the clustered form
 constexpr int kFsList = 256;  // candidates for the threshold that are compared pairwise
-constexpr size_t kFsSmem =
-    sizeof(unsigned long long) * (kFsKeys + kFsWarps) + sizeof(unsigned) * (kFsPieces + 1) * kFsBins;
+template <int C>
+constexpr size_t kFsSmem = sizeof(unsigned long long) * (kFsKeys<C> + kFsWarps) +
+                           sizeof(unsigned) * (kFsPieces + 1) * (kFsBins + (C > 1 ? (kFsBins + C - 1) / C : 0));
 
 struct FrontSmallArgs {
   const double *gamma, *x, *y;
@@ -140,16 +151,63 @@ struct Run {
   }
 };
 
-__global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constant__ FrontSmallArgs a) {
+// The blocks of a cluster of C (1: one block) as k_front_small uses them.
+template <int C>
+__device__ __forceinline__ void all_sync() {
+  if constexpr (C > 1)
+    cooperative_groups::this_cluster().sync();
+  else
+    __syncthreads();
+}
+template <int C, class T>
+__device__ __forceinline__ T* of_block(T* p, int r) {
+  if constexpr (C > 1)
+    return cooperative_groups::this_cluster().map_shared_rank(p, r);
+  else
+    return p;
+}
+// Every block's digit sums become those of all blocks: block r adds up its
+// share of the bins into `merged`, then every block copies all shares.
+template <int C, int BINS>
+__device__ __forceinline__ void merge_sums(unsigned* h, unsigned* merged, int rank) {
+  all_sync<C>();
+  if constexpr (C > 1) {
+    constexpr int kShare = (BINS + C - 1) / C;
+    for (int k = threadIdx.x; k < kShare * (kFsPieces + 1); k += kFsThreads) {
+      const int piece = k / kShare, b = rank * kShare + k % kShare;
+      unsigned v = 0;
+      if (b < BINS) {
+#pragma unroll
+        for (int r = 0; r < C; ++r) v += of_block<C>(h, r)[piece * BINS + b];
+      }
+      merged[k] = v;
+    }
+    all_sync<C>();
+    for (int k = threadIdx.x; k < BINS * (kFsPieces + 1); k += kFsThreads) {
+      const int piece = k / BINS, b = k % BINS;
+      h[k] = of_block<C>(merged, b / kShare)[piece * kShare + b % kShare];
+    }
+    __syncthreads();
+  }
+}
+
+template <int C>
+__device__ __forceinline__ void front_small_block(const FrontSmallArgs& a) {
   extern __shared__ unsigned long long s_dyn[];
   unsigned long long* const s_key = s_dyn;
-  DigitSums H{reinterpret_cast<unsigned*>(s_dyn + kFsKeys + kFsWarps), kFsBins};
+  unsigned* const s_merged = reinterpret_cast<unsigned*>(s_dyn + kFsKeys<C> + kFsWarps) + (kFsPieces + 1) * kFsBins;
+  __shared__ unsigned long long s_x[5];
+  __shared__ int s_xflag, s_xties, s_xgt;
+  const int rank = C > 1 ? (int)blockIdx.x : 0;
+  DigitSums H{reinterpret_cast<unsigned*>(s_dyn + kFsKeys<C> + kFsWarps), kFsBins};
   __shared__ unsigned long long s_red[5][kFsWarps], s_tau[2], s_rem[2], s_T;
   __shared__ unsigned long long s_list[kFsList], s_qlo[kFsList], s_qhi[kFsList];
   __shared__ int s_flag[kFsWarps], s_sel, s_cnt, s_ktie, s_gt[kFsWarps], s_tie[kFsWarps], s_nlist;
   __shared__ Grid s_grid;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int n = *a.n_dev;
+  // the block's share of the particles: [c0, c0 + n) of n_all
+  const int n_all = *a.n_dev, per = (n_all + C - 1) / C;
+  const int c0 = rank * per < n_all ? rank * per : n_all, n = n_all - c0 < per ? n_all - c0 : per;
   // The particles in 32 segments of 32 `chunk`s: warp w takes segment w where a
   // warp works together, and where every thread takes a chunk of its own, lane
   // l of warp w has chunk w of segment l, so that a warp's lanes are far apart
@@ -158,7 +216,7 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
   const int chunk = (n + kFsThreads - 1) / kFsThreads;
   const int seg = 32 * chunk;
   auto key_of = [&](int i, int sg) {
-    if (i < kFsKeys) return s_key[i + sg];
+    if (C > 1 || i < kFsKeys<C>) return s_key[i + sg];
     const unsigned long long b = (unsigned long long)__double_as_longlong(a.gamma[i]) & 0x7FFFFFFFFFFFFFFFull;
     return b < 0x7FF0000000000000ull ? b : 0ull;
   };
@@ -168,13 +226,13 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
   int flags = 0;  // 1: a circulation is NaN or Inf, 2: a position is
 #pragma unroll 4
   for (int i = tid; i < n; i += kFsThreads) {
-    unsigned long long b = (unsigned long long)__double_as_longlong(a.gamma[i]) & 0x7FFFFFFFFFFFFFFFull;
-    const double xi = a.x[i], yi = a.y[i];
+    unsigned long long b = (unsigned long long)__double_as_longlong(a.gamma[c0 + i]) & 0x7FFFFFFFFFFFFFFFull;
+    const double xi = a.x[c0 + i], yi = a.y[c0 + i];
     if (b >= 0x7FF0000000000000ull) {
       flags |= 1;
       b = 0;
     }
-    if (i < kFsKeys) s_key[i + i / seg] = b;
+    if (C > 1 || i < kFsKeys<C>) s_key[i + i / seg] = b;
     amax = b > amax ? b : amax;
     // (exponent bits: a test in FP64 would take the one SM's FP64 pipe 10 us for
     // 20,449 particles)
@@ -213,22 +271,41 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
     s_flag[w] = flags;
   }
   __syncthreads();
-  amax = s_red[0][lane];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long t = __shfl_xor_sync(0xffffffffu, amax, o);
-    amax = t > amax ? t : amax;
-  }
-  if (tid == kFsThreads - 32) {  // the last warp's first lane: the grid, beside the selection
+  if (tid == kFsThreads - 32) {
     for (int k = 0; k < kFsWarps; ++k) {
+      amax = s_red[0][k] > amax ? s_red[0][k] : amax;
       mnx = s_red[1][k] < mnx ? s_red[1][k] : mnx;
       mxx = s_red[2][k] > mxx ? s_red[2][k] : mxx;
       mny = s_red[3][k] < mny ? s_red[3][k] : mny;
       mxy = s_red[4][k] > mxy ? s_red[4][k] : mxy;
       flags |= s_flag[k];
     }
+    s_x[0] = amax;
+    s_x[1] = mnx;
+    s_x[2] = mxx;
+    s_x[3] = mny;
+    s_x[4] = mxy;
+    s_xflag = flags;
+  }
+  all_sync<C>();
+  amax = 0;
+#pragma unroll
+  for (int r = 0; r < C; ++r) {
+    const unsigned long long t = of_block<C>(s_x, r)[0];
+    amax = t > amax ? t : amax;
+  }
+  if (rank == 0 && tid == kFsThreads - 32) {  // the last warp's first lane: the grid, beside the selection
+#pragma unroll
+    for (int r = 1; r < C; ++r) {
+      const unsigned long long* const o = of_block<C>(s_x, r);
+      mnx = o[1] < mnx ? o[1] : mnx;
+      mxx = o[2] > mxx ? o[2] : mxx;
+      mny = o[3] < mny ? o[3] : mny;
+      mxy = o[4] > mxy ? o[4] : mxy;
+      flags |= *of_block<C>(&s_xflag, r);
+    }
     if (flags & 1) atomicOr(&a.ds->nonfinite, 1);
-    s_grid = grid_geometry(mnx, mxx, mny, mxy, (flags & 2) != 0, n, a.Rh, a.lo2, a.hi2, a.ncell_cap);
+    s_grid = grid_geometry(mnx, mxx, mny, mxy, (flags & 2) != 0, n_all, a.Rh, a.lo2, a.hi2, a.ncell_cap);
     *a.g = s_grid;
   }
 
@@ -257,7 +334,7 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
       }
       run.flush(H);
     }
-    __syncthreads();
+    merge_sums<C, kFsBins>(H.h, s_merged, rank);
     const int b0 = 2 * tid;
     const u128 v0 = b0 < kFsBins ? H.sum(b0) : (u128)0, v1 = b0 + 1 < kFsBins ? H.sum(b0 + 1) : (u128)0;
     u128 total;
@@ -304,7 +381,7 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
           run.add(key);
         }
         run.flush(B);
-        __syncthreads();
+        merge_sums<C, 256>(B.h, s_merged, rank);
         const u128 v = tid < 256 ? B.sum(tid) : (u128)0;
         u128 all;
         const u128 inc = block_scan_u128(v, &all);
@@ -339,18 +416,21 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
         // the key at which the sum of the q up to it passes the rest
         const int shift = 64 - 8 * pass;
         if (tid == 0) s_nlist = 0;
-        __syncthreads();
+        all_sync<C>();
+        unsigned long long *const l_key = of_block<C>(s_list, 0), *const l_lo = of_block<C>(s_qlo, 0),
+                           *const l_hi = of_block<C>(s_qhi, 0);
+        int* const l_n = of_block<C>(&s_nlist, 0);
         for (int i = i0; i < i1; ++i) {
           const unsigned long long key = key_of(i, lane);
           if ((key >> shift) != prefix) continue;
-          const int k = atomicAdd(&s_nlist, 1);
+          const int k = atomicAdd(l_n, 1);
           const u128 q = q_of_key(key, E);
-          s_list[k] = key;
-          s_qlo[k] = (unsigned long long)q;
-          s_qhi[k] = (unsigned long long)(q >> 64);
+          l_key[k] = key;
+          l_lo[k] = (unsigned long long)q;
+          l_hi[k] = (unsigned long long)(q >> 64);
         }
-        __syncthreads();
-        if (tid < count) {
+        all_sync<C>();
+        if (rank == 0 && tid < count) {
           const unsigned long long mine = s_list[tid];
           u128 less = 0, q = 0;
           unsigned same = 0;
@@ -377,9 +457,9 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
           }
         }
       }
-      __syncthreads();
-      T = s_T;
-      k_tie = s_ktie;
+      all_sync<C>();
+      T = *of_block<C>(&s_T, 0);
+      k_tie = *of_block<C>(&s_ktie, 0);
     }
   }
 
@@ -400,6 +480,11 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
   __syncthreads();
   int all_ties, total;
   int tie_at = warps_before(s_tie, w, &all_ties);  // ties before this warp's segment
+  if (C > 1) {
+    if (tid == 0) s_xties = all_ties;
+    all_sync<C>();
+    for (int r = 0; r < rank; ++r) tie_at += *of_block<C>(&s_xties, r);
+  }
   {
     // ties of rank k_tie and above diffuse
     const int first = tie_at > k_tie ? tie_at : k_tie;
@@ -407,6 +492,17 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
   }
   __syncthreads();
   int at = warps_before(s_gt, w, &total);
+  if (C > 1) {
+    if (tid == 0) s_xgt = total;
+    all_sync<C>();
+    total = 0;
+#pragma unroll
+    for (int r = 0; r < C; ++r) {
+      const int t = *of_block<C>(&s_xgt, r);
+      if (r < rank) at += t;
+      total += t;
+    }
+  }
 #pragma unroll 4
   for (int base = r0; base < r1; base += 32) {
     const int i = base + lane;
@@ -415,25 +511,35 @@ __global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constan
     const unsigned tb = __ballot_sync(0xffffffffu, tie);
     const bool d = i < r1 && !all_out && (key > T || (tie && tie_at + __popc(tb & ((1u << lane) - 1u)) >= k_tie));
     const unsigned db = __ballot_sync(0xffffffffu, d);
-    if (i < r1) a.diffused[i] = d;
-    if (d) a.dlist[at + __popc(db & ((1u << lane) - 1u))] = i;
+    if (i < r1) a.diffused[c0 + i] = d;
+    if (d) a.dlist[at + __popc(db & ((1u << lane) - 1u))] = c0 + i;
     at += __popc(db);
     tie_at += __popc(tb);
   }
+  const int g_tid = rank * kFsThreads + tid, g_threads = C * kFsThreads;
   {  // flags past the particles: 0, in words where they are whole
     const uintptr_t d0 = (uintptr_t)a.diffused;
-    const int head = (int)(((d0 + n + 15) & ~(uintptr_t)15) - d0);
+    const int head = (int)(((d0 + n_all + 15) & ~(uintptr_t)15) - d0);
     const int v0 = head < a.cap ? head : a.cap, v1 = v0 + ((a.cap - v0) & ~15);
-    for (int i = v0 + 16 * tid; i < v1; i += 16 * kFsThreads)
+    for (int i = v0 + 16 * g_tid; i < v1; i += 16 * g_threads)
       *reinterpret_cast<uint4*>(a.diffused + i) = make_uint4(0, 0, 0, 0);
-    for (int i = n + tid; i < v0; i += kFsThreads) a.diffused[i] = 0;
-    for (int i = v1 + tid; i < a.cap; i += kFsThreads) a.diffused[i] = 0;
+    for (int i = n_all + g_tid; i < v0; i += g_threads) a.diffused[i] = 0;
+    for (int i = v1 + g_tid; i < a.cap; i += g_threads) a.diffused[i] = 0;
   }
-  if (tid == 0) *a.dcount = total;
+  if (g_tid == 0) *a.dcount = total;
   // the grid's cells empty (s_grid was written before the barriers above)
-  const int ncell = s_grid.ncell;
-  for (int k = tid; k < ncell; k += kFsThreads) a.cell_count[k] = 0;
-  for (int k = tid; k <= ncell / kScanTile; k += kFsThreads) a.cell_ts[k] = 0;
+  const int ncell = of_block<C>(&s_grid, 0)->ncell;
+  if (C > 1) all_sync<C>();  // no block ends while another reads it
+  for (int k = g_tid; k < ncell; k += g_threads) a.cell_count[k] = 0;
+  for (int k = g_tid; k <= ncell / kScanTile; k += g_threads) a.cell_ts[k] = 0;
+}
+
+__global__ void __launch_bounds__(kFsThreads) k_front_small(const __grid_constant__ FrontSmallArgs a) {
+  front_small_block<1>(a);
+}
+__global__ void __cluster_dims__(kFsCluster, 1, 1) __launch_bounds__(kFsThreads)
+    k_front_small_cluster(const __grid_constant__ FrontSmallArgs a) {
+  front_small_block<kFsCluster>(a);
 }
 
 // Open list of the first round (the diffused particles whose mask is not
@@ -514,19 +620,31 @@ __global__ void __launch_bounds__(kFsThreads) k_open_small(const int* __restrict
 
 }  // namespace
 
+// From this capacity on the front takes a cluster: steps of 3,600 particles
+// (8,224 of capacity) 221 us in one block and 229 in a cluster, of 10,000
+// (21,024) 228 and 222, of 20,449 302 and 281, of 32,041 377 and 327.
+constexpr int kFsClusterCap = 16384;
+
 cudaError_t front_small(const double* gamma, const double* x, const double* y, int cap, const int* n_dev,
                         double c_bound, double Rh, double lo2, double hi2, int ncell_cap, uint8_t* diffused,
                         int* dlist, int* dcount, DevStats* ds, Grid* g, int* cell_count, int* cell_ts,
                         cudaStream_t s) {
   static bool attr_set = false;
   if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_front_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFsSmem);
+    cudaError_t e =
+        cudaFuncSetAttribute(k_front_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFsSmem<1>);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_front_small_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kFsSmem<kFsCluster>);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   const FrontSmallArgs a{gamma, x, y, cap, n_dev, c_bound, Rh, lo2, hi2, ncell_cap, diffused, dlist, dcount, ds, g,
                          cell_count, cell_ts};
-  k_front_small<<<1, kFsThreads, kFsSmem, s>>>(a);
+  if (cap >= kFsClusterCap)
+    k_front_small_cluster<<<kFsCluster, kFsThreads, kFsSmem<kFsCluster>, s>>>(a);
+  else
+    k_front_small<<<1, kFsThreads, kFsSmem<1>, s>>>(a);
   note_launch();
   return cudaGetLastError();
 }
