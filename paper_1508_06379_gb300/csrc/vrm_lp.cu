@@ -571,9 +571,10 @@ __global__ void __launch_bounds__(128) k_lp_small(Consts c, const double* __rest
                                                   int* __restrict__ cols, double* __restrict__ f,
                                                   double* __restrict__ fii, uint8_t* __restrict__ status,
                                                   int* __restrict__ fail_list, DevStats* __restrict__ ds,
-                                                  double nu_dt, const double* __restrict__ dt_dev, double nu) {
+                                                  double nu_dt, const double* __restrict__ dt_dev, double nu, int least) {
   if (dt_dev) nu_dt = nu * *dt_dev;
   const int m = *list_count;
+  if (m < least) return;  // left to the pairs
   const double inv_h2 = 1.0 / (c.h * c.h);
   LpTally tl;
   // grid-stride over whole warps so that the warp-level statistics below run converged
@@ -1747,7 +1748,7 @@ __global__ void __launch_bounds__(128, kDfBlocks<M, FULL>) k_lp_df(Consts c, con
                                                const int* __restrict__ nbr_count, const int* __restrict__ nbr_idx,
                                                const int* __restrict__ small, int* __restrict__ cols,
                                                int* __restrict__ retry_list, uint8_t* __restrict__ pending,
-                                               DevStats* __restrict__ ds, bool count_retries) {
+                                               DevStats* __restrict__ ds, bool count_retries, int most) {
   constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int kNone = 1 << 20;
@@ -1763,6 +1764,7 @@ __global__ void __launch_bounds__(128, kDfBlocks<M, FULL>) k_lp_df(Consts c, con
   const f32x2 m1 = pack2(-1.0f, -1.0f), fma_u = pack2(kDfFma, kDfFma);
   unsigned it_all = 0;
   const int m = *list_count;
+  if (m > most) return;  // left to FP64
   const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long nwarps = ((long)gridDim.x * blockDim.x) >> 5;
   for (long t0 = warp * (32 / G); t0 < m; t0 += nwarps * (32 / G)) {
@@ -2198,7 +2200,8 @@ __global__ void __launch_bounds__(64) k_lp_small_end(Consts c, const double* __r
                                                       int* __restrict__ cols, double* __restrict__ f,
                                                       double* __restrict__ fii, uint8_t* __restrict__ status,
                                                       int* __restrict__ fail_list, DevStats* __restrict__ ds,
-                                                      double nu_dt, const double* __restrict__ dt_dev, double nu) {
+                                                      double nu_dt, const double* __restrict__ dt_dev, double nu, int most) {
+  if (*list_count > most) return;
   if (dt_dev) nu_dt = nu * *dt_dev;
   const int solve_blocks = (int)gridDim.x - retry_blocks;
   if ((int)blockIdx.x < solve_blocks)
@@ -2421,10 +2424,10 @@ static cudaError_t lp_pairs(const Consts& c, const double* x, const double* y, c
   if (!fp64) {
     if (M == 5 || small)
       k_lp_df<M, G, false><<<grid(128 / G, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small,
-                                                             cols, retry_list, nullptr, ds, count_retries);
+                                                             cols, retry_list, nullptr, ds, count_retries, INT_MAX);
     else
       k_lp_df<9, 32, true><<<grid(4, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
-                                                       retry_list, nullptr, ds, false);
+                                                       retry_list, nullptr, ds, false, INT_MAX);
     note_launch();
     list = retry_list;
   }
@@ -2460,6 +2463,13 @@ static cudaError_t lp_finish_list(const Consts& c, const double* x, const double
 // to 300,000 particles: 4.49 ms, 4.60 when each went by its own).
 constexpr int kPairsCap = 65536;
 constexpr int kPairsRetryCap = 6 * 65536;
+// The longest list of hand-backs that goes to the pairs in that range, decided
+// on the device (the other form's launch returns at once).  Jittered clouds
+// hand back 2%, lattices a quarter to all of their LPs, many of which the pairs
+// cannot certify either: steps of a lattice of 53,000 particles with 18,229
+// hand-backs 396 us in FP64 and 536 in pairs, of a jittered cloud of 184,900
+// with 4,177 605 and 590, RK3 steps with 5,000 a stage 1,083 and 1,037.
+constexpr int kPairsRetries = 6144;
 // Smallest capacity that takes the 8 + 4-warp form where no schedule was set:
 // steps of 640,000 particles 1,075 us against 1,114 with one kind of warp, of a
 // million 1,469 against 1,581; 787 and 797 at 360,000.  The form fills every SM,
@@ -2489,11 +2499,12 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
   if (blocks > c.lp_blocks_per_sm * sm_count()) blocks = c.lp_blocks_per_sm * sm_count();
   if (c.lp_fp64_pivots || !(c.inv_h > 1e-20 && c.inv_h < 1e20)) {
     k_lp_small<5, 8><<<blocks, tb, 0, s>>>(c, x, y, list, list_count, small, cols, f, fii, status, fail_list, ds,
-                                           nu_dt, dt_dev, nu);
+                                           nu_dt, dt_dev, nu, 0);
     note_launch();
     return cudaGetLastError();
   }
   const int load = c.load > cap ? c.load : cap;
+  int most = INT_MAX;  // the pairs take no longer lists
   if (load > kPairsCap) {
     // certified binary32 pivots, then the uncertain particles in pairs or in FP64
     const int form = c.lp_auto && c.load == 0 && cap >= kWsCap ? kLpWsThreadsWide : c.lp_block;
@@ -2510,16 +2521,16 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
                                                retry_list, ds, nu_dt, dt_dev, nu);
     }
     note_launch();
-    if (load > kPairsRetryCap) {
-      // the re-run list is a few percent of the LPs: one-warp blocks spread it
-      // over every SM instead of over the first few hundred blocks
-      int rblocks = (int)(((long)cap + 31) / 32);
-      if (rblocks > 32 * sm_count()) rblocks = 32 * sm_count();
-      k_lp_small<5, 8><<<rblocks, 32, 0, s>>>(c, x, y, retry_list, &ds->n_retry, small, cols, f, fii, status,
-                                              fail_list, ds, nu_dt, dt_dev, nu);
-      note_launch();
-      return cudaGetLastError();
-    }
+    // the re-run list is a few percent of the LPs, or, on lattices, a quarter:
+    // one-warp blocks spread it over every SM instead of over the first few
+    // hundred blocks
+    most = load > kPairsRetryCap ? -1 : kPairsRetries;
+    int rblocks = (int)(((long)cap + 31) / 32);
+    if (rblocks > 32 * sm_count()) rblocks = 32 * sm_count();
+    k_lp_small<5, 8><<<rblocks, 32, 0, s>>>(c, x, y, retry_list, &ds->n_retry, small, cols, f, fii, status, fail_list,
+                                            ds, nu_dt, dt_dev, nu, most + 1);
+    note_launch();
+    if (most < 0) return cudaGetLastError();
     list = retry_list;
     list_count = &ds->n_retry;
   }
@@ -2529,12 +2540,12 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
     return (int)(b < per_sm * sms ? b : per_sm * sms);
   };
   k_lp_df<5, 8, false><<<blocks_of(16, 16), 128, 0, s>>>(c, x, y, list, list_count, nullptr, nullptr, small, cols,
-                                                         retry_list2, pending, ds, load <= kPairsCap);
+                                                         retry_list2, pending, ds, load <= kPairsCap, most);
   note_launch();
   const int retry_blocks = blocks_of(2, 4);
   k_lp_small_end<5, 8><<<retry_blocks + blocks_of(64, 16), 64, 0, s>>>(
       c, x, y, list, list_count, pending, retry_list2, small, retry_blocks, cols, f, fii, status, fail_list, ds, nu_dt,
-      dt_dev, nu);
+      dt_dev, nu, most);
   note_launch();
   return cudaGetLastError();
 }

@@ -51,3 +51,27 @@ def test_noisy_lattices(lib, orc, inv_h, holes, bits, fallback):
         assert torch.equal(got[0][key], got[1][key]), key
     a, b = ({k: v for k, v in g["stats"].items() if k != "lp_small_rechecked"} for g in got)
     assert a == b
+
+
+@pytest.mark.parametrize("bits,rechecked", [(2, (1, 6144)), (26, (6145, 10 ** 9)), (52, (6145, 10 ** 9))])
+def test_short_and_long_lists_of_mid_sized_clouds(lib, orc, bits, rechecked):
+    # above the small clouds' size: the hand-backs in pairs or, past 6144 of them, in FP64
+    h = 1.0 / 140
+    x, y = vrm_inputs.lattice(h)
+    rng = np.random.default_rng(bits)
+    n = len(x)
+    assert 65536 < n < 6 * 65536
+    x = x + rng.uniform(-1, 1, n) * h * 2.0 ** -bits
+    y = y + rng.uniform(-1, 1, n) * h * 2.0 ** -bits
+    nb = orc.neighbours(x, y, h)
+    nbt = dict(count=cu(nb["count"]), idx=cu(nb["idx"].reshape(-1)), small=cu(nb["small"].reshape(-1)))
+    got = []
+    for k in (0, 1):
+        ctx = lib.VRM(h=h, nu=1e-3)
+        ctx.set_schedule(dict(ctx.get_schedule(), lp_fp64_pivots=k))
+        got.append(ctx.solve_weights(cu(x), cu(y), n, cu(np.ones(n, np.uint8)), nbt))
+    assert rechecked[0] <= got[0]["stats"]["lp_small_rechecked"] <= rechecked[1]
+    for key in ("status", "cols", "f", "fii"):
+        assert torch.equal(got[0][key], got[1][key]), key
+    a, b = ({k: v for k, v in g["stats"].items() if k != "lp_small_rechecked"} for g in got)
+    assert a == b
