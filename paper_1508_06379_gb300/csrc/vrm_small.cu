@@ -9,12 +9,12 @@
 // Bound by latency and, from some ten thousand particles on, by the one SM's
 // issue: 870 particles take 13 us, 20,449 43 us and 32,041 80 us, the ten
 // kernels of the front 75 us either way.  k_front_small_cluster shares the
-// particles out to the eight blocks of a cluster: each takes
-// its own into its shared memory and sums their digits, the blocks exchange
-// digit sums, candidates and counts through distributed shared memory, and every
-// block takes the same decisions; its six cluster barriers make it slower for
-// few particles.  The open list and the rounds' state take 5 and 11 us against
-// 17.
+// particles out to the eight blocks of a cluster: each takes its own into its
+// shared memory and sums their digits, the blocks exchange digit sums,
+// candidates and counts through distributed shared memory, and every block
+// takes the same decisions (20,449 particles: 25 us); its seven cluster
+// barriers make it slower for few particles.  The open list and the rounds'
+// state take 5 and 12 us against 17.
 #include <cooperative_groups.h>
 
 #include "vrm_internal.cuh"
