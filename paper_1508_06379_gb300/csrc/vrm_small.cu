@@ -25,10 +25,13 @@ namespace {
 
 constexpr int kFsThreads = 1024;
 constexpr int kFsWarps = kFsThreads / 32;
-// keys kept in shared memory: as many as fit, further ones are read again; in
-// a cluster all of them
+// From this capacity on the front takes a cluster: steps of 3,600 particles
+// (8,224 of capacity) 221 us in one block and 229 in a cluster, of 10,000
+// (21,024) 228 and 222, of 20,449 302 and 281, of 32,041 377 and 327.
+constexpr int kFsClusterCap = 16384;
+// a block's keys, kept in shared memory
 template <int C>
-constexpr int kFsKeys = C == 1 ? 21504 : kSmallCap / C;
+constexpr int kFsKeys = C == 1 ? kFsClusterCap : kSmallCap / C;
 // The first selection takes the keys' top 16 bits (sixteenths of a binade)
 // below those of the largest key: q is 0 more than 96 binades below it.
 constexpr int kFsBins = 97 * 16;
@@ -215,11 +218,7 @@ __device__ __forceinline__ void front_small_block(const FrontSmallArgs& a) {
   // are shifted by its number, which spreads those lanes over the banks.
   const int chunk = (n + kFsThreads - 1) / kFsThreads;
   const int seg = 32 * chunk;
-  auto key_of = [&](int i, int sg) {
-    if (C > 1 || i < kFsKeys<C>) return s_key[i + sg];
-    const unsigned long long b = (unsigned long long)__double_as_longlong(a.gamma[i]) & 0x7FFFFFFFFFFFFFFFull;
-    return b < 0x7FF0000000000000ull ? b : 0ull;
-  };
+  auto key_of = [&](int i, int sg) { return s_key[i + sg]; };
 
   // keys, their maximum, the bounding box (ordered bit patterns)
   unsigned long long amax = 0, mnx = ~0ull, mxx = 0, mny = ~0ull, mxy = 0;
@@ -232,7 +231,7 @@ __device__ __forceinline__ void front_small_block(const FrontSmallArgs& a) {
       flags |= 1;
       b = 0;
     }
-    if (C > 1 || i < kFsKeys<C>) s_key[i + i / seg] = b;
+    s_key[i + i / seg] = b;
     amax = b > amax ? b : amax;
     // (exponent bits: a test in FP64 would take the one SM's FP64 pipe 10 us for
     // 20,449 particles)
@@ -619,11 +618,6 @@ __global__ void __launch_bounds__(kFsThreads) k_open_small(const int* __restrict
 }
 
 }  // namespace
-
-// From this capacity on the front takes a cluster: steps of 3,600 particles
-// (8,224 of capacity) 221 us in one block and 229 in a cluster, of 10,000
-// (21,024) 228 and 222, of 20,449 302 and 281, of 32,041 377 and 327.
-constexpr int kFsClusterCap = 16384;
 
 cudaError_t front_small(const double* gamma, const double* x, const double* y, int cap, const int* n_dev,
                         double c_bound, double Rh, double lo2, double hi2, int ncell_cap, uint8_t* diffused,
