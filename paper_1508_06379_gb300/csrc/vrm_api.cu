@@ -1016,7 +1016,7 @@ vrm_status vrm_remove_close(vrm_ctx* ctx, const double* x, const double* y, cons
   VRM_CUDA(lp_identity(c, x, y, ctx->rm_clist, s.counters + 3, n, s.small, ctx->rm_removed, ctx->rm_cols4, ctx->rm_w4,
                        stream));
   // (the rows are not needed here: their buffers hold the lists)
-  VRM_CUDA(remove_apply(ctx->rm_clist, s.counters + 3, n, gamma, ctx->rm_removed, ctx->rm_cols4, ctx->rm_w4, s.pos,
+  VRM_CUDA(remove_apply(c, ctx->rm_clist, s.counters + 3, n, gamma, ctx->rm_removed, ctx->rm_cols4, ctx->rm_w4, s.pos,
                         s.nbr_idx, ctx->rm_gnew, ctx->rm_keep, s.ds, stream));
   VRM_CUDA(compact_flags(ctx->rm_keep, n, ctx->rm_klist, s.counters + 4, s.pos, s.scan_tmp, stream));
   VRM_CUDA(remove_out(n, s.counters + 4, ctx->rm_klist, x, y, ctx->rm_gnew, x_out, y_out, gamma_out, stream));

@@ -588,10 +588,10 @@ cudaError_t remove_close_flags(const Consts& c, const Grid* g, const int* cell_s
                                const float2* sorted_loc, const int* sorted_idx, int n, const double* gamma,
                                uint8_t* close, DevStats* ds, cudaStream_t s);
 // The removed particles' circulation moved to their targets through lists of
-// entries (head[n], next[4 n]: scratch).
-cudaError_t remove_apply(const int* clist, const int* n_cand, int n, const double* gamma, const uint8_t* removed,
-                         const int* cols4, const double* w4, int* head, int* next, double* gnew, uint8_t* keep,
-                         DevStats* ds, cudaStream_t s);
+// entries (head[n], next[4 n]: scratch), of at most k_cap entries each.
+cudaError_t remove_apply(const Consts& c, const int* clist, const int* n_cand, int n, const double* gamma,
+                         const uint8_t* removed, const int* cols4, const double* w4, int* head, int* next,
+                         double* gnew, uint8_t* keep, DevStats* ds, cudaStream_t s);
 cudaError_t remove_out(int n, const int* n_keep, const int* klist, const double* x, const double* y,
                        const double* gnew, double* x_out, double* y_out, double* g_out, cudaStream_t s);
 

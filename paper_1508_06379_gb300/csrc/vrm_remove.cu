@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kBlock) k_remove_link(const int* __restrict__ 
   }
 }
 
-__global__ void __launch_bounds__(kBlock) k_remove_apply(int n, const double* __restrict__ gamma,
+__global__ void __launch_bounds__(kBlock) k_remove_apply(int n, int k_cap, const double* __restrict__ gamma,
                                                          const uint8_t* __restrict__ removed,
                                                          const double* __restrict__ w4, const int* __restrict__ head,
                                                          const int* __restrict__ next, double* __restrict__ gnew,
@@ -121,17 +121,21 @@ __global__ void __launch_bounds__(kBlock) k_remove_apply(int n, const double* __
     keep[j] = gone ? 0 : 1;
     if (gone) continue;
     // the list's entries in ascending order (the sources differ, so that is
-    // the sources' order): the smallest one above the last, a few times
+    // the sources' order): the smallest one above the last, a few times.  The
+    // sources are neighbours of j, so a list beyond k_cap belongs to a call that
+    // ends in the capacity error: it is left alone at its k_cap-th entry (a spot
+    // of 20,000 particles puts most of them in one list, 4e8 dependent loads of
+    // one thread)
     double acc = gj;
     const int first = head[j];
     if (first >= 0 && next[first] < 0) {  // one entry: most targets that have any
       acc = __dadd_rn(acc, __dmul_rn(w4[first], gamma[first >> 2]));
     } else {
       for (int last = -1; first >= 0;) {
-        int best = INT_MAX;
-        for (int e = first; e >= 0; e = next[e])
+        int best = INT_MAX, seen = 0;
+        for (int e = first; e >= 0 && seen <= k_cap; e = next[e], ++seen)
           if (e > last && e < best) best = e;
-        if (best == INT_MAX) break;
+        if (best == INT_MAX || seen > k_cap) break;
         acc = __dadd_rn(acc, __dmul_rn(w4[best], gamma[best >> 2]));
         last = best;
       }
@@ -170,15 +174,15 @@ cudaError_t remove_close_flags(const Consts& c, const Grid* g, const int* cell_s
   return cudaGetLastError();
 }
 
-cudaError_t remove_apply(const int* clist, const int* n_cand, int n, const double* gamma, const uint8_t* removed,
-                         const int* cols4, const double* w4, int* head, int* next, double* gnew, uint8_t* keep,
-                         DevStats* ds, cudaStream_t s) {
+cudaError_t remove_apply(const Consts& c, const int* clist, const int* n_cand, int n, const double* gamma,
+                         const uint8_t* removed, const int* cols4, const double* w4, int* head, int* next,
+                         double* gnew, uint8_t* keep, DevStats* ds, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const cudaError_t e = cudaMemsetAsync(head, 0xFF, sizeof(int) * (size_t)n, s);
   if (e != cudaSuccess) return e;
   k_remove_link<<<blocks_for(n), kBlock, 0, s>>>(clist, n_cand, removed, cols4, head, next);
   note_launch();
-  k_remove_apply<<<blocks_for(n), kBlock, 0, s>>>(n, gamma, removed, w4, head, next, gnew, keep, ds);
+  k_remove_apply<<<blocks_for(n), kBlock, 0, s>>>(n, c.k_cap, gamma, removed, w4, head, next, gnew, keep, ds);
   note_launch();
   return cudaGetLastError();
 }
