@@ -31,6 +31,7 @@
 
 #include "vrm_internal.cuh"
 #include "vrm_mlp.cuh"
+#include "vrm_smem.cuh"
 #include "vrm_umma.cuh"
 
 using namespace vrm;
@@ -1163,12 +1164,8 @@ bool mlp_input_map(CUtensorMap* m, const bf16* X, int rows_pad) { return make_ma
 cudaError_t mlp_forward(vrm_mlp* net, const CUtensorMap& mX, int rows, const int* rows_dev, float* Y,
                         cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t r = cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
-    if (r != cudaSuccess) return r;
-    attr_set = true;
-  }
+  const cudaError_t r = allow_smem<k_mlp_fused>(kFusedSmem);
+  if (r != cudaSuccess) return r;
   const int ntiles = (rows + 2 * kBM - 1) / (2 * kBM), npair = sm_count() / 2;
   const int grid = 2 * (ntiles < npair ? ntiles : npair);
   FusedArgs fa;
@@ -1205,14 +1202,9 @@ cudaError_t zalloc(T** p, size_t count) {
 // Forward and backward pass of the current batch (Xb, Xbt, Tb) up to the
 // partial weight gradients.
 cudaError_t forward_backward(vrm_mlp* n, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t r = cudaFuncSetAttribute(k_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem);
-    if (r == cudaSuccess)
-      r = cudaFuncSetAttribute(k_weight_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
-    if (r != cudaSuccess) return r;
-    attr_set = true;
-  }
+  cudaError_t r = allow_smem<k_chain>(kChainSmem);
+  if (r == cudaSuccess) r = allow_smem<k_weight_grad>(kWgSmem);
+  if (r != cudaSuccess) return r;
   ChainArgs a;
   a.theta = n->theta;
   a.Xb = n->Xb;

@@ -27,6 +27,7 @@
 #include <climits>
 
 #include "vrm_internal.cuh"
+#include "vrm_smem.cuh"
 
 namespace vrm {
 
@@ -566,16 +567,20 @@ cudaError_t search_all(const Consts& c, const Grid* g, const int* cell_start, co
   if (n <= 0) return cudaSuccess;
   const int tb = c.search_block;
   const int blocks = (int)(((long)n + tb - 1) / tb);
-  const auto kernel = c.row_cap <= 16   ? k_search_all<16>
-                      : c.row_cap <= 24 ? k_search_all<24>
-                                        : k_search_all<VRM_KCAP_MAX>;
-  const size_t smem = search_smem(tb, c.row_cap <= 16 ? 16 : c.row_cap <= 24 ? 24 : VRM_KCAP_MAX);
-  if (smem > 40 * 1024) {  // (beside the static part, more than a launch may ask for without this)
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  kernel<<<blocks, tb, smem, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, n, nullptr, nbr_count, nbr_idx,
-                                  seg_mask, small, ds, nullptr, nullptr, nullptr, nullptr);
+#define VRM_SEARCH_LAUNCH(K)                                                                                      \
+  do {                                                                                                            \
+    const cudaError_t e = allow_smem<k_search_all<K>>(search_smem(kBlock, K));                                    \
+    if (e != cudaSuccess) return e;                                                                               \
+    k_search_all<K><<<blocks, tb, search_smem(tb, K), s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, n, \
+                                                           nullptr, nbr_count, nbr_idx, seg_mask, small, ds);     \
+  } while (0)
+  if (c.row_cap <= 16)
+    VRM_SEARCH_LAUNCH(16);
+  else if (c.row_cap <= 24)
+    VRM_SEARCH_LAUNCH(24);
+  else
+    VRM_SEARCH_LAUNCH(VRM_KCAP_MAX);
+#undef VRM_SEARCH_LAUNCH
   note_launch();
   return cudaGetLastError();
 }

@@ -18,6 +18,7 @@
 #include <cooperative_groups.h>
 
 #include "vrm_internal.cuh"
+#include "vrm_smem.cuh"
 
 namespace vrm {
 
@@ -623,22 +624,16 @@ cudaError_t front_small(const double* gamma, const double* x, const double* y, i
                         double c_bound, double Rh, double lo2, double hi2, int ncell_cap, uint8_t* diffused,
                         int* dlist, int* dcount, DevStats* ds, Grid* g, int* cell_count, int* cell_ts,
                         cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_front_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFsSmem<1>);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_front_small_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kFsSmem<kFsCluster>);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
   const FrontSmallArgs a{gamma, x, y, cap, n_dev, c_bound, Rh, lo2, hi2, ncell_cap, diffused, dlist, dcount, ds, g,
                          cell_count, cell_ts};
-  if (cap >= kFsClusterCap)
+  cudaError_t e;
+  if (cap >= kFsClusterCap) {
+    if ((e = allow_smem<k_front_small_cluster>(kFsSmem<kFsCluster>)) != cudaSuccess) return e;
     k_front_small_cluster<<<kFsCluster, kFsThreads, kFsSmem<kFsCluster>, s>>>(a);
-  else
+  } else {
+    if ((e = allow_smem<k_front_small>(kFsSmem<1>)) != cudaSuccess) return e;
     k_front_small<<<1, kFsThreads, kFsSmem<1>, s>>>(a);
+  }
   note_launch();
   return cudaGetLastError();
 }
