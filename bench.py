@@ -403,7 +403,7 @@ def run_ours(args):
     dom = max(mean_stage, key=mean_stage.get)
     sch = ctx.get_schedule()
     roofline = (roofline_for(dom, mean_stage[dom], stats, n, desc["order"], sch["lp_fp64_pivots"], peaks,
-                             sch["lp_block"], rows=bool(getattr(args, "learned", False)))
+                             lp_block_run(sch, xb.numel()), rows=bool(getattr(args, "learned", False)))
                 if mean_stage[dom] > 0 else None)
     learned = None
     if args.workload == "mixture_1m" and not args.no_learned and world == 1:
@@ -587,6 +587,12 @@ def binding_for(kernel):
         return ent.get("binding")
     except Exception:
         return None
+
+
+def lp_block_run(sch, cap):
+    """lp_block of the form that the small LPs of a cloud by itself run in: the default pair leaves it to the capacity."""
+    by_capacity = sch["lp_block"] == 128 and sch["lp_blocks_per_sm"] == 16 and cap >= 18 * 65536
+    return 384 if by_capacity else sch["lp_block"]
 
 
 def roofline_for(stage, ms, stats, n, order=1, lp_fp64_pivots=1, peaks=None, lp_block=128, rows=False):

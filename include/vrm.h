@@ -126,7 +126,7 @@ typedef struct vrm_stats {
   int64_t learned_screens; /* five-slot supports screened by the learned path (binary32 solves) */
   int64_t remove_candidates; /* vrm_remove_close: particles closer than r h to one of larger key */
   int64_t lp_small_rechecked; /* of lp_small_solved: LPs whose binary32 pivot decisions (of pairs of
-                                 binary32 numbers in calls of at most 65,536 capacity) were not all
+                                 binary32 numbers where each particle has eight lanes) were not all
                                  certain and that were re-run with FP64 pivots (same result either way) */
 } vrm_stats;
 
@@ -311,17 +311,25 @@ typedef struct vrm_batch vrm_batch;
  *                     up to k_cap (32 by default).  A step whose rows need
  *                     more than row_cap but at most k_cap is repeated once
  *                     with row_cap = k_cap, which the context then keeps.
- *   search_block:     threads per block of the neighbourhood search (32..256, multiple of 32).
+ *   search_block:     threads per block of the neighbourhood search (32..256, multiple of 32), a particle per
+ *                     thread; 256 (default): capacities of at most 65,536 give each particle a warp instead
+ *                     (where no rows are written: n = 1 without a network).
  *   lp_block:         threads per block of the small-neighbourhood LP, one particle per thread (32..128, multiple of 32);
  *                     192 and 384 select the warp-specialised form of the binary32 LP (4 pivot and 2 FP64 warps
  *                     per block, two blocks per SM; 8 pivot and 4 FP64 warps, one block per SM).
  *   lp_blocks_per_sm: the small LP's grid is capped at this many blocks per SM (1..64).
+ *                     lp_block = 128 with lp_blocks_per_sm = 16 (default) leaves the binary32 LP's form to
+ *                     the capacity: eight lanes per particle up to 65,536, the 384 form from 1,179,648 on
+ *                     (not in a batch, where the clouds' capacities add up for the first line), else one
+ *                     particle per thread.  Any other pair holds at every capacity.  n = 2 has one form of
+ *                     its own and uses neither field.
  *   apply_block:      threads per block of the application (32..256, multiple of 32).
  *   lp_fp64_pivots:   0 (default): the small-neighbourhood LPs (n = 1) pivot
  *                     in binary32 with certified decisions, and the few whose
  *                     decisions are not all certain are re-run with FP64
  *                     pivots; 1: every LP pivots in FP64.  The final basis,
  *                     hence every weight, is the same bit for bit.
+ * Setting what vrm_get_schedule answered changes nothing.
  * Setting a schedule drops any captured step graph; VRM_ERR_ARG if a field
  * is out of range.
  */

@@ -23,7 +23,9 @@ Every candidate's output (positions and Gamma after the step) is checked to
 be bit-identical to the default schedule's; a difference is an error.
 Results are cached as JSON per device, k_cap, consistency order and size
 bucket (nearest power of two of the particle count); batches take the
-schedule of each cloud's bucket.
+schedule of each cloud's bucket.  Files without a "version" are older than the
+forms that small clouds choose by themselves: the launch options of their small
+buckets, which were timed against other kernels, go back to the defaults.
 """
 import json
 import math
@@ -38,6 +40,10 @@ GROUPS = (
     ("lp_small", [dict(lp_fp64_pivots=v) for v in (0, 1)]),
     ("apply", [dict(apply_block=b) for b in (64, 128, 256)]),
 )
+# groups of n = 2, whose LP has one launch
+GROUPS_N2 = tuple(g for g in GROUPS if "lp_block" not in g[1][0])
+VERSION = 2
+SMALL_BUCKET = 16  # buckets up to this one hold the clouds of at most 65,536 of capacity
 
 
 def bucket(n):
@@ -118,7 +124,8 @@ def tune_context(ctx, x, y, n, gamma_in, gamma_out, dt, reps=5):
         return {k: statistics.median(v) for k, v in per_stage.items()}, same
 
     try:
-        best, report = descend(measure, ctx.k_cap, max_count)
+        groups = GROUPS_N2 if getattr(ctx, "order", 1) == 2 else GROUPS
+        best, report = descend(measure, ctx.k_cap, max_count, groups=groups)
     finally:
         ctx.set_timing(False)
     ctx.set_schedule(best)
@@ -138,11 +145,17 @@ class Autotuner:
                 self.table = json.load(open(self.path))
             except (OSError, ValueError):
                 self.table = {}
+            if self.table and "version" not in self.table:
+                for key, s in self.table.items():
+                    b = key.rsplit("^", 1)[-1]
+                    if b.isdigit() and int(b) <= SMALL_BUCKET and isinstance(s, dict):
+                        s.update({f: DEFAULT[f] for f in ("search_block", "lp_block", "lp_blocks_per_sm")})
 
     def save(self):
         d = os.path.dirname(self.path)
         if d:
             os.makedirs(d, exist_ok=True)
+        self.table["version"] = VERSION
         tmp = self.path + ".tmp"
         with open(tmp, "w") as f:
             json.dump(self.table, f, indent=1, sort_keys=True)

@@ -643,7 +643,6 @@ void put_schedule(Consts& c, const vrm_schedule& s) {
   c.row_cap = s.row_cap;
   c.search_block = s.search_block;
   c.lp_block = s.lp_block;
-  c.lp_auto = 0;
   c.lp_blocks_per_sm = s.lp_blocks_per_sm;
   c.lp_fp64_pivots = s.lp_fp64_pivots;
   c.apply_block = s.apply_block;

@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include "../../include/vrm.h"
+#include "vrm_schedule.cuh"
 
 namespace vrm {
 
@@ -39,7 +40,6 @@ struct Consts {
   int row_cap;           // neighbour entries kept per row (<= k_cap)
   int search_block;      // threads per block of k_search_all
   int lp_block;          // threads per block of k_lp_small
-  int lp_auto;           // 1: no schedule was set, the LP's form follows the capacity
   int lp_blocks_per_sm;  // grid cap of k_lp_small
   int lp_fp64_pivots;    // 1: small LPs pivot in FP64; 0: certified binary32 pivots, FP64 re-runs
   int apply_block;       // threads per block of k_apply
@@ -47,22 +47,15 @@ struct Consts {
   int load;
 };
 
-// Largest capacity (of all clouds that run at the same time) whose cell scans
-// give a warp to each particle or proposal instead of a thread: at 870
-// particles a thread's chain of dependent loads over nine cells takes 33 us in
-// the neighbourhood search and in the masks (7 and 9 by warps), 17 in the mask
-// update (10) and 8 in the conflict test (5); at 20,449 34, 14, 21 and 11
-// against 20, 11, 21 and 7.
-constexpr int kWarpScanCap = 65536;
+// The cell scans of the masks and the insertion rounds, which no schedule names.
 inline bool warp_scans(const Consts& c, int cap) { return (c.load > cap ? c.load : cap) <= kWarpScanCap; }
 
 // The schedule every context starts with.
 inline void default_schedule(Consts& c) {
   c.row_cap = c.k_cap;
-  c.search_block = 256;
-  c.lp_block = 128;
-  c.lp_auto = 1;
-  c.lp_blocks_per_sm = 16;
+  c.search_block = kSearchBlockDefault;
+  c.lp_block = kLpBlockDefault;
+  c.lp_blocks_per_sm = kLpBlocksPerSmDefault;
   c.lp_fp64_pivots = 0;
   c.apply_block = 256;
 }

@@ -1066,8 +1066,7 @@ __global__ void __launch_bounds__(128, 3) k_lp_small32(Consts c, const double* _
 // with one block per SM (the same 12 warps per SM at 168 registers; the
 // wider block is 6% faster on the 1M-particle workload).
 // ---------------------------------------------------------------------------
-constexpr int kLpWsThreads = 32 * (4 + 2);
-constexpr int kLpWsThreadsWide = 32 * (8 + 4);
+static_assert(kLpWsThreads == 32 * (4 + 2) && kLpWsThreadsWide == 32 * (8 + 4), "warps of the two forms");
 
 // Hand-over of the warp-specialised LP: kWsSlots buffers, and per buffer two
 // named barriers over every thread of the block.  FULL (1 + slot): the pivot
@@ -2449,34 +2448,13 @@ static cudaError_t lp_finish_list(const Consts& c, const double* x, const double
   return cudaGetLastError();
 }
 
-// Largest particle capacities whose n = 1 LPs all go to the pairs kernel, eight
-// lanes per LP, and whose hand-backs do.  One LP per thread takes 32 us in
-// binary32 and 43 for the re-run of a few in FP64 however few they are, the
-// pairs and their solves 35 for all; but they take seven times the
-// instructions.  Steps of 3,600, 20,449 and 32,400 particles: 290, 323 and 386
-// us with all LPs in pairs, 346, 371 and 409 with binary32 and FP64 (65,536:
-// 435 and 446, 90,000: 511 and 483).  Hand-backs in pairs: 423, 474, 509 and
-// 578 us at 65,536, 90,000, 129,600 and 184,900 particles against 446, 483,
-// 531 and 582, but 1,675 against 1,664 at a million.  The capacity is what the
-// host knows; twice the particles is usual.  The clouds of a batch run at the
-// same time, so the sum of their capacities counts there (32 clouds of 10,000
-// to 300,000 particles: 4.49 ms, 4.60 when each went by its own).
-constexpr int kPairsCap = 65536;
-constexpr int kPairsRetryCap = 6 * 65536;
-// The longest list of hand-backs that goes to the pairs in that range, decided
+// The longest list of hand-backs that goes to the pairs up to kPairsRetryCap, decided
 // on the device (the other form's launch returns at once).  Jittered clouds
 // hand back 2%, lattices a quarter to all of their LPs, many of which the pairs
 // cannot certify either: steps of a lattice of 53,000 particles with 18,229
 // hand-backs 396 us in FP64 and 536 in pairs, of a jittered cloud of 184,900
 // with 4,177 605 and 590, RK3 steps with 5,000 a stage 1,083 and 1,037.
 constexpr int kPairsRetries = 6144;
-// Smallest capacity that takes the 8 + 4-warp form where no schedule was set:
-// steps of 640,000 particles 1,075 us against 1,114 with one kind of warp, of a
-// million 1,469 against 1,581; 787 and 797 at 360,000.  The form fills every SM,
-// so batches, whose clouds run beside each other, keep the other (4.54 ms
-// against 4.66), as do capacities that may hold fewer LPs than this (an RK3
-// step of 500,000 in 730,000: 2.41 against 2.47 ms).
-constexpr int kWsCap = 18 * 65536;
 
 cudaError_t lp_small(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
                      int cap, const int* small, int* cols, double* f, double* fii, uint8_t* status, int* fail_list,
@@ -2503,16 +2481,16 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
     note_launch();
     return cudaGetLastError();
   }
+  const LpForm form = small_lp_form(c.lp_block, c.lp_blocks_per_sm, cap, c.load);
   const int load = c.load > cap ? c.load : cap;
   int most = INT_MAX;  // the pairs take no longer lists
-  if (load > kPairsCap) {
+  if (form != kLpPairs) {
     // certified binary32 pivots, then the uncertain particles in pairs or in FP64
-    const int form = c.lp_auto && c.load == 0 && cap >= kWsCap ? kLpWsThreadsWide : c.lp_block;
-    if (form == kLpWsThreads) {
+    if (form == kLpWs) {
       // warp-specialised form, 4 + 2 warps: two resident blocks per SM
       k_lp_small32_ws<5, 8, 4, 2, 2><<<2 * sm_count(), kLpWsThreads, 0, s>>>(
           c, x, y, list, list_count, small, cols, f, fii, status, fail_list, retry_list, ds, nu_dt, dt_dev, nu);
-    } else if (form == kLpWsThreadsWide) {
+    } else if (form == kLpWsWide) {
       // 8 + 4 warps: one resident block per SM
       k_lp_small32_ws<5, 8, 8, 4, 1><<<sm_count(), kLpWsThreadsWide, 0, s>>>(
           c, x, y, list, list_count, small, cols, f, fii, status, fail_list, retry_list, ds, nu_dt, dt_dev, nu);
@@ -2540,7 +2518,7 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
     return (int)(b < per_sm * sms ? b : per_sm * sms);
   };
   k_lp_df<5, 8, false><<<blocks_of(16, 16), 128, 0, s>>>(c, x, y, list, list_count, nullptr, nullptr, small, cols,
-                                                         retry_list2, pending, ds, load <= kPairsCap, most);
+                                                         retry_list2, pending, ds, form == kLpPairs, most);
   note_launch();
   const int retry_blocks = blocks_of(2, 4);
   k_lp_small_end<5, 8><<<retry_blocks + blocks_of(64, 16), 64, 0, s>>>(

@@ -591,7 +591,7 @@ cudaError_t search_list_dev(const Consts& c, const Grid* g, const int* cell_star
                             int* nbr_count, int* nbr_idx, uint8_t* seg_mask, int* small, DevStats* ds,
                             cudaStream_t s, bool rows, const uint8_t* skip) {
   if (m_bound <= 0) return cudaSuccess;
-  if (!rows && !skip && warp_scans(c, m_bound)) {
+  if (!rows && !skip && search_by_warps(c.search_block, m_bound, c.load)) {
     k_search_warp<<<warp_grid(m_bound), 128, 0, s>>>(c, g, cell_start, sorted_xy, sorted_loc, sorted_idx, list,
                                                      list_count, cell_key, cell_rank, nbr_count, seg_mask, small, ds);
     note_launch();

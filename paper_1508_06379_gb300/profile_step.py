@@ -42,7 +42,8 @@ def main(argv=None):
     gi = torch.from_numpy(g).cuda()
     go = torch.zeros_like(xb)
     ctx = vrm.VRM(h=h, nu=nu)
-    per_sm = {384: 1, 192: 2}.get(a.lp_block, autotune.DEFAULT["lp_blocks_per_sm"])
+    # (128 x 16 would leave the form to the capacity)
+    per_sm = {384: 1, 192: 2, 128: 17}.get(a.lp_block, autotune.DEFAULT["lp_blocks_per_sm"])
     ctx.set_schedule(dict(autotune.DEFAULT, lp_block=a.lp_block, lp_blocks_per_sm=per_sm))
     n2, st = n, {}
     for _ in range(a.steps):
