@@ -49,6 +49,14 @@ constexpr int kBK = 64;       // K per slab
 constexpr long long kWaitCycles = 2000000000LL;  // about one second
 constexpr long long kDrainCycles = 4000000LL;    // about 2 ms
 
+// Copies that nothing waited for (after a wait that gave up) arrive before the
+// CTA ends.
+__device__ __forceinline__ void wait_for_copies() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < kDrainCycles) {
+  }
+}
+
 constexpr long kOffW1 = 0, kOffB1 = kOffW1 + (long)kHid * kIn;
 constexpr long kOffW2 = kOffB1 + kHid, kOffB2 = kOffW2 + (long)kHid * kHid;
 constexpr long kOffW3 = kOffB2 + kHid, kOffB3 = kOffW3 + (long)kHid * kHid;
@@ -125,9 +133,10 @@ __device__ __forceinline__ f32x2 gelu_grad2(f32x2 z) {
 // per 128-row tile: issue 4,600 -> 1,100 with an elected thread (a branch on
 // the lane makes every MMA wait for its operands to move to uniform
 // registers); the pair halves what shared memory takes in and L2 gives out per
-// MMA, 448 KB a tile before.  The arrivals keep their default scope: the
-// activations cross to the async proxy by the proxy fence before them, and an
-// arrival released at cluster scope waits for all the CTA's stores (300 us).
+// MMA, 448 KB a tile before.  The arrivals keep their default scope (CTA):
+// what orders the activations, which only MMAs read, is the proxy fence before
+// the arrival and not its release, and one released at cluster scope waits for
+// all the CTA's stores (300 us).
 // What bounds it now: of a tile's 11,000 clocks the epilogues take 9,000, three
 // times about 3,000, at 1,600 of the FMA pipe (six operations a value) and
 // 2,400 of shared memory (64 KB of A, 64 KB of the half weight slabs read, 64 KB
@@ -332,9 +341,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFusedThreads, 1)
         }
       }
       if (fail) *abort_flag = 1;
-      // every MMA issued completes before the TMEM is released
-      umma::mma_commit_pair(drain);
-      if (!umma::mbar_wait(drain, 0u, kWaitCycles)) *abort_flag = 1;
+      umma::mma_commit_pair(drain);  // (after a failure too)
     }
   } else {
     // ---- epilogue warps ----
@@ -412,14 +419,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFusedThreads, 1)
   __syncwarp();
   umma::fence_before_sync();
   __syncthreads();
+  // Every MMA issued completes before the TMEM is released, and every commit
+  // arrives in this CTA before it ends: the leading CTA sees its own arrivals,
+  // not its peer's, so each waits for those it gets.  (The producers have waited
+  // for all commits of a ring stage or slot but the last one, so its parity
+  // cannot be that of an earlier one; accf is waited for by the epilogues.)
+  if (threadIdx.x == 0) {
+    bool ok = umma::mbar_wait(drain, 0u, 2 * kWaitCycles);
+    if (ok && !*abort_flag) {
+      for (int st = 0; st < kRing && st < total; ++st)
+        ok = ok && umma::mbar_wait(&wempty[st], (uint32_t)((total - 1 - st) / kRing) & 1u, kWaitCycles);
+      for (int s = 0; s < 2 && s < my_tiles; ++s)
+        ok = ok && umma::mbar_wait(&hfree[s], (uint32_t)((my_tiles - 1 - s) / 2) & 1u, kWaitCycles);
+    }
+    if (!ok) *abort_flag = 1;
+  }
+  __syncthreads();
   if (*abort_flag) {
     if (threadIdx.x == 0 && a.error) atomicExch(a.error, 1);
-    // copies that nothing waited for arrive before the CTA ends
-    const long long t0 = clock64();
-    while (clock64() - t0 < kDrainCycles) {
-    }
+    wait_for_copies();
   }
-  umma::cluster_sync();  // no MMA, copy or arrival of the peer is under way
+  umma::cluster_sync();  // the peer is as far: nothing it sent here is under way
   if (warp == 0) {
     umma::fence_after_sync();
     umma::tmem_dealloc_pair(tmem, 512);
@@ -642,7 +662,11 @@ __global__ void __launch_bounds__(kChainThreads, 1)
       }
       if (fail) *abort_flag = 1;
       umma::mma_commit(drain);
-      if (!umma::mbar_wait(drain, 0u, kWaitCycles)) *abort_flag = 1;
+      bool ok = umma::mbar_wait(drain, 0u, kWaitCycles);
+      // and the last commit of every ring stage
+      for (int st = 0; st < kChainRing && st < g && !fail; ++st)
+        ok = ok && umma::mbar_wait(&wempty[st], (uint32_t)((g - 1 - st) / kChainRing) & 1u, kWaitCycles);
+      if (!ok) *abort_flag = 1;
     }
   } else {
     const int q = warp & 3, cg = warp >> 2;
@@ -809,7 +833,10 @@ __global__ void __launch_bounds__(kChainThreads, 1)
   }
   umma::fence_before_sync();
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag && a.error) atomicExch(a.error, 1);
+  if (*abort_flag) {
+    if (threadIdx.x == 0 && a.error) atomicExch(a.error, 1);
+    wait_for_copies();
+  }
   if (warp == 0) {
     umma::fence_after_sync();
     umma::tmem_dealloc(tmem, 512);
@@ -892,6 +919,9 @@ __global__ void __launch_bounds__(128, 2)
       }
     }
     umma::mma_commit(done);
+    // the last commit of every stage
+    for (int s = 0; s < kWgStages && s < k_slabs; ++s)
+      ok = ok && umma::mbar_wait(&empty[s], (uint32_t)((k_slabs - 1 - s) / kWgStages) & 1u, kWaitCycles);
     if (!ok) s_fail = 1;
   }
   const bool got = umma::mbar_wait(done, 0, 2 * kWaitCycles);
@@ -899,6 +929,7 @@ __global__ void __launch_bounds__(128, 2)
   const bool failed = __syncthreads_or(!got || s_fail) != 0;  // uniform: the TMEM loads below are warp-wide
   if (failed) {
     if (threadIdx.x == 0 && error) atomicExch(error, 1);
+    wait_for_copies();
   } else if (layer < 3 || warp == 0) {
     float* const out = part + (size_t)blockIdx.x * kPartSplit + (size_t)piece * kHid * kBM + warp * 32 + lane;
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);

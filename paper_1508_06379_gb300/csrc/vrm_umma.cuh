@@ -156,7 +156,9 @@ __device__ __forceinline__ uint32_t lead_addr(const void* p) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
   return a;
 }
-// One arrival at a barrier of either CTA of the cluster.
+// One arrival at a barrier of either CTA of the cluster, of the default scope
+// (CTA): what the other CTA may use after it has to be ordered otherwise, as the
+// operands of its MMAs are by fence_proxy_async_smem.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
