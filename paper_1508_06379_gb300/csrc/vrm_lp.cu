@@ -1315,12 +1315,11 @@ __device__ __forceinline__ void lp_recorded(const int* row, int (&basis)[M], int
 // swaps, multipliers times the pivot's reciprocal, separately rounded
 // updates), forward substitution in column order, back substitution row by
 // row; the result is bit-identical to the oracle's basis solve.
-// For n = 2 (M = 9) and for the columns of small neighbourhoods (small given)
+// small: the columns are those of the small neighbourhoods.  For n = 2 (M = 9)
 // the kernel stops at the final basis and leaves it in the particle's stencil
 // row (lp_record), for k_lp_finish.
-// SMALL_END: the columns of small neighbourhoods, solved here all the same,
-// an infeasible LP queued for the full neighbourhoods (next_list) as the small
-// LPs' other kernels do.  warp of nwarps warps.
+// SMALL_END (n = 1): an infeasible LP is queued for the full neighbourhoods
+// (next_list) as the small LPs' other kernels do.  warp of nwarps warps.
 template <int M, int W, bool SMALL_END>
 __device__ __forceinline__ void lp_by_warps(const Consts& c, const double* __restrict__ x,
                                             const double* __restrict__ y, const int* __restrict__ fail_list,
@@ -1465,7 +1464,7 @@ __device__ __forceinline__ void lp_by_warps(const Consts& c, const double* __res
       if (lane == leave) bas = M + q;
       ++it;
     }
-    if (M == 9 || (!SMALL_END && small)) {
+    if (M == 9) {
       const int bj = __shfl_sync(kAll, j, bas >= M && bas != INT_MAX ? bas - M : 0);
       lp_record<M, 32>(cols + (size_t)i * W, lane, bas, bas >= M ? bj : -1, code, it);
       continue;
@@ -2170,7 +2169,7 @@ __device__ __forceinline__ void lp_finish_recorded(const Consts& c, const double
     }
   }
 }
-template <int M, bool FULL>
+template <bool FULL>
 __global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __restrict__ x,
                                                    const double* __restrict__ y, const int* __restrict__ list,
                                                    const int* __restrict__ list_count,
@@ -2180,7 +2179,7 @@ __global__ void __launch_bounds__(64) k_lp_finish(Consts c, const double* __rest
                                                    DevStats* __restrict__ ds, double nu_dt,
                                                    const double* __restrict__ dt_dev, double nu) {
   if (dt_dev) nu_dt = nu * *dt_dev;
-  lp_finish_recorded<M, FULL>(c, x, y, list, list_count, nullptr, nbr_count, cols, f, fii, status, fail_list, ds, nu_dt,
+  lp_finish_recorded<9, FULL>(c, x, y, list, list_count, nullptr, nbr_count, cols, f, fii, status, fail_list, ds, nu_dt,
                               blockIdx.x, gridDim.x);
 }
 
@@ -2406,44 +2405,32 @@ __global__ void k_lp_clear(int n, int w, bool vec, const uint8_t* __restrict__ d
   }
 }
 
-// The LPs of a list in pairs of binary32 numbers (small neighbourhoods, or
-// for n = 2 full ones: small null), the uncertain ones in FP64, then the final
-// solves.  fp64: every LP in FP64.  ds->n_retry_pairs is 0 on entry.
-template <int M>
-static cudaError_t lp_pairs(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
-                            int cap, const int* nbr_count, const int* nbr_idx, const int* small, int* cols, double* f,
-                            double* fii, uint8_t* status, int* fail_list, int* retry_list, DevStats* ds, double nu_dt,
-                            cudaStream_t s, const double* dt_dev, double nu, bool fp64, bool count_retries) {
-  constexpr int W = M == 9 ? VRM_STENCIL_W2 : VRM_STENCIL_W, G = M == 9 ? 16 : 8;
+// The n = 2 LPs of a list, on small neighbourhoods or (small null) on full ones:
+// pivots in pairs of binary32 numbers, the uncertain ones in FP64 (fp64: every
+// LP), then the final solves.  ds->n_retry_pairs is 0 on entry.
+template <bool FULL>
+static cudaError_t lp_order2(const Consts& c, const double* x, const double* y, const int* list, const int* list_count,
+                             int cap, const int* nbr_count, const int* nbr_idx, const int* small, int* cols, double* f,
+                             double* fii, uint8_t* status, int* fail_list, int* retry_list, DevStats* ds,
+                             double nu_dt, cudaStream_t s, const double* dt_dev, double nu) {
+  constexpr int G = FULL ? 32 : 16;
+  const bool fp64 = c.lp_fp64_pivots != 0;
   const int sms = sm_count();
   auto grid = [&](long per_block, int per_sm) {
     const long b = ((long)cap + per_block - 1) / per_block, most = (long)per_sm * sms;
     return (int)(b < most ? b : most);
   };
   if (!fp64) {
-    if (M == 5 || small)
-      k_lp_df<M, G, false><<<grid(128 / G, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small,
-                                                             cols, retry_list, nullptr, ds, count_retries, INT_MAX);
-    else
-      k_lp_df<9, 32, true><<<grid(4, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
-                                                       retry_list, nullptr, ds, false, INT_MAX);
+    k_lp_df<9, G, FULL><<<grid(128 / G, 16), 128, 0, s>>>(c, x, y, list, list_count, nbr_count, nbr_idx, small, cols,
+                                                          retry_list, nullptr, ds, false, INT_MAX);
     note_launch();
-    list = retry_list;
   }
-  const int* const all = list_count;
-  k_lp_full<M, W><<<grid(4, 4), 128, 0, s>>>(c, x, y, list, fp64 ? all : &ds->n_retry_pairs, nbr_count, nbr_idx, small,
-                                             cols, f, fii, status, ds, nu_dt, dt_dev, nu);
+  k_lp_full<9, VRM_STENCIL_W2><<<grid(4, 4), 128, 0, s>>>(c, x, y, fp64 ? list : retry_list,
+                                                          fp64 ? list_count : &ds->n_retry_pairs, nbr_count, nbr_idx,
+                                                          small, cols, f, fii, status, ds, nu_dt, dt_dev, nu);
   note_launch();
-  return cudaGetLastError();
-}
-template <int M, bool FULL>
-static cudaError_t lp_finish_list(const Consts& c, const double* x, const double* y, const int* list,
-                                  const int* list_count, int cap, const int* nbr_count, int* cols, double* f,
-                                  double* fii, uint8_t* status, int* fail_list, DevStats* ds, double nu_dt,
-                                  cudaStream_t s, const double* dt_dev, double nu) {
-  const long b = ((long)cap + 63) / 64, most = 16L * sm_count();
-  k_lp_finish<M, FULL><<<(int)(b < most ? b : most), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii,
-                                                                 status, fail_list, ds, nu_dt, dt_dev, nu);
+  k_lp_finish<FULL><<<grid(64, 16), 64, 0, s>>>(c, x, y, list, list_count, nbr_count, cols, f, fii, status, fail_list,
+                                                ds, nu_dt, dt_dev, nu);
   note_launch();
   return cudaGetLastError();
 }
@@ -2461,14 +2448,9 @@ cudaError_t lp_small(const Consts& c, const double* x, const double* y, const in
                      int* retry_list, int* retry_list2, uint8_t* pending, DevStats* ds, double nu_dt,
                      cudaStream_t s, const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
-  cudaError_t e;
-  if (c.order == 2) {
-    e = lp_pairs<9>(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list,
-                    retry_list2, ds, nu_dt, s, dt_dev, nu, c.lp_fp64_pivots != 0, false);
-    if (e != cudaSuccess) return e;
-    return lp_finish_list<9, false>(c, x, y, list, list_count, cap, nullptr, cols, f, fii, status, fail_list, ds,
-                                    nu_dt, s, dt_dev, nu);
-  }
+  if (c.order == 2)
+    return lp_order2<false>(c, x, y, list, list_count, cap, nullptr, nullptr, small, cols, f, fii, status, fail_list,
+                            retry_list2, ds, nu_dt, s, dt_dev, nu);
   // lp_block = kLpWsThreads or kLpWsThreadsWide selects the warp-specialised
   // binary32 LP; the other LP kernels then run with 128 threads per block
   const bool ws = c.lp_block == kLpWsThreads || c.lp_block == kLpWsThreadsWide;
@@ -2534,13 +2516,10 @@ cudaError_t lp_full(const Consts& c, const double* x, const double* y, const int
                     const double* dt_dev, double nu) {
   if (cap <= 0) return cudaSuccess;
   if (c.order == 2) {
-    cudaError_t e = cudaMemsetAsync(&ds->n_retry_pairs, 0, sizeof(int), s);
-    if (e == cudaSuccess)
-      e = lp_pairs<9>(c, x, y, fail_list, fail_count, cap, nbr_count, nbr_idx, nullptr, cols, f, fii, status, nullptr,
-                      retry_list2, ds, nu_dt, s, dt_dev, nu, c.lp_fp64_pivots != 0, false);
+    const cudaError_t e = cudaMemsetAsync(&ds->n_retry_pairs, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    return lp_finish_list<9, true>(c, x, y, fail_list, fail_count, cap, nbr_count, cols, f, fii, status, nullptr, ds,
-                                   nu_dt, s, dt_dev, nu);
+    return lp_order2<true>(c, x, y, fail_list, fail_count, cap, nbr_count, nbr_idx, nullptr, cols, f, fii, status,
+                           nullptr, retry_list2, ds, nu_dt, s, dt_dev, nu);
   }
   long warps = cap;
   long blocks = (warps * 32 + 127) / 128;
