@@ -484,7 +484,10 @@ typedef struct vrm_velocity {
  * u and v receive m values.  Pair terms in fp32 on hi/lo-split positions,
  * tile sums in FP64: relative error about 1e-6 of sum_j |Gamma_j K_eps|.
  * O(n m) work (the fast multipole method of the paper is not part of this
- * library).  Asynchronous.
+ * library).  The context keeps the tile sums' workspace until it is destroyed:
+ * 8 bytes per target and tile of 256 sources, at most 256 MB (8 bytes per target where
+ * those alone are more); an RK3 step with VRM_VEL_BIOT_SAVART holds the same.
+ * Asynchronous.
  */
 vrm_status vrm_biot_savart(vrm_ctx* ctx, const double* xs, const double* ys, const double* gamma, int32_t n,
                            const double* xt, const double* yt, int32_t m, double eps, double* u, double* v,

@@ -1624,9 +1624,9 @@ __global__ void __launch_bounds__(128) k_lp_full(Consts c, const double* __restr
 // pipes, about 15 operations per tableau entry and pivot and five for its
 // bound: 96% of the full LPs and 99.9% of the small ones are certified.
 // Bound by issue (66% of the slots, the integer pipe half busy with selects
-// and votes).  175,000 LPs of 251,001 particles: full 1.71 ms + 0.27 ms of
-// FP64 re-runs + 0.42 ms of final solves, 7.87 ms when a warp did pivots and
-// solve in FP64; small 0.78 + 0.03 + 0.41 ms, 1.15 ms with one FP64 LP per
+// and votes).  229,000 LPs of 251,001 particles: full 1.65 ms + 0.27 ms of
+// FP64 re-runs + 0.43 ms of final solves, 8.26 ms when a warp did pivots and
+// solve in FP64; small 0.73 + 0.03 + 0.08 ms, 1.22 ms with one FP64 LP per
 // thread (9 x 8 tableau, spilled).
 //
 // The bounds follow k_lp_small32 with u^2 = 2^-48 in place of u:
