@@ -485,8 +485,9 @@ typedef struct vrm_velocity {
  * tile sums in FP64: relative error about 1e-6 of sum_j |Gamma_j K_eps|.
  * O(n m) work (the fast multipole method of the paper is not part of this
  * library).  The context keeps the tile sums' workspace until it is destroyed:
- * 8 bytes per target and tile of 256 sources, at most 256 MB (8 bytes per target where
- * those alone are more); an RK3 step with VRM_VEL_BIOT_SAVART holds the same.
+ * 8 bytes per target and tile of 256 sources for the largest numbers of both so
+ * far, at most 256 MB (8 bytes per target where those alone are more); an RK3
+ * step with VRM_VEL_BIOT_SAVART holds the same for its capacity.
  * Asynchronous.
  */
 vrm_status vrm_biot_savart(vrm_ctx* ctx, const double* xs, const double* ys, const double* gamma, int32_t n,

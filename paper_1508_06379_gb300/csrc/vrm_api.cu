@@ -134,7 +134,6 @@ struct vrm_ctx {
   int bs_src_cap = 0, bs_tgt_cap = 0;
   float4 *bs_src = nullptr, *bs_tgt = nullptr;
   float* bs_g = nullptr;
-  size_t bs_part_cap = 0;
   float2* bs_part = nullptr;  // tile sums of the direct summation
   // particle removal (vrm_remove_close)
   int rm_cap = 0;
@@ -290,7 +289,6 @@ void free_bs(vrm_ctx* ctx) {
   if (ctx->bs_g) cudaFree(ctx->bs_g);
   if (ctx->bs_part) cudaFree(ctx->bs_part);
   ctx->bs_part = nullptr;
-  ctx->bs_part_cap = 0;
   ctx->bs_src = ctx->bs_tgt = nullptr;
   ctx->bs_g = nullptr;
   ctx->bs_src_cap = ctx->bs_tgt_cap = 0;
@@ -331,14 +329,15 @@ cudaError_t ensure_rm(vrm_ctx* ctx, int n, cudaStream_t st) {
 }
 
 // Buffers of the direct summation of n sources at m targets (grown, never
-// shrunk; the tile sums' workspace is bounded by bs_part_count).
+// shrunk).  The tile sums' workspace is sized for the largest numbers of both
+// (bs_part_count grows with either), so that a call within them allocates
+// nothing, whichever came together before.
 cudaError_t ensure_bs(vrm_ctx* ctx, int n, int m, cudaStream_t st) {
-  const size_t want = bs_part_count(n, m);
-  if (n <= ctx->bs_src_cap && m <= ctx->bs_tgt_cap && want <= ctx->bs_part_cap) return cudaSuccess;
+  if (n <= ctx->bs_src_cap && m <= ctx->bs_tgt_cap) return cudaSuccess;
   cudaStreamSynchronize(st);
   const int ns = n > ctx->bs_src_cap ? n : ctx->bs_src_cap;
   const int mt = m > ctx->bs_tgt_cap ? m : ctx->bs_tgt_cap;
-  const size_t np = want > ctx->bs_part_cap ? want : ctx->bs_part_cap;
+  const size_t np = bs_part_count(ns, mt);
   free_bs(ctx);
   cudaError_t e = cudaMalloc(&ctx->bs_src, sizeof(float4) * (size_t)(ns > 0 ? ns : 1));
   if (e == cudaSuccess) e = cudaMalloc(&ctx->bs_g, sizeof(float) * (size_t)(ns > 0 ? ns : 1));
@@ -351,7 +350,6 @@ cudaError_t ensure_bs(vrm_ctx* ctx, int n, int m, cudaStream_t st) {
   }
   ctx->bs_src_cap = ns;
   ctx->bs_tgt_cap = mt;
-  ctx->bs_part_cap = np;
   return cudaSuccess;
 }
 
