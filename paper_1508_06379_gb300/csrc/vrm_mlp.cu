@@ -274,6 +274,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFusedThreads, 1)
         umma::tma_load_2d_pair(ring + (size_t)st * kSlabBytes, wmap[layer], umma::lead_addr(&wfull[st]), kb * kBK,
                                rank * half);
       }
+      // Every commit arrives in this CTA before it ends: the leading CTA sees its
+      // own arrivals, not its peer's, so each waits for those it gets (here and
+      // beside the inputs; accf is waited for by the epilogues).  And every MMA
+      // issued completes before the TMEM is released.
+      for (int g = total < kRing ? 0 : total - kRing; g < total && !*abort_flag; ++g)
+        if (!umma::mbar_wait(&wempty[g % kRing], (uint32_t)(g / kRing) & 1u, 2 * kWaitCycles)) *abort_flag = 1;
+      if (!umma::mbar_wait(drain, 0u, 2 * kWaitCycles)) *abort_flag = 1;
     }
   } else if (warp == kEpiWarps + 2) {
     // ---- input tiles (one thread) ----
@@ -294,6 +301,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFusedThreads, 1)
         umma::tma_load_2d_pair(h, &tx, bar, 0, row0);
         umma::tma_load_2d_pair(h + kSlabBytes, &tx, bar, kBK, row0);
       }
+      for (int i = my_tiles < 2 ? 0 : my_tiles - 2; i < my_tiles && !*abort_flag; ++i)
+        if (!umma::mbar_wait(&hfree[i & 1], (uint32_t)(i / 2) & 1u, 2 * kWaitCycles)) *abort_flag = 1;
     }
   } else if (warp == kEpiWarps) {
     // ---- MMA issue (one thread of the pair) ----
@@ -419,22 +428,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFusedThreads, 1)
   }
   __syncwarp();
   umma::fence_before_sync();
-  __syncthreads();
-  // Every MMA issued completes before the TMEM is released, and every commit
-  // arrives in this CTA before it ends: the leading CTA sees its own arrivals,
-  // not its peer's, so each waits for those it gets.  (The producers have waited
-  // for all commits of a ring stage or slot but the last one, so its parity
-  // cannot be that of an earlier one; accf is waited for by the epilogues.)
-  if (threadIdx.x == 0) {
-    bool ok = umma::mbar_wait(drain, 0u, 2 * kWaitCycles);
-    if (ok && !*abort_flag) {
-      for (int st = 0; st < kRing && st < total; ++st)
-        ok = ok && umma::mbar_wait(&wempty[st], (uint32_t)((total - 1 - st) / kRing) & 1u, kWaitCycles);
-      for (int s = 0; s < 2 && s < my_tiles; ++s)
-        ok = ok && umma::mbar_wait(&hfree[s], (uint32_t)((my_tiles - 1 - s) / 2) & 1u, kWaitCycles);
-    }
-    if (!ok) *abort_flag = 1;
-  }
   __syncthreads();
   if (*abort_flag) {
     if (threadIdx.x == 0 && a.error) atomicExch(a.error, 1);
@@ -613,6 +606,10 @@ __global__ void __launch_bounds__(kChainThreads, 1)
           }
         }
       }
+      // the last commit of every ring stage lands before the CTA ends
+      for (int k = g < kChainRing ? 0 : g - kChainRing; k < g && !fail && !*abort_flag; ++k)
+        if (!umma::mbar_wait(&wempty[k % kChainRing], (uint32_t)(k / kChainRing) & 1u, 2 * kWaitCycles))
+          *abort_flag = 1;
     }
   } else if (warp == kEpiWarps) {
     // ---- inputs and MMA issue (one thread) ----
@@ -663,11 +660,7 @@ __global__ void __launch_bounds__(kChainThreads, 1)
       }
       if (fail) *abort_flag = 1;
       umma::mma_commit(drain);
-      bool ok = umma::mbar_wait(drain, 0u, kWaitCycles);
-      // and the last commit of every ring stage
-      for (int st = 0; st < kChainRing && st < g && !fail; ++st)
-        ok = ok && umma::mbar_wait(&wempty[st], (uint32_t)((g - 1 - st) / kChainRing) & 1u, kWaitCycles);
-      if (!ok) *abort_flag = 1;
+      if (!umma::mbar_wait(drain, 0u, kWaitCycles)) *abort_flag = 1;
     }
   } else {
     const int q = warp & 3, cg = warp >> 2;

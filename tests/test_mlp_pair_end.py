@@ -63,11 +63,15 @@ def run(my_tiles, rng, waits):
     for rank, c in enumerate(cta):
         end = t
         if waits == "all":
+            # the weights' thread, and beside it the inputs'
+            end = c["load"]
+            for k in range(max(total - RING, 0), total):
+                end = c["wempty"][k % RING].wait(end, (k // RING) & 1)
             end = c["drain"].wait(end, 0)
-            for st in range(min(RING, total)):
-                end = c["wempty"][st].wait(end, ((total - 1 - st) // RING) & 1)
-            for s in range(min(2, my_tiles)):
-                end = c["hfree"][s].wait(end, ((my_tiles - 1 - s) // 2) & 1)
+            tile = c["tile"]
+            for i in range(max(my_tiles - 2, 0), my_tiles):
+                tile = c["hfree"][i % 2].wait(tile, (i // 2) & 1)
+            end = max(end, tile)
         elif rank == 0:
             end = c["drain"].wait(end, 0)
         ends.append(end)
